@@ -135,19 +135,26 @@ WsLayout ws_layout(const kvp_handle* h, int64_t Bm, int64_t Tm) {
   w.attn = take(Tm * A.max_dq * es);
   w.gu = take(Tm * 2 * (size_t)A.max_ffn * es);
   w.act = take(Tm * (size_t)A.max_ffn * es);
+  const size_t step0 = off;
   w.xb = take(Bm * B.d * 4);
   w.hb = take(Bm * B.d * 4);
   w.qkvb = take(Bm * B.max_nqkv * 4);
   w.ab = take(Bm * B.max_dq * 4);
   w.actb = take(Bm * (size_t)B.max_ffn * 4);
-  w.part = take((size_t)(2 * 148 + Bm * B.max_nkv) * B.max_group * (B.L[0].hd + 2) * 4);
-  w.tok_stage = take(Tm * 4);
-  w.first_stage = take(Bm * 4);
   // tensor-core step projections: operand rows (hi + lo) of the widest input, fp32 gate/up outputs
   const int64_t Bp = step_tc_rows((int)Bm);
   const int64_t k_max = std::max((int64_t)B.d, std::max((int64_t)B.max_dq, (int64_t)B.max_ffn));
   w.xbt = take(2 * Bp * k_max * 2);
   w.gub = take(Bm * 2 * (size_t)B.max_ffn * 4);
+  // The persistent kernel of small batches uses none of the seven buffers above: its tagged values (64 bits each) take
+  // their place, at the end, so that they and its split partials in w.part are cleared as one range.
+  const size_t Bq = (size_t)std::min<int64_t>(Bm, 4);
+  const size_t ll = h->opt.dtype == KVP_BF16 ? Bq * ((size_t)B.max_nqkv + B.max_dq + 2 * (size_t)B.d + B.max_ffn) * 8 + 5 * 256 : 0;
+  off = std::max(off, align_up(step0 + ll, 256));
+  w.ll = off - align_up(ll, 256);
+  w.part = take((size_t)(2 * std::max(148, h->n_sm) + Bm * B.max_nkv) * B.max_group * (B.L[0].hd + 2) * 4);
+  w.tok_stage = take(Tm * 4);
+  w.first_stage = take(Bm * 4);
   w.attn_sched = take((size_t)(Tm / 128 + Bm + 1) * 8);
   w.attn_done = take((size_t)Bm * B.max_nkv * 4);
   // fused RMSNorm: per auxiliary layer two vectors of row sums of squares (one memset clears all)
@@ -284,6 +291,16 @@ void base_layer_step(kvp_handle* h, const LaunchCtx& ctx, int i, const kvp_cache
   KVP_TIMED(KVP_CLASS_STEP_GEMV, launch_step_gemv(ctx, P + L.wd, L.ffn, B.d, L.ffn, actb, L.ffn, batch, xb, B.d, GEMV_RESID, 0, 0));
 }
 
+// Which persistent step kernel a call takes: with 16-bit weights and head_dim 64 / 128 the one that multiplies on the
+// warp-level tensor cores, in fp32 mode and for other head widths the one on the CUDA cores.
+bool mega_uses_mma(const kvp_handle* h, int batch) {
+  return h->opt.dtype == KVP_BF16 && step_mega_mma_supported(batch, h->base.L[0].hd, h->base.max_group, h->base.d, h->step_sms > 0 ? h->step_sms : h->n_sm);
+}
+cudaError_t launch_mega(kvp_handle* h, const MegaParams& p, int k_max, int n_sm, cudaStream_t st) {
+  return mega_uses_mma(h, p.batch) ? launch_step_mega_mma(p, h->base.max_group, n_sm, st, &h->n_launch)
+                                   : launch_step_mega(p, h->opt.dtype, k_max, n_sm, st, &h->n_launch);
+}
+
 // Parameters of the persistent step kernel for this call; false = the kernel does not apply.
 bool mega_prepare(kvp_handle* h, const LaunchCtx& ctx, const kvp_cache* cache, const WsLayout& w, char* ws, int batch,
                   int max_keys, bool generation, const int* tokens, const int* gather_idx, float* logits,
@@ -293,7 +310,8 @@ bool mega_prepare(kvp_handle* h, const LaunchCtx& ctx, const kvp_cache* cache, c
   // its attention phase reads cache pages with plain loads: fine for a few thousand keys, several times
   // slower than the ring-fed kernel beyond that
   if (max_keys > 4096) return false;
-  if (B.n_layers > MEGA_MAX_LAYERS || !step_mega_supported(batch, B.L[0].hd, k_max, B.max_group, h->es)) return false;
+  if (B.n_layers > MEGA_MAX_LAYERS) return false;
+  if (!mega_uses_mma(h, batch) && !step_mega_supported(batch, B.L[0].hd, k_max, B.max_group, h->es)) return false;
   // bulk copies need 16-byte rows: every projection's row length must be a multiple of 16 bytes
   for (int i = 0; i < B.n_layers; ++i)
     if ((B.d * h->es) % 16 || (B.L[i].dq * h->es) % 16 || (B.L[i].ffn * h->es) % 16) return false;
@@ -315,6 +333,12 @@ bool mega_prepare(kvp_handle* h, const LaunchCtx& ctx, const kvp_cache* cache, c
 #else
   p.trace = nullptr;
 #endif
+  {
+    size_t at = w.ll;
+    auto ll = [&](size_t n) { unsigned long long* q = (unsigned long long*)(ws + at); at = align_up(at + (size_t)batch * n * 8, 256); return q; };
+    p.ll_q = ll(B.max_nqkv); p.ll_a = ll(B.max_dq); p.ll_x1 = ll(B.d); p.ll_x2 = ll(B.d); p.ll_h = ll(B.max_ffn);
+    p.ll_part = (unsigned long long*)(ws + w.part);
+  }
   int min_nkv = B.L[0].nkv;
   for (int i = 0; i < B.n_layers; ++i) {
     const LayerPlan& L = B.L[i];
@@ -333,6 +357,16 @@ bool mega_prepare(kvp_handle* h, const LaunchCtx& ctx, const kvp_cache* cache, c
   return true;
 }
 
+// What has to be zero in the workspace before the first launch of a step: the tagged values of the tensor-core kernel (with
+// its split partials behind them), or the split counters of the other one.
+void mega_clear(kvp_handle* h, const MegaParams& p, const WsLayout& w, char* ws, cudaStream_t st) {
+  const ModelPlan& B = h->base;
+  if (mega_uses_mma(h, p.batch))
+    cudaMemsetAsync(ws + w.ll, 0, w.part - w.ll + (size_t)h->n_sm * B.max_group * (B.L[0].hd + 2) * 8, st);
+  else
+    cudaMemsetAsync(p.attn_done, 0, (size_t)p.batch * B.max_nkv * 4, st);
+}
+
 // The whole base step (all layers, LM head, argmax) as one persistent kernel; false = not applicable.
 // The caller has cleared the first MEGA_STATUS_BYTES of the status block (or at least its counters).
 bool base_step_fused(kvp_handle* h, const LaunchCtx& ctx, const kvp_cache* cache, const WsLayout& w, char* ws, int batch,
@@ -341,9 +375,9 @@ bool base_step_fused(kvp_handle* h, const LaunchCtx& ctx, const kvp_cache* cache
   MegaParams p;
   int k_max = 0;
   if (!mega_prepare(h, ctx, cache, w, ws, batch, max_keys, generation, tokens, gather_idx, logits, token_out, &p, &k_max)) return false;
-  cudaMemsetAsync(p.attn_done, 0, (size_t)batch * h->base.max_nkv * 4, ctx.st);
+  mega_clear(h, p, w, ws, ctx.st);
   TimedScope ts(h, ctx.st, KVP_CLASS_STEP_FUSED);
-  cudaError_t e = launch_step_mega(p, h->opt.dtype, k_max, h->n_sm, ctx.st, ctx.n_launch);
+  cudaError_t e = launch_mega(h, p, k_max, h->n_sm, ctx.st);
   if (e != cudaSuccess && *err == cudaSuccess) *err = e;
   return true;
 }
@@ -660,7 +694,7 @@ static kvp_status prefill_direct(kvp_handle* h, const int32_t* tokens, const int
       while (i < h->base.n_layers && std::max(dep, h->map[i]) <= j) { dep = std::max(dep, h->map[i]); ++i; }
       ready_after[j] = i;
     }
-    cudaMemsetAsync(mp.attn_done, 0, (size_t)batch * h->base.max_nkv * 4, s);
+    mega_clear(h, mp, w, ws, s);
     h->gemm_sms = h->n_sm - h->step_sms;
     // key-range splits of the pieces: one attention item per CTA of the piece (measured: 2.72 against 2.83 ms at C2
     // with the 16 splits chosen for the whole GPU, which make two rounds on 72 SMs)
@@ -792,7 +826,7 @@ static kvp_status prefill_direct(kvp_handle* h, const int32_t* tokens, const int
         q.do_embed = base_done == 0; q.do_head = last; q.counter_idx = piece++;
         q.n_split = piece_split;
         // the last piece starts when the prefill has nothing left to run: it takes every SM
-        cudaError_t e = launch_step_mega(q, h->opt.dtype, mega_kmax, last ? h->n_sm : h->step_sms, h->step_st, ctx.n_launch);
+        cudaError_t e = launch_mega(h, q, mega_kmax, last ? h->n_sm : h->step_sms, h->step_st);
         if (e != cudaSuccess && tc_err == cudaSuccess) tc_err = e;
         base_done = q.layer_end;
       }
@@ -989,7 +1023,7 @@ kvp_status kvp_decode_step(kvp_handle* h, const int32_t* tokens, const int32_t* 
   char* ws = (char*)workspace;
   LaunchCtx ctx{(cudaStream_t)stream, &h->n_launch, (int*)(ws + w.status), h->opt.dtype};
   cudaError_t mega_err = cudaSuccess;
-  cudaMemsetAsync((char*)(ws + w.status) + 128, 0, MEGA_COUNTERS * 4, ctx.st);     // barrier counters of the persistent kernel
+  cudaMemsetAsync(ws + w.status + 64, 0, MEGA_STATUS_BYTES - 64, ctx.st);     // argmax slots and counters of the persistent kernel
   if (base_step_fused(h, ctx, cache, w, ws, batch, cs.max_len + 1, true, tokens, nullptr, logits_out, next_token, &mega_err)) {
     if (mega_err != cudaSuccess) return fail(h, KVP_ERR_CUDA, "base step launch: %s", cudaGetErrorString(mega_err));
     return check_cuda(h, "kvp_decode_step");

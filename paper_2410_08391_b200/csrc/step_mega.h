@@ -23,6 +23,9 @@ struct MegaParams {
   const int* block_table; int mpps, n_pages;
   int* seq_lens;
   float *xb, *qkvb, *ab, *actb, *part;           // workspace: residual, projections, attention out, FFN act, partials
+  // step_mega_mma_kernel: {value, tag} words instead of the buffers above (cleared before a step): q(kv) rows, attention out,
+  // residual after attention / after the FFN, FFN act, split partials
+  unsigned long long *ll_q, *ll_a, *ll_x1, *ll_x2, *ll_h, *ll_part;
   int* attn_done;                                // [batch * max n_kv] splits finished per (sequence, kv head); zero on entry, left zero
   float* logits; int* token_out;
   // One launch may cover only base layers [layer_begin, layer_end): the residual stream stays in xb between
@@ -37,3 +40,7 @@ struct MegaParams {
 
 bool step_mega_supported(int batch, int hd, int k_max, int max_group, int es);
 cudaError_t launch_step_mega(MegaParams p, int dtype, int k_max, int n_sm, cudaStream_t st, int64_t* n_launch);
+
+// The same step on the warp-level tensor cores (16-bit weights, head_dim 64 / 128): step_mega_mma.cu.
+bool step_mega_mma_supported(int batch, int hd, int max_group, int d, int n_sm);
+cudaError_t launch_step_mega_mma(MegaParams p, int max_group, int n_sm, cudaStream_t st, int64_t* n_launch);
