@@ -339,7 +339,6 @@ bool mega_prepare(kvp_handle* h, const LaunchCtx& ctx, const kvp_cache* cache, c
     p.ll_q = ll(B.max_nqkv); p.ll_a = ll(B.max_dq); p.ll_x1 = ll(B.d); p.ll_x2 = ll(B.d); p.ll_h = ll(B.max_ffn);
     p.ll_part = (unsigned long long*)(ws + w.part);
   }
-  int min_nkv = B.L[0].nkv;
   for (int i = 0; i < B.n_layers; ++i) {
     const LayerPlan& L = B.L[i];
     MegaLayer& m = p.layers[i];
@@ -349,9 +348,10 @@ bool mega_prepare(kvp_handle* h, const LaunchCtx& ctx, const kvp_cache* cache, c
     m.k_norm = B.qk_norm ? (const float*)(P + L.k_norm) : nullptr;
     m.kpool = cache->k_pools[i]; m.vpool = cache->v_pools[i];
     m.nq = L.nq; m.nkv = L.nkv; m.dq = L.dq; m.nqkv = L.nqkv; m.ffn = L.ffn; m.G = L.G;
-    min_nkv = std::min(min_nkv, L.nkv);
+    // From the layer's own kv heads: w.part holds the partial results of 2 CTAs per SM and one more split per (sequence, kv
+    // head), which the split count of a layer with fewer kv heads would exceed.
+    m.n_split = step_attn_splits(batch, L.nkv, max_keys);
   }
-  p.n_split = step_attn_splits(batch, min_nkv, max_keys);   // sized for the layer with the fewest kv heads
   p.layer_begin = 0; p.layer_end = B.n_layers; p.do_embed = 1; p.do_head = 1; p.counter_idx = 0;
   *k_max_out = k_max;
   return true;
@@ -684,7 +684,7 @@ static kvp_status prefill_direct(kvp_handle* h, const int32_t* tokens, const int
   // The base step in pieces beside the prefill: piece j = the base layers whose cache (and that of every
   // layer below them) is complete once auxiliary layer j has gone through the predictor.
   MegaParams mp;
-  int mega_kmax = 0, piece = 0, base_done = 0, piece_split = 1;
+  int mega_kmax = 0, piece = 0, base_done = 0;
   bool piped = fork && h->step_sms > 0 && h->j_max + 1 <= MEGA_COUNTERS &&
                mega_prepare(h, ctx, cache, w, ws, batch, cs.max_len, false, tokens, last_idx, logits_out, first_token, &mp, &mega_kmax);
   std::vector<int> ready_after(h->j_max + 2, 0);      // ready_after[j] = base layers runnable after auxiliary layer j
@@ -696,11 +696,9 @@ static kvp_status prefill_direct(kvp_handle* h, const int32_t* tokens, const int
     }
     mega_clear(h, mp, w, ws, s);
     h->gemm_sms = h->n_sm - h->step_sms;
-    // key-range splits of the pieces: one attention item per CTA of the piece (measured: 2.72 against 2.83 ms at C2
-    // with the 16 splits chosen for the whole GPU, which make two rounds on 72 SMs)
-    int min_nkv = h->base.L[0].nkv;
-    for (int i = 0; i < h->base.n_layers; ++i) min_nkv = std::min(min_nkv, h->base.L[i].nkv);
-    piece_split = std::max(1, std::min(mp.n_split, h->step_sms / (batch * min_nkv)));
+    // key-range splits of the pieces: one attention item per CTA of the piece (more make two rounds)
+    for (int i = 0; i < h->base.n_layers; ++i)
+      mp.layers[i].n_split = std::max(1, std::min(mp.layers[i].n_split, h->step_sms / (batch * h->base.L[i].nkv)));
   }
   // More than 4 sequences: the step is a chain of short per-layer kernels bound by launch latency; the same
   // pieces go to the step stream as plain launches.  Their projections size their grids for step_tc_sms SMs;
@@ -824,7 +822,6 @@ static kvp_status prefill_direct(kvp_handle* h, const int32_t* tokens, const int
         MegaParams q = mp;
         q.layer_begin = base_done; q.layer_end = last ? h->base.n_layers : ready_after[j];
         q.do_embed = base_done == 0; q.do_head = last; q.counter_idx = piece++;
-        q.n_split = piece_split;
         // the last piece starts when the prefill has nothing left to run: it takes every SM
         cudaError_t e = launch_mega(h, q, mega_kmax, last ? h->n_sm : h->step_sms, h->step_st);
         if (e != cudaSuccess && tc_err == cudaSuccess) tc_err = e;

@@ -518,17 +518,17 @@ __global__ void __launch_bounds__(NT, 1) step_mega_kernel(const __grid_constant_
     // (sequence, kv head) merges that group's partial results on the spot (a counter per group tells
     // it so), which saves a separate merge phase and its grid barrier.
     {
-      const int n_items = batch * L.nkv * p.n_split;
+      const int n_split = L.n_split, n_items = batch * L.nkv * n_split;
       const int group = L.nq / L.nkv, ldr = p.hd + 2;
       for (int it = blockIdx.x; it < n_items; it += gridDim.x) {
-        const int sp = it % p.n_split, r = it / p.n_split;
-        attn_item<T>(p, L, r / L.nkv, r % L.nkv, sp, p.n_split, p.qkvb, n_out, sm_raw, p.part, p.ab);
-        if (p.n_split > 1) {
+        const int sp = it % n_split, r = it / n_split;
+        attn_item<T>(p, L, r / L.nkv, r % L.nkv, sp, n_split, p.qkvb, n_out, sm_raw, p.part, p.ab);
+        if (n_split > 1) {
           __threadfence();                       // this CTA's partial results are visible before it counts itself done
           __syncthreads();
           if (tid == 0) {
             const int before = atomicAdd(p.attn_done + r, 1);
-            s_last = before == p.n_split - 1;
+            s_last = before == n_split - 1;
             if (s_last) atomicExch(p.attn_done + r, 0);      // ready for the next layer
           }
           __syncthreads();
@@ -536,14 +536,14 @@ __global__ void __launch_bounds__(NT, 1) step_mega_kernel(const __grid_constant_
             __threadfence();
             if (warp < group) {                  // one warp per q head of the group
               const int head = (r / L.nkv) * L.nq + (r % L.nkv) * group + warp;
-              const float* pr = p.part + (size_t)head * p.n_split * ldr;
+              const float* pr = p.part + (size_t)head * n_split * ldr;
               float mm = -INFINITY;
-              for (int s = lane; s < p.n_split; s += 32) mm = fmaxf(mm, __ldcg(pr + (size_t)s * ldr + p.hd));
+              for (int s = lane; s < n_split; s += 32) mm = fmaxf(mm, __ldcg(pr + (size_t)s * ldr + p.hd));
               mm = warp_max(mm);
               // the loads of different splits do not depend on one another: unrolled, they are in flight together
               float ll = 0.f, o0 = 0.f, o1 = 0.f, o2 = 0.f, o3 = 0.f;
 #pragma unroll 8
-              for (int s = 0; s < p.n_split; ++s) {
+              for (int s = 0; s < n_split; ++s) {
                 const float* rr = pr + (size_t)s * ldr;
                 const float ms = __ldcg(rr + p.hd);
                 const float f = (ms == -INFINITY) ? 0.f : __expf(ms - mm);

@@ -12,10 +12,11 @@ struct MegaLayer {
   const float *q_norm, *k_norm;          // query / key norm gains [hd], or null
   void *kpool, *vpool;                   // cache pools of the layer
   int nq, nkv, dq, nqkv, ffn, G;
+  int n_split;                           // step_mega_kernel: key-range splits of this layer's attention
 };
 
 struct MegaParams {
-  int n_layers, d, vocab, hd, batch, generation, n_split;
+  int n_layers, d, vocab, hd, batch, generation;
   float eps;
   InvFreq inv;
   const int* tokens; const int* gather_idx;      // token of row b = tokens[gather_idx ? gather_idx[b] : b]
