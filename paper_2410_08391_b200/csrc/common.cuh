@@ -58,6 +58,24 @@ inline cudaError_t launch_overlapped(void (*kernel)(KArgs...), dim3 grid, dim3 b
   return cudaLaunchKernelEx(&cfg, kernel, static_cast<KArgs>(args)...);
 }
 
+// Host side.  A kernel's dynamic shared-memory limit is an attribute that all threads of the process share: it is raised once per
+// device, to the most that any launch of the kernel takes.  (Set to each launch's own size, a second thread could lower it
+// between another's setting and launch.)
+constexpr int TC_MAX_DEVICES = 64;
+template <class K>
+inline cudaError_t tc_raise_smem_limit(K kernel, int bytes, bool (&done)[TC_MAX_DEVICES]) {
+  int dev = 0;
+  cudaError_t e = cudaGetDevice(&dev);
+  if (e != cudaSuccess) return e;
+  if (dev < 0 || dev >= TC_MAX_DEVICES) return cudaErrorInvalidDevice;
+  if (!done[dev]) {
+    e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, bytes);
+    if (e != cudaSuccess) return e;
+    done[dev] = true;
+  }
+  return cudaSuccess;
+}
+
 __device__ __forceinline__ float warp_sum(float v) {
 #pragma unroll
   for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);

@@ -96,6 +96,7 @@ void launch_gemm_simt(const LaunchCtx& ctx, const GemmArgs& g, int epi) {
 // ---------------------------------------------------------------------------------------
 namespace {
 constexpr int AQ = 8, AKV = 64;
+constexpr int ATTN_SMEM_MAX = (2 * AKV * 129 + AQ * 128) * 4;      // head_dim 128, the widest
 
 template <class T>
 __global__ void __launch_bounds__(256) attn_prefill_simt_kernel(const T* __restrict__ qkv, int ld, int nq, int nkv, int hd,
@@ -190,10 +191,12 @@ void launch_attn_prefill_simt(const LaunchCtx& ctx, const void* qkv, int ld, int
   float scale = 1.f / sqrtf((float)hd);
   ++*ctx.n_launch;
   if (ctx.dtype == 0) {
-    cudaFuncSetAttribute(attn_prefill_simt_kernel<float>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    static bool raised[TC_MAX_DEVICES] = {};
+    tc_raise_smem_limit(attn_prefill_simt_kernel<float>, ATTN_SMEM_MAX, raised);
     attn_prefill_simt_kernel<float><<<grid, 256, smem, ctx.st>>>((const float*)qkv, ld, nq, nkv, hd, cu_dev, batch, (float*)out, ldo, scale);
   } else {
-    cudaFuncSetAttribute(attn_prefill_simt_kernel<bf16>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    static bool raised[TC_MAX_DEVICES] = {};
+    tc_raise_smem_limit(attn_prefill_simt_kernel<bf16>, ATTN_SMEM_MAX, raised);
     attn_prefill_simt_kernel<bf16><<<grid, 256, smem, ctx.st>>>((const bf16*)qkv, ld, nq, nkv, hd, cu_dev, batch, (bf16*)out, ldo, scale);
   }
 }

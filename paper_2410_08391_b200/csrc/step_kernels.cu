@@ -199,6 +199,8 @@ __global__ void __launch_bounds__(256) step_gemv_smem_kernel(const T* __restrict
   }
 }
 
+constexpr int GEMV_SMEM_MAX = 96 * 1024;      // activation rows in shared memory, at most
+
 template <class T, int BB, bool NORM>
 void gemv_smem_go(const LaunchCtx& ctx, const void* W, int ldw, int N, int K, const float* x, int ldx, const float* gain,
                   float eps, float* y, int ldy, int mode, int G, int ffn) {
@@ -209,8 +211,8 @@ void gemv_smem_go(const LaunchCtx& ctx, const void* W, int ldw, int N, int K, co
   RowMap mg{0, G, 0, ffn}, mu{G == 0 ? ffn : 0, G, 1, ffn};
 #define GO(MODE)                                                                                                        \
   do {                                                                                                                  \
-    if (smem > 48 * 1024)                                                                                               \
-      cudaFuncSetAttribute(step_gemv_smem_kernel<T, BB, MODE, NORM>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem); \
+    static bool raised[TC_MAX_DEVICES] = {};                                                                            \
+    if (smem > 48 * 1024) tc_raise_smem_limit(step_gemv_smem_kernel<T, BB, MODE, NORM>, GEMV_SMEM_MAX, raised);         \
     step_gemv_smem_kernel<T, BB, MODE, NORM><<<grid, 256, smem, ctx.st>>>((const T*)W, ldw, N, K, x, ldx, gain, eps, y, ldy, mg, mu, rows); \
   } while (0)
   if (mode == GEMV_STORE) GO(GEMV_STORE); else if (mode == GEMV_RESID) GO(GEMV_RESID); else GO(GEMV_SWIGLU);
@@ -235,7 +237,7 @@ void gemv_smem_dispatch(const LaunchCtx& ctx, const void* W, int ldw, int N, int
 void launch_step_gemv(const LaunchCtx& ctx, const void* W, int ldw, int N, int K, const float* x, int ldx, int batch,
                       float* y, int ldy, int mode, int G, int ffn, const float* gain, float eps, float* scratch_h) {
   if (batch == 0 || N == 0) return;
-  const bool smem_path = batch <= 4 && (batch == 3 ? 4 : batch) * (size_t)K * 4 <= 96 * 1024 && K % 8 == 0 && ldw % 8 == 0 &&
+  const bool smem_path = batch <= 4 && (batch == 3 ? 4 : batch) * (size_t)K * 4 <= GEMV_SMEM_MAX && K % 8 == 0 && ldw % 8 == 0 &&
                          ldx % 4 == 0;
   if (smem_path) {
     // a batch of 3 runs the 4-row kernel on a zero-extended view: handled by clamping rows inside via batch==4 only
@@ -633,7 +635,9 @@ void launch_step_attn(const LaunchCtx& ctx, const float* q, int ldq, int nq, int
     int es = ctx.dtype == 0 ? 4 : 2;
     size_t smem = (size_t)2 * PAGE_TOKENS * (hd * es + 16) + (size_t)(MAXG * hd + MAXG * PAGE_TOKENS + 3 * MAXG) * sizeof(float);
     if (ctx.dtype == 0) {
-      cudaFuncSetAttribute(step_attn_paged_kernel<float>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+      constexpr int smem_max = 2 * PAGE_TOKENS * (128 * 4 + 16) + (MAXG * 128 + MAXG * PAGE_TOKENS + 3 * MAXG) * 4;   // head_dim 128
+      static bool raised[TC_MAX_DEVICES] = {};
+      tc_raise_smem_limit(step_attn_paged_kernel<float>, smem_max, raised);
       step_attn_paged_kernel<float><<<grid, 128, smem, ctx.st>>>(q, ldq, nq, nkv, hd, inv, (const float*)kpool, (const float*)vpool,
                                                                  block_table, mpps, n_pages, seq_lens, extra, n_split, part, out, ctx.status, q_gain, eps);
     } else {

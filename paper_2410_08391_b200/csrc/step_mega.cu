@@ -607,7 +607,8 @@ size_t stage_region_bytes(int batch, int hd, int k_max, int es) {
 template <class T, int BB>
 cudaError_t go(MegaParams& p, size_t smem, cudaStream_t st, int n_sm) {
   auto kern = step_mega_kernel<T, BB>;
-  cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+  static bool raised[TC_MAX_DEVICES] = {};
+  cudaError_t e = tc_raise_smem_limit(kern, SMEM_LIMIT, raised);
   if (e != cudaSuccess) return e;
   int per_sm = 0;
   e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kern, NT, smem);

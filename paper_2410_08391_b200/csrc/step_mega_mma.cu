@@ -933,6 +933,8 @@ __global__ void __launch_bounds__(NT, 1) step_mega_mma_kernel(const __grid_const
   }
 }
 
+constexpr size_t SMEM_ROOM = SMEM_LIMIT - sizeof(Shared) - 256;      // dynamic shared memory of a CTA
+
 // Shared-memory plan: scratch and page slots first, the weight ring takes what is left (at least 3 slots).
 bool make_plan(int batch, int hd, int max_group, Plan* pl, size_t* bytes) {
   const int bb = batch <= 1 ? 1 : (batch == 2 ? 2 : 4);
@@ -940,11 +942,10 @@ bool make_plan(int batch, int hd, int max_group, Plan* pl, size_t* bytes) {
   const size_t attn = (size_t)((max_group <= 4 ? 4 : MAXG) + CW * max_group) * hd * 4 + (size_t)2 * CW * max_group * 4;
   const size_t scr = (proj + attn + 127) / 128 * 128;
   const int STAGE = bb == 4 ? Geo<4>::STAGE : Geo<1>::STAGE;
-  const size_t room = SMEM_LIMIT - sizeof(Shared) - 256;
   for (int n_kv = 2; n_kv >= 1; --n_kv) {
     const size_t kv = (size_t)n_kv * 2 * PAGE_TOKENS * hd * 2;
-    if (scr + kv + 3 * (size_t)STAGE > room) continue;
-    int n = (int)((room - scr - kv) / STAGE);
+    if (scr + kv + 3 * (size_t)STAGE > SMEM_ROOM) continue;
+    int n = (int)((SMEM_ROOM - scr - kv) / STAGE);
     if (n > MAX_SLOTS) n = MAX_SLOTS;
     pl->n_stage = n; pl->n_kv = n_kv; pl->kv_off = n * STAGE; pl->scr_off = pl->kv_off + (int)kv;
     *bytes = (size_t)pl->scr_off + scr;
@@ -956,7 +957,8 @@ bool make_plan(int batch, int hd, int max_group, Plan* pl, size_t* bytes) {
 template <int BB, int HD, int GQ>
 cudaError_t go(MegaParams& p, Plan& pl, size_t smem, cudaStream_t st, int n_sm) {
   auto kern = step_mega_mma_kernel<BB, HD, GQ>;
-  cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+  static bool raised[TC_MAX_DEVICES] = {};
+  cudaError_t e = tc_raise_smem_limit(kern, SMEM_ROOM, raised);
   if (e != cudaSuccess) return e;
   void* args[] = {(void*)&p, (void*)&pl};
   return cudaLaunchCooperativeKernel((const void*)kern, dim3(n_sm), dim3(NT), args, smem, st);

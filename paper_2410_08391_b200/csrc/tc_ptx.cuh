@@ -158,22 +158,6 @@ __device__ __forceinline__ uint64_t desc_kmajor(uint32_t smem_addr) {
 
 }  // namespace tcp
 
-// Host side.  A kernel's dynamic shared-memory limit is a per-device attribute: raise it once per device.
-constexpr int TC_MAX_DEVICES = 64;
-template <class K>
-inline cudaError_t tc_raise_smem_limit(K kernel, int bytes, bool (&done)[TC_MAX_DEVICES]) {
-  int dev = 0;
-  cudaError_t e = cudaGetDevice(&dev);
-  if (e != cudaSuccess) return e;
-  if (dev < 0 || dev >= TC_MAX_DEVICES) return cudaErrorInvalidDevice;
-  if (!done[dev]) {
-    e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, bytes);
-    if (e != cudaSuccess) return e;
-    done[dev] = true;
-  }
-  return cudaSuccess;
-}
-
 // The driver's tensor-map encoder, resolved once through the runtime.
 inline PFN_cuTensorMapEncodeTiled_v12000 tc_encode_fn() {
   static PFN_cuTensorMapEncodeTiled_v12000 fn = nullptr;
