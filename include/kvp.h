@@ -281,8 +281,8 @@ kvp_status kvp_train_forward(kvp_handle* h, const int32_t* tokens /* dev [sum(le
 kvp_status kvp_poll_status(kvp_handle* h, void* workspace, void* stream);
 
 /* Self-test of the error path behind KVP_ERR_TIMEOUT (the paper has no counterpart).  Enqueues a one-block
- * kernel that waits, with the same bounded wait every kernel of the library uses but a limit of a few thousand
- * polls, on a barrier that nothing completes.  The wait runs out, the kernel returns normally and records its code
+ * kernel that waits, with the library's own bounded waits but a 64th of their limits, for what never comes
+ * (a few hundredths of a second).  The waits run out, the kernel returns normally and records its code
  * in the status word of `workspace` (dev, >= 16 bytes, as passed to the compute calls; the three words behind the status
  * word receive the outcomes of the step kernel's own waits); kvp_poll_status then
  * returns KVP_ERR_TIMEOUT and clears the word, and the handle and the context stay usable. */

@@ -1,31 +1,38 @@
-// Self-test of the bounded device-side waits: a one-block kernel waits on a barrier that nothing will ever complete, with a
-// limit of a few thousand polls.  The wait must run out, the kernel must return, and the status word must read DEV_TIMEOUT,
-// which kvp_poll_status reports as KVP_ERR_TIMEOUT.  A further warp plays a loader of the barrier-free step kernel whose slot is
-// free but whose consumers have given up: its wait must say so (word 3 of the status block then reads 1).
+// Self-test of the bounded device-side waits: a one-block kernel waits, with a 64th of each kind's limit, for what never comes.
+// Every wait must run out, the kernel must return, and the status word must read DEV_TIMEOUT, which kvp_poll_status reports as
+// KVP_ERR_TIMEOUT.  The kinds: the mbarrier wait of most kernels (status word), the tagged value (word 1) and the sleeping loader
+// (word 2) of the barrier-free step kernel.  A last warp plays such a loader whose slot is free but whose consumers have given
+// up: its wait must say so (word 3 then reads 1).
 #include "kvp_internal.h"
 #include "step_waits.cuh"
 
 namespace {
 using namespace tcp;
 
-__global__ void __launch_bounds__(96) wait_timeout_kernel(int* status, uint32_t limit) {
+__global__ void __launch_bounds__(160) wait_timeout_kernel(int* status) {
   __shared__ __align__(8) unsigned long long bar, free_bar;
-  __shared__ int abort_mem, given_up;
+  __shared__ int abort_mem, given_up, abort_tag, abort_lazy;
   volatile int* abort_flag = &abort_mem;
   if (threadIdx.x == 0) {
     mbar_init(smem_u32(&bar), 1);
     mbar_init(smem_u32(&free_bar), 1);
     *abort_flag = 0;
     given_up = 1;
+    abort_tag = abort_lazy = 0;
     status[1] = status[2] = status[3] = 0;
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
   }
   __syncthreads();
   // thread 0 plays a consumer whose producer never arrives; thread 32 a second role that watches the abort flag
-  if (threadIdx.x == 0 || threadIdx.x == 32) mbar_wait(smem_u32(&bar), 0, abort_flag, status, limit);
-  if (threadIdx.x >= 64) {       // phase "minus one" of a fresh barrier counts as complete: a loader's first wait
+  if (threadIdx.x == 0 || threadIdx.x == 32) mbar_wait(smem_u32(&bar), 0, abort_flag, status, TRY_WAIT_LIMIT / 64);
+  if (threadIdx.x == 64) {       // a value whose tag never arrives: the tag would be the upper half of the first two words
+    bool dead = false;
+    ll_wait(reinterpret_cast<const u64*>(status), 0xffffffffu, dead, &abort_tag, status + 1, L2_POLL_LIMIT / 64);
+  }
+  if (threadIdx.x >= 96 && threadIdx.x < 128) lazy_wait(smem_u32(&bar), 0, &abort_lazy, status + 2, LAZY_LIMIT / 64);
+  if (threadIdx.x >= 128) {       // phase "minus one" of a fresh barrier counts as complete: a loader's first wait
     const bool go = lazy_wait(smem_u32(&free_bar), 1, &given_up, status + 2);
-    if (threadIdx.x == 64) status[3] = go ? 2 : 1;
+    if (threadIdx.x == 128) status[3] = go ? 2 : 1;
   }
   __syncthreads();
 }
@@ -41,7 +48,7 @@ extern "C" kvp_status kvp_selftest_wait_timeout(kvp_handle* h, void* workspace, 
     return KVP_ERR_INVALID_ARG;
   }
   ++h->n_launch;
-  wait_timeout_kernel<<<1, 96, 0, (cudaStream_t)stream>>>((int*)workspace, 4096u);
+  wait_timeout_kernel<<<1, 160, 0, (cudaStream_t)stream>>>((int*)workspace);
   cudaError_t e = cudaGetLastError();
   if (e != cudaSuccess) {
     h->err = std::string("kvp_selftest_wait_timeout: ") + cudaGetErrorString(e);

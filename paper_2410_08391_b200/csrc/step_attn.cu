@@ -122,7 +122,7 @@ __global__ void __launch_bounds__(512) step_attn_ring_wide_kernel(const float* _
     {
       const uint32_t bar = smem_u32(&bars[it % ST]), parity = (it / ST) & 1;
       bool got = false;
-      for (uint32_t spin = 0; spin < SPIN_LIMIT; ++spin) {
+      for (uint32_t spin = 0; spin < TRY_WAIT_LIMIT; ++spin) {
         if (mbar_test(bar, parity)) { got = true; break; }
         if ((spin & 1023u) == 1023u && *(volatile int*)&s_ok == 0) break;
       }
@@ -357,7 +357,7 @@ step_attn_ring_kernel(const float* __restrict__ q, int ldq, int nq, int nkv, con
     {                                             // wait for this page's copies (every thread polls; bounded)
       const uint32_t bar = smem_u32(&bars[it % STG]), parity = (it / STG) & 1;
       bool got = false;
-      for (uint32_t spin = 0; spin < SPIN_LIMIT; ++spin) {
+      for (uint32_t spin = 0; spin < TRY_WAIT_LIMIT; ++spin) {
         if (mbar_test(bar, parity)) { got = true; break; }
         if ((spin & 1023u) == 1023u && *(volatile int*)&s_ok == 0) break;
       }

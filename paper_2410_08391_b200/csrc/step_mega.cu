@@ -41,7 +41,7 @@ __device__ __forceinline__ bool grid_barrier(unsigned* counter, unsigned target,
       unsigned v;
       asm volatile("ld.acquire.gpu.global.u32 %0, [%1];" : "=r"(v) : "l"(counter) : "memory");
       if (v >= target) break;
-      if (++it > SPIN_LIMIT) { dev_flag(status, DEV_TIMEOUT); ok = 0; break; }
+      if (++it > L2_POLL_LIMIT) { dev_flag(status, DEV_TIMEOUT); ok = 0; break; }
       if ((it & 255u) == 0u && *reinterpret_cast<volatile int*>(status) == DEV_TIMEOUT) { ok = 0; break; }
     }
     if (ok && *reinterpret_cast<volatile int*>(status) == DEV_TIMEOUT) ok = 0;
@@ -171,7 +171,7 @@ __device__ __forceinline__ void gemv_phase(const MegaParams& p, const GemvDesc g
         const uint32_t bar = ws.bars + 8u * slot, parity = (ws.consumed / NSLOT) & 1u;
         bool got = false;
         if (!*s_abort) {
-          for (unsigned it = 0; it < SPIN_LIMIT; ++it) {
+          for (unsigned it = 0; it < TRY_WAIT_LIMIT; ++it) {
             if (mbar_test(bar, parity)) { got = true; break; }
             if ((it & 1023u) == 1023u && *s_abort) break;
           }

@@ -6,6 +6,8 @@
 
 namespace tcp {
 
+constexpr unsigned LAZY_LIMIT = 10u * 1000u * 1000u;         // polls with a sleep between them: 0.2 us each (measured), two seconds
+
 typedef unsigned long long u64;
 
 // Wait on an mbarrier: the test of a phase that is complete already costs 20 cycles, the bounded loop is kept out of line.
@@ -20,13 +22,13 @@ __device__ __forceinline__ bool quick_wait(uint32_t bar, uint32_t parity, volati
 // issue slots nor shared-memory cycles from them.  Consumers that have given up run on without waiting and release slots whose
 // copies are still in flight, so a phase that is complete counts only while nobody has given up (a warp sets the flag before it
 // releases anything unseen, and the completed phase makes that visible): the loader never arms a barrier a second time.
-__device__ __forceinline__ bool lazy_wait(uint32_t bar, uint32_t parity, volatile int* s_abort, int* status) {
+__device__ __forceinline__ bool lazy_wait(uint32_t bar, uint32_t parity, volatile int* s_abort, int* status, unsigned limit = LAZY_LIMIT) {
   int ok = 1;
   if ((threadIdx.x & 31) == 0) {
     unsigned it = 0;
     while (!mbar_poll(bar, parity)) {
       if (*s_abort) { ok = 0; break; }
-      if (++it > SPIN_LIMIT) { *s_abort = 1; dev_flag(status, DEV_TIMEOUT); ok = 0; break; }
+      if (++it > limit) { *s_abort = 1; dev_flag(status, DEV_TIMEOUT); ok = 0; break; }
       __nanosleep(100);
     }
     if (*s_abort) ok = 0;
@@ -49,21 +51,22 @@ __device__ __forceinline__ void ll_load2(const u64* p, u64& a, u64& b) {
 __device__ __forceinline__ float ll_val(u64 v) { return __uint_as_float((uint32_t)v); }
 __device__ __forceinline__ uint32_t ll_tag(u64 v) { return (uint32_t)(v >> 32); }
 // One poll more; false = the wait is over without its value (ran out, or another role gave up).
-__device__ __forceinline__ bool poll_more(unsigned& it, volatile int* s_abort, int* status) {
+__device__ __forceinline__ bool poll_more(unsigned& it, volatile int* s_abort, int* status, unsigned limit = L2_POLL_LIMIT) {
   ++it;
   if ((it & 63u) == 0u) {
     if (*s_abort) return false;
     if (*reinterpret_cast<volatile int*>(status) == DEV_TIMEOUT) { *s_abort = 1; return false; }
   }
-  if (it > SPIN_LIMIT) { *s_abort = 1; dev_flag(status, DEV_TIMEOUT); return false; }
+  if (it > limit) { *s_abort = 1; dev_flag(status, DEV_TIMEOUT); return false; }
   return true;
 }
 // A value of the wanted tag.
-__device__ __forceinline__ float ll_wait(const u64* p, uint32_t tag, bool& dead, volatile int* s_abort, int* status) {
+__device__ __forceinline__ float ll_wait(const u64* p, uint32_t tag, bool& dead, volatile int* s_abort, int* status,
+                                         unsigned limit = L2_POLL_LIMIT) {
   u64 v = ll_load(p);
   unsigned it = 0;
   while (ll_tag(v) != tag && !dead) {
-    if (!poll_more(it, s_abort, status)) dead = true;
+    if (!poll_more(it, s_abort, status, limit)) dead = true;
     v = ll_load(p);
   }
   return ll_val(v);

@@ -9,7 +9,10 @@
 
 namespace tcp {
 
-constexpr uint32_t SPIN_LIMIT = 20u * 1000u * 1000u;      // ~1-2 s of polling
+// After how many failing polls a wait gives up: about two seconds each.
+constexpr uint32_t SPIN_LIMIT = 20u * 1000u * 1000u;         // rounds of a loop that looks at several barriers (test_wait)
+constexpr uint32_t TRY_WAIT_LIMIT = 250u * 1000u;            // mbarrier.try_wait: parks the thread, 8.0 us a failing poll (measured)
+constexpr uint32_t L2_POLL_LIMIT = 4u * 1000u * 1000u;       // dependent loads that miss L1: 0.45 us each (measured)
 
 __device__ __forceinline__ uint32_t smem_u32(const void* p) { return (uint32_t)__cvta_generic_to_shared(p); }
 
@@ -48,7 +51,7 @@ __device__ __forceinline__ bool mbar_poll(uint32_t bar, uint32_t parity) {
 }
 // Bounded wait.  Returns false if the kernel is aborting (this or another role gave up).
 __device__ __forceinline__ bool mbar_wait(uint32_t bar, uint32_t parity, volatile int* abort_flag, int* status,
-                                          uint32_t limit = SPIN_LIMIT) {
+                                          uint32_t limit = TRY_WAIT_LIMIT) {
   for (uint32_t it = 0; it < limit; ++it) {
     if (mbar_test(bar, parity)) return true;
     if ((it & 63u) == 63u) {

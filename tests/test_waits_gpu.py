@@ -8,7 +8,9 @@ from parity_util import make_session
 pytestmark = pytest.mark.gpu
 
 
-def _outcomes():
+@pytest.fixture(scope="module")
+def outcomes():
+    """The four words, and how long the self-test kernel took (seconds)."""
     import torch
 
     import paper_2410_08391_b200 as kvp
@@ -17,14 +19,28 @@ def _outcomes():
     try:
         s.workspace[:256].zero_()
         torch.cuda.synchronize()
-        kvp.kvp_selftest_wait_timeout(s.h, s.workspace, s.stream)
+        kvp.kvp_selftest_wait_timeout(s.h, s.workspace, s.stream)      # (the first launch loads the kernel)
         torch.cuda.synchronize()
-        return s.workspace[:16].view(torch.int32).cpu().tolist()
+        s.workspace[:256].zero_()
+        torch.cuda.synchronize()
+        a, b = (torch.cuda.Event(enable_timing=True) for _ in range(2))
+        a.record(s.torch_stream)
+        kvp.kvp_selftest_wait_timeout(s.h, s.workspace, s.stream)
+        b.record(s.torch_stream)
+        torch.cuda.synchronize()
+        return s.workspace[:16].view(torch.int32).cpu().tolist(), a.elapsed_time(b) * 1e-3
     finally:
         s.close()
 
 
-def test_loader_stops_when_its_consumers_gave_up():
-    words = _outcomes()
-    assert words[0] == 1      # the wait that nobody satisfies ran out (DEV_TIMEOUT)
-    assert words[3] == 1      # a free slot is not filled any more once the consumers have given up
+def test_loader_stops_when_its_consumers_gave_up(outcomes):
+    assert outcomes[0][3] == 1      # a free slot is not filled any more once the consumers have given up
+
+
+def test_every_kind_of_wait_runs_out(outcomes):
+    assert outcomes[0][:3] == [1, 1, 1]      # DEV_TIMEOUT from the mbarrier wait, the tagged value, the sleeping loader
+
+
+def test_limits_are_a_few_seconds(outcomes):
+    """The kernel waits with a 64th of the limits, which are meant to be two seconds: at most five with room for a slower clock."""
+    assert 0.005 < outcomes[1] < 5.0 / 64
