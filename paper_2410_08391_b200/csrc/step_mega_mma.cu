@@ -21,6 +21,11 @@
 //   - Products are mma.sync m16n8k16 with the weights as A (read once from shared memory, no unpacking) and the activations
 //     as B.  An fp32 activation enters as three bf16 terms (x = hi + mid + lo, 24 significant bits: nothing of the fp32
 //     value is dropped) in three of four columns, so one 8-column instruction serves two sequences.
+//   - The accumulation inside an instruction rounds towards zero: one sum over a warp's whole share of K left a step's logits
+//     twice as far from 64 bits as fp32 multiply-adds do (1.1B shape 3.1e-6 against 1.5e-6, 3B shape 4.7e-6 against 2.1e-6, on
+//     the same cache).  So a sum goes through few instructions: with one sequence the hi terms of successive blocks of 32 k
+//     take turns in four columns, with two sequences in two; with two and more sequences a chunk is summed apart and added in
+//     fp32.  Now 1.3e-6 .. 1.7e-6 and 1.8e-6 .. 1.9e-6, for up to 1 % of a step's time (two sequences: 2 .. 4 %).
 //   - The cache pages of an attention item are brought into shared memory by a warp of their own, ahead of the query; the
 //     step's own key and value are taken from the projection's output by the CTA whose key range ends with them (no separate
 //     append phase); RoPE angles are computed once per launch.
@@ -83,6 +88,11 @@ __device__ __forceinline__ uint4 lds128(uint32_t a) {
 __device__ __forceinline__ void mma16816(float (&d)[4], uint32_t a0, uint32_t a1, uint32_t a2, uint32_t a3, uint32_t b0, uint32_t b1) {
   asm volatile("mma.sync.aligned.m16n8k16.row.col.f32.bf16.bf16.f32 {%0, %1, %2, %3}, {%4, %5, %6, %7}, {%8, %9}, {%0, %1, %2, %3};"
                : "+f"(d[0]), "+f"(d[1]), "+f"(d[2]), "+f"(d[3]) : "r"(a0), "r"(a1), "r"(a2), "r"(a3), "r"(b0), "r"(b1));
+}
+// The first product of a sum: no accumulator goes in.
+__device__ __forceinline__ void mma16816_first(float (&d)[4], uint32_t a0, uint32_t a1, uint32_t a2, uint32_t a3, uint32_t b0, uint32_t b1) {
+  asm volatile("mma.sync.aligned.m16n8k16.row.col.f32.bf16.bf16.f32 {%0, %1, %2, %3}, {%4, %5, %6, %7}, {%8, %9}, {%10, %10, %10, %10};"
+               : "=f"(d[0]), "=f"(d[1]), "=f"(d[2]), "=f"(d[3]) : "r"(a0), "r"(a1), "r"(a2), "r"(a3), "r"(b0), "r"(b1), "f"(0.f));
 }
 
 // A projection phase: 4 per layer (q(kv), O, gate/up, down), then the LM head.
@@ -165,6 +175,7 @@ struct Shared {
   int kv_rows[2];                              // cached rows in a page slot, -1 = bad page
   int max_pages, abort;
   int issued;                                  // a ring slot lately asked for
+  __align__(16) unsigned zeros[16];
   __align__(16) kv16 knew[128];                // the step's own key and value (of one kv head)
   __align__(16) kv16 vnew[128];
 };
@@ -214,12 +225,20 @@ __device__ __forceinline__ void proj_phase(const MegaParams& p, const Work& g, R
   const int kws = g.kc / CW;                   // k elements of a warp's share of a chunk
   constexpr int RS = TG * TR * BB;
   constexpr int NJ = KW / 32;                  // 32-k blocks of a warp's share of a chunk
+  constexpr bool OWN_PART = BB > 1;            // chunks are summed apart
   constexpr int NH = KW / KS, QJ = KS / 32;    // ... handled as NH pieces of QJ blocks
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, gr = lane >> 2, t = lane & 3;
   volatile int* s_abort = &sh.abort;
   const bool sw = g.mode == GEMV_SWIGLU;
   const int TO = sw ? TR / 2 : TR;
   const int nch = g.nch;
+  // Columns 4 b .. 4 b + 2 of an instruction hold sequence b's hi, mid and lo terms.  With one or two sequences, the hi terms of
+  // successive blocks of 32 k take turns in the columns that are left (0 and 3, and 4 and 5 beside one sequence; zeros where it
+  // is another column's turn); with four, column 3 holds the lo term again and is not used.
+  constexpr int TURNS = BB == 1 ? 4 : 2;
+  const int cpart = BB == 1 ? gr : gr & 3, cterm = cpart == 1 || cpart == 2 ? cpart : (BB == 4 && cpart == 3 ? 2 : 0);
+  const int cturn = cpart ? cpart - 2 : 0;
+  const uint32_t cbase = xp + (3 * (BB == 1 ? 0 : gr >> 2) + cterm) * XCOL + t * 16, czero = smem_u32(sh.zeros) + t * 16;
   const int ss_par = par >> 1;                 // par: bit 0 = half of the partial sums, bit 1 = half of the sums of squares
   u64 xr[NH][BB][4];
   float4 gv[NH];
@@ -310,10 +329,8 @@ __device__ __forceinline__ void proj_phase(const MegaParams& p, const Work& g, R
         for (int i = 0; i < NH; ++i)
           if (!ready(i)) fetch_x(i, c);
       }
-      // column 4 b + part of an instruction is sequence b's hi / mid / lo term
       auto column = [&](int nb, int j) {
-        const int b = (gr >> 2) + 2 * nb;
-        return (gr & 3) != 3 && b < BB ? lds128(xp + (3 * b + (gr & 3)) * XCOL + j * 64 + t * 16) : make_uint4(0, 0, 0, 0);
+        return lds128(BB == 4 || cterm || cturn == (j & (TURNS - 1)) ? cbase + 6 * nb * XCOL + j * 64 : czero);
       };
       uint4 bq[NJ];
 #pragma unroll
@@ -341,6 +358,13 @@ __device__ __forceinline__ void proj_phase(const MegaParams& p, const Work& g, R
       }
       fetch(c + 1 < nch ? c + 1 : 0);
       const int kw = min(kws, g.K - c * g.kc - warp * kws);      // of them within the row
+      float part[NB][4];                       // a tile's share of the chunk
+      auto add_part = [&](int ti) {
+#pragma unroll
+        for (int nb = 0; nb < NB; ++nb)
+#pragma unroll
+          for (int e = 0; e < 4; ++e) acc[ti][nb][e] += part[nb][e];
+      };
 #pragma unroll
       for (int ti = 0; ti < TG; ++ti) {
         if (ti < ntg) {
@@ -363,6 +387,7 @@ __device__ __forceinline__ void proj_phase(const MegaParams& p, const Work& g, R
               uint4 ua[2], ub[2];
 #pragma unroll
               for (int j = 0; j < 2; ++j) { ua[j] = lds128(a + (jh + j) * 64); ub[j] = lds128(b + (jh + j) * 64); }
+              if (OWN_PART && jh == 0 && ti > 0) add_part(ti - 1);      // (its last product has long been finished by now)
               if (kw < kws) {                  // k beyond the rows' end
 #pragma unroll
                 for (int j = 0; j < 2; ++j)
@@ -373,13 +398,16 @@ __device__ __forceinline__ void proj_phase(const MegaParams& p, const Work& g, R
 #pragma unroll
                 for (int nb = 0; nb < NB; ++nb) {
                   const uint4 bb = NB == 1 ? bq[jh + j] : column(nb, jh + j);
-                  mma16816(acc[ti][nb], ua[j].x, ub[j].x, ua[j].y, ub[j].y, bb.x, bb.y);
-                  mma16816(acc[ti][nb], ua[j].z, ub[j].z, ua[j].w, ub[j].w, bb.z, bb.w);
+                  float (&d)[4] = OWN_PART ? part[nb] : acc[ti][nb];
+                  if (OWN_PART && jh + j == 0) mma16816_first(d, ua[j].x, ub[j].x, ua[j].y, ub[j].y, bb.x, bb.y);
+                  else mma16816(d, ua[j].x, ub[j].x, ua[j].y, ub[j].y, bb.x, bb.y);
+                  mma16816(d, ua[j].z, ub[j].z, ua[j].w, ub[j].w, bb.z, bb.w);
                 }
             }
           }
           __syncwarp();
           if (lane == 0) { mbar_arrive(bar_a); if (two) mbar_arrive(bar_b); }
+          if (OWN_PART && ti + 1 == ntg && kw > 0) add_part(ti);
         }
       }
       dead = __any_sync(0xffffffffu, dead);    // (also: every lane has read this chunk's columns)
@@ -390,9 +418,14 @@ __device__ __forceinline__ void proj_phase(const MegaParams& p, const Work& g, R
       if (ti < ntg) {
 #pragma unroll
         for (int nb = 0; nb < NB; ++nb) {
-          float v0 = acc[ti][nb][0] + acc[ti][nb][1], v1 = acc[ti][nb][2] + acc[ti][nb][3];
+          const bool pair = BB < 4 || !(t & 1);
+          float v0 = acc[ti][nb][0] + (pair ? acc[ti][nb][1] : 0.f), v1 = acc[ti][nb][2] + (pair ? acc[ti][nb][3] : 0.f);
           v0 += __shfl_xor_sync(0xffffffffu, v0, 1);
           v1 += __shfl_xor_sync(0xffffffffu, v1, 1);
+          if (BB == 1) {
+            v0 += __shfl_xor_sync(0xffffffffu, v0, 2);
+            v1 += __shfl_xor_sync(0xffffffffu, v1, 2);
+          }
           const int b = nb * 2 + (t >> 1);
           if (!(t & 1) && b < BB) {
             red[warp * RS + (ti * TR + gr) * BB + b] = v0;
@@ -714,6 +747,7 @@ __global__ void __launch_bounds__(NT, 1) step_mega_mma_kernel(const __grid_const
   Ring wr{smem_u32(sm), bars, bars + 8u * pl.n_stage, pl.n_stage, 0, 0u, STAGE};
   Ring kr{smem_u32(sm) + pl.kv_off, bars + 16u * pl.n_stage, bars + 16u * pl.n_stage + 8u * pl.n_kv, pl.n_kv, 0, 0u, 2 * PAGE_TOKENS * HD * 2};
   const uint32_t rope_bar = bars + 16u * pl.n_stage + 16u * pl.n_kv;
+  if (tid < 16) sh.zeros[tid] = 0u;
   if (tid == 0) {
     sh.abort = 0; sh.issued = 0;
     for (int i = 0; i < pl.n_stage; ++i) { mbar_init(wr.full + 8u * i, 1); mbar_init(wr.empty + 8u * i, CW); }
