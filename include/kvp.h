@@ -283,7 +283,7 @@ kvp_status kvp_poll_status(kvp_handle* h, void* workspace, void* stream);
 /* Self-test of the error path behind KVP_ERR_TIMEOUT (the paper has no counterpart).  Enqueues a one-block
  * kernel that waits, with the library's own bounded waits but a 64th of their limits, for what never comes
  * (a few hundredths of a second).  The waits run out, the kernel returns normally and records its code
- * in the status word of `workspace` (dev, >= 16 bytes, as passed to the compute calls; the three words behind the status
+ * in the status word of `workspace` (dev, >= 16 bytes, as passed to the compute calls; the two words behind the status
  * word receive the outcomes of the step kernel's own waits); kvp_poll_status then
  * returns KVP_ERR_TIMEOUT and clears the word, and the handle and the context stay usable. */
 kvp_status kvp_selftest_wait_timeout(kvp_handle* h, void* workspace, void* stream);

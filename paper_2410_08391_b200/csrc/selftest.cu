@@ -1,25 +1,22 @@
 // Self-test of the bounded device-side waits: a one-block kernel waits, with a 64th of each kind's limit, for what never comes.
 // Every wait must run out, the kernel must return, and the status word must read DEV_TIMEOUT, which kvp_poll_status reports as
 // KVP_ERR_TIMEOUT.  The kinds: the mbarrier wait of most kernels (status word), the tagged value (word 1) and the sleeping loader
-// (word 2) of the barrier-free step kernel.  A last warp plays such a loader whose slot is free but whose consumers have given
-// up: its wait must say so (word 3 then reads 1).
+// (word 2) of the barrier-free step kernel.
 #include "kvp_internal.h"
 #include "step_waits.cuh"
 
 namespace {
 using namespace tcp;
 
-__global__ void __launch_bounds__(160) wait_timeout_kernel(int* status) {
-  __shared__ __align__(8) unsigned long long bar, free_bar;
-  __shared__ int abort_mem, given_up, abort_tag, abort_lazy;
+__global__ void __launch_bounds__(128) wait_timeout_kernel(int* status) {
+  __shared__ __align__(8) unsigned long long bar;
+  __shared__ int abort_mem, abort_tag, abort_lazy;
   volatile int* abort_flag = &abort_mem;
   if (threadIdx.x == 0) {
     mbar_init(smem_u32(&bar), 1);
-    mbar_init(smem_u32(&free_bar), 1);
     *abort_flag = 0;
-    given_up = 1;
     abort_tag = abort_lazy = 0;
-    status[1] = status[2] = status[3] = 0;
+    status[1] = status[2] = 0;
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
   }
   __syncthreads();
@@ -29,11 +26,7 @@ __global__ void __launch_bounds__(160) wait_timeout_kernel(int* status) {
     bool dead = false;
     ll_wait(reinterpret_cast<const u64*>(status), 0xffffffffu, dead, &abort_tag, status + 1, L2_POLL_LIMIT / 64);
   }
-  if (threadIdx.x >= 96 && threadIdx.x < 128) lazy_wait(smem_u32(&bar), 0, &abort_lazy, status + 2, LAZY_LIMIT / 64);
-  if (threadIdx.x >= 128) {       // phase "minus one" of a fresh barrier counts as complete: a loader's first wait
-    const bool go = lazy_wait(smem_u32(&free_bar), 1, &given_up, status + 2);
-    if (threadIdx.x == 128) status[3] = go ? 2 : 1;
-  }
+  if (threadIdx.x >= 96) lazy_wait(smem_u32(&bar), 0, &abort_lazy, status + 2, LAZY_LIMIT / 64);
   __syncthreads();
 }
 }  // namespace
@@ -48,7 +41,7 @@ extern "C" kvp_status kvp_selftest_wait_timeout(kvp_handle* h, void* workspace, 
     return KVP_ERR_INVALID_ARG;
   }
   ++h->n_launch;
-  wait_timeout_kernel<<<1, 160, 0, (cudaStream_t)stream>>>((int*)workspace);
+  wait_timeout_kernel<<<1, 128, 0, (cudaStream_t)stream>>>((int*)workspace);
   cudaError_t e = cudaGetLastError();
   if (e != cudaSuccess) {
     h->err = std::string("kvp_selftest_wait_timeout: ") + cudaGetErrorString(e);

@@ -34,8 +34,8 @@
 // Measured against the CUDA-core kernel of step_mega.cu (generation step, ms): 1.1B shape 1 x 1100 keys 1.55 -> 0.81,
 // 4 x 300 2.90 -> 1.12 (that kernel's multiply-adds grow with the batch); of the 0.42 ms that the first one's bytes take,
 // the rest is the chain of ~170 hand-overs.
-// Every wait is bounded: on expiry DEV_TIMEOUT is recorded, no further wait is started, every CTA runs through its
-// remaining phases without waiting and leaves after copies in flight have had time to land.
+// Every wait is bounded: on expiry DEV_TIMEOUT is recorded, no further wait is started, every CTA runs through its remaining
+// phases without waiting or releasing slots, its loaders stop, and it leaves after copies in flight have had time to land.
 #include <math.h>
 
 #include "common.cuh"
@@ -406,7 +406,7 @@ __device__ __forceinline__ void proj_phase(const MegaParams& p, const Work& g, R
             }
           }
           __syncwarp();
-          if (lane == 0) { mbar_arrive(bar_a); if (two) mbar_arrive(bar_b); }
+          if (lane == 0 && !dead) { mbar_arrive(bar_a); if (two) mbar_arrive(bar_b); }
           if (OWN_PART && ti + 1 == ntg && kw > 0) add_part(ti);
         }
       }
@@ -669,7 +669,7 @@ __device__ __forceinline__ void attn_phase(const MegaParams& p, const MegaLayer&
         }
       }
       __syncwarp();
-      if (lane == 0) mbar_arrive(rg.empty + 8u * rg.slot);
+      if (lane == 0 && !dead) mbar_arrive(rg.empty + 8u * rg.slot);
       rg.next();
     }
     // merge the warps

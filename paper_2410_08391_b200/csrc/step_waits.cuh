@@ -19,9 +19,8 @@ __device__ __forceinline__ bool quick_wait(uint32_t bar, uint32_t parity, volati
 }
 
 // Wait of a loader warp, which is far ahead of its consumers: one lane looks now and then, so that the wait takes neither
-// issue slots nor shared-memory cycles from them.  Consumers that have given up run on without waiting and release slots whose
-// copies are still in flight, so a phase that is complete counts only while nobody has given up (a warp sets the flag before it
-// releases anything unseen, and the completed phase makes that visible): the loader never arms a barrier a second time.
+// issue slots nor shared-memory cycles from them.  (A consumer that has given up releases no slot: the copy into it
+// may still be in flight, and the loader would arm its barrier a second time.)
 __device__ __forceinline__ bool lazy_wait(uint32_t bar, uint32_t parity, volatile int* s_abort, int* status, unsigned limit = LAZY_LIMIT) {
   int ok = 1;
   if ((threadIdx.x & 31) == 0) {
@@ -31,7 +30,6 @@ __device__ __forceinline__ bool lazy_wait(uint32_t bar, uint32_t parity, volatil
       if (++it > limit) { *s_abort = 1; dev_flag(status, DEV_TIMEOUT); ok = 0; break; }
       __nanosleep(100);
     }
-    if (*s_abort) ok = 0;
   }
   return __shfl_sync(0xffffffffu, ok, 0) != 0;
 }

@@ -1,4 +1,4 @@
-"""The bounded waits of the barrier-free step kernel, through the library's self-test kernel: words 1 to 3 behind the status word
+"""The bounded waits of the barrier-free step kernel, through the library's self-test kernel: the two words behind the status word
 hold what each of them did."""
 import pytest
 
@@ -10,7 +10,7 @@ pytestmark = pytest.mark.gpu
 
 @pytest.fixture(scope="module")
 def outcomes():
-    """The four words, and how long the self-test kernel took (seconds)."""
+    """The status block's first words, and how long the self-test kernel took (seconds)."""
     import torch
 
     import paper_2410_08391_b200 as kvp
@@ -31,10 +31,6 @@ def outcomes():
         return s.workspace[:16].view(torch.int32).cpu().tolist(), a.elapsed_time(b) * 1e-3
     finally:
         s.close()
-
-
-def test_loader_stops_when_its_consumers_gave_up(outcomes):
-    assert outcomes[0][3] == 1      # a free slot is not filled any more once the consumers have given up
 
 
 def test_every_kind_of_wait_runs_out(outcomes):
