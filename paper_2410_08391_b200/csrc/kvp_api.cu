@@ -307,8 +307,13 @@ bool mega_prepare(kvp_handle* h, const LaunchCtx& ctx, const kvp_cache* cache, c
                   int32_t* token_out, MegaParams* out, int* k_max_out) {
   const ModelPlan& B = h->base;
   int k_max = std::max(B.d, std::max(B.max_dq, B.max_ffn));
-  // its attention phase reads cache pages with plain loads: fine for a few thousand keys, several times
-  // slower than the ring-fed kernel beyond that
+  // Beyond some thousand keys the chain of launches around the tensor-core attention kernel (step_attn_mma.cu) is the faster one.
+  // The CUDA-core kernel reads cache pages with plain loads, several times slower than that kernel.  The other one brings them in
+  // by bulk copy, but multiplies them on the CUDA cores; where it falls behind depends on the sequences and kv heads.  Generation
+  // step, chain of launches / step_mega_mma_kernel, us: 1.1B shape 1 x 8000 1983 / 1054, 2 x 16000 2154 / 1833, 4 x 4200 1953 /
+  // 1570, 4 x 8000 2070 / 2026, 4 x 16000 2335 / 2941; 3B shape 1 x 16000 3928 / 2584, 2 x 8000 3490 / 2817, 4 x 4200 3399 / 3289,
+  // 4 x 6000 3443 / 3723, 4 x 16000 4117 / 6015; 32 kv heads of 64 1 x 8000 1287 / 999, 4 x 4200 1449 / 1734.  The line is
+  // where four sequences of the 3B shape cross; a single sequence of it would gain up to 16000 keys.
   if (max_keys > 4096) return false;
   if (B.n_layers > MEGA_MAX_LAYERS) return false;
   if (!mega_uses_mma(h, batch) && !step_mega_supported(batch, B.L[0].hd, k_max, B.max_group, h->es)) return false;
@@ -696,7 +701,8 @@ static kvp_status prefill_direct(kvp_handle* h, const int32_t* tokens, const int
     }
     mega_clear(h, mp, w, ws, s);
     h->gemm_sms = h->n_sm - h->step_sms;
-    // key-range splits of the pieces: one attention item per CTA of the piece (more make two rounds)
+    // key-range splits of the CUDA-core kernel's pieces: one attention item per CTA of the piece (more make two rounds); the other
+    // kernel splits by its own grid
     for (int i = 0; i < h->base.n_layers; ++i)
       mp.layers[i].n_split = std::max(1, std::min(mp.layers[i].n_split, h->step_sms / (batch * h->base.L[i].nkv)));
   }

@@ -3,7 +3,7 @@
 #include "common.cuh"
 
 constexpr int MEGA_MAX_LAYERS = 64;
-constexpr int MEGA_COUNTERS = 32;      // grid-barrier counter words in the status block (one per launch of a step)
+constexpr int MEGA_COUNTERS = 32;      // counter words in the status block, one per launch of a step: grid barrier (step_mega_kernel), finished CTAs (step_mega_mma_kernel)
 constexpr int MEGA_STATUS_BYTES = 256; // what a caller clears before a step: status word, argmax slots, counters
 
 struct MegaLayer {
@@ -29,13 +29,13 @@ struct MegaParams {
   unsigned long long *ll_q, *ll_a, *ll_x1, *ll_x2, *ll_h, *ll_part;
   int* attn_done;                                // [batch * max n_kv] splits finished per (sequence, kv head); zero on entry, left zero
   float* logits; int* token_out;
-  // One launch may cover only base layers [layer_begin, layer_end): the residual stream stays in xb between
+  // One launch may cover only base layers [layer_begin, layer_end): the residual stream stays in xb (ll_x2) between
   // launches.  do_embed: start from the token embeddings; do_head: end with the LM head and the token.
   int layer_begin, layer_end, do_embed, do_head;
-  int counter_idx;                               // which grid-barrier counter word this launch uses (zero on entry)
+  int counter_idx;                               // which counter word this launch uses (zero on entry)
   int stage_bytes, slot_bytes;                   // shared-memory plan (set by the launcher)
-  long long* trace;                              // optional: clock64 of CTA 0 around every barrier (debugging aid)
-  int* status;                                   // [0] status word, +64 bytes: argmax slots, +128 bytes: MEGA_COUNTERS barrier counters
+  long long* trace;                              // optional: clock64 of CTA 0 around every barrier / after every phase (debugging aid)
+  int* status;                                   // [0] status word, +64 bytes: argmax slots, +128 bytes: MEGA_COUNTERS counters
   MegaLayer layers[MEGA_MAX_LAYERS];
 };
 

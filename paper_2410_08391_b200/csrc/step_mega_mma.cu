@@ -1,7 +1,7 @@
 // The base model's single-token step as ONE persistent cooperative kernel for 16-bit weights (batch <= 4), with the
 // multiply on the warp-level tensor cores and without grid-wide barriers.
 //
-// What bounds it: the step is ~140 dependent matrix-vector phases (5 per layer) whose weights stream from HBM once; a
+// What bounds it: the step is a chain of dependent phases (5 per layer, 141 in the 1.1B shape) whose weights stream from HBM once; a
 // phase's own bytes take 1-7 us, so whatever sits in series between two phases counts as much as the bytes do.  Hence:
 //   - No barrier.  Every value that one CTA hands to others (projections, attention, residual stream) is stored as ONE
 //     64-bit word {fp32 value, tag}, the tag being the layer; whoever needs a value polls the value itself.  That takes the
@@ -14,7 +14,7 @@
 //     pieces of 2 KB; HBM's share of an SM is 23.  Two loader warps walk the static schedule of the whole step, so the ring is
 //     full again before a phase's input exists, and a third asks the rows behind the ring into L2 (per line, not through the
 //     copy engine, which works in order), so that HBM streams on while the ring is full (1 x 1100 keys, 1.1B shape:
-//     0.83 -> 0.80 ms).  Rows lie 4160 bytes apart: the 16-byte reads of two rows then cover all 32 banks.
+//     4 % of the step).  Rows lie 4160 bytes apart: the 16-byte reads of two rows then cover all 32 banks.
 //   - The 8 consumer warps cut K: warp w owns an eighth of every chunk.  A warp therefore needs only its own eighth of the
 //     activations, which it fetches and converts by itself: no staging of the whole input.  The 1 / rms of RMSNorm is
 //     applied to the outputs (its sum of squares falls out of the fetch), so nothing waits for it.
@@ -25,15 +25,18 @@
 //     twice as far from 64 bits as fp32 multiply-adds do (1.1B shape 3.1e-6 against 1.5e-6, 3B shape 4.7e-6 against 2.1e-6, on
 //     the same cache).  So a sum goes through few instructions: with one sequence the hi terms of successive blocks of 32 k
 //     take turns in four columns, with two sequences in two; with two and more sequences a chunk is summed apart and added in
-//     fp32.  Now 1.3e-6 .. 1.7e-6 and 1.8e-6 .. 1.9e-6, for up to 1 % of a step's time (two sequences: 2 .. 4 %).
+//     fp32.  Now 1.3e-6 .. 1.7e-6 and 1.8e-6 .. 1.9e-6, for up to 1 % of a step's time (8 heads of 128 a group: 3 %; two sequences:
+//     1 .. 5 %).
 //   - The cache pages of an attention item are brought into shared memory by a warp of their own, ahead of the query; the
 //     step's own key and value are taken from the projection's output by the CTA whose key range ends with them (no separate
 //     append phase); RoPE angles are computed once per launch.
 //   - 12 warps of up to 168 registers: next to 220 KB of shared memory there is almost no L1, so every spilled register
-//     is a round trip to L2.
-// Measured against the CUDA-core kernel of step_mega.cu (generation step, ms): 1.1B shape 1 x 1100 keys 1.55 -> 0.81,
-// 4 x 300 2.90 -> 1.12 (that kernel's multiply-adds grow with the batch); of the 0.42 ms that the first one's bytes take,
-// the rest is the chain of ~170 hand-overs.
+//     is a round trip to L2.  One and four sequences with up to 4 heads a group fit; two sequences, and groups of 5 to 8 heads,
+//     spill 8 to 48 bytes (ptxas), which is part of what those take longer.
+// Measured against the CUDA-core kernel of step_mega.cu (generation step): 1.1B shape 1 x 1100 keys 1557 -> 838 us, 4 x 300
+// 2990 -> 1123 us (that kernel's multiply-adds grow with the batch); 3B shape 1 x 300 2966 -> 2003 us, 4 x 300 5578 -> 2415 us.
+// The bytes of the first take 416 us.  Of the rest, its 169 hand-overs between CTAs (a phase each, two in attention) of about
+// 0.5 us are 85 us; what the other 340 us go to has not been measured phase by phase.
 // Every wait is bounded: on expiry DEV_TIMEOUT is recorded, no further wait is started, every CTA runs through its remaining
 // phases without waiting or releasing slots, its loaders stop, and it leaves after copies in flight have had time to land.
 #include <math.h>
@@ -215,7 +218,7 @@ __device__ __forceinline__ Work work_of(const MegaParams& p, int i, int kind, bo
 
 // ---- projection: y[b, o] (op)= sum_k W[o, k] x[b, k] for this CTA's outputs --------------------------------------------
 // xp: this warp's private shared memory (3 BB columns of XCOL bytes); red: [2][CW][TG * 16 * BB] floats.
-// The loop over chunks of 1024 k is kept rolled: every phase runs through this code once per layer, and straight-line
+// The loop over chunks is kept rolled: every phase runs through this code once per layer, and straight-line
 // copies of it cost more in instruction fetches than the loop does.
 template <int BB>
 __device__ __forceinline__ void proj_phase(const MegaParams& p, const Work& g, Ring& rg, uint32_t xp, float* red0, int& par, Shared& sh, bool& dead,
@@ -911,6 +914,8 @@ __global__ void __launch_bounds__(NT, 1) step_mega_mma_kernel(const __grid_const
 constexpr size_t SMEM_ROOM = SMEM_LIMIT - sizeof(Shared) - 256;      // dynamic shared memory of a CTA
 
 // Shared-memory plan: scratch and page slots first, the weight ring takes what is left (at least 3 slots).
+// (head_dim 128 with four sequences has room for one page slot and three weight slots only, so that a page's load does not overlap
+// the arithmetic on the one before.)
 bool make_plan(int batch, int hd, int max_group, Plan* pl, size_t* bytes) {
   const int bb = batch <= 1 ? 1 : (batch == 2 ? 2 : 4);
   const size_t proj = (size_t)CW * 3 * bb * XCOL + (size_t)2 * CW * TG * TR * bb * 4;
