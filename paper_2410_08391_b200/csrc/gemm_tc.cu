@@ -1,8 +1,7 @@
 // Tensor-core GEMM for sm_100a:  D[M,N] = A[M,K] W[N,K]^T (+ A_lo W^T on split tiles), bf16
 // operands, fp32 accumulation in tensor memory.
 //
-// One persistent CTA per SM walks output tiles of 128 x BN (BN = 256, or 128 when the problem
-// has too few wide tiles to fill the SMs).  Operand tiles travel through a ring of shared-
+// One persistent CTA per SM walks output tiles of 128 x BN, BN = 128 to 256 (choose_cut).  Operand tiles travel through a ring of shared-
 // memory stages (128-byte swizzle, 64 k-elements per stage) filled by TMA.  A thread that
 // issues a tensor copy is held for a few hundred cycles per copy, which caps one issuing thread
 // at about 120 GB/s; a 128 x 256 tile needs 48 KiB per 512 tensor-pipe cycles (about 180 GB/s),
@@ -12,8 +11,8 @@
 // (bf16 store / fp32 residual add / RoPE + hi-lo split / SwiGLU / scatter into cache pages),
 // so the epilogue of tile i overlaps the main loop of tile i+1.
 // Tiles are visited in groups of 16 row blocks so that a wave's A and W tiles stay in L2.
-// The residual GEMMs (x += A W^T) add with red.global, so when they have fewer tiles than
-// two per SM their k loops are cut into equal contiguous shares, one per CTA (stream-K).
+// The residual GEMMs (x += A W^T) add in L2, so where whole tiles would leave SMs idle their
+// k loops are cut into equal contiguous shares, one per CTA (stream-K).
 // Every mbarrier wait is bounded: on expiry the kernel records DEV_TIMEOUT, all roles leave
 // their loops, in-flight copies are given time to land, tensor memory is freed.
 #include <cuda.h>
@@ -32,16 +31,17 @@ constexpr int GROUP_M = 16;                                // row blocks per ras
 constexpr int N_THREADS = 224;                             // warps: 0 A loads, 1 MMA, 2 W loads, 3-6 epilogue
 constexpr int N_THREADS_NORM = 352;                        // fused-norm residual kernel: 8 epilogue warps (3-10), two per lane quarter
 constexpr int TC_RESID_NORM = 100;                         // internal: TC_RESID with the folded RMSNorm producer (own shared-memory plan)
+constexpr int SMEM_LIMIT = 227 * 1024;
 template <int BN, int EPI = TC_STORE> struct Tile {
-  // the fused-norm residual epilogue needs a deeper prefetch ring for the old values of X: one operand stage less
-  static constexpr int STAGES = (BN == 256 ? 4 : 6) - (EPI == TC_RESID_NORM ? 1 : 0);
   static constexpr int XS = (EPI == TC_PAGED || EPI == TC_QKV) ? 1 : 2;        // 4 KiB slots per epilogue warp
   // epilogues that move every element through shared memory get eight warps (two per tensor-memory lane quarter)
   static constexpr int EPI_WARPS = (EPI == TC_RESID_NORM || EPI == TC_PAGED || EPI == TC_QKV || EPI == TC_SWIGLU) ? 8 : 4;
   static constexpr int THREADS = EPI_WARPS == 8 ? N_THREADS_NORM : N_THREADS;
   static constexpr int XRING = (EPI == TC_RESID || EPI == TC_RESID_NORM || EPI == TC_PAGED || EPI == TC_QKV) ? EPI_WARPS * XS * 4096 : 0;
   static constexpr int A_BYTES = BM * BK * 2, W_BYTES = BN * BK * 2;
-  static constexpr int STAGE_BYTES = A_BYTES + W_BYTES;    // 48 KiB / 32 KiB
+  static constexpr int STAGE_BYTES = A_BYTES + W_BYTES;    // 32 KiB (128 columns) to 48 KiB (256)
+  static constexpr int STAGES_FIT = (SMEM_LIMIT - 1536 - XRING) / STAGE_BYTES, STAGES = STAGES_FIT < 6 ? STAGES_FIT : 6;
+  static constexpr int ACC_STRIDE = BN > 128 ? 256 : 128;  // tensor-memory columns between the two accumulators
   static constexpr int SMEM_BYTES = STAGES * STAGE_BYTES + XRING + 1024 /*align*/ + 512 /*barriers*/;
 };
 // Fused-norm residual epilogue: each epilogue warp prefetches the residual stream's old values of its 32 rows,
@@ -314,8 +314,8 @@ gemm_tc_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_constant_
     *abort_flag = 0;
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
   }
-  if (warp == 1) {   // tensor memory: two accumulators of BN columns
-    tmem_alloc(smem_u32(tmem_slot), 2 * BN);
+  if (warp == 1) {   // tensor memory: two accumulators of BN columns (a power of two is allocated)
+    tmem_alloc(smem_u32(tmem_slot), 2 * T::ACC_STRIDE);
   }
   tc_fence_before();
   __syncthreads();
@@ -365,7 +365,7 @@ gemm_tc_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_constant_
         ok = mbar_wait(tempty_bar(acc), acc_phase ^ 1u, abort_flag, p.status);
         if (!ok) break;
         tc_fence_after();
-        const uint32_t d_tmem = tmem_base + acc * BN;
+        const uint32_t d_tmem = tmem_base + acc * T::ACC_STRIDE;
         for (int it = w.kb0; it < w.kb1 && ok; ++it) {
           ok = mbar_wait(full_bar(stage), phase, abort_flag, p.status);
           if (!ok) break;
@@ -420,7 +420,7 @@ gemm_tc_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_constant_
       if (!ok) break;
       tc_fence_after();
       const int m = w.m0 + quarter * 32 + lane;
-      const uint32_t tmem_acc = tmem_base + ((uint32_t)(quarter * 32) << 16) + acc * BN;
+      const uint32_t tmem_acc = tmem_base + ((uint32_t)(quarter * 32) << 16) + acc * T::ACC_STRIDE;
       if (fused) {
         float row_ss = 0.f;
 #pragma unroll 1
@@ -652,7 +652,7 @@ gemm_tc_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_constant_
   __syncthreads();
   if (warp == 1) {
     tc_fence_after();
-    tmem_dealloc(tmem_base, 2 * BN);
+    tmem_dealloc(tmem_base, 2 * T::ACC_STRIDE);
   }
 }
 
@@ -671,33 +671,62 @@ cudaError_t go(const CUtensorMap& a, const CUtensorMap& a2, const CUtensorMap& w
   return launch_overlapped(gemm_tc_kernel<EPI, BN>, dim3(grid), dim3(Tile<BN, EPI>::THREADS), SMEM, st, a, a2, w, x, p);
 }
 
+// Which widths an epilogue takes: whole heads (TC_QKV: 192 only with head_dim 64), whole gate / up blocks (TC_SWIGLU), whole 64-column
+// pieces of a cache row (TC_PAGED).
+bool width_ok(const TcGemm& g, int bn) {
+  if (bn == 128 || bn == 256) return true;
+  if (g.epi == TC_RESID) return bn == 160 || bn == 192 || bn == 224;
+  return bn == 192 && ((g.epi == TC_QKV && g.hd == 64) || g.epi == TC_PAGED);
+}
+
+template <int BN>
+cudaError_t go_resid(const CUtensorMap& a, const CUtensorMap& a2, const CUtensorMap& w, const CUtensorMap& x, const Params& p, int grid, cudaStream_t st) {
+  return p.H ? go<TC_RESID_NORM, BN>(a, a2, w, x, p, grid, st) : go<TC_RESID, BN>(a, a2, w, x, p, grid, st);
+}
+
 template <int BN>
 cudaError_t go_epi(int epi, const CUtensorMap& a, const CUtensorMap& a2, const CUtensorMap& w, const CUtensorMap& x, const Params& p, int grid, cudaStream_t st) {
   switch (epi) {
     case TC_STORE: return go<TC_STORE, BN>(a, a2, w, x, p, grid, st);
-    case TC_RESID: return p.H ? go<TC_RESID_NORM, BN>(a, a2, w, x, p, grid, st) : go<TC_RESID, BN>(a, a2, w, x, p, grid, st);
+    case TC_RESID: return go_resid<BN>(a, a2, w, x, p, grid, st);
     case TC_SWIGLU: return go<TC_SWIGLU, BN>(a, a2, w, x, p, grid, st);
     case TC_QKV: return go<TC_QKV, BN>(a, a2, w, x, p, grid, st);
     default: return go<TC_PAGED, BN>(a, a2, w, x, p, grid, st);
   }
 }
 
-// Relative time of a launch with tile width bn on n_sm SMs: waves of tiles, each tile costing
-// the larger of its tensor-pipe time and its operand-feed time (two issuing threads deliver
-// about 100 bytes per cycle).
-double tile_cost(const TcGemm& g, int bn, bool stream_k) {
-  const double tiles = (double)((g.M + BM - 1) / BM) * ((g.N + bn - 1) / bn);
-  const double mma = 2.0 * bn, feed = (BM + bn) * 128.0 / 100.0;      // cycles per k block
-  const double per_tile = mma > feed ? mma : feed;
-  const double waves = stream_k ? tiles / g.n_sm : (double)(((long long)tiles + g.n_sm - 1) / g.n_sm);
-  return waves * per_tile;
+// How a launch is cut: tile width, and whether the CTAs take whole tiles or (residual GEMM with one operand pass) equal shares of all
+// k blocks.  Costs in units of a k block of a 256-wide tile on one SM (0.41 us).  A CTA is bound by its shared-memory port (operands
+// written once and read once), so a k block costs almost the same whatever the width, and what counts is how many waves of tiles a
+// width leaves: with 128 and 256 columns only, 3776 x 1280 x 3456 took 3 waves or 2.03.  Fitted to 118 launches of 59 to 8192 rows,
+// N 1280 to 32000, K 1280 to 5632, 76 and 148 SMs, one and two passes: the geometric mean of the chosen cuts is 0.9 % above
+// that of the best ones (the rule before, 128 or 256 columns by tensor time: 18 %).
+struct Cut { int bn; bool shares; };
+Cut choose_cut(const TcGemm& g) {
+  static const struct { int bn; double cost; } widths[] = {{256, 1.00}, {224, 0.95}, {192, 0.90}, {160, 0.87}, {128, 0.84}};
+  const double kb = (double)((g.K + BK - 1) / BK) * (g.A2 ? 2 : 1);
+  Cut best{256, false};
+  double least = -1.0;
+  for (const auto& w : widths) {
+    if (!width_ok(g, w.bn)) continue;
+    const long long tiles = (long long)((g.M + BM - 1) / BM) * ((g.N + w.bn - 1) / w.bn), waves = (tiles + g.n_sm - 1) / g.n_sm;
+    const double own = waves * (kb * w.cost + 2.0 + 2.0 * w.bn / 256);
+    if (least < 0 || own < least) { least = own; best = Cut{w.bn, false}; }
+    if (g.epi != TC_RESID || g.A2 || g.H || (w.bn != 128 && w.bn != 256)) continue;
+    const double per_sm = tiles * kb / g.n_sm, share = (per_sm > 1.0 ? per_sm : 1.0) * w.cost * 1.1 + 8.0 + 8.0 * w.bn / 256;
+    if (share < least) { least = share; best = Cut{w.bn, true}; }
+  }
+  return best;
 }
 
 }  // namespace
 
-bool tc_gemm_resid_can_fuse(int M, int N, int n_sm) {
-  // with fewer than two 128 x 128 tiles per SM the k loops are shared among CTAs and no CTA sees a final value
-  return ((M + BM - 1) / BM) * ((N + 127) / 128) >= 2 * n_sm;
+bool tc_gemm_resid_folds_norm(long long M, long long N) {
+  // The folded epilogue reads, adds and writes x in place and takes 10-25 us more than a reduce-add of the same product (8192 x 1536 x
+  // 4096: 111 against 88 us); the RMSNorm launch it saves reads x once.  While x stays in L2 that launch is the cheaper one
+  // (3776 x 1280: whole call 4362 -> 4282 us without folding), from HBM it is not (25240 x 1536: 28.2 -> 27.9 ms with folding, 65536 x 1280:
+  // 38.6 -> 37.5, 65536 x 1536: 128.3 -> 125.5).  Lines between 19 and 155 MB were not tried; L2 holds 126.
+  return M * N * 4 > (80LL << 20);
 }
 
 bool tc_gemm_supported(const TcGemm& g) {
@@ -708,8 +737,7 @@ bool tc_gemm_supported(const TcGemm& g) {
   switch (g.epi) {
     case TC_STORE: return g.N % 8 == 0 && g.ldc % 8 == 0 && al16(g.C);
     case TC_RESID:
-      if (g.H && (g.N % 8 || g.ldh % 8 || !al16(g.H) || (g.H_lo && !al16(g.H_lo)) || !g.gain_next || !g.ss_out || g.A2 ||
-                  !tc_gemm_resid_can_fuse(g.M, g.N, g.n_sm))) return false;
+      if (g.H && (g.N % 8 || g.ldh % 8 || !al16(g.H) || (g.H_lo && !al16(g.H_lo)) || !g.gain_next || !g.ss_out || g.A2)) return false;
       return g.N % 4 == 0 && g.ldx % 4 == 0 && al16(g.X);
     case TC_SWIGLU:
       return g.ffn % 64 == 0 && g.N == 2 * g.ffn && g.ldc % 8 == 0 && al16(g.C) && (!g.C_lo || (g.ld_lo % 8 == 0 && al16(g.C_lo)));
@@ -728,12 +756,11 @@ bool tc_gemm_supported(const TcGemm& g) {
 
 cudaError_t launch_gemm_tc(const TcGemm& g, int* status, cudaStream_t st, int64_t* n_launch) {
   if (!tc_encode_fn()) return cudaErrorNotSupported;
-  const int tiles128 = ((g.M + BM - 1) / BM) * ((g.N + 127) / 128);
-  const bool stream_k = g.epi == TC_RESID && !g.A2 && tiles128 < 2 * g.n_sm;
-  int bn = g.bn;
-  if (bn != 128 && bn != 256) bn = tile_cost(g, 256, stream_k) <= tile_cost(g, 128, stream_k) ? 256 : 128;
+  const Cut cut = choose_cut(g);
+  const int bn = cut.bn;
+  const bool stream_k = cut.shares;
   CUtensorMap ma, ma2, mw, mx;
-  if (g.H && (stream_k || g.epi != TC_RESID)) return cudaErrorInvalidValue;     // see tc_gemm_resid_can_fuse()
+  if (g.H && g.epi != TC_RESID) return cudaErrorInvalidValue;
   if (!make_map(&ma, g.A, g.M, g.K, g.lda, BM)) return cudaErrorInvalidValue;
   if (!make_map(&mw, g.W, g.N, g.K, g.ldw, bn)) return cudaErrorInvalidValue;
   if (g.A2) { if (!make_map(&ma2, g.A2, g.M, g.K, g.lda2, BM)) return cudaErrorInvalidValue; }
@@ -758,7 +785,16 @@ cudaError_t launch_gemm_tc(const TcGemm& g, int* status, cudaStream_t st, int64_
   const long long kblocks = (long long)tiles * ((g.K + BK - 1) / BK);
   int grid = stream_k ? (int)(kblocks < g.n_sm ? kblocks : g.n_sm) : (tiles < g.n_sm ? tiles : g.n_sm);
   ++*n_launch;
-  return bn == 256 ? go_epi<256>(g.epi, ma, ma2, mw, mx, p, grid, st) : go_epi<128>(g.epi, ma, ma2, mw, mx, p, grid, st);
+  switch (bn) {
+    case 160: return go_resid<160>(ma, ma2, mw, mx, p, grid, st);
+    case 224: return go_resid<224>(ma, ma2, mw, mx, p, grid, st);
+    case 192:
+      if (g.epi == TC_QKV) return go<TC_QKV, 192>(ma, ma2, mw, mx, p, grid, st);
+      if (g.epi == TC_PAGED) return go<TC_PAGED, 192>(ma, ma2, mw, mx, p, grid, st);
+      return go_resid<192>(ma, ma2, mw, mx, p, grid, st);
+    case 128: return go_epi<128>(g.epi, ma, ma2, mw, mx, p, grid, st);
+    default: return go_epi<256>(g.epi, ma, ma2, mw, mx, p, grid, st);
+  }
 }
 
 // ---- RoPE table: entry [c / 2][pos] = (cos, sin)(pos * theta^(-2c/hd)) for c and c + 1 (16 bytes), positions contiguous ----

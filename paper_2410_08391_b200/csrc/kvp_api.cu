@@ -653,14 +653,11 @@ static kvp_status prefill_direct(kvp_handle* h, const int32_t* tokens, const int
 
   KVP_TIMED(KVP_CLASS_OTHER, launch_build_index(ctx, cs.cu.data(), batch, T, cu_dev, tok_pos, tok_slot, last_idx, cache->block_table,
                      cache->max_pages_per_seq, cache->n_pages, cache->seq_lens));
-  // RMSNorm is folded into the GEMMs around it wherever both neighbours run on the tensor cores: the residual GEMM
+  // With many tokens RMSNorm is folded into the GEMMs around it wherever both neighbours run on the tensor cores: the residual GEMM
   // that completes x writes bf16(x * gain) and the rows' sums of squares, the next GEMM scales its accumulator rows
   // by 1 / rms.  fused_in[j][0 / 1]: layer j's QKV / gate-up projection takes its operand that way.
   float* norm_ss = (float*)(ws + w.norm_ss);
-  // (the producer needs every output tile to belong to one CTA: enough tiles for the SMs the GEMMs of this call get)
-  const int sms_for_gemms = (h->side != nullptr && !h->timing && T <= 4096 && h->step_sms > 0) ? h->n_sm - h->step_sms : h->n_sm;
-  const bool can_fuse = (h->opt.flags & KVP_OPT_SEPARATE_NORM) == 0 && tc_gemm_resid_can_fuse(T, A.d, h->n_sm) &&
-                        tc_gemm_resid_can_fuse(T, A.d, sms_for_gemms);
+  const bool can_fuse = (h->opt.flags & KVP_OPT_SEPARATE_NORM) == 0 && tc_gemm_resid_folds_norm(T, A.d);
   if (can_fuse) cudaMemsetAsync(norm_ss, 0, (size_t)2 * A.n_layers * T * 4, s);
   auto shape_ok = [&](int K, int N) { return can_fuse && h->opt.dtype == KVP_BF16 && K % 8 == 0 && N % 8 == 0 && A.d % 8 == 0; };
   std::vector<char> fused_in(2 * (h->j_max + 1), 0);
