@@ -9,6 +9,7 @@
 #include <algorithm>
 #include <new>
 
+#include "attn_mma.h"
 #include "attn_tc.h"
 #include "gemm_tc.h"
 #include "kvp_internal.h"
@@ -669,15 +670,13 @@ static kvp_status prefill_direct(kvp_handle* h, const int32_t* tokens, const int
     if (j < h->j_max && L.ffn % 64 == 0 && shape_ok(A.d, 2 * L.ffn) && shape_ok(L.dq, A.d)) fused_in[2 * j + 1] = 1;
   }
   int2* attn_sched = (int2*)(ws + w.attn_sched);
-  // two query tiles per CTA share their K/V tiles; with so few tokens that even the widest layer's pairs
-  // would leave SMs idle, one tile per CTA finishes sooner
   int max_nq = 1;
   for (int j = 0; j <= h->j_max; ++j) max_nq = std::max(max_nq, A.L[j].nq);
-  const int attn_tiles = attn_tc_items(cs.cu.data(), batch, 2) * max_nq < h->n_sm ? 1 : 2;
-  const int attn_items = attn_tc_items(cs.cu.data(), batch, attn_tiles);
+  const int attn_tiles = attn_choose(cs.cu.data(), batch, max_nq, A.L[0].hd);
+  const int attn_items = attn_tiles ? attn_tc_items(cs.cu.data(), batch, attn_tiles) : 0;
   if (h->opt.dtype == KVP_BF16 && (A.L[0].hd == 64 || A.L[0].hd == 128)) {
     KVP_TIMED(KVP_CLASS_OTHER, launch_rope_table(ctx, rope_tab, cs.max_len, A.L[0].hd, A.theta));
-    KVP_TIMED(KVP_CLASS_OTHER, launch_attn_schedule(cu_dev, batch, attn_tiles, attn_sched, ctx.st, ctx.n_launch));
+    if (attn_tiles) KVP_TIMED(KVP_CLASS_OTHER, launch_attn_schedule(cu_dev, batch, attn_tiles, attn_sched, ctx.st, ctx.n_launch));
   }
   // ---- stage 1 + 2: auxiliary prefill, each layer's K/V pushed through the predictor ----
   // (only worth it while a layer's kernels leave SMs idle: with many tokens every kernel fills the GPU by itself)
@@ -846,8 +845,9 @@ static kvp_status prefill_direct(kvp_handle* h, const int32_t* tokens, const int
     if (last) break;
     if (split && attn_items <= 65535 && attn_tc_supported(L.hd, L.nqkv, qkv, L.dq, attn)) {
       TimedScope ts(h, ctx.st, KVP_CLASS_AUX_ATTN);
-      cudaError_t e = launch_attn_tc((const bf16*)qkv, L.nqkv, T, L.nq, L.nkv, L.hd, cu_dev, attn_sched, attn_items, attn_tiles, (bf16*)attn,
-                                     L.dq, ctx.status, ctx.st, ctx.n_launch);
+      cudaError_t e = attn_tiles ? launch_attn_tc((const bf16*)qkv, L.nqkv, T, L.nq, L.nkv, L.hd, cu_dev, attn_sched, attn_items, attn_tiles, (bf16*)attn,
+                                                  L.dq, ctx.status, ctx.st, ctx.n_launch)
+                                 : launch_attn_mma((const bf16*)qkv, L.nqkv, L.nq, L.nkv, L.hd, cu_dev, batch, cs.max_len, (bf16*)attn, L.dq, ctx.st, ctx.n_launch);
       if (e != cudaSuccess && tc_err == cudaSuccess) tc_err = e;
     } else {
       KVP_TIMED(KVP_CLASS_AUX_ATTN, launch_attn_prefill_simt(ctx, qkv, L.nqkv, L.nq, L.nkv, L.hd, cu_dev, batch, T, attn, L.dq));
@@ -1170,11 +1170,11 @@ extern "C" kvp_status kvp_train_forward(kvp_handle* h, const int32_t* tokens, co
                      cache->max_pages_per_seq, cache->n_pages, cache->seq_lens);
   int max_nq = 1;
   for (int i = 0; i < B.n_layers; ++i) max_nq = std::max(max_nq, B.L[i].nq);
-  const int attn_tiles = attn_tc_items(cs.cu.data(), batch, 2) * max_nq < h->n_sm ? 1 : 2;
-  const int attn_items = attn_tc_items(cs.cu.data(), batch, attn_tiles);
+  const int attn_tiles = attn_choose(cs.cu.data(), batch, max_nq, B.L[0].hd);
+  const int attn_items = attn_tiles ? attn_tc_items(cs.cu.data(), batch, attn_tiles) : 0;
   if (h->opt.dtype == KVP_BF16 && (B.L[0].hd == 64 || B.L[0].hd == 128)) {
     launch_rope_table(ctx, rope_tab, cs.max_len, B.L[0].hd, B.theta);
-    launch_attn_schedule(cu_dev, batch, attn_tiles, attn_sched, ctx.st, ctx.n_launch);
+    if (attn_tiles) launch_attn_schedule(cu_dev, batch, attn_tiles, attn_sched, ctx.st, ctx.n_launch);
   }
   // pass 0: the base model's ordinary forward, for its own cache KV_B (consistency terms against the predicted one);
   // pass 1: the forward whose attention reads the predicted cache, for the logits
@@ -1214,8 +1214,10 @@ extern "C" kvp_status kvp_train_forward(kvp_handle* h, const int32_t* tokens, co
         launch_kv_take(ctx, qkv, L.nqkv, L.dq, T, L.nkv, L.hd, tok_slot, cache->k_pools[i], cache->v_pools[i], hp);
       }
       if (split && attn_items <= 65535 && attn_tc_supported(L.hd, L.nqkv, qkv, L.dq, attn)) {
-        cudaError_t e = launch_attn_tc((const bf16*)qkv, L.nqkv, T, L.nq, L.nkv, L.hd, cu_dev, attn_sched, attn_items, attn_tiles,
-                                       (bf16*)attn, L.dq, ctx.status, ctx.st, ctx.n_launch, hp, (bf16*)attn_lo);
+        cudaError_t e = attn_tiles ? launch_attn_tc((const bf16*)qkv, L.nqkv, T, L.nq, L.nkv, L.hd, cu_dev, attn_sched, attn_items, attn_tiles,
+                                                    (bf16*)attn, L.dq, ctx.status, ctx.st, ctx.n_launch, hp, (bf16*)attn_lo)
+                                   : launch_attn_mma((const bf16*)qkv, L.nqkv, L.nq, L.nkv, L.hd, cu_dev, batch, cs.max_len, (bf16*)attn, L.dq, ctx.st,
+                                                     ctx.n_launch, hp, (bf16*)attn_lo);
         if (e != cudaSuccess && tc_err == cudaSuccess) tc_err = e;
       } else {
         if (hp) return fail(h, KVP_ERR_CUDA, "internal: the tensor-core attention refused the training-time forward");
