@@ -199,11 +199,21 @@ enum StepGemvMode : int { GEMV_STORE = 0, GEMV_RESID = 1, GEMV_SWIGLU = 2 };
 void launch_step_gemv(const LaunchCtx&, const void* W, int ldw, int N, int K, const float* x, int ldx,
                       int batch, float* y, int ldy, int mode, int G, int ffn, const float* gain = nullptr,
                       float eps = 0.f, float* scratch_h = nullptr);
-void launch_step_attn(const LaunchCtx&, const float* q, int ldq, int nq, int nkv, int hd, float theta,
-                      const void* kpool, const void* vpool, const int* block_table,
-                      int max_pages_per_seq, int n_pages, const int* seq_lens, int extra, int batch,
-                      int max_keys, float* part, float* out, const float* q_gain = nullptr, float eps = 0.f,
-                      int* split_done = nullptr /* [batch * nkv] ints: lets the attention kernel merge its own key-range splits */);
+// Attention of a single-token step over the paged cache: sequence b attends to seq_lens[b] + extra keys (max_keys bounds that).
+struct StepAttn {
+  const float* q; int ldq;             // query rows (before norm and RoPE); with append, followed by the step's own keys and values
+  int nq, nkv, hd; float theta;
+  void *kpool, *vpool;
+  const int* block_table; int mpps, n_pages;
+  const int* seq_lens; int extra, batch, max_keys;
+  int append;                          // the step's own keys (norm, RoPE) and values join the cache at position seq_lens[b]
+  float* part; float* out;             // split partials; output rows [batch, nq * hd]
+  bf16* xb;                            // or null: the output goes here instead, as bf16 value and remainder rows (step_tc.h)
+  const float *q_gain, *k_gain; float eps;
+  int* split_done;                     // [batch * nkv] ints, zero, left zero; or null (the kernels that merge their own splits need it)
+};
+// true: the output is in xb; false: in out (xb null, or a kernel that writes fp32 rows ran)
+bool launch_step_attn(const LaunchCtx&, const StepAttn&);
 void launch_step_append(const LaunchCtx&, const float* qkv, int nq, int nkv, int hd, float theta,
                         void* kpool, void* vpool, const int* block_table, int max_pages_per_seq,
                         int n_pages, const int* seq_lens, int batch, const float* k_gain = nullptr, float eps = 0.f);
@@ -211,12 +221,9 @@ void launch_argmax(const LaunchCtx&, const float* logits, int batch, int vocab, 
 void launch_add_int(const LaunchCtx&, int* v, int n, int delta);
 int step_attn_splits(int batch, int nkv, int max_keys);
 // warp-level tensor-core variant for the half-precision cache (pages fetched through a swizzling tensor map)
-int step_attn_mma_splits(int batch, int nkv, int max_keys, int upper);
+int step_attn_mma_splits(int batch, int nkv, int hd, int max_keys, int upper);
 bool step_attn_mma_supported(int dtype, int nq, int nkv, int hd, const void* kpool, const void* vpool, int n_pages);
-cudaError_t launch_step_attn_mma(const LaunchCtx&, const float* q, int ldq, int nq, int nkv, int hd, float theta, const void* kpool,
-                                 const void* vpool, const int* block_table, int max_pages_per_seq, int n_pages, const int* seq_lens,
-                                 int extra, int batch, int n_split, int max_keys, float* part, float* out, const float* q_gain,
-                                 float eps, int* split_done);
+cudaError_t launch_step_attn_mma(const LaunchCtx&, const StepAttn& a, int n_split);
 // bandwidth-bound variant for the bf16 cache (pages fetched with bulk asynchronous copies)
 int step_attn_ring_splits(int nq, int nkv, int hd, int batch, int max_keys, int upper);
 bool step_attn_ring_supported(int dtype, int nq, int nkv, int hd, const void* kpool, const void* vpool);

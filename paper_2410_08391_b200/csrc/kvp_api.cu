@@ -234,12 +234,12 @@ bool step_uses_tc(const kvp_handle* h, int batch) {
 }
 
 // y += W x on the tensor cores: operand rows from `src` (RMS-normalised with `gain`, or SwiGLU of a
-// gate/up row, or as they are), output cleared first unless it is the residual stream.
+// gate/up row, or as they are; null: they are there already), output cleared first unless it is the residual stream.
 void step_proj_tc(kvp_handle* h, const LaunchCtx& ctx, const WsLayout& w, char* ws, int mode, const float* src, int ld_src,
                   int K, int batch, const float* gain, int G, const void* W, int N, float* Y, int ldy, bool clear,
                   cudaError_t* err, const void* next_w = nullptr, size_t next_bytes = 0) {
   bf16* XB = (bf16*)(ws + w.xbt);
-  KVP_TIMED(KVP_CLASS_STEP_GEMV, launch_step_prep(ctx, mode, src, ld_src, K, batch, gain, h->base.eps, G, XB, clear ? Y : nullptr, ldy, N));
+  if (src) KVP_TIMED(KVP_CLASS_STEP_GEMV, launch_step_prep(ctx, mode, src, ld_src, K, batch, gain, h->base.eps, G, XB, clear ? Y : nullptr, ldy, N));
   TimedScope ts(h, ctx.st, KVP_CLASS_STEP_GEMV);
   cudaError_t e = launch_step_gemm_tc((const bf16*)W, K, N, K, XB, batch, Y, ldy, h->step_grid_sms, ctx.status, ctx.st, ctx.n_launch, next_w, next_bytes);
   if (e != cudaSuccess && *err == cudaSuccess) *err = e;
@@ -270,17 +270,19 @@ void base_layer_step(kvp_handle* h, const LaunchCtx& ctx, int i, const kvp_cache
   else
     KVP_TIMED(KVP_CLASS_STEP_GEMV, launch_step_gemv(ctx, P + L.wqkv, B.d, n_out, B.d, xb, B.d, batch, qkvb, n_out, GEMV_STORE, 0, 0,
                                                     (const float*)(P + L.attn_norm), B.eps, hb));
-  const float* qn = B.qk_norm ? (const float*)(P + L.q_norm) : nullptr;
-  const float* kn = B.qk_norm ? (const float*)(P + L.k_norm) : nullptr;
-  if (generation)
-    KVP_TIMED(KVP_CLASS_OTHER, launch_step_append(ctx, qkvb, L.nq, L.nkv, L.hd, B.theta, cache->k_pools[i], cache->v_pools[i], cache->block_table,
-                       cache->max_pages_per_seq, cache->n_pages, cache->seq_lens, batch, kn, B.eps));
-  KVP_TIMED(KVP_CLASS_STEP_ATTN, launch_step_attn(ctx, qkvb, n_out, L.nq, L.nkv, L.hd, B.theta, cache->k_pools[i], cache->v_pools[i], cache->block_table,
-                   cache->max_pages_per_seq, cache->n_pages, cache->seq_lens, generation ? 1 : 0, batch, max_keys,
-                   (float*)(ws + w.part), ab, qn, B.eps, (int*)(ws + w.attn_done)));
+  StepAttn a{};
+  a.q = qkvb; a.ldq = n_out; a.nq = L.nq; a.nkv = L.nkv; a.hd = L.hd; a.theta = B.theta; a.kpool = cache->k_pools[i]; a.vpool = cache->v_pools[i];
+  a.block_table = cache->block_table; a.mpps = cache->max_pages_per_seq; a.n_pages = cache->n_pages; a.seq_lens = cache->seq_lens;
+  a.extra = a.append = generation ? 1 : 0; a.batch = batch; a.max_keys = max_keys; a.part = (float*)(ws + w.part); a.out = ab;
+  a.xb = tc ? (bf16*)(ws + w.xbt) : nullptr;      // (the queries' own operand rows have been read)
+  a.q_gain = B.qk_norm ? (const float*)(P + L.q_norm) : nullptr;
+  a.k_gain = B.qk_norm ? (const float*)(P + L.k_norm) : nullptr;
+  a.eps = B.eps; a.split_done = (int*)(ws + w.attn_done);
+  bool in_xb = false;
+  KVP_TIMED(KVP_CLASS_STEP_ATTN, in_xb = launch_step_attn(ctx, a));
   if (tc) {
     float* gub = (float*)(ws + w.gub);
-    step_proj_tc(h, ctx, w, ws, PREP_PLAIN, ab, L.dq, L.dq, batch, nullptr, 0, P + L.wo, B.d, xb, B.d, false, err, P + L.wgu, (size_t)2 * L.ffn * B.d * es);
+    step_proj_tc(h, ctx, w, ws, PREP_PLAIN, in_xb ? nullptr : ab, L.dq, L.dq, batch, nullptr, 0, P + L.wo, B.d, xb, B.d, false, err, P + L.wgu, (size_t)2 * L.ffn * B.d * es);
     step_proj_tc(h, ctx, w, ws, PREP_NORM, xb, B.d, B.d, batch, (const float*)(P + L.ffn_norm), 0, P + L.wgu, 2 * L.ffn, gub, 2 * L.ffn, true, err,
                  P + L.wd, (size_t)B.d * L.ffn * es);
     step_proj_tc(h, ctx, w, ws, PREP_SWIGLU, gub, 2 * L.ffn, L.ffn, batch, nullptr, L.G, P + L.wd, B.d, xb, B.d, false, err, w_after, b_after);
@@ -290,6 +292,13 @@ void base_layer_step(kvp_handle* h, const LaunchCtx& ctx, int i, const kvp_cache
   KVP_TIMED(KVP_CLASS_STEP_GEMV, launch_step_gemv(ctx, P + L.wgu, B.d, L.ffn, B.d, xb, B.d, batch, actb, L.ffn, GEMV_SWIGLU, L.G, L.ffn,
                                                   (const float*)(P + L.ffn_norm), B.eps, hb));
   KVP_TIMED(KVP_CLASS_STEP_GEMV, launch_step_gemv(ctx, P + L.wd, L.ffn, B.d, L.ffn, actb, L.ffn, batch, xb, B.d, GEMV_RESID, 0, 0));
+}
+
+// The start of a step that runs as a chain of launches.
+void base_step_begin(kvp_handle* h, const LaunchCtx& ctx, const WsLayout& w, char* ws, const int* tokens, const int* gather_idx, int batch) {
+  const ModelPlan& B = h->base;
+  cudaMemsetAsync(ws + w.attn_done, 0, (size_t)batch * B.max_nkv * 4, ctx.st);
+  KVP_TIMED(KVP_CLASS_OTHER, launch_embed(ctx, tokens, gather_idx, batch, h->packed + B.embed, B.vocab, B.d, (float*)(ws + w.xb)));
 }
 
 // Which persistent step kernel a call takes: with 16-bit weights and head_dim 64 / 128 the one that multiplies on the
@@ -836,7 +845,7 @@ static kvp_status prefill_direct(kvp_handle* h, const int32_t* tokens, const int
         const int end = last ? h->base.n_layers : ready_after[j];
         if (last) h->step_grid_sms = h->n_sm;          // the prefill has nothing left to run
         if (base_done == 0)
-          launch_embed(sctx, tokens, last_idx, batch, P + h->base.embed, h->base.vocab, h->base.d, (float*)(ws + w.xb));
+          base_step_begin(h, sctx, w, ws, tokens, last_idx, batch);
         for (int i = base_done; i < end; ++i) base_layer_step(h, sctx, i, cache, w, ws, batch, cs.max_len, false, &tc_err);
         if (last) base_head(h, sctx, w, ws, batch, logits_out, first_token, &tc_err);
         base_done = end;
@@ -903,7 +912,7 @@ static kvp_status prefill_direct(kvp_handle* h, const int32_t* tokens, const int
   if (tc_err != cudaSuccess) return fail(h, KVP_ERR_CUDA, "kernel launch: %s", cudaGetErrorString(tc_err));
   // ---- stage 3: one base step per sequence on its last prompt token ----
   if (!piped && !piped_tc && !base_step_fused(h, ctx, cache, w, ws, batch, cs.max_len, false, tokens, last_idx, logits_out, first_token, &tc_err)) {
-    KVP_TIMED(KVP_CLASS_OTHER, launch_embed(ctx, tokens, last_idx, batch, P + h->base.embed, h->base.vocab, h->base.d, (float*)(ws + w.xb)));
+    base_step_begin(h, ctx, w, ws, tokens, last_idx, batch);
     for (int i = 0; i < h->base.n_layers; ++i) base_layer_step(h, ctx, i, cache, w, ws, batch, cs.max_len, false, &tc_err);
     base_head(h, ctx, w, ws, batch, logits_out, first_token, &tc_err);
   }
@@ -1028,7 +1037,7 @@ kvp_status kvp_decode_step(kvp_handle* h, const int32_t* tokens, const int32_t* 
     if (mega_err != cudaSuccess) return fail(h, KVP_ERR_CUDA, "base step launch: %s", cudaGetErrorString(mega_err));
     return check_cuda(h, "kvp_decode_step");
   }
-  KVP_TIMED(KVP_CLASS_OTHER, launch_embed(ctx, tokens, nullptr, batch, h->packed + h->base.embed, h->base.vocab, h->base.d, (float*)(ws + w.xb)));
+  base_step_begin(h, ctx, w, ws, tokens, nullptr, batch);
   for (int i = 0; i < h->base.n_layers; ++i) base_layer_step(h, ctx, i, cache, w, ws, batch, cs.max_len + 1, true, &mega_err);
   base_head(h, ctx, w, ws, batch, logits_out, next_token, &mega_err);
   KVP_TIMED(KVP_CLASS_OTHER, launch_add_int(ctx, cache->seq_lens, batch, 1));

@@ -599,24 +599,24 @@ int step_attn_splits(int batch, int nkv, int max_keys) {
   return n;
 }
 
-void launch_step_attn(const LaunchCtx& ctx, const float* q, int ldq, int nq, int nkv, int hd, float theta,
-                      const void* kpool, const void* vpool, const int* block_table, int mpps, int n_pages,
-                      const int* seq_lens, int extra, int batch, int max_keys, float* part, float* out, const float* q_gain,
-                      float eps, int* split_done) {
-  // every sequence attends to seq_lens[b] + extra keys; max_keys bounds that count (host copy).
-  InvFreq inv;
-  fill_inv_freq(&inv, hd, theta);
-  int n_split = step_attn_splits(batch, nkv, max_keys);
-  dim3 grid(n_split, nkv, batch);
-  if (split_done && step_attn_mma_supported(ctx.dtype, nq, nkv, hd, kpool, vpool, n_pages)) {
+bool launch_step_attn(const LaunchCtx& ctx, const StepAttn& a) {
+  int n_split = step_attn_splits(a.batch, a.nkv, a.max_keys);
+  if (a.split_done && step_attn_mma_supported(ctx.dtype, a.nq, a.nkv, a.hd, a.kpool, a.vpool, a.n_pages)) {
     // half-precision cache, head_dim 64 / 128: warp-level tensor-core kernel (pages through a swizzling tensor map)
-    const int ns = step_attn_mma_splits(batch, nkv, max_keys, n_split);
-    if (ns > 1) cudaMemsetAsync(split_done, 0, (size_t)batch * nkv * sizeof(int), ctx.st);
-    if (launch_step_attn_mma(ctx, q, ldq, nq, nkv, hd, theta, kpool, vpool, block_table, mpps, n_pages, seq_lens, extra, batch, ns, max_keys, part, out,
-                             q_gain, eps, split_done) == cudaSuccess)
-      return;
+    if (launch_step_attn_mma(ctx, a, step_attn_mma_splits(a.batch, a.nkv, a.hd, a.max_keys, n_split)) == cudaSuccess) return a.xb != nullptr;
     cudaGetLastError();      // (a tensor map could not be made: the kernels below take plain pointers)
   }
+  const float *q = a.q, *q_gain = a.q_gain;
+  const void *kpool = a.kpool, *vpool = a.vpool;
+  const int *block_table = a.block_table, *seq_lens = a.seq_lens;
+  const int ldq = a.ldq, nq = a.nq, nkv = a.nkv, hd = a.hd, mpps = a.mpps, n_pages = a.n_pages, extra = a.extra, batch = a.batch, max_keys = a.max_keys;
+  const float theta = a.theta, eps = a.eps;
+  float *part = a.part, *out = a.out;
+  int* split_done = a.split_done;
+  if (a.append) launch_step_append(ctx, q, nq, nkv, hd, theta, a.kpool, a.vpool, block_table, mpps, n_pages, seq_lens, batch, a.k_gain, eps);
+  InvFreq inv;
+  fill_inv_freq(&inv, hd, theta);
+  dim3 grid(n_split, nkv, batch);
   if (step_attn_ring_supported(ctx.dtype, nq, nkv, hd, kpool, vpool)) {
     n_split = step_attn_ring_splits(nq, nkv, hd, batch, max_keys, n_split);
     // up to 4 heads per kv head: the CTA that finishes a group's last split merges it (counters cleared here)
@@ -628,7 +628,8 @@ void launch_step_attn(const LaunchCtx& ctx, const float* q, int ldq, int nq, int
       ++*ctx.n_launch;
       step_attn_merge_kernel<<<dim3(nq, batch), 64, 0, ctx.st>>>(part, nq, hd, n_split, out);
     }
-    return;
+    if (fused) cudaMemsetAsync(split_done, 0, (size_t)batch * nkv * sizeof(int), ctx.st);
+    return false;
   }
   ++*ctx.n_launch;
   if (hd == 16 || hd == 32 || hd == 64 || hd == 128) {
@@ -657,6 +658,7 @@ void launch_step_attn(const LaunchCtx& ctx, const float* q, int ldq, int nq, int
     ++*ctx.n_launch;
     step_attn_merge_kernel<<<dim3(nq, batch), 64, 0, ctx.st>>>(part, nq, hd, n_split, out);
   }
+  return false;
 }
 
 // ---------------------------------------------------------------------------------------

@@ -21,6 +21,10 @@ constexpr int BM = 128, BK = 64;
 constexpr int W_BYTES = BM * BK * 2;
 constexpr int N_THREADS = 192;
 constexpr int SMEM_LIMIT = 220 * 1024;
+// Fewest k blocks of a CTA: a narrow projection (2048 x 2048: 512 blocks) takes 52 SMs, not all.  Every CTA adds a block of partial sums
+// to the output for each tile it touches and holds its SM through the wait for the launch before it, so more CTAs cost other work more
+// than they give: 64 x 123 keys among steps of other batches 1191 -> 1093 us, 8 x 300 974 -> 877; a step by itself 1549 -> 1714.
+constexpr int MIN_KB = 10;
 constexpr size_t STEP_PREFETCH_MAX = 32u << 20;   // bytes of the next weight matrix asked into L2 (L2 holds 126 MB; this kernel streams through it too)
 
 struct Params {
@@ -77,6 +81,7 @@ step_gemm_kernel(const __grid_constant__ CUtensorMap map_w, const __grid_constan
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const uint32_t tmem_cols = max(32, 2 * p.acc_stride);
   pdl_trigger();      // the next kernel's CTAs may take SMs as this kernel's CTAs leave them
+  if (threadIdx.x == 32) { prefetch_tensormap(&map_w); prefetch_tensormap(&map_x); }   // on their way while the rest is set up
 
   if (threadIdx.x == 0) {
     for (int s = 0; s < S; ++s) { mbar_init(full_bar(s), 1); mbar_init(empty_bar(s), 1); }
@@ -318,7 +323,8 @@ cudaError_t launch_step_gemm_tc(const bf16* W, int ldw, int N, int K, const bf16
   cudaError_t e = tc_raise_smem_limit(step_gemm_kernel, SMEM_LIMIT, raised);
   if (e != cudaSuccess) return e;
   const long long total = (long long)((N + BM - 1) / BM) * ((K + BK - 1) / BK);
-  const int grid = (int)(total < n_sm ? total : n_sm);
+  const long long want = (total + MIN_KB - 1) / MIN_KB;
+  const int grid = (int)(want < n_sm ? want : n_sm);
   ++*n_launch;
   return launch_overlapped(step_gemm_kernel, dim3(grid), dim3(N_THREADS), (size_t)smem, st, mw, mx, p);
 }
