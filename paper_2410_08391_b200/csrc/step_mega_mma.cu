@@ -24,19 +24,22 @@
 //   - The accumulation inside an instruction rounds towards zero: one sum over a warp's whole share of K left a step's logits
 //     twice as far from 64 bits as fp32 multiply-adds do (1.1B shape 3.1e-6 against 1.5e-6, 3B shape 4.7e-6 against 2.1e-6, on
 //     the same cache).  So a sum goes through few instructions: with one sequence the hi terms of successive blocks of 32 k
-//     take turns in four columns, with two sequences in two; with two and more sequences a chunk is summed apart and added in
-//     fp32.  Now 1.3e-6 .. 1.7e-6 and 1.8e-6 .. 1.9e-6, for up to 1 % of a step's time (8 heads of 128 a group: 3 %; two sequences:
+//     take turns in four columns, with two sequences in two; a chunk is summed apart and added in fp32.  Now 1.3e-6 .. 1.7e-6 and 1.8e-6 .. 1.9e-6, for up to 1 % of a step's time (8 heads of 128 a group: 3 %; two sequences:
 //     1 .. 5 %).
 //   - The cache pages of an attention item are brought into shared memory by a warp of their own, ahead of the query; the
 //     step's own key and value are taken from the projection's output by the CTA whose key range ends with them (no separate
 //     append phase); RoPE angles are computed once per launch.
 //   - 12 warps of up to 168 registers: next to 220 KB of shared memory there is almost no L1, so every spilled register
-//     is a round trip to L2.  One and four sequences with up to 4 heads a group fit; two sequences, and groups of 5 to 8 heads,
-//     spill 8 to 48 bytes (ptxas), which is part of what those take longer.
-// Measured against the CUDA-core kernel of step_mega.cu (generation step): 1.1B shape 1 x 1100 keys 1557 -> 838 us, 4 x 300
-// 2990 -> 1123 us (that kernel's multiply-adds grow with the batch); 3B shape 1 x 300 2966 -> 2003 us, 4 x 300 5578 -> 2415 us.
-// The bytes of the first take 416 us.  Of the rest, its 169 hand-overs between CTAs (a phase each, two in attention) of about
-// 0.5 us are 85 us; what the other 340 us go to has not been measured phase by phase.
+//     is a round trip to L2.  Up to 4 heads a group nothing spills; groups of 5 to 8 heads spill 16 to 92 bytes (ptxas).
+//   - The instructions of a layer's phases are fetched anew in every layer: a clock trace showed 1080 cycles a tile where its shared-memory
+//     reads take 512, and more of them in proportion to the code's length.  So a group's tiles are ONE loop whose sums wait in shared
+//     memory, not five straight-line copies with their sums in registers.  Generation step, 1.1B shape: 1 x 1100 keys 840 -> 807 us,
+//     2 x 300 888 -> 824, 4 x 300 1109 -> 1075; on the 72 SMs of a piece, with twice the tiles a CTA, more (first token of 1 x 59 1532 -> 1363 us,
+//     1 x 1024 1733 -> 1649); 3B shape 2 x 300 2242 -> 2126, but 1 x 300 1985 -> 2009, 4 x 300 2410 -> 2430 (more chunks of K a tile).
+// Measured against the CUDA-core kernel of step_mega.cu (generation step): 1.1B shape 1 x 1100 keys 1557 -> 807 us, 4 x 300
+// 2990 -> 1075 us (that kernel's multiply-adds grow with the batch); 3B shape 1 x 300 2966 -> 2009 us, 4 x 300 5578 -> 2430 us.
+// The bytes of the first take 416 us.  Of the rest, per layer of 26 us: waits for inputs 0.4-0.7 us a phase, attention's exchange between
+// key ranges 2.8, its wait for the queries 1.3, the tiles of O and down (4.0 us, weights 4.8 on HBM) and gate / up (3.9, 7.0).
 // Every wait is bounded: on expiry DEV_TIMEOUT is recorded, no further wait is started, every CTA runs through its remaining
 // phases without waiting or releasing slots, its loaders stop, and it leaves after copies in flight have had time to land.
 #include <math.h>
@@ -63,6 +66,7 @@ template <int BB> struct Geo {
   static constexpr int KW = KC / CW;         // k elements of a consumer warp
   static constexpr int PITCH = KC * 2 + 64;  // bytes between rows of a slot (64 mod 128: no bank conflicts)
   static constexpr int STAGE = HR * PITCH;
+  static constexpr int TG = BB == 4 ? 5 : 8; // tiles whose sums a CTA holds at a time (the input is fetched anew for every group of them)
   static constexpr int AHEAD = 5;            // slots that the L2 prefetch runs ahead of the loaders (25 MB on 148 SMs)
   // k elements of a chunk of a row of K: as few chunks as possible, of about equal size, whole 64s for every consumer warp
   __device__ __forceinline__ static int chunk(int K) {
@@ -70,7 +74,6 @@ template <int BB> struct Geo {
     return min(KC, ((K + n - 1) / n + 64 * CW - 1) / (64 * CW) * (64 * CW));
   }
 };
-constexpr int TG = 5;                        // tiles whose accumulators a warp holds at a time
 constexpr int MAXG = 8;                      // query heads per kv head (kernels for up to 4 and up to 8)
 constexpr int XCOL = KS * 2 + 64;            // bytes between activation columns of a warp (64 mod 128)
 constexpr int MAX_SLOTS = 12;
@@ -92,12 +95,6 @@ __device__ __forceinline__ void mma16816(float (&d)[4], uint32_t a0, uint32_t a1
   asm volatile("mma.sync.aligned.m16n8k16.row.col.f32.bf16.bf16.f32 {%0, %1, %2, %3}, {%4, %5, %6, %7}, {%8, %9}, {%0, %1, %2, %3};"
                : "+f"(d[0]), "+f"(d[1]), "+f"(d[2]), "+f"(d[3]) : "r"(a0), "r"(a1), "r"(a2), "r"(a3), "r"(b0), "r"(b1));
 }
-// The first product of a sum: no accumulator goes in.
-__device__ __forceinline__ void mma16816_first(float (&d)[4], uint32_t a0, uint32_t a1, uint32_t a2, uint32_t a3, uint32_t b0, uint32_t b1) {
-  asm volatile("mma.sync.aligned.m16n8k16.row.col.f32.bf16.bf16.f32 {%0, %1, %2, %3}, {%4, %5, %6, %7}, {%8, %9}, {%10, %10, %10, %10};"
-               : "=f"(d[0]), "=f"(d[1]), "=f"(d[2]), "=f"(d[3]) : "r"(a0), "r"(a1), "r"(a2), "r"(a3), "r"(b0), "r"(b1), "f"(0.f));
-}
-
 // A projection phase: 4 per layer (q(kv), O, gate/up, down), then the LM head.
 struct Proj { const char* W; int N, K, mode, G, ffn; };
 __device__ __forceinline__ Proj proj_of(const MegaParams& p, int s) {
@@ -145,8 +142,8 @@ __device__ __forceinline__ bool walk_slots(const MegaParams& p, F f) {
     cta_range(g.N, o0, o1);
     const bool sw = g.mode == GEMV_SWIGLU;
     const int TO = sw ? TR / 2 : TR, nt = (o1 - o0 + TO - 1) / TO, kc = Geo<BB>::chunk(g.K), nch = (g.K + kc - 1) / kc;
-    for (int g0 = 0; g0 < nt; g0 += TG) {
-      const int ntg = min(TG, nt - g0);
+    for (int g0 = 0; g0 < nt; g0 += Geo<BB>::TG) {
+      const int ntg = min(Geo<BB>::TG, nt - g0);
       for (int c = 0; c < nch; ++c)
         for (int hs = 0; hs < TR / HR * ntg; ++hs) {
           const int r = (hs * HR & (TR - 1)) + lane;              // row of the tile
@@ -226,9 +223,8 @@ __device__ __forceinline__ void proj_phase(const MegaParams& p, const Work& g, R
   constexpr int NB = BB == 4 ? 2 : 1;          // 8-column groups: two sequences each
   constexpr int HR = Geo<BB>::HR, KW = Geo<BB>::KW, PITCH = Geo<BB>::PITCH, STAGE = Geo<BB>::STAGE;   // (KW: most that a warp's share can be)
   const int kws = g.kc / CW;                   // k elements of a warp's share of a chunk
-  constexpr int RS = TG * TR * BB;
+  constexpr int TG = Geo<BB>::TG, RS = TG * TR * BB;
   constexpr int NJ = KW / 32;                  // 32-k blocks of a warp's share of a chunk
-  constexpr bool OWN_PART = BB > 1;            // chunks are summed apart
   constexpr int NH = KW / KS, QJ = KS / 32;    // ... handled as NH pieces of QJ blocks
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, gr = lane >> 2, t = lane & 3;
   volatile int* s_abort = &sh.abort;
@@ -292,13 +288,6 @@ __device__ __forceinline__ void proj_phase(const MegaParams& p, const Work& g, R
   for (int t0 = 0; t0 < g.nt; t0 += TG) {
     const int ntg = min(TG, g.nt - t0);
     float* red = red0 + (par & 1) * (CW * RS);
-    float acc[TG][NB][4];
-#pragma unroll
-    for (int ti = 0; ti < TG; ++ti)
-#pragma unroll
-      for (int nb = 0; nb < NB; ++nb)
-#pragma unroll
-        for (int e = 0; e < 4; ++e) acc[ti][nb][e] = 0.f;
 #pragma unroll 1
     for (int c = 0; c < nch; ++c) {
       // the chunk's activations: poll until every value carries the wanted tag
@@ -361,82 +350,73 @@ __device__ __forceinline__ void proj_phase(const MegaParams& p, const Work& g, R
       }
       fetch(c + 1 < nch ? c + 1 : 0);
       const int kw = min(kws, g.K - c * g.kc - warp * kws);      // of them within the row
-      float part[NB][4];                       // a tile's share of the chunk
-      auto add_part = [&](int ti) {
+      // One copy of a tile's code for all of them (see the head of the file)
+#pragma unroll 1
+      for (int ti = 0; ti < ntg; ++ti) {
+        // the tile's two slots: rows 0-7 and 8-15 (SwiGLU: the gate rows and the up rows); a last tile may have the first only
+        const bool two = HR < TR && (sw || g.o0 + (t0 + ti) * TR + HR < g.o1);
+        const uint32_t off = gr * PITCH + warp * (kws * 2) + t * 16;
+        const uint32_t a = rg.base + rg.slot * STAGE + off, bar_a = rg.empty + 8u * rg.slot;
+        if (!dead) dead = !quick_wait(rg.full + 8u * rg.slot, rg.phase, s_abort, p.status);
+        rg.next();
+        const uint32_t b = HR == TR ? a + 8 * PITCH : (two ? rg.base + rg.slot * STAGE + off : a), bar_b = rg.empty + 8u * rg.slot;
+        if (two) {
+          if (!dead) dead = !quick_wait(rg.full + 8u * rg.slot, rg.phase, s_abort, p.status);
+          rg.next();
+        }
+        __syncwarp();
+        float part[NB][4];                     // the tile's share of the chunk
 #pragma unroll
         for (int nb = 0; nb < NB; ++nb)
 #pragma unroll
-          for (int e = 0; e < 4; ++e) acc[ti][nb][e] += part[nb][e];
-      };
+          for (int e = 0; e < 4; ++e) part[nb][e] = 0.f;
+        if (kw > 0) {
 #pragma unroll
-      for (int ti = 0; ti < TG; ++ti) {
-        if (ti < ntg) {
-          // the tile's two slots: rows 0-7 and 8-15 (SwiGLU: the gate rows and the up rows); a last tile may have the first only
-          const bool two = HR < TR && (sw || g.o0 + (t0 + ti) * TR + HR < g.o1);
-          const uint32_t off = gr * PITCH + warp * (kws * 2) + t * 16;
-          const uint32_t a = rg.base + rg.slot * STAGE + off, bar_a = rg.empty + 8u * rg.slot;
-          if (!dead) dead = !quick_wait(rg.full + 8u * rg.slot, rg.phase, s_abort, p.status);
-          rg.next();
-          const uint32_t b = HR == TR ? a + 8 * PITCH : (two ? rg.base + rg.slot * STAGE + off : a), bar_b = rg.empty + 8u * rg.slot;
-          if (two) {
-            if (!dead) dead = !quick_wait(rg.full + 8u * rg.slot, rg.phase, s_abort, p.status);
-            rg.next();
-          }
-          __syncwarp();
-          if (kw > 0) {
+          for (int jh = 0; jh < NJ; jh += 2) {
+            if (jh * 32 >= kws) break;
+            uint4 ua[2], ub[2];
 #pragma unroll
-            for (int jh = 0; jh < NJ; jh += 2) {
-              if (jh * 32 >= kws) break;
-              uint4 ua[2], ub[2];
-#pragma unroll
-              for (int j = 0; j < 2; ++j) { ua[j] = lds128(a + (jh + j) * 64); ub[j] = lds128(b + (jh + j) * 64); }
-              if (OWN_PART && jh == 0 && ti > 0) add_part(ti - 1);      // (its last product has long been finished by now)
-              if (kw < kws) {                  // k beyond the rows' end
-#pragma unroll
-                for (int j = 0; j < 2; ++j)
-                  if ((jh + j) * 32 + t * 8 >= kw) { ua[j] = make_uint4(0, 0, 0, 0); ub[j] = ua[j]; }
-              }
+            for (int j = 0; j < 2; ++j) { ua[j] = lds128(a + (jh + j) * 64); ub[j] = lds128(b + (jh + j) * 64); }
+            if (kw < kws) {                    // k beyond the rows' end
 #pragma unroll
               for (int j = 0; j < 2; ++j)
-#pragma unroll
-                for (int nb = 0; nb < NB; ++nb) {
-                  const uint4 bb = NB == 1 ? bq[jh + j] : column(nb, jh + j);
-                  float (&d)[4] = OWN_PART ? part[nb] : acc[ti][nb];
-                  if (OWN_PART && jh + j == 0) mma16816_first(d, ua[j].x, ub[j].x, ua[j].y, ub[j].y, bb.x, bb.y);
-                  else mma16816(d, ua[j].x, ub[j].x, ua[j].y, ub[j].y, bb.x, bb.y);
-                  mma16816(d, ua[j].z, ub[j].z, ua[j].w, ub[j].w, bb.z, bb.w);
-                }
+                if ((jh + j) * 32 + t * 8 >= kw) { ua[j] = make_uint4(0, 0, 0, 0); ub[j] = ua[j]; }
             }
-          }
-          __syncwarp();
-          if (lane == 0 && !dead) { mbar_arrive(bar_a); if (two) mbar_arrive(bar_b); }
-          if (OWN_PART && ti + 1 == ntg && kw > 0) add_part(ti);
-        }
-      }
-      dead = __any_sync(0xffffffffu, dead);    // (also: every lane has read this chunk's columns)
-    }
-    // ---- the group's outputs: hi + mid + lo columns, then the sum over the warps' k ranges
 #pragma unroll
-    for (int ti = 0; ti < TG; ++ti) {
-      if (ti < ntg) {
+            for (int j = 0; j < 2; ++j)
+#pragma unroll
+              for (int nb = 0; nb < NB; ++nb) {
+                const uint4 bb = NB == 1 ? bq[jh + j] : column(nb, jh + j);
+                mma16816(part[nb], ua[j].x, ub[j].x, ua[j].y, ub[j].y, bb.x, bb.y);
+                mma16816(part[nb], ua[j].z, ub[j].z, ua[j].w, ub[j].w, bb.z, bb.w);
+              }
+          }
+        }
+        __syncwarp();
+        if (lane == 0 && !dead) { mbar_arrive(bar_a); if (two) mbar_arrive(bar_b); }
+        // hi + mid + lo columns; the chunks of K add up in this warp's part of `red`
 #pragma unroll
         for (int nb = 0; nb < NB; ++nb) {
           const bool pair = BB < 4 || !(t & 1);
-          float v0 = acc[ti][nb][0] + (pair ? acc[ti][nb][1] : 0.f), v1 = acc[ti][nb][2] + (pair ? acc[ti][nb][3] : 0.f);
+          float v0 = part[nb][0] + (pair ? part[nb][1] : 0.f), v1 = part[nb][2] + (pair ? part[nb][3] : 0.f);
           v0 += __shfl_xor_sync(0xffffffffu, v0, 1);
           v1 += __shfl_xor_sync(0xffffffffu, v1, 1);
           if (BB == 1) {
             v0 += __shfl_xor_sync(0xffffffffu, v0, 2);
             v1 += __shfl_xor_sync(0xffffffffu, v1, 2);
           }
-          const int b = nb * 2 + (t >> 1);
-          if (!(t & 1) && b < BB) {
-            red[warp * RS + (ti * TR + gr) * BB + b] = v0;
-            red[warp * RS + (ti * TR + gr + 8) * BB + b] = v1;
+          const int bs = nb * 2 + (t >> 1);
+          if (!(t & 1) && bs < BB) {
+            float* d0 = red + warp * RS + (ti * TR + gr) * BB + bs;
+            float* d1 = d0 + 8 * BB;
+            if (c > 0) { v0 += *d0; v1 += *d1; }
+            *d0 = v0; *d1 = v1;
           }
         }
       }
+      dead = __any_sync(0xffffffffu, dead);    // (also: every lane has read this chunk's columns)
     }
+    // ---- the group's outputs: the sum over the warps' k ranges
     if (t0 == 0 && g.gain) {
 #pragma unroll
       for (int b = 0; b < BB; ++b) {
@@ -858,7 +838,7 @@ __global__ void __launch_bounds__(NT, 1) step_mega_mma_kernel(const __grid_const
   unsigned char* scr = sm + pl.scr_off;
   const uint32_t xp = smem_u32(scr) + warp * (3 * BB * XCOL);
   float* red = reinterpret_cast<float*>(scr + CW * 3 * BB * XCOL);
-  unsigned char* attn_scr = scr + CW * 3 * BB * XCOL + 2 * CW * TG * TR * BB * 4;
+  unsigned char* attn_scr = scr + CW * 3 * BB * XCOL + 2 * CW * Geo<BB>::TG * TR * BB * 4;
   bool dead = false;
   int par = 0;
   {
@@ -918,7 +898,7 @@ constexpr size_t SMEM_ROOM = SMEM_LIMIT - sizeof(Shared) - 256;      // dynamic 
 // the arithmetic on the one before.)
 bool make_plan(int batch, int hd, int max_group, Plan* pl, size_t* bytes) {
   const int bb = batch <= 1 ? 1 : (batch == 2 ? 2 : 4);
-  const size_t proj = (size_t)CW * 3 * bb * XCOL + (size_t)2 * CW * TG * TR * bb * 4;
+  const size_t proj = (size_t)CW * 3 * bb * XCOL + (size_t)2 * CW * (bb == 4 ? Geo<4>::TG : Geo<1>::TG) * TR * bb * 4;
   const size_t attn = (size_t)((max_group <= 4 ? 4 : MAXG) + CW * max_group) * hd * 4 + (size_t)2 * CW * max_group * 4;
   const size_t scr = (proj + attn + 127) / 128 * 128;
   const int STAGE = bb == 4 ? Geo<4>::STAGE : Geo<1>::STAGE;
