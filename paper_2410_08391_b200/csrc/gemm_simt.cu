@@ -4,53 +4,83 @@
 #include "common.cuh"
 
 namespace {
-constexpr int BM = 64, BN = 64, BK = 16;
-
-// 64x64 tile, K step 16, 256 threads, 4x4 outputs per thread.
-template <class T, int EPI>
-__global__ void __launch_bounds__(256) gemm_simt_kernel(GemmArgs g) {
-  __shared__ float As[BK][BM + 4];
-  __shared__ float Ws[BK][BN + 4];
+// TS x TS tile, 256 threads, R x R outputs per thread (R = TS / 16).  A thread stages 8 consecutive k of one row of each operand; the
+// next k block is on its way to registers while this one is multiplied.  Small problems are a chain of memory latencies: 32 x 32
+// tiles with 64 k at a time give them four times the CTAs and a quarter of the trips.
+// Every output is one chain of multiply-adds in the order of k, whatever the tile.
+template <class T, int EPI, int TS>
+__global__ void __launch_bounds__(256) gemm_simt_kernel(GemmArgs g, int vec) {
+  constexpr int R = TS / 16, BK = 2048 / TS, KT = BK / 8;
+  __shared__ __align__(16) float As[BK][TS + 4];
+  __shared__ __align__(16) float Ws[BK][TS + 4];
+  pdl_trigger();
   const T* __restrict__ A = (const T*)g.A;
   const T* __restrict__ W = (const T*)g.W;
-  int m0 = blockIdx.y * BM, n0 = blockIdx.x * BN;
-  const T* __restrict__ A2 = (g.A2 && n0 + BN > g.split_begin) ? (const T*)g.A2 : nullptr;
+  int m0 = blockIdx.y * TS, n0 = blockIdx.x * TS;
+  const T* __restrict__ A2 = (g.A2 && n0 + TS > g.split_begin) ? (const T*)g.A2 : nullptr;
   int tid = threadIdx.x;
   int tx = tid & 15, ty = tid >> 4;
-  float acc[4][4] = {};
-  int lr = tid >> 2, lk = (tid & 3) * 4;   // each thread stages 4 consecutive k of one row
+  float acc[R][R] = {};
+  const int lr = tid / KT, lk = (tid % KT) * 8, am = m0 + lr, wn = n0 + lr;
+  float av[8], wv[8];
+  auto load8 = [&](const T* row, bool ok, int k, float* v) {
+    if (!ok || k >= g.K) {
+#pragma unroll
+      for (int i = 0; i < 8; ++i) v[i] = 0.f;
+    } else if (vec) {                        // rows of whole 16-byte pieces: K, the strides and the addresses allow it
+#pragma unroll
+      for (int i = 0; i < 8; i += 16 / (int)sizeof(T)) {
+        const uint4 u = k + i < g.K ? *reinterpret_cast<const uint4*>(row + k + i) : make_uint4(0, 0, 0, 0);
+        const T* e = reinterpret_cast<const T*>(&u);
+#pragma unroll
+        for (int q = 0; q < 16 / (int)sizeof(T); ++q) v[i + q] = to_f(e[q]);
+      }
+    } else {
+#pragma unroll
+      for (int i = 0; i < 8; ++i) v[i] = k + i < g.K ? to_f(row[k + i]) : 0.f;
+    }
+  };
+  auto load = [&](int k0) {
+    load8(A + (size_t)am * g.lda, am < g.M, k0 + lk, av);
+    if (A2) {
+      float a2[8];
+      load8(A2 + (size_t)am * g.lda2, am < g.M, k0 + lk, a2);
+#pragma unroll
+      for (int i = 0; i < 8; ++i) av[i] += a2[i];
+    }
+  };
+  load8(W + (size_t)wn * g.ldw, wn < g.N, lk, wv);      // a weight: does not wait for the kernel before this one
+  pdl_wait();
+  load(0);
   for (int k0 = 0; k0 < g.K; k0 += BK) {
 #pragma unroll
-    for (int i = 0; i < 4; ++i) {
-      int k = k0 + lk + i;
-      int am = m0 + lr, wn = n0 + lr;
-      float av = (am < g.M && k < g.K) ? to_f(A[(size_t)am * g.lda + k]) : 0.f;
-      if (A2 && am < g.M && k < g.K) av += to_f(A2[(size_t)am * g.lda2 + k]);
-      As[lk + i][lr] = av;
-      Ws[lk + i][lr] = (wn < g.N && k < g.K) ? to_f(W[(size_t)wn * g.ldw + k]) : 0.f;
-    }
+    for (int i = 0; i < 8; ++i) { As[lk + i][lr] = av[i]; Ws[lk + i][lr] = wv[i]; }
     __syncthreads();
-#pragma unroll
+    if (k0 + BK < g.K) {
+      load(k0 + BK);
+      load8(W + (size_t)wn * g.ldw, wn < g.N, k0 + BK + lk, wv);
+    }
+#pragma unroll 16
     for (int k = 0; k < BK; ++k) {
-      float a[4], w[4];
+      float a[R], w[R];
 #pragma unroll
-      for (int i = 0; i < 4; ++i) { a[i] = As[k][ty * 4 + i]; w[i] = Ws[k][tx * 4 + i]; }
+      for (int i = 0; i < R; ++i) { a[i] = As[k][ty * R + i]; w[i] = Ws[k][tx * R + i]; }
 #pragma unroll
-      for (int i = 0; i < 4; ++i)
+      for (int i = 0; i < R; ++i)
 #pragma unroll
-        for (int j = 0; j < 4; ++j) acc[i][j] = fmaf(a[i], w[j], acc[i][j]);
+        for (int j = 0; j < R; ++j) acc[i][j] = fmaf(a[i], w[j], acc[i][j]);
     }
     __syncthreads();
   }
 #pragma unroll
-  for (int i = 0; i < 4; ++i) {
-    int m = m0 + ty * 4 + i;
+  for (int i = 0; i < R; ++i) {
+    int m = m0 + ty * R + i;
     if (m >= g.M) continue;
     int slot = 0;
     if (EPI == EPI_PAGED) { slot = g.paged.tok_slot[m]; if (slot < 0) continue; }
 #pragma unroll
-    for (int j = 0; j < 4; ++j) {
-      int n = n0 + tx * 4 + j;
+    for (int j = 0; j < R; ++j) {
+      int n = n0 + tx * R + j;
       if (n >= g.N) continue;
       float v = acc[i][j];
       if (EPI == EPI_STORE) {
@@ -78,9 +108,15 @@ __global__ void __launch_bounds__(256) gemm_simt_kernel(GemmArgs g) {
 
 void launch_gemm_simt(const LaunchCtx& ctx, const GemmArgs& g, int epi) {
   if (g.M == 0 || g.N == 0) return;
-  dim3 grid((g.N + BN - 1) / BN, (g.M + BM - 1) / BM);
+  // 64 x 64 tiles where they give every SM one
+  const bool small = (long long)((g.N + 63) / 64) * ((g.M + 63) / 64) < 148;
+  const int ts = small ? 32 : 64, per = ctx.dtype == 0 ? 4 : 8;
+  const dim3 grid((g.N + ts - 1) / ts, (g.M + ts - 1) / ts);
+  const int vec = g.K % per == 0 && g.lda % per == 0 && g.ldw % per == 0 && (!g.A2 || g.lda2 % per == 0) &&
+                  (((uintptr_t)g.A | (uintptr_t)g.W | (uintptr_t)g.A2) & 15) == 0;
   ++*ctx.n_launch;
-#define GO(T, E) gemm_simt_kernel<T, E><<<grid, 256, 0, ctx.st>>>(g)
+#define GO(T, E) (small ? launch_overlapped(gemm_simt_kernel<T, E, 32>, grid, dim3(256), 0, ctx.st, g, vec) \
+                        : launch_overlapped(gemm_simt_kernel<T, E, 64>, grid, dim3(256), 0, ctx.st, g, vec))
   if (ctx.dtype == 0) {
     if (epi == EPI_STORE) GO(float, EPI_STORE); else if (epi == EPI_RESID) GO(float, EPI_RESID); else if (epi == EPI_STORE32) GO(float, EPI_STORE32); else GO(float, EPI_PAGED);
   } else {
@@ -103,6 +139,8 @@ __global__ void __launch_bounds__(256) attn_prefill_simt_kernel(const T* __restr
                                                                 const int* __restrict__ cu, int batch, T* __restrict__ out,
                                                                 int ldo, float scale) {
   extern __shared__ float smem[];
+  pdl_trigger();
+  pdl_wait();
   int ldk = hd + 1;
   float* Ks = smem;                       // [AKV][hd+1]
   float* Vs = Ks + AKV * ldk;             // [AKV][hd+1]
@@ -193,10 +231,10 @@ void launch_attn_prefill_simt(const LaunchCtx& ctx, const void* qkv, int ld, int
   if (ctx.dtype == 0) {
     static bool raised[TC_MAX_DEVICES] = {};
     tc_raise_smem_limit(attn_prefill_simt_kernel<float>, ATTN_SMEM_MAX, raised);
-    attn_prefill_simt_kernel<float><<<grid, 256, smem, ctx.st>>>((const float*)qkv, ld, nq, nkv, hd, cu_dev, batch, (float*)out, ldo, scale);
+    launch_overlapped(attn_prefill_simt_kernel<float>, grid, dim3(256), smem, ctx.st, (const float*)qkv, ld, nq, nkv, hd, cu_dev, batch, (float*)out, ldo, scale);
   } else {
     static bool raised[TC_MAX_DEVICES] = {};
     tc_raise_smem_limit(attn_prefill_simt_kernel<bf16>, ATTN_SMEM_MAX, raised);
-    attn_prefill_simt_kernel<bf16><<<grid, 256, smem, ctx.st>>>((const bf16*)qkv, ld, nq, nkv, hd, cu_dev, batch, (bf16*)out, ldo, scale);
+    launch_overlapped(attn_prefill_simt_kernel<bf16>, grid, dim3(256), smem, ctx.st, (const bf16*)qkv, ld, nq, nkv, hd, cu_dev, batch, (bf16*)out, ldo, scale);
   }
 }

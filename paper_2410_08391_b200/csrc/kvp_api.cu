@@ -307,8 +307,12 @@ bool mega_uses_mma(const kvp_handle* h, int batch) {
   return h->opt.dtype == KVP_BF16 && step_mega_mma_supported(batch, h->base.L[0].hd, h->base.max_group, h->base.d, h->step_sms > 0 ? h->step_sms : h->n_sm);
 }
 cudaError_t launch_mega(kvp_handle* h, const MegaParams& p, int k_max, int n_sm, cudaStream_t st) {
-  return mega_uses_mma(h, p.batch) ? launch_step_mega_mma(p, h->base.max_group, n_sm, st, &h->n_launch)
-                                   : launch_step_mega(p, h->opt.dtype, k_max, n_sm, st, &h->n_launch);
+  if (mega_uses_mma(h, p.batch)) return launch_step_mega_mma(p, h->base.max_group, n_sm, st, &h->n_launch);
+  // The CUDA-core kernel gives a row to a warp, 16 warps to a CTA, and its grid-wide barriers cost the more the more CTAs meet (and a
+  // launch that takes every SM keeps other calls off them): a model whose widest projection has fewer rows takes fewer CTAs.
+  // fp32 pair of test size, 1 x 64 tokens: 148 and 72 CTAs 102 us, 43 CTAs 50 us (among other calls).
+  const int rows = std::max(std::max(2 * h->base.max_ffn, h->base.max_nqkv), std::max(h->base.d, h->base.vocab));
+  return launch_step_mega(p, h->opt.dtype, k_max, std::min(n_sm, std::max(16, (rows + 15) / 16)), st, &h->n_launch);
 }
 
 // Parameters of the persistent step kernel for this call; false = the kernel does not apply.
