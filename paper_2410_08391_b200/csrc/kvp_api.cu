@@ -628,10 +628,34 @@ kvp_status kvp_load_weights(kvp_handle* h, const kvp_tensor* tensors, int32_t n,
   return check_cuda(h, "kvp_load_weights");
 }
 
+// SMs that the step's pieces take beside the prefill of a call; 0: the step runs after it, on all of them.  Both are estimated in
+// microseconds, the prefill from its launches and operations, the step (on all SMs) from its weights.  Prompts whose prefill is the
+// longer by far want the SMs themselves; where it is over long before the step, a caller that waits is served sooner by one after the
+// other (while other calls keep the GPU busy, 72 SMs get more done).  Alone / among other calls, us, with 0, 48, 72, 88 SMs:
+//   1.1B 1 x 59 (prefill / step 0.7): 1394 / 1056, 1606 / 880, 1354 / 948, 1349 / 1234;  1 x 1024 (1.6): 2064 / 1708, 1963 / 1603,
+//   1893 / 1628, 2000 / 1889;  3 x 1000 (2.5): 3486 / 3266, 3227 / 3038, 3446 / 3211, 3755 / 3398;  1 x 3500 (3.7): 4001 / 3878, 3904 / 3849,
+//   4151 / 3810, 4807 / 3919;  layer-pruned 1 x 1000 (2.5): 2567 / 2356, 2313 / 2170, 2605 / 2252, 2892 / 2437;
+//   3B 1 x 59 (0.35): 2931 / 2561, 4957 / 2615, 3782 / 2446, 3361 / 3342;  1 x 800 (0.8): 3916 / 3461, 5237 / 3092, 4124 / 3274, 3912 / 3724.
+int step_piece_sms(const kvp_handle* h, int batch, const CallShape& cs, bool blocking) {
+  if (h->step_sms == 0 || h->opt.dtype != KVP_BF16) return h->step_sms;
+  const ModelPlan &A = h->aux, &B = h->base;
+  double pairs = 0, ops = 0, bytes = (double)B.vocab * B.d * h->es;
+  for (int b = 0; b < batch; ++b) { const double n = cs.cu[b + 1] - cs.cu[b]; pairs += n * (n + 1) / 2; }
+  for (int j = 0; j <= h->j_max; ++j) ops += 2.0 * cs.total * A.d * (A.L[j].nqkv + A.L[j].dq + 3.0 * A.L[j].ffn) + 4.0 * A.L[j].dq * pairs;
+  for (const LayerPlan& L : B.L) bytes += (2.0 * L.dq + 3.0 * L.ffn) * B.d * h->es;
+  const double prefill = 36.0 * (h->j_max + 1) + ops / 8e8, step = bytes / 3.2e6 * (1.0 + 0.1 * (batch - 1));      // microseconds
+  if (prefill > 1.9 * step) {
+    const int few = 48;
+    return few < h->step_sms && step_mega_mma_supported(batch, B.L[0].hd, B.max_group, B.d, few) ? few : h->step_sms;
+  }
+  if (blocking && prefill < 0.5 * step) return 0;
+  return h->step_sms;
+}
+
 // Enqueues every kernel of the time-to-first-token path on `stream` (validates first).
 static kvp_status prefill_direct(kvp_handle* h, const int32_t* tokens, const int32_t* lengths, int32_t batch,
                                  const kvp_cache* cache, void* workspace, size_t workspace_bytes, float* logits_out,
-                                 int32_t* first_token, void* stream) {
+                                 int32_t* first_token, void* stream, bool blocking) {
   CallShape cs;
   kvp_status st = common_checks(h, lengths, batch, cache, workspace, 0, &cs);
   if (st != KVP_OK) return st;
@@ -699,8 +723,10 @@ static kvp_status prefill_direct(kvp_handle* h, const int32_t* tokens, const int
   // layer below them) is complete once auxiliary layer j has gone through the predictor.
   MegaParams mp;
   int mega_kmax = 0, piece = 0, base_done = 0;
-  bool piped = fork && h->step_sms > 0 && h->j_max + 1 <= MEGA_COUNTERS &&
-               mega_prepare(h, ctx, cache, w, ws, batch, cs.max_len, false, tokens, last_idx, logits_out, first_token, &mp, &mega_kmax);
+  const bool one_kernel = fork && h->step_sms > 0 && h->j_max + 1 <= MEGA_COUNTERS &&
+                          mega_prepare(h, ctx, cache, w, ws, batch, cs.max_len, false, tokens, last_idx, logits_out, first_token, &mp, &mega_kmax);
+  const int piece_sms = one_kernel ? step_piece_sms(h, batch, cs, blocking) : 0;
+  const bool piped = piece_sms > 0;
   std::vector<int> ready_after(h->j_max + 2, 0);      // ready_after[j] = base layers runnable after auxiliary layer j
   if (piped) {
     int dep = 0, i = 0;
@@ -709,16 +735,16 @@ static kvp_status prefill_direct(kvp_handle* h, const int32_t* tokens, const int
       ready_after[j] = i;
     }
     mega_clear(h, mp, w, ws, s);
-    h->gemm_sms = h->n_sm - h->step_sms;
+    h->gemm_sms = h->n_sm - piece_sms;
     // key-range splits of the CUDA-core kernel's pieces: one attention item per CTA of the piece (more make two rounds); the other
     // kernel splits by its own grid
     for (int i = 0; i < h->base.n_layers; ++i)
-      mp.layers[i].n_split = std::max(1, std::min(mp.layers[i].n_split, h->step_sms / (batch * h->base.L[i].nkv)));
+      mp.layers[i].n_split = std::max(1, std::min(mp.layers[i].n_split, piece_sms / (batch * h->base.L[i].nkv)));
   }
   // More than 4 sequences: the step is a chain of short per-layer kernels bound by launch latency; the same
   // pieces go to the step stream as plain launches.  Their projections size their grids for step_tc_sms SMs;
   // the prefill's GEMMs keep the whole GPU (measured: restricting them costs more than the step gains).
-  const bool piped_tc = !piped && fork && h->step_sms > 0 && h->step_tc_sms > 0 && step_uses_tc(h, batch);
+  const bool piped_tc = !one_kernel && fork && h->step_sms > 0 && h->step_tc_sms > 0 && step_uses_tc(h, batch);
   if (piped_tc) {
     int dep = 0, i = 0;
     for (int j = 0; j <= h->j_max; ++j) {
@@ -838,7 +864,7 @@ static kvp_status prefill_direct(kvp_handle* h, const int32_t* tokens, const int
         q.layer_begin = base_done; q.layer_end = last ? h->base.n_layers : ready_after[j];
         q.do_embed = base_done == 0; q.do_head = last; q.counter_idx = piece++;
         // the last piece starts when the prefill has nothing left to run: it takes every SM
-        cudaError_t e = launch_mega(h, q, mega_kmax, last ? h->n_sm : h->step_sms, h->step_st);
+        cudaError_t e = launch_mega(h, q, mega_kmax, last ? h->n_sm : piece_sms, h->step_st);
         if (e != cudaSuccess && tc_err == cudaSuccess) tc_err = e;
         base_done = q.layer_end;
       }
@@ -928,9 +954,10 @@ static kvp_status prefill_direct(kvp_handle* h, const int32_t* tokens, const int
 // time.  The first call with a given set of arguments records the schedule into a CUDA graph;
 // later calls with the same arguments replay it (token values may change, they are read on the
 // device).  Everything baked into the kernels' parameters is part of the key.
-kvp_status kvp_prefill_predict(kvp_handle* h, const int32_t* tokens, const int32_t* lengths, int32_t batch,
-                               const kvp_cache* cache, void* workspace, size_t workspace_bytes, float* logits_out,
-                               int32_t* first_token, void* stream) {
+// blocking: the caller waits for the result (kvp_prefill_predict_host).
+static kvp_status prefill_recorded(kvp_handle* h, const int32_t* tokens, const int32_t* lengths, int32_t batch, const kvp_cache* cache,
+                                   void* workspace, size_t workspace_bytes, float* logits_out, int32_t* first_token, void* stream,
+                                   bool blocking) {
   cudaStream_t s = (cudaStream_t)stream;
   cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
   // (the legacy default stream cannot record)
@@ -938,16 +965,16 @@ kvp_status kvp_prefill_predict(kvp_handle* h, const int32_t* tokens, const int32
                   batch <= KVP_MAX_BATCH && cudaStreamIsCapturing(s, &cap) == cudaSuccess && cap == cudaStreamCaptureStatusNone;
   if (!graph_ok) {
     cudaGetLastError();
-    return prefill_direct(h, tokens, lengths, batch, cache, workspace, workspace_bytes, logits_out, first_token, stream);
+    return prefill_direct(h, tokens, lengths, batch, cache, workspace, workspace_bytes, logits_out, first_token, stream, blocking);
   }
   std::vector<uint64_t> key;
-  key.reserve(12 + batch + 2 * h->base.n_layers);
+  key.reserve(13 + batch + 2 * h->base.n_layers);
   key.push_back((uint64_t)(uintptr_t)tokens); key.push_back((uint64_t)batch);
   key.push_back((uint64_t)(uintptr_t)workspace); key.push_back((uint64_t)workspace_bytes);
   key.push_back((uint64_t)(uintptr_t)logits_out); key.push_back((uint64_t)(uintptr_t)first_token);
   key.push_back((uint64_t)(uintptr_t)cache->block_table); key.push_back((uint64_t)(uintptr_t)cache->seq_lens);
   key.push_back((uint64_t)cache->max_pages_per_seq); key.push_back((uint64_t)cache->n_pages);
-  key.push_back((uint64_t)(uintptr_t)h->packed); key.push_back((uint64_t)(uintptr_t)s);
+  key.push_back((uint64_t)(uintptr_t)h->packed); key.push_back((uint64_t)(uintptr_t)s); key.push_back((uint64_t)blocking);
   for (int b = 0; b < batch; ++b) key.push_back((uint64_t)(uint32_t)lengths[b]);
   for (int i = 0; i < h->base.n_layers; ++i) {
     key.push_back((uint64_t)(uintptr_t)cache->k_pools[i]);
@@ -965,9 +992,9 @@ kvp_status kvp_prefill_predict(kvp_handle* h, const int32_t* tokens, const int32
   int64_t n0 = h->n_launch;
   if (cudaStreamBeginCapture(s, cudaStreamCaptureModeThreadLocal) != cudaSuccess) {
     cudaGetLastError();
-    return prefill_direct(h, tokens, lengths, batch, cache, workspace, workspace_bytes, logits_out, first_token, stream);
+    return prefill_direct(h, tokens, lengths, batch, cache, workspace, workspace_bytes, logits_out, first_token, stream, blocking);
   }
-  kvp_status st = prefill_direct(h, tokens, lengths, batch, cache, workspace, workspace_bytes, logits_out, first_token, stream);
+  kvp_status st = prefill_direct(h, tokens, lengths, batch, cache, workspace, workspace_bytes, logits_out, first_token, stream, blocking);
   cudaGraph_t graph = nullptr;
   cudaError_t ce = cudaStreamEndCapture(s, &graph);
   if (st != KVP_OK) {               // argument error: nothing was launched, drop the empty capture
@@ -982,7 +1009,7 @@ kvp_status kvp_prefill_predict(kvp_handle* h, const int32_t* tokens, const int32
     cudaGetLastError();
     h->n_launch = n0;
     h->use_graph = false;           // this context cannot record: run directly from now on
-    return prefill_direct(h, tokens, lengths, batch, cache, workspace, workspace_bytes, logits_out, first_token, stream);
+    return prefill_direct(h, tokens, lengths, batch, cache, workspace, workspace_bytes, logits_out, first_token, stream, blocking);
   }
   cudaGraphDestroy(graph);
   int64_t launches = h->n_launch - n0;
@@ -997,6 +1024,12 @@ kvp_status kvp_prefill_predict(kvp_handle* h, const int32_t* tokens, const int32
   if (cudaGraphLaunch(exec, s) != cudaSuccess) return check_cuda(h, "cudaGraphLaunch");
   h->n_launch += launches;
   return KVP_OK;
+}
+
+kvp_status kvp_prefill_predict(kvp_handle* h, const int32_t* tokens, const int32_t* lengths, int32_t batch,
+                               const kvp_cache* cache, void* workspace, size_t workspace_bytes, float* logits_out,
+                               int32_t* first_token, void* stream) {
+  return prefill_recorded(h, tokens, lengths, batch, cache, workspace, workspace_bytes, logits_out, first_token, stream, false);
 }
 
 kvp_status kvp_prefill_predict_host(kvp_handle* h, const int32_t* tokens_host, const int32_t* lengths, int32_t batch,
@@ -1014,7 +1047,7 @@ kvp_status kvp_prefill_predict_host(kvp_handle* h, const int32_t* tokens_host, c
   int32_t* first_dev = (int32_t*)(ws + w.first_stage);
   if (cudaMemcpyAsync(tok_dev, tokens_host, (size_t)cs.total * 4, cudaMemcpyHostToDevice, s) != cudaSuccess)
     return check_cuda(h, "token upload");
-  st = kvp_prefill_predict(h, tok_dev, lengths, batch, cache, workspace, workspace_bytes, logits_dev, first_dev, stream);
+  st = prefill_recorded(h, tok_dev, lengths, batch, cache, workspace, workspace_bytes, logits_dev, first_dev, stream, true);
   if (st != KVP_OK) return st;
   if (logits_host)
     cudaMemcpyAsync(logits_host, logits_dev, (size_t)batch * h->base.vocab * 4, cudaMemcpyDeviceToHost, s);

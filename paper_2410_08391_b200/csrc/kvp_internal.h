@@ -83,9 +83,8 @@ struct kvp_handle {
   // The base step at small batch is one persistent kernel, a chain of short phases, the auxiliary prefill a chain
   // of tensor-core kernels: base layer i only needs the predicted cache of layers <= i, so the step runs in
   // pieces (one per auxiliary layer that completes some base layers' cache) on a stream of its own, on
-  // `step_sms` SMs, while the prefill's kernels size their grids for the others.  0 = the step runs after the prefill.
-  // 72 of 148: the compromise over eight calls of 59 to 4000 tokens (48 / 60 / 84 / 96 SMs run at 0.86-1.20 / 0.92-1.19 / 0.90-1.01 /
-  // 0.81-1.00 of its speed on the 1.1B pair, 0.76-1.05 / 0.87-1.01 / 0.92-1.09 / 0.84-1.19 on the 3B pair).
+  // `step_sms` SMs (most calls; step_piece_sms() chooses), while the prefill's kernels size their grids for the others.  0 = the step runs
+  // after the prefill.
   cudaStream_t step_st = nullptr;
   cudaEvent_t ev_step = nullptr;
   int step_sms = 72;
