@@ -100,8 +100,8 @@ typedef struct {
  *                          is the projection's epilogue; K_A / V_A reach it through shared memory), used for calls
  *                          with at least one 128-token block per SM.  Off by default: it measured slower than the
  *                          projection GEMM followed by a predictor GEMM.
- *   KVP_OPT_SEPARATE_NORM  RMSNorm as a kernel of its own in front of every projection.  By default, wherever every
- *                          output tile of the residual GEMMs belongs to one CTA (calls of some thousand tokens and
+ *   KVP_OPT_SEPARATE_NORM  RMSNorm as a kernel of its own in front of every projection.  By default, where the residual
+ *                          stream outgrows L2 (80 MB; calls of some ten thousand tokens and
  *                          more), RMSNorm is folded into the GEMMs around it: the residual GEMM that completes x also
  *                          writes x * gain as the next GEMM's 16-bit operand and the rows' sums of squares, the next GEMM
  *                          scales its rows by 1 / rms. */
