@@ -762,6 +762,10 @@ static kvp_status prefill_direct(kvp_handle* h, const int32_t* tokens, const int
     const bool qkv_half = h->qkv_half[j] != 0;
     if (!qkv_fused)
       KVP_TIMED(KVP_CLASS_OTHER, launch_rmsnorm(ctx, x, (const float*)(P + L.attn_norm), A.eps, T, A.d, hbuf, h->opt.dtype, qkv_half ? nullptr : h_lo, qkv_half));
+    if (pending_join) {      // the predictor of the layer before reads the key and value buffers that this projection overwrites
+      cudaStreamWaitEvent(s, h->ev_join, 0);
+      pending_join = false;
+    }
     // predictor of this layer: K_hat_i = K_A,j FK_i^T, V_hat_i = V_A,j FV_i^T for every base layer i with j_i = j
     const PredGroup& pg = h->groups[j];
     const bool half_path = pg.half_path;
