@@ -41,8 +41,14 @@ __device__ __forceinline__ void dev_flag(int* status, int code) { atomicCAS(stat
 
 // Programmatic dependent launch.  A kernel started with launch_overlapped() may begin while the
 // kernel before it in the stream is still running (once every CTA of that kernel has called
-// pdl_trigger() or exited); it must call pdl_wait() before its first access to global memory,
-// which returns when the earlier kernel has finished and its writes are visible.  Both calls do
+// pdl_trigger() or exited), and so may the kernels behind it in a chain of such launches.  pdl_wait()
+// returns when the earlier kernel has finished and its writes, and those of all before it, are
+// visible.  Every kernel of a chain calls it, in at least one CTA, before it writes or reads what a kernel
+// of the chain writes.  Before it a kernel may read only what was complete when the chain's last ordinary
+// launch started: weights (RMSNorm's gain, the matrices of the CUDA-core GEMM and of the step's projections), and,
+// in the step's attention, lengths, block table and cache pages.  So the embedding, with which every pass starts, and the
+// first launch behind a wait for another stream are ordinary launches: recorded into a graph, a dependent
+// launch behind such a wait may start while the other stream's kernel still runs.  Both calls do
 // nothing in a kernel launched the ordinary way.
 __device__ __forceinline__ void pdl_trigger() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
 __device__ __forceinline__ void pdl_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }

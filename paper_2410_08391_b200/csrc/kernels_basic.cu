@@ -92,6 +92,7 @@ void launch_build_index(const LaunchCtx& ctx, const int* cu_host, int batch, int
 // ---------------------------------------------------------------------------------------
 // embedding gather: x[r, :] = table[tokens[idx(r)], :] as fp32.  Latency-bound (a row is a few KB from HBM): a thread asks
 // for 16 bytes at a time, so that a row takes one or two trips instead of one per 128 elements (64 rows of 2048: 12.2 -> 4.0 us).
+// An ordinary launch, not a dependent one: kernels behind it read lengths and cache pages before their own waits.
 // ---------------------------------------------------------------------------------------
 template <class T, bool VEC>
 __global__ void __launch_bounds__(128) embed_kernel(const int* __restrict__ tokens, const int* __restrict__ gather_idx,

@@ -237,17 +237,20 @@ bool step_uses_tc(const kvp_handle* h, int batch) {
 // gate/up row, or as they are; null: they are there already), output cleared first unless it is the residual stream.
 void step_proj_tc(kvp_handle* h, const LaunchCtx& ctx, const WsLayout& w, char* ws, int mode, const float* src, int ld_src,
                   int K, int batch, const float* gain, int G, const void* W, int N, float* Y, int ldy, bool clear,
-                  cudaError_t* err, const void* next_w = nullptr, size_t next_bytes = 0) {
+                  cudaError_t* err, const void* next_w = nullptr, size_t next_bytes = 0, bool overlapped = true) {
   bf16* XB = (bf16*)(ws + w.xbt);
-  if (src) KVP_TIMED(KVP_CLASS_STEP_GEMV, launch_step_prep(ctx, mode, src, ld_src, K, batch, gain, h->base.eps, G, XB, clear ? Y : nullptr, ldy, N));
+  if (src) KVP_TIMED(KVP_CLASS_STEP_GEMV, launch_step_prep(ctx, mode, src, ld_src, K, batch, gain, h->base.eps, G, XB, clear ? Y : nullptr, ldy, N, overlapped));
   TimedScope ts(h, ctx.st, KVP_CLASS_STEP_GEMV);
   cudaError_t e = launch_step_gemm_tc((const bf16*)W, K, N, K, XB, batch, Y, ldy, h->step_grid_sms, ctx.status, ctx.st, ctx.n_launch, next_w, next_bytes);
   if (e != cudaSuccess && *err == cudaSuccess) *err = e;
 }
 
 // one base-model layer of a single-token step (shared by the first step and generation)
+// after_event: the launch before it on this stream is a wait for another stream's kernels, which wrote the cache pages.  A dependent
+// launch behind such a wait may start while they run (the recorded edge is a programmatic one like any other), and so may the
+// dependent launches behind it, up to the attention, which asks for pages before its own wait: the first launch is an ordinary one.
 void base_layer_step(kvp_handle* h, const LaunchCtx& ctx, int i, const kvp_cache* cache, const WsLayout& w, char* ws,
-                     int batch, int max_keys, bool generation, cudaError_t* err) {
+                     int batch, int max_keys, bool generation, cudaError_t* err, bool after_event = false) {
   const ModelPlan& B = h->base;
   const LayerPlan& L = B.L[i];
   const char* P = h->packed;
@@ -266,7 +269,7 @@ void base_layer_step(kvp_handle* h, const LaunchCtx& ctx, int i, const kvp_cache
   const size_t b_after = last_layer ? (size_t)B.vocab * B.d * es : (size_t)(generation ? B.L[i + 1].nqkv : B.L[i + 1].dq) * B.d * es;
   if (tc)
     step_proj_tc(h, ctx, w, ws, PREP_NORM, xb, B.d, B.d, batch, (const float*)(P + L.attn_norm), 0, P + L.wqkv, n_out, qkvb, n_out, true, err,
-                 P + L.wo, (size_t)B.d * L.dq * es);
+                 P + L.wo, (size_t)B.d * L.dq * es, !after_event);
   else
     KVP_TIMED(KVP_CLASS_STEP_GEMV, launch_step_gemv(ctx, P + L.wqkv, B.d, n_out, B.d, xb, B.d, batch, qkvb, n_out, GEMV_STORE, 0, 0,
                                                     (const float*)(P + L.attn_norm), B.eps, hb));
@@ -880,7 +883,7 @@ static kvp_status prefill_direct(kvp_handle* h, const int32_t* tokens, const int
         if (last) h->step_grid_sms = h->n_sm;          // the prefill has nothing left to run
         if (base_done == 0)
           base_step_begin(h, sctx, w, ws, tokens, last_idx, batch);
-        for (int i = base_done; i < end; ++i) base_layer_step(h, sctx, i, cache, w, ws, batch, cs.max_len, false, &tc_err);
+        for (int i = base_done; i < end; ++i) base_layer_step(h, sctx, i, cache, w, ws, batch, cs.max_len, false, &tc_err, i == base_done);
         if (last) base_head(h, sctx, w, ws, batch, logits_out, first_token, &tc_err);
         base_done = end;
       }

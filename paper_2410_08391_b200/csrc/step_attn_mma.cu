@@ -125,9 +125,9 @@ step_attn_mma_kernel(const __grid_constant__ CUtensorMap map_k, const __grid_con
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
   }
   if (tid == 32) { prefetch_tensormap(&map_k); prefetch_tensormap(&map_v); }
-  // Lengths, block table and cached pages do not come from the kernel before this one: a step starts with a launch that waits for
-  // everything in front of it, and within the step a layer's pages are written by this kernel only.  So the pages are on their way
-  // before the wait for the queries.
+  // Lengths, block table and cached pages do not come from the kernel before this one.  A step, and every piece of a step that waits
+  // for a predictor on another stream, starts with an ordinary launch, behind which all of them are complete, and within the step a
+  // layer's pages are written by this kernel only.  So the pages are on their way before the wait for the queries.
   const int n_keys = p.seq_lens[b] + p.extra;
   const int pos = n_keys - 1;
   const int n_pg = (n_keys + PAGE_TOKENS - 1) / PAGE_TOKENS;

@@ -296,12 +296,13 @@ bool step_tc_supported(int batch, int K, int ldw, const void* W, const void* XB)
 }
 
 void launch_step_prep(const LaunchCtx& ctx, int mode, const float* x, int ldx, int K, int batch, const float* gain, float eps,
-                      int G, bf16* XB, float* zero_ptr, int zero_ld, int zero_n) {
+                      int G, bf16* XB, float* zero_ptr, int zero_ld, int zero_n, bool overlapped) {
   const int Bp = step_tc_rows(batch);
   RowMap mg{0, G, 0, K}, mu{G == 0 ? K : 0, G, 1, K};
+  const dim3 grid(Bp, (K + PREP_CHUNK - 1) / PREP_CHUNK);
   ++*ctx.n_launch;
-  launch_overlapped(step_prep_kernel, dim3(Bp, (K + PREP_CHUNK - 1) / PREP_CHUNK), dim3(256), 0, ctx.st, mode, x, ldx, K, batch, Bp, gain, eps,
-                    mg, mu, XB, zero_ptr, zero_ld, zero_n);
+  if (overlapped) launch_overlapped(step_prep_kernel, grid, dim3(256), 0, ctx.st, mode, x, ldx, K, batch, Bp, gain, eps, mg, mu, XB, zero_ptr, zero_ld, zero_n);
+  else step_prep_kernel<<<grid, 256, 0, ctx.st>>>(mode, x, ldx, K, batch, Bp, gain, eps, mg, mu, XB, zero_ptr, zero_ld, zero_n);
 }
 
 cudaError_t launch_step_gemm_tc(const bf16* W, int ldw, int N, int K, const bf16* XB, int batch, float* Y, int ldy, int n_sm,

@@ -15,7 +15,7 @@ bool step_tc_supported(int batch, int K, int ldw, const void* W, const void* XB)
 //   PREP_SWIGLU: v_b[c] = silu(x[b, gate row c]) * x[b, up row c], c < K = ffn, rows placed as in the packed w_gate/w_up
 // Also clears zero_ptr[b, 0:zero_n] (row stride zero_ld) for b < batch when zero_ptr is given.
 void launch_step_prep(const LaunchCtx&, int mode, const float* x, int ldx, int K, int batch, const float* gain, float eps,
-                      int G, bf16* XB, float* zero_ptr, int zero_ld, int zero_n);
+                      int G, bf16* XB, float* zero_ptr, int zero_ld, int zero_n, bool overlapped = true);
 
 // Y[b, n] += sum_k W[n, k] (XB[b, k] + XB[Bp + b, k]) for b < batch, n < N; fp32 atomic adds.
 // next_w / next_bytes: the weight matrix the next projection will read (or null): its first megabytes are asked into L2.

@@ -1,6 +1,6 @@
 """Order of the kernels that a call of up to 4096 prompt tokens puts on three streams, read from the recorded graph (nothing is
 launched): the predictor of an auxiliary layer runs beside the layer's attention and FFN and reads buffers that the next layer's
-projection overwrites."""
+projection overwrites; the base step's layers run beside the auxiliary layers after them and read what the predictor wrote."""
 import ctypes as C
 import re
 
@@ -51,13 +51,20 @@ class Recorded:
                 self.edges[b[i]].append((a[i], data[i][2] != 0))      # (node, whether it may still be running)
         finally:
             cu.cuGraphDestroy(graph)
-        self._before = {}
+        self._before, self._complete = {}, {}
 
     def before(self, x):
         """Every node on a path to x."""
         if x not in self._before:
             self._before[x] = set().union(*({y} | self.before(y) for y, _ in self.edges[x]))
         return self._before[x]
+
+    def complete(self, x):
+        """The nodes that have finished when x starts.  One whose launch does not wait for the end of the node before it starts
+        no earlier than that one; no kernel ends before those in front of it have."""
+        if x not in self._complete:
+            self._complete[x] = set().union(*(self.complete(y) if early else {y} | self.before(y) for y, early in self.edges[x]))
+        return self._complete[x]
 
     def find(self, pattern):
         return [x for x, n in self.name.items() if pattern.search(n)]
@@ -89,3 +96,16 @@ def test_predictor_is_ordered_against_every_projection(name, lens):
     for r in predictors:
         for w in projections:
             assert r in g.before(w) or w in g.before(r), "a projection may overwrite keys and values that a predictor kernel still reads"
+
+
+@pytest.mark.parametrize("name,lens", [("t_small", [9] * 6), ("t_small_gap", [40, 9, 130, 17, 64, 65]), ("t_hd128_qkn", [70] * 9), ("t_small", [600] * 6)], ids=str)
+def test_pages_are_complete_when_the_steps_attention_starts(name, lens):
+    """It asks for cache pages (and reads lengths) before it waits for the kernel in front of it."""
+    pair = wl.pair(name)
+    g = _recorded(pair, lens)
+    attention, predictors, lengths = g.find(re.compile("step_attn_mma_kernel")), g.find(PREDICTOR), g.find(re.compile("build_index_kernel"))
+    assert len(attention) == pair.base.n_layers and len(predictors) == 2 * len(set(pair.layer_map)) and len(lengths) == 1
+    first = min(len(set(predictors) & g.before(x)) for x in attention)
+    assert first == 2      # its first layers do run beside the auxiliary layers
+    for x in attention:
+        assert set(lengths + predictors) & g.before(x) <= g.complete(x), "a page may be read while a predictor kernel writes it"
