@@ -13,7 +13,6 @@ __global__ void __launch_bounds__(256) gemm_simt_kernel(GemmArgs g, int vec) {
   constexpr int R = TS / 16, BK = 2048 / TS, KT = BK / 8;
   __shared__ __align__(16) float As[BK][TS + 4];
   __shared__ __align__(16) float Ws[BK][TS + 4];
-  pdl_trigger();
   const T* __restrict__ A = (const T*)g.A;
   const T* __restrict__ W = (const T*)g.W;
   int m0 = blockIdx.y * TS, n0 = blockIdx.x * TS;
@@ -49,8 +48,7 @@ __global__ void __launch_bounds__(256) gemm_simt_kernel(GemmArgs g, int vec) {
       for (int i = 0; i < 8; ++i) av[i] += a2[i];
     }
   };
-  load8(W + (size_t)wn * g.ldw, wn < g.N, lk, wv);      // a weight: does not wait for the kernel before this one
-  pdl_wait();
+  load8(W + (size_t)wn * g.ldw, wn < g.N, lk, wv);
   load(0);
   for (int k0 = 0; k0 < g.K; k0 += BK) {
 #pragma unroll
@@ -115,8 +113,11 @@ void launch_gemm_simt(const LaunchCtx& ctx, const GemmArgs& g, int epi) {
   const int vec = g.K % per == 0 && g.lda % per == 0 && g.ldw % per == 0 && (!g.A2 || g.lda2 % per == 0) &&
                   (((uintptr_t)g.A | (uintptr_t)g.W | (uintptr_t)g.A2) & 15) == 0;
   ++*ctx.n_launch;
-#define GO(T, E) (small ? launch_overlapped(gemm_simt_kernel<T, E, 32>, grid, dim3(256), 0, ctx.st, g, vec) \
-                        : launch_overlapped(gemm_simt_kernel<T, E, 64>, grid, dim3(256), 0, ctx.st, g, vec))
+  // Ordinary launches.  As programmatic dependents (with this path's attention, RoPE and SwiGLU) they held SMs while they waited and
+  // took longer to record: fp32 test pair, 1 x 1024 tokens 206 us a call and 700 a first one, now 144 and 572; 1 x 64 49 and 469, now
+  // 45 and 438; 8 x 100 97, now 86.
+#define GO(T, E) (small ? (gemm_simt_kernel<T, E, 32><<<grid, 256, 0, ctx.st>>>(g, vec)) \
+                        : (gemm_simt_kernel<T, E, 64><<<grid, 256, 0, ctx.st>>>(g, vec)))
   if (ctx.dtype == 0) {
     if (epi == EPI_STORE) GO(float, EPI_STORE); else if (epi == EPI_RESID) GO(float, EPI_RESID); else if (epi == EPI_STORE32) GO(float, EPI_STORE32); else GO(float, EPI_PAGED);
   } else {
@@ -139,8 +140,6 @@ __global__ void __launch_bounds__(256) attn_prefill_simt_kernel(const T* __restr
                                                                 const int* __restrict__ cu, int batch, T* __restrict__ out,
                                                                 int ldo, float scale) {
   extern __shared__ float smem[];
-  pdl_trigger();
-  pdl_wait();
   int ldk = hd + 1;
   float* Ks = smem;                       // [AKV][hd+1]
   float* Vs = Ks + AKV * ldk;             // [AKV][hd+1]
@@ -231,10 +230,10 @@ void launch_attn_prefill_simt(const LaunchCtx& ctx, const void* qkv, int ld, int
   if (ctx.dtype == 0) {
     static bool raised[TC_MAX_DEVICES] = {};
     tc_raise_smem_limit(attn_prefill_simt_kernel<float>, ATTN_SMEM_MAX, raised);
-    launch_overlapped(attn_prefill_simt_kernel<float>, grid, dim3(256), smem, ctx.st, (const float*)qkv, ld, nq, nkv, hd, cu_dev, batch, (float*)out, ldo, scale);
+    attn_prefill_simt_kernel<float><<<grid, 256, smem, ctx.st>>>((const float*)qkv, ld, nq, nkv, hd, cu_dev, batch, (float*)out, ldo, scale);
   } else {
     static bool raised[TC_MAX_DEVICES] = {};
     tc_raise_smem_limit(attn_prefill_simt_kernel<bf16>, ATTN_SMEM_MAX, raised);
-    launch_overlapped(attn_prefill_simt_kernel<bf16>, grid, dim3(256), smem, ctx.st, (const bf16*)qkv, ld, nq, nkv, hd, cu_dev, batch, (bf16*)out, ldo, scale);
+    attn_prefill_simt_kernel<bf16><<<grid, 256, smem, ctx.st>>>((const bf16*)qkv, ld, nq, nkv, hd, cu_dev, batch, (bf16*)out, ldo, scale);
   }
 }

@@ -245,8 +245,6 @@ __global__ void rope_split_kernel(const float* __restrict__ in, int ld_in, int r
                                   T* __restrict__ out, int ld_out, T* __restrict__ out_lo, int ld_lo,
                                   int lo_head_begin, int n_q_heads, const float* __restrict__ q_gain,
                                   const float* __restrict__ k_gain, float eps) {
-  pdl_trigger();
-  pdl_wait();
   int half = hd >> 1;
   size_t n = (size_t)rows * n_heads * half;
   for (size_t i = blockIdx.x * (size_t)blockDim.x + threadIdx.x; i < n; i += (size_t)gridDim.x * blockDim.x) {
@@ -292,9 +290,9 @@ void launch_rope_split(const LaunchCtx& ctx, const float* in, int ld_in, int row
   int grid = grid_for(n, 256);
   LAUNCH_COUNT(ctx);
   if (ctx.dtype == 0)
-    launch_overlapped(rope_split_kernel<float>, dim3(grid), dim3(256), 0, ctx.st, in, ld_in, rows, n_heads, n_heads_rot, hd, tok_pos, inv, (float*)out, ld_out, (float*)nullptr, 0, 0, n_q_heads, q_gain, k_gain, eps);
+    rope_split_kernel<float><<<grid, 256, 0, ctx.st>>>(in, ld_in, rows, n_heads, n_heads_rot, hd, tok_pos, inv, (float*)out, ld_out, (float*)nullptr, 0, 0, n_q_heads, q_gain, k_gain, eps);
   else
-    launch_overlapped(rope_split_kernel<bf16>, dim3(grid), dim3(256), 0, ctx.st, in, ld_in, rows, n_heads, n_heads_rot, hd, tok_pos, inv, (bf16*)out, ld_out, (bf16*)out_lo, ld_lo, lo_head_begin, n_q_heads, q_gain, k_gain, eps);
+    rope_split_kernel<bf16><<<grid, 256, 0, ctx.st>>>(in, ld_in, rows, n_heads, n_heads_rot, hd, tok_pos, inv, (bf16*)out, ld_out, (bf16*)out_lo, ld_lo, lo_head_begin, n_q_heads, q_gain, k_gain, eps);
 }
 
 // ---------------------------------------------------------------------------------------
@@ -302,8 +300,6 @@ void launch_rope_split(const LaunchCtx& ctx, const float* in, int ld_in, int row
 // ---------------------------------------------------------------------------------------
 template <class T>
 __global__ void swiglu_kernel(const T* __restrict__ gu, int rows, int ffn, RowMap mg, RowMap mu, T* __restrict__ act) {
-  pdl_trigger();
-  pdl_wait();
   size_t n = (size_t)rows * ffn;
   for (size_t i = blockIdx.x * (size_t)blockDim.x + threadIdx.x; i < n; i += (size_t)gridDim.x * blockDim.x) {
     int r = (int)(i / ffn), c = (int)(i - (size_t)r * ffn);
@@ -319,8 +315,8 @@ void launch_swiglu(const LaunchCtx& ctx, const void* gu, int rows, int ffn, int 
   RowMap mg{0, G, 0, ffn}, mu{G == 0 ? ffn : 0, G, 1, ffn};
   int grid = grid_for(n, 256);
   LAUNCH_COUNT(ctx);
-  if (ctx.dtype == 0) launch_overlapped(swiglu_kernel<float>, dim3(grid), dim3(256), 0, ctx.st, (const float*)gu, rows, ffn, mg, mu, (float*)act);
-  else launch_overlapped(swiglu_kernel<bf16>, dim3(grid), dim3(256), 0, ctx.st, (const bf16*)gu, rows, ffn, mg, mu, (bf16*)act);
+  if (ctx.dtype == 0) swiglu_kernel<float><<<grid, 256, 0, ctx.st>>>((const float*)gu, rows, ffn, mg, mu, (float*)act);
+  else swiglu_kernel<bf16><<<grid, 256, 0, ctx.st>>>((const bf16*)gu, rows, ffn, mg, mu, (bf16*)act);
 }
 
 // ---------------------------------------------------------------------------------------

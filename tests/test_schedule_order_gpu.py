@@ -109,3 +109,12 @@ def test_pages_are_complete_when_the_steps_attention_starts(name, lens):
     assert first == 2      # its first layers do run beside the auxiliary layers
     for x in attention:
         assert set(lengths + predictors) & g.before(x) <= g.complete(x), "a page may be read while a predictor kernel writes it"
+
+
+@pytest.mark.parametrize("name,lens", [("t_small_f32", [70, 63]), ("t_small_f32", [9] * 6), ("narrow", [30, 7])], ids=str)
+def test_kernels_of_the_cuda_core_path_are_ordinary_launches(name, lens):
+    """Recorded as dependent launches they made first calls and, while they waited, other kernels slower."""
+    g = _recorded(_narrow() if name == "narrow" else wl.pair(name), lens)
+    nodes = g.find(re.compile("gemm_simt_kernel|attn_prefill_simt_kernel|rope_split_kernel|swiglu_kernel"))
+    assert len(nodes) >= 7
+    assert not any(early for x in nodes for _, early in g.edges[x])
