@@ -7,6 +7,7 @@ import pytest
 import workloads as wl
 from oracle import kvp_oracle as orc
 from parity_util import TOL, make_session, rel_fro
+from recorded_graph import Recorded, recorded_prefill
 
 pytestmark = pytest.mark.gpu
 TAIL = 1 << 20
@@ -51,3 +52,27 @@ def test_splits_of_layers_with_few_and_many_kv_heads(dtype, hd, lens):
         assert bool((whole[n:] == 0xA5).all()), "bytes behind the workspace were written"
     finally:
         s.close()
+
+
+@pytest.mark.parametrize("lens,ctas", [([64], 43), ([300], 43), ([999], 64), ([300] * 4, 80), ([3999], 148)], ids=str)
+def test_every_attention_item_of_a_step_has_a_cta(lens, ctas):
+    """A small model takes fewer CTAs than there are SMs (16 rows of its widest projection each: 688 / 16), but a key range of a
+    sequence and kv head is not left to a second round while SMs are free."""
+    import torch
+
+    import paper_2410_08391_b200 as kvp
+    pair = wl.pair("c1")
+    s = make_session(pair, wl.make_weights(pair, seed=1), wl.custom_prompts(pair.base.vocab, lens, seed=1), extra_len=1)
+    try:
+        tok = torch.zeros(len(lens), dtype=torch.int32, device=s.device)
+        g = Recorded(s, lambda: kvp.kvp_decode_step(s.h, tok, lens, s.cache, s.workspace, s.logits, s.first, s.stream))
+        assert g.grids("step_mega_kernel") == [(ctas, 1, 1)]
+    finally:
+        s.close()
+
+
+@pytest.mark.parametrize("lens,ctas", [([64], 43), ([999], 64), ([300] * 4, 64), ([3999], 72)], ids=str)
+def test_every_attention_item_of_a_piece_has_a_cta(lens, ctas):
+    """The same beside a prefill, where the pieces take at most 72 SMs and the key ranges go by that."""
+    grids = recorded_prefill(wl.pair("c1"), lens).grids("step_mega_kernel")
+    assert len(grids) == 2 and all(g == (ctas, 1, 1) for g in grids)
