@@ -101,7 +101,7 @@ typedef struct {
  *                          with at least one 128-token block per SM.  Off by default: it measured slower than the
  *                          projection GEMM followed by a predictor GEMM.
  *   KVP_OPT_SEPARATE_NORM  RMSNorm as a kernel of its own in front of every projection.  By default, where the residual
- *                          stream outgrows L2 (80 MB; calls of some ten thousand tokens and
+ *                          stream outgrows 32 MB (calls of some five thousand tokens and
  *                          more), RMSNorm is folded into the GEMMs around it: the residual GEMM that completes x also
  *                          writes x * gain as the next GEMM's 16-bit operand and the rows' sums of squares, the next GEMM
  *                          scales its rows by 1 / rms. */

@@ -723,10 +723,11 @@ Cut choose_cut(const TcGemm& g) {
 
 bool tc_gemm_resid_folds_norm(long long M, long long N) {
   // The folded epilogue reads, adds and writes x in place and takes 10-25 us more than a reduce-add of the same product (8192 x 1536 x
-  // 4096: 111 against 88 us); the RMSNorm launch it saves reads x once.  While x stays in L2 that launch is the cheaper one
-  // (3776 x 1280: whole call 4362 -> 4282 us without folding), from HBM it is not (25240 x 1536: 28.2 -> 27.9 ms with folding, 65536 x 1280:
-  // 38.6 -> 37.5, 65536 x 1536: 128.3 -> 125.5).  Lines between 19 and 155 MB were not tried; L2 holds 126.
-  return M * N * 4 > (80LL << 20);
+  // 4096: 111 against 88 us); the RMSNorm launch it saves reads x once.  While x stays in L2 beside the operands that launch is the
+  // cheaper one, beyond it is not.  First token with folding against without, by MB of x (M x N x 4): 18 (1.1B pair 64 x 59) 0.98,
+  // 26 0.994, 31 0.990, 42 1.007 and 1.012, 50 1.013, 52 0.998, 63 1.011 and 0.994, 67 1.062 (layer-pruned pair 8 x 1024, 12102 against
+  // 11395 us), 75 1.013, 84 1.054 and 1.039, 101 1.050 and 1.028, 126 1.038, 134 0.986, 201 1.003.
+  return M * N * 4 > (32LL << 20);
 }
 
 bool tc_gemm_supported(const TcGemm& g) {

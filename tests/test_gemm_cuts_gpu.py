@@ -5,6 +5,7 @@ import pytest
 
 import workloads as wl
 from parity_util import TOL, assert_first_tokens, compare_prefill, make_session
+from recorded_graph import recorded_prefill
 
 pytestmark = pytest.mark.gpu
 TWO = [1000, 999]                # 1999 rows = 15.6 row blocks
@@ -39,6 +40,7 @@ def test_folded_norm_with_ragged_columns_matches_oracle():
     W = wl.make_weights(pair, seed=6, regime="fanin")
     lens = [500] * 82 + [412]
     pr = wl.custom_prompts(300, lens, seed=6)
+    assert recorded_prefill(pair, lens, W).find("gemm_tc_kernelILi100E")
     s = make_session(pair, W, pr)
     try:
         ek, ev, el, tally = compare_prefill(s, pair, W, pr, seqs=[0, 41, 82])

@@ -7,6 +7,7 @@ import workloads as wl
 from oracle import kvp_oracle as orc
 from parity_util import (GAP, TOL, ArgmaxTally, assert_first_tokens, check_cache_layer, compare_prefill, compare_with_golden, load_golden,
                          make_session, rel_fro, run_prefill)
+from recorded_graph import recorded_prefill
 
 pytestmark = pytest.mark.gpu
 
@@ -84,18 +85,21 @@ def test_prefill_predict_matches_oracle(name, lens, regime):
         s.close()
 
 
-@pytest.mark.parametrize("flags", [1, 2, 3])
-@pytest.mark.parametrize("name,lens,regime", [("t_small", [1900] * 9 + [1901], "fanin"), ("t_hd128", [1300] * 9 + [1207], "n002"),
-                                              ("t_small_qkn", [1900] * 10, "fanin"), ("t_bias", [1900] * 10, "fanin"),
-                                              ("t_scaled", [1500] * 13, "fanin")],
+# tokens x d_model x 4 bytes above the line from which the norm is folded in (32 MB)
+@pytest.mark.parametrize("flags", [0, 1, 2, 3])
+@pytest.mark.parametrize("name,lens,regime", [("t_small", [1900] * 23 + [1901], "fanin"), ("t_hd128", [1300] * 17 + [1207], "n002"),
+                                              ("t_small_qkn", [1900] * 24, "fanin"), ("t_hd128_qkn", [1300] * 17 + [1207], "fanin"),
+                                              ("t_bias", [1900] * 24, "fanin"), ("t_scaled", [1500] * 23, "fanin")],
                          ids=lambda v: str(v).replace(" ", "")[:40])
 def test_kernel_variants_match_oracle(name, lens, regime, flags):
     """The schedule variants (kvp_options.flags: K/V projection + predictor as one kernel; RMSNorm as its own kernel
-    instead of folded into the GEMMs around it) on calls large enough for the choice to matter (flags = 0, the default, is
-    what every other many-token case runs): same results within the same tolerances."""
+    instead of folded into the GEMMs around it) on calls large enough for the choice to matter: the variant's kernels are
+    the ones that run, with the same results within the same tolerances."""
     pair = wl.pair(name)
     W = wl.make_weights(pair, seed=1, regime=regime)
     pr = wl.custom_prompts(pair.base.vocab, lens, seed=1)
+    g = recorded_prefill(pair, lens, W, flags=flags)
+    assert bool(g.find("gemm_tc_kernelILi100E")) == (not flags & 2) and bool(g.find("kvpred_tc_kernel")) == bool(flags & 1)
     s = make_session(pair, W, pr, flags=flags)
     try:
         ek, ev, el, tally = compare_prefill(s, pair, W, pr, seqs=[0, len(lens) - 1])
