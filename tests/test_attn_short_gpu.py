@@ -1,11 +1,12 @@
 """Prompt attention of short sequences: lengths at the edges of its 64-query and 64-key tiles and of a warp's 16 rows, both head widths,
-bfloat16 (prefill) and IEEE-half operands with a remainder (training-time forward), against the oracle.  The rule that picks the form
-of a call is looked at on the sizes themselves: these calls take the short form."""
+bfloat16 (prefill) and IEEE-half operands with a remainder (training-time forward), against the oracle.  The recorded graph says that
+these calls take the short form, and that each of the three forms is taken by the calls it was measured to be the fastest for."""
 import pytest
 
 import workloads as wl
 from oracle import kvp_oracle as orc
 from parity_util import TOL, assert_first_tokens, compare_prefill, make_session, rel_fro
+from recorded_graph import Recorded, recorded_prefill
 
 pytestmark = pytest.mark.gpu
 
@@ -17,6 +18,8 @@ def test_short_prompts_match_oracle(hd, heads, lens):
     pair = wl.PairCfg("short", aux, wl.uniform_model(3, 128, 2, 1, hd, 128, 300), (0, 1, 2))
     W = wl.make_weights(pair, seed=8, regime="fanin")
     pr = wl.custom_prompts(300, lens, seed=8)
+    g = recorded_prefill(pair, lens, W)
+    assert len(g.find("attn_mma_kernelILi%dELb0E" % hd)) == 2 and not g.find("attn_tc_kernel")
     s = make_session(pair, W, pr)
     try:
         ek, ev, el, tally = compare_prefill(s, pair, W, pr)
@@ -29,6 +32,8 @@ def test_short_prompts_match_oracle(hd, heads, lens):
 @pytest.mark.parametrize("hd,lens", [(64, [65, 1, 64, 100, 16]), (128, [64, 65, 3])], ids=str)
 def test_training_forward_of_short_prompts_matches_oracle(hd, lens):
     import torch
+
+    import paper_2410_08391_b200 as kvp
     pair = wl.PairCfg("short", wl.uniform_model(2, 128, 2, 1, hd, 128, 300), wl.uniform_model(3, 192, 4, 2, hd, 192, 300), (0, 1, 1))
     W = wl.make_weights(pair, seed=8, regime="fanin")
     pr = wl.custom_prompts(300, lens, seed=8)
@@ -38,6 +43,9 @@ def test_training_forward_of_short_prompts_matches_oracle(hd, lens):
         s.prefill_predict(toks, lens)
         logits, l1_k, l1_v = s.train_forward(toks, lens)
         s.poll()
+        g = Recorded(s, lambda: kvp.kvp_train_forward(s.h, toks, lens, s.cache, s.train_ws, logits, l1_k, l1_v, s.stream))
+        assert len(g.find("attn_mma_kernelILi%dELb1E" % hd)) == 2 * 3 - 1 and not g.find("attn_tc_kernel")
+        s.poll()
         logits, t0 = logits.cpu().numpy(), 0
         for b in range(pr.batch):
             want = orc.train_forward(pair, W, pr.seq(b))[0]
@@ -45,3 +53,18 @@ def test_training_forward_of_short_prompts_matches_oracle(hd, lens):
             t0 += lens[b]
     finally:
         s.close()
+
+
+@pytest.mark.parametrize("heads,hd,lens,form", [((20, 5), 64, [59] * 64, 0), ((20, 5), 64, [59], 0), ((20, 5), 64, [1024], 1), ((20, 5), 64, [700], 1),
+                                                ((12, 3), 128, [4096], 2), ((12, 3), 128, [3500, 1200, 2000], 2)], ids=str)
+def test_form_of_the_prompt_attention(heads, hd, lens, form):
+    """0: this file's kernel; 1, 2: the tcgen05 kernel with that many 128-query tiles a CTA (its grid: query heads x such pieces of the prompts)."""
+    aux = wl.uniform_model(2, heads[0] * hd, heads[0], heads[1], hd, 128, 300)
+    pair = wl.PairCfg("form", aux, wl.uniform_model(2, 128, 2, 1, hd, 128, 300), (0, 1))
+    g = recorded_prefill(pair, lens)
+    short, tc = g.find("attn_mma_kernelILi%dELb0E" % hd), g.grids("attn_tc_kernel")
+    if form == 0:
+        assert len(short) == 1 and not tc
+    else:
+        items = sum((n + 128 * form - 1) // (128 * form) for n in lens)
+        assert not short and len(tc) == 1 and items in tc[0] and heads[0] in tc[0]

@@ -1,6 +1,8 @@
 """The tensor-core GEMM at every tile width and both ways of cutting the work: rows, columns and k that leave the last tile, the last
-piece of a cache row and the last k block ragged, against the oracle.  Which width a size takes is the launcher's rule (76 SMs beside
-a step of up to four sequences, 148 otherwise); the sizes are some that it cuts that way."""
+piece of a cache row and the last k block ragged, against the oracle.  Which width and cut a call takes is the launcher's rule; the
+recorded graph says that it is the one meant here."""
+import re
+
 import pytest
 
 import workloads as wl
@@ -8,22 +10,35 @@ from parity_util import TOL, assert_first_tokens, compare_prefill, make_session
 from recorded_graph import recorded_prefill
 
 pytestmark = pytest.mark.gpu
-TWO = [1000, 999]                # 1999 rows = 15.6 row blocks
+TWO = [1000, 999]                # 1999 rows = 15.6 row blocks, on 100 SMs beside the step's 48
+SIX = [301, 200, 190, 64, 35, 1000]      # 1790 rows = 14 row blocks, on 148
 
 
-@pytest.mark.parametrize("d,ffn,heads,base_kv,lens", [
-    (72, 128, (1, 1), 1, [70]),             # 128 columns, one ragged tile
-    (520, 200, (3, 1), 2, TWO),             # residual 160: 3.25 tiles
-    (648, 136, (7, 1), 9, TWO),             # residual 192: 3.4 tiles; q / k / v 576 = 3 x 192; predictor 576
-    (776, 72, (3, 3), 3, TWO),              # residual 224: 3.5 tiles
-    (904, 64, (2, 1), 1, TWO),              # residual 256: 3.5 tiles
-    (264, 4104, (2, 2), 2, [70, 3]),        # shares of the k blocks: 65 k blocks of three 128-wide tiles
-    (1032, 2056, (4, 1), 9, [301, 200, 190, 64, 35, 1000]),     # 148 SMs, shares of 256-wide tiles
+def _launches(g, epilogue):
+    """(tile width, CTAs) of the GEMMs with this epilogue, in order"""
+    found = [(int(re.search("gemm_tc_kernelILi%dELi(\\d+)E" % epilogue, g.name[x]).group(1)), g.grid[x][0]) for x in sorted(
+        g.find("gemm_tc_kernelILi%dE" % epilogue), key=lambda x: len(g.before(x)))]
+    return found
+
+
+# residual: O and down projection of the first layer, (width, CTAs): whole tiles take a CTA each here, shares of the k blocks every SM;
+# widths of its QKV projection and of its predictor
+@pytest.mark.parametrize("d,ffn,heads,base_kv,lens,residual,qkv,predictor", [
+    (72, 128, (1, 1), 1, [70], [(128, 1), (128, 1)], 128, 128),                         # one ragged tile
+    (264, 2056, (2, 2), 2, TWO, [(128, 48), (128, 100)], 128, 128),                     # down: 33 k blocks of 48 tiles, shared by 100 CTAs
+    (520, 4104, (2, 2), 2, TWO, [(128, 80), (256, 100)], 128, 128),                     # shares of 256-wide tiles, the last of 8 columns
+    (840, 200, (3, 1), 2, TWO, [(160, 96), (160, 96)], 128, 128),                       # 5.25 tiles
+    (1032, 136, (10, 2), 13, TWO, [(192, 96), (192, 96)], 192, 192),                    # 5.4; 896 = 4.7 x 192; 832 = 4.3 x 192
+    (1224, 72, (3, 3), 3, TWO, [(224, 96), (224, 96)], 128, 128),                       # 5.5
+    (1368, 64, (15, 3), 19, TWO, [(256, 96), (256, 96)], 256, 256),                     # 5.3; 1344 = 5.25 x 256; 1216 = 4.75 x 256
+    (1032, 4104, (4, 1), 9, SIX, [(128, 126), (256, 148)], 128, 128),                   # 148 SMs, shares of 256-wide tiles
 ], ids=str)
-def test_every_cut_matches_oracle(d, ffn, heads, base_kv, lens):
+def test_every_cut_matches_oracle(d, ffn, heads, base_kv, lens, residual, qkv, predictor):
     aux = wl.uniform_model(2, d, heads[0], heads[1], 64, ffn, 500)
     pair = wl.PairCfg("cuts", aux, wl.uniform_model(2, 128, base_kv, base_kv, 64, 128, 500), (0, 1))
     W = wl.make_weights(pair, seed=6, regime="fanin")
+    g = recorded_prefill(pair, lens, W)
+    assert _launches(g, 1) == residual and _launches(g, 3)[0][0] == qkv and {w for w, _ in _launches(g, 4)} == {predictor}
     pr = wl.custom_prompts(500, lens, seed=6)
     s = make_session(pair, W, pr)
     try:

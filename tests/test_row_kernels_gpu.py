@@ -43,18 +43,39 @@ def test_row_widths_match_oracle(dtype, d, vocab):
         s.close()
 
 
-def test_argmax_takes_the_lowest_index_of_a_tie():
-    """Zero weights in front of the head: every logit is the same, in every row."""
+def _first_tokens(pair, W, pr):
     import torch
-    pair = wl.PairCfg("tie", wl.uniform_model(1, 64, 1, 1, 64, 64, 16390), wl.uniform_model(1, 64, 1, 1, 64, 64, 16390), (0,))
-    W = wl.make_weights(pair, seed=4)
-    W["base.lm_head"] = np.zeros_like(W["base.lm_head"])
-    lens = [3, 4, 5, 6, 7]
-    pr = wl.custom_prompts(16390, lens, seed=4)
     s = make_session(pair, W, pr)
     try:
-        logits, first = s.prefill_predict(torch.from_numpy(pr.tokens).to(s.device), lens)
+        logits, first = s.prefill_predict(torch.from_numpy(pr.tokens).to(s.device), [int(n) for n in pr.lengths])
         s.poll()
-        assert first.cpu().tolist() == [0] * 5 and float(logits.abs().max()) == 0.0
+        return logits.cpu().numpy(), first.cpu().tolist()
     finally:
         s.close()
+
+
+# 16390: element by element; 16388, 32000: 16-byte pieces, four a thread and trip of 16384 elements
+@pytest.mark.parametrize("vocab,tied", [(16390, range(16390)), (16388, range(16388)), (32000, range(32000)),
+                                        (32000, [4 * 40 + 16384, 4 * 40]),             # one thread, on two trips
+                                        (32000, [4 * 7 + 4096, 4 * 7 + 8192 + 3]),     # one thread, two of a trip's four pieces
+                                        (32000, [4 * 9 + 1, 4 * 9 + 2]),               # one piece
+                                        (32000, [4 * 33, 4 * 34 + 3]),                 # neighbouring lanes
+                                        (32000, [4 * 1023 + 3, 4 * 31 + 16384]),       # two warps, the lower index in the later one
+                                        (32000, [31999, 16000, 20000]), (16388, [16387, 16384]), (16390, [16389, 5001])],
+                         ids=lambda v: str(v)[:30].replace(" ", ""))
+def test_argmax_takes_the_lowest_index_of_a_tie(vocab, tied):
+    """Rows of the head that are the same give logits that are the same (one k block: d_model 64)."""
+    pair = wl.PairCfg("tie", wl.uniform_model(1, 64, 1, 1, 64, 64, vocab), wl.uniform_model(1, 64, 1, 1, 64, 64, vocab), (0,))
+    W = wl.make_weights(pair, seed=4)
+    pr = wl.custom_prompts(vocab, [5] * 5, seed=4)
+    pr.tokens[:] = np.tile(pr.tokens[:5], 5)
+    head = W["base.lm_head"].copy()
+    if len(tied) < vocab:        # four times the row whose logit is the largest, and so far above all others
+        head[list(tied)] = 4 * head[_first_tokens(pair, W, pr)[1][0]]
+    else:
+        head[:] = 0
+    W["base.lm_head"] = head
+    logits, first = _first_tokens(pair, W, pr)
+    assert first == [min(tied)] * 5
+    for row in logits:
+        assert sorted(np.flatnonzero(row == row.max())) == sorted(tied)
