@@ -35,9 +35,11 @@
 //     reads take 512, and more of them in proportion to the code's length.  So a group's tiles are ONE loop whose sums wait in shared
 //     memory, not five straight-line copies with their sums in registers.  Generation step, 1.1B shape: 1 x 1100 keys 840 -> 807 us,
 //     2 x 300 888 -> 824, 4 x 300 1109 -> 1075; on the 72 SMs of a piece, with twice the tiles a CTA, more (first token of 1 x 59 1532 -> 1363 us,
-//     1 x 1024 1733 -> 1649); 3B shape 2 x 300 2242 -> 2126, but 1 x 300 1985 -> 2009, 4 x 300 2410 -> 2430 (more chunks of K a tile).
+//     1 x 1024 1733 -> 1649); 3B shape 2 x 300 2242 -> 2126.  The price is a sum over columns with every chunk of a
+//     tile, not one a tile (3B shape 1 x 300 1979 -> 2016, 4 x 300 2401 -> 2407); lanes that share it by rows took half of that back
+//     (2000, 2374; 1.1B shape 4 x 300 1075 -> 1067; the same bits).
 // Measured against the CUDA-core kernel of step_mega.cu (generation step): 1.1B shape 1 x 1100 keys 1557 -> 807 us, 4 x 300
-// 2990 -> 1075 us (that kernel's multiply-adds grow with the batch); 3B shape 1 x 300 2966 -> 2009 us, 4 x 300 5578 -> 2430 us.
+// 2990 -> 1067 us (that kernel's multiply-adds grow with the batch); 3B shape 1 x 300 2966 -> 2000 us, 4 x 300 5578 -> 2374 us.
 // The bytes of the first take 416 us.  Of the rest, per layer of 26 us: waits for inputs 0.4-0.7 us a phase, attention's exchange between
 // key ranges 2.8, its wait for the queries 1.3, the tiles of O and down (4.0 us, weights 4.8 on HBM) and gate / up (3.9, 7.0).
 // Every wait is bounded: on expiry DEV_TIMEOUT is recorded, no further wait is started, every CTA runs through its remaining
@@ -398,19 +400,17 @@ __device__ __forceinline__ void proj_phase(const MegaParams& p, const Work& g, R
 #pragma unroll
         for (int nb = 0; nb < NB; ++nb) {
           const bool pair = BB < 4 || !(t & 1);
-          float v0 = part[nb][0] + (pair ? part[nb][1] : 0.f), v1 = part[nb][2] + (pair ? part[nb][3] : 0.f);
-          v0 += __shfl_xor_sync(0xffffffffu, v0, 1);
-          v1 += __shfl_xor_sync(0xffffffffu, v1, 1);
-          if (BB == 1) {
-            v0 += __shfl_xor_sync(0xffffffffu, v0, 2);
-            v1 += __shfl_xor_sync(0xffffffffu, v1, 2);
-          }
-          const int bs = nb * 2 + (t >> 1);
-          if (!(t & 1) && bs < BB) {
-            float* d0 = red + warp * RS + (ti * TR + gr) * BB + bs;
-            float* d1 = d0 + 8 * BB;
-            if (c > 0) { v0 += *d0; v1 += *d1; }
-            *d0 = v0; *d1 = v1;
+          const float v0 = part[nb][0] + (pair ? part[nb][1] : 0.f), v1 = part[nb][2] + (pair ? part[nb][3] : 0.f);
+          // an even lane of the quad goes on with row gr, an odd one with row gr + 8
+          const float out = t & 1 ? v0 : v1;
+          float v = t & 1 ? v1 : v0;
+          v += __shfl_xor_sync(0xffffffffu, out, 1);
+          if (BB == 1) v += __shfl_xor_sync(0xffffffffu, v, 2);
+          const int bs = BB == 1 ? 0 : nb * 2 + (t >> 1);
+          if (BB == 1 ? t < 2 : bs < BB) {
+            float* d = red + warp * RS + (ti * TR + gr + 8 * (t & 1)) * BB + bs;
+            if (c > 0) v += *d;
+            *d = v;
           }
         }
       }
