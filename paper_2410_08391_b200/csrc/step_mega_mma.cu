@@ -39,7 +39,7 @@
 //     tile, not one a tile (3B shape 1 x 300 1979 -> 2016, 4 x 300 2401 -> 2407); lanes that share it by rows took half of that back
 //     (2000, 2374; 1.1B shape 4 x 300 1075 -> 1067; the same bits).
 // Measured against the CUDA-core kernel of step_mega.cu (generation step): 1.1B shape 1 x 1100 keys 1557 -> 807 us, 4 x 300
-// 2990 -> 1067 us (that kernel's multiply-adds grow with the batch); 3B shape 1 x 300 2966 -> 2000 us, 4 x 300 5578 -> 2374 us.
+// 2990 -> 1067 us (that kernel's multiply-adds grow with the batch); 3B shape 1 x 300 2966 -> 1787 us, 4 x 300 5578 -> 2374 us.
 // The bytes of the first take 416 us.  Of the rest, per layer of 26 us: waits for inputs 0.4-0.7 us a phase, attention's exchange between
 // key ranges 2.8, its wait for the queries 1.3, the tiles of O and down (4.0 us, weights 4.8 on HBM) and gate / up (3.9, 7.0).
 // Every wait is bounded: on expiry DEV_TIMEOUT is recorded, no further wait is started, every CTA runs through its remaining
@@ -893,9 +893,12 @@ __global__ void __launch_bounds__(NT, 1) step_mega_mma_kernel(const __grid_const
 
 constexpr size_t SMEM_ROOM = SMEM_LIMIT - sizeof(Shared) - 256;      // dynamic shared memory of a CTA
 
-// Shared-memory plan: scratch and page slots first, the weight ring takes what is left (at least 3 slots).
-// (head_dim 128 with four sequences has room for one page slot and three weight slots only, so that a page's load does not overlap
-// the arithmetic on the one before.)
+// Shared-memory plan: scratch and page slots first, the weight ring takes what is left (at least 3 slots).  A second page slot, which lets
+// a page's load overlap the arithmetic on the one before, is not worth the weight slots of a tile: where tiles take two slots (up to
+// two sequences), fewer than four would be left beside it and head_dim is 128, there is one.  Generation step, 3B shape, with two page
+// slots and 3 weight slots / with one and 4: 1 x 300 keys 2000 / 1787 us, 1 x 4090 2133 / 2025, 2 x 300 2111 / 1899, 2 x 4000 2380 / 2360; eight
+// heads of 128 a group, 8 layers of 4096, 1 x 300 726 / 632, 1 x 4000 751 / 663.  (Four sequences of head_dim 128, and two with more
+// than 4 heads a group, have room for one page slot and three weight slots only.)
 bool make_plan(int batch, int hd, int max_group, Plan* pl, size_t* bytes) {
   const int bb = batch <= 1 ? 1 : (batch == 2 ? 2 : 4);
   const size_t proj = (size_t)CW * 3 * bb * XCOL + (size_t)2 * CW * (bb == 4 ? Geo<4>::TG : Geo<1>::TG) * TR * bb * 4;
@@ -904,7 +907,7 @@ bool make_plan(int batch, int hd, int max_group, Plan* pl, size_t* bytes) {
   const int STAGE = bb == 4 ? Geo<4>::STAGE : Geo<1>::STAGE;
   for (int n_kv = 2; n_kv >= 1; --n_kv) {
     const size_t kv = (size_t)n_kv * 2 * PAGE_TOKENS * hd * 2;
-    if (scr + kv + 3 * (size_t)STAGE > SMEM_ROOM) continue;
+    if (scr + kv + (n_kv > 1 && bb < 4 ? 4 : 3) * (size_t)STAGE > SMEM_ROOM) continue;
     int n = (int)((SMEM_ROOM - scr - kv) / STAGE);
     if (n > MAX_SLOTS) n = MAX_SLOTS;
     pl->n_stage = n; pl->n_kv = n_kv; pl->kv_off = n * STAGE; pl->scr_off = pl->kv_off + (int)kv;

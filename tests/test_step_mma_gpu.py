@@ -25,6 +25,8 @@ def _pair(name):
     if name.startswith("g"):     # g<query heads per kv head>x<head_dim>
         g, hd = (int(n) for n in name[1:].split("x"))
         return wl.PairCfg(name, wl.uniform_model(2, 192, 2, 1, hd, 320, 500), wl.uniform_model(2, 264, 2 * g, 2, hd, 520, 500), (0, 1))
+    if name == "kv4x128":    # a long cache is more pages than CTAs: several pages a key range, through one page slot
+        return wl.PairCfg(name, wl.uniform_model(2, 192, 2, 1, 128, 320, 500), wl.uniform_model(2, 264, 8, 4, 128, 520, 500), (0, 1))
     # more (sequence, kv head) pairs than CTAs can split: one split per item; layers of different widths
     return wl.PairCfg(name, wl.uniform_model(2, 192, 4, 1, 64, 320, 1000), wl.uniform_model(2, 256, 48, 48, 64, 192, 1000), (0, 1))
 
@@ -97,7 +99,8 @@ def _step(pair, W, token, cache, cut=lambda v: v):
 ALONE = [("wide", [1]), ("wide", [64, 191]), ("wide", [130, 64, 3]), ("hd128", [700]), ("hd128", [321, 64]), ("hd128", [63, 320, 1, 65]),
          ("many", [200, 64, 65, 129]), ("small", [70]), ("small", [5, 127]), ("small", [64, 1, 300]), ("small", [130, 63, 64, 65]),
          ("deep", [70]), ("deep", [65, 3]), ("deep", [64, 5, 9, 130]), ("g5x64", [200]), ("g6x64", [66, 300]), ("g7x64", [3, 64, 190]),
-         ("g8x64", [127, 64, 1, 320]), ("g1x128", [130]), ("g3x128", [63, 200]), ("g5x128", [300, 64]), ("g8x128", [65, 2, 129])]
+         ("g8x64", [127, 64, 1, 320]), ("g1x128", [130]), ("g3x128", [63, 200]), ("g5x128", [300, 64]), ("g8x128", [65, 2, 129]),
+         ("kv4x128", [4000]), ("kv4x128", [1990, 2050]), ("g8x128", [4030, 3900])]
 
 
 @pytest.mark.parametrize("name,lens", ALONE, ids=str)
