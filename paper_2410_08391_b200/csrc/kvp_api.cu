@@ -332,10 +332,11 @@ bool mega_prepare(kvp_handle* h, const LaunchCtx& ctx, const kvp_cache* cache, c
   // Beyond some thousand keys the chain of launches around the tensor-core attention kernel (step_attn_mma.cu) is the faster one.
   // The CUDA-core kernel reads cache pages with plain loads, several times slower than that kernel.  The other one brings them in
   // by bulk copy, but multiplies them on the CUDA cores; where it falls behind depends on the sequences and kv heads.  Generation
-  // step, chain of launches / step_mega_mma_kernel, us: 1.1B shape 1 x 8000 1983 / 1054, 2 x 16000 2154 / 1833, 4 x 4200 1953 /
-  // 1570, 4 x 8000 2070 / 2026, 4 x 16000 2335 / 2941; 3B shape 1 x 16000 3928 / 2584, 2 x 8000 3490 / 2817, 4 x 4200 3399 / 3289,
-  // 4 x 6000 3443 / 3723, 4 x 16000 4117 / 6015; 32 kv heads of 64 1 x 8000 1287 / 999, 4 x 4200 1449 / 1734.  The line is
-  // where four sequences of the 3B shape cross; a single sequence of it would gain up to 16000 keys.
+  // step by itself, chain of launches / step_mega_mma_kernel, us: 1.1B shape 1 x 8000 1715 / 1062, 1 x 16000 1806 / 1252, 2 x 16000 1835 / 1728,
+  // 4 x 4200 1629 / 1555, 4 x 8000 1764 / 2025; 3B shape 1 x 16000 3447 / 2793, 2 x 8000 3017 / 2838, 4 x 4000 2884 / 3270, 4 x 6000
+  // 2943 / 3705.  Among other calls: 1.1B shape 1 x 8000 977 / 1013, 1 x 16000 1119 / 1211, 4 x 4200 1063 / 1516; 3B shape 1 x 16000 2785 / 2741,
+  // 2 x 8000 2288 / 2798, 4 x 4000 2211 / 3231.  One line for all: four sequences cross below it since the chain has eight launches a layer,
+  // one sequence would gain by itself up to 16000 keys.
   if (max_keys > 4096) return false;
   if (B.n_layers > MEGA_MAX_LAYERS) return false;
   if (!mega_uses_mma(h, batch) && !step_mega_supported(batch, B.L[0].hd, k_max, B.max_group, h->es)) return false;
@@ -640,10 +641,10 @@ kvp_status kvp_load_weights(kvp_handle* h, const kvp_tensor* tensors, int32_t n,
 // microseconds, the prefill from its launches and operations, the step (on all SMs) from its weights.  Prompts whose prefill is the
 // longer by far want the SMs themselves; where it is over long before the step, a caller that waits is served sooner by one after the
 // other (while other calls keep the GPU busy, 72 SMs get more done).  Alone / among other calls, us, with 0, 48, 72, 88 SMs:
-//   1.1B 1 x 59 (prefill / step 0.7): 1394 / 1056, 1606 / 880, 1354 / 948, 1349 / 1234;  1 x 1024 (1.6): 2064 / 1708, 1963 / 1603,
-//   1893 / 1628, 2000 / 1889;  3 x 1000 (2.5): 3486 / 3266, 3227 / 3038, 3446 / 3211, 3755 / 3398;  1 x 3500 (3.7): 4001 / 3878, 3904 / 3849,
+//   1.1B 1 x 59 (prefill / step 0.7): 1394 / 1107, 1562 / 885, 1370 / 969, 1295 / 1230;  1 x 1024 (1.6): 2087 / 1756, 1911 / 1606,
+//   1911 / 1677, 2027 / 1858;  3 x 1000 (2.5): 3486 / 3266, 3227 / 3038, 3446 / 3211, 3755 / 3398;  1 x 3500 (3.7): 4001 / 3878, 3904 / 3849,
 //   4151 / 3810, 4807 / 3919;  layer-pruned 1 x 1000 (2.5): 2567 / 2356, 2313 / 2170, 2605 / 2252, 2892 / 2437;
-//   3B 1 x 59 (0.35): 2931 / 2561, 4957 / 2615, 3782 / 2446, 3361 / 3342;  1 x 800 (0.8): 3916 / 3461, 5237 / 3092, 4124 / 3274, 3912 / 3724.
+//   3B 1 x 59 (0.35): 2678 / 2281, 4053 / 1912, 3113 / 2057, 2840 / 2769;  1 x 800 (0.8): 3677 / 3126, 4449 / 2872, 3550 / 2931, 3431 / 3263.
 int step_piece_sms(const kvp_handle* h, int batch, const CallShape& cs, bool blocking) {
   if (h->step_sms == 0 || h->opt.dtype != KVP_BF16) return h->step_sms;
   const ModelPlan &A = h->aux, &B = h->base;
