@@ -1,7 +1,11 @@
 // Tensor-core GEMM for sm_100a:  D[M,N] = A[M,K] W[N,K]^T (+ A_lo W^T on split tiles), bf16
 // operands, fp32 accumulation in tensor memory.
 //
-// One persistent CTA per SM walks output tiles of 128 x BN, BN = 128 to 256 (choose_cut).  Operand tiles travel through a ring of shared-
+// One persistent CTA per SM walks output tiles of 128 x BN, BN = 128 to 256, or a pair of CTAs tiles of 256 x 256 (choose_cut).  In a pair
+// (a cluster of two) each CTA loads its own 128 rows of A and half of the tile's W rows; one thread of the first CTA issues
+// tcgen05.mma.cta_group::2, which reads the operands of both and leaves each CTA the accumulator rows of its A rows, so that the
+// epilogues are those of single CTAs.  The copies of both are counted on the first CTA's barriers; its commits free the
+// stages of both.  Operand tiles travel through a ring of shared-
 // memory stages (128-byte swizzle, 64 k-elements per stage) filled by TMA.  A thread that
 // issues a tensor copy is held for a few hundred cycles per copy, which caps one issuing thread
 // at about 120 GB/s; a 128 x 256 tile needs 48 KiB per 512 tensor-pipe cycles (about 180 GB/s),
@@ -32,15 +36,15 @@ constexpr int N_THREADS = 224;                             // warps: 0 A loads, 
 constexpr int N_THREADS_NORM = 352;                        // fused-norm residual kernel: 8 epilogue warps (3-10), two per lane quarter
 constexpr int TC_RESID_NORM = 100;                         // internal: TC_RESID with the folded RMSNorm producer (own shared-memory plan)
 constexpr int SMEM_LIMIT = 227 * 1024;
-template <int BN, int EPI = TC_STORE> struct Tile {
+template <int BN, int EPI = TC_STORE, bool PAIR = false> struct Tile {
   static constexpr int XS = (EPI == TC_PAGED || EPI == TC_QKV) ? 1 : 2;        // 4 KiB slots per epilogue warp
   // epilogues that move every element through shared memory get eight warps (two per tensor-memory lane quarter)
   static constexpr int EPI_WARPS = (EPI == TC_RESID_NORM || EPI == TC_PAGED || EPI == TC_QKV || EPI == TC_SWIGLU) ? 8 : 4;
   static constexpr int THREADS = EPI_WARPS == 8 ? N_THREADS_NORM : N_THREADS;
   static constexpr int XRING = (EPI == TC_RESID || EPI == TC_RESID_NORM || EPI == TC_PAGED || EPI == TC_QKV) ? EPI_WARPS * XS * 4096 : 0;
-  static constexpr int A_BYTES = BM * BK * 2, W_BYTES = BN * BK * 2;
+  static constexpr int A_BYTES = BM * BK * 2, W_ROWS = PAIR ? BN / 2 : BN, W_BYTES = W_ROWS * BK * 2;    // (a CTA's own)
   static constexpr int STAGE_BYTES = A_BYTES + W_BYTES;    // 32 KiB (128 columns) to 48 KiB (256)
-  static constexpr int STAGES_FIT = (SMEM_LIMIT - 1536 - XRING) / STAGE_BYTES, STAGES = STAGES_FIT < 6 ? STAGES_FIT : 6;
+  static constexpr int STAGES_FIT = (SMEM_LIMIT - 1536 - XRING) / STAGE_BYTES, MOST = PAIR ? 8 : 6, STAGES = STAGES_FIT < MOST ? STAGES_FIT : MOST;
   static constexpr int ACC_STRIDE = BN > 128 ? 256 : 128;  // tensor-memory columns between the two accumulators
   static constexpr int SMEM_BYTES = STAGES * STAGE_BYTES + XRING + 1024 /*align*/ + 512 /*barriers*/;
 };
@@ -81,6 +85,7 @@ struct Params {
   int M, N, K;
   int split_begin;       // tiles with n0 + BN > split_begin run the k loop a second time over A2
   int has_a2;
+  int pair;              // CTA pairs: tiles of 256 rows
   int stream_k;          // residual GEMM only: CTAs take equal shares of all k blocks
   int* status;
   // epilogue
@@ -108,26 +113,29 @@ struct Params {
 // ---- work list: every role of a CTA walks the same sequence of (tile, k-block range) ---------
 struct Work { int m0, n0, kb0, kb1, tile; };
 
-template <int BN>
+template <int BN, bool PAIR>
 struct Sched {
+  static constexpr int ROWS = PAIR ? 2 * BM : BM, GROUP = GROUP_M * BM / ROWS;
+
   int tiles_m, tiles_n, n_tiles, num_kb;
   int tile;                 // tile mode: next tile of this CTA
   long long g, g_end;       // stream-K mode: this CTA's share of the global k-block sequence
   const Params& p;
   __device__ __forceinline__ explicit Sched(const Params& p_) : p(p_) {
-    tiles_m = (p.M + BM - 1) / BM; tiles_n = (p.N + BN - 1) / BN;
+    tiles_m = (p.M + ROWS - 1) / ROWS; tiles_n = (p.N + BN - 1) / BN;
     n_tiles = tiles_m * tiles_n;
     num_kb = (p.K + BK - 1) / BK;
-    tile = blockIdx.x;
+    const int unit = blockIdx.x / (PAIR ? 2 : 1), units = gridDim.x / (PAIR ? 2 : 1);
+    tile = unit;
     long long total = (long long)n_tiles * num_kb;
-    g = total * blockIdx.x / gridDim.x;
-    g_end = total * (blockIdx.x + 1) / gridDim.x;
+    g = total * unit / units;
+    g_end = total * (unit + 1) / units;
   }
   __device__ __forceinline__ void coords(int t, Work& w) const {
-    const int per_group = GROUP_M * tiles_n;
+    const int per_group = GROUP * tiles_n;
     const int grp = t / per_group, r = t - grp * per_group;
-    const int gm = min(GROUP_M, tiles_m - grp * GROUP_M);
-    w.m0 = (grp * GROUP_M + r % gm) * BM;
+    const int gm = min(GROUP, tiles_m - grp * GROUP);
+    w.m0 = (grp * GROUP + r % gm) * ROWS + (PAIR ? (int)(blockIdx.x & 1) * BM : 0);      // this CTA's rows
     w.n0 = (r / gm) * BN;
     w.tile = t;
   }
@@ -145,7 +153,7 @@ struct Sched {
     coords(tile, w);
     w.kb0 = 0;
     w.kb1 = ((p.has_a2 && w.n0 + BN > p.split_begin) ? 2 : 1) * num_kb;
-    tile += gridDim.x;
+    tile += gridDim.x / (PAIR ? 2 : 1);
     return true;
   }
 };
@@ -277,11 +285,11 @@ __device__ __forceinline__ void epilogue_tile(const Params& p, uint32_t tmem_acc
   }
 }
 
-template <int EPI, int BN>
-__global__ void __launch_bounds__((Tile<BN, EPI>::THREADS), 1)
+template <int EPI, int BN, bool PAIR>
+__global__ void __launch_bounds__((Tile<BN, EPI, PAIR>::THREADS), 1)
 gemm_tc_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_constant__ CUtensorMap map_a2,
                const __grid_constant__ CUtensorMap map_w, const __grid_constant__ CUtensorMap map_x, const Params p) {
-  using T = Tile<BN, EPI>;
+  using T = Tile<BN, EPI, PAIR>;
   constexpr int STAGES = T::STAGES, STAGE_BYTES = T::STAGE_BYTES, XS = T::XS;
   extern __shared__ uint8_t smem_raw[];
   uint8_t* smem = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~uintptr_t(1023));
@@ -300,7 +308,8 @@ gemm_tc_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_constant_
   auto xfull_bar = [&](int q, int s) { return bar_base + 8u * (2 * STAGES + 4 + q * XS + s); };
 
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  pdl_trigger();      // the next kernel's CTAs may take SMs as this kernel's CTAs leave them
+  const bool leader = !PAIR || (blockIdx.x & 1) == 0;      // issues the pair's MMAs; its barriers count the operands of both CTAs
+  if (!PAIR) pdl_trigger();      // the next kernel's CTAs may take SMs as this kernel's CTAs leave them
   if (threadIdx.x == 32) {   // tensor maps on their way while the barriers and tensor memory are set up
     prefetch_tensormap(&map_a);
     prefetch_tensormap(&map_w);
@@ -309,17 +318,20 @@ gemm_tc_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_constant_
 
   if (threadIdx.x == 0) {
     for (int s = 0; s < STAGES; ++s) { mbar_init(full_bar(s), 2); mbar_init(empty_bar(s), 1); }   // two loaders per stage
-    for (int a = 0; a < 2; ++a) { mbar_init(tfull_bar(a), 1); mbar_init(tempty_bar(a), EW); }
+    for (int a = 0; a < 2; ++a) { mbar_init(tfull_bar(a), 1); mbar_init(tempty_bar(a), PAIR ? 2 * EW : EW); }
     for (int q = 0; q < EW; ++q) for (int x = 0; x < XS; ++x) mbar_init(xfull_bar(q, x), 1);
     *abort_flag = 0;
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
   }
   if (warp == 1) {   // tensor memory: two accumulators of BN columns (a power of two is allocated)
-    tmem_alloc(smem_u32(tmem_slot), 2 * T::ACC_STRIDE);
+    if constexpr (PAIR) tmem_alloc_pair(smem_u32(tmem_slot), 2 * T::ACC_STRIDE);
+    else tmem_alloc(smem_u32(tmem_slot), 2 * T::ACC_STRIDE);
   }
   tc_fence_before();
-  __syncthreads();
+  if constexpr (PAIR) cluster_sync();      // (the other CTA's barriers are there from here on)
+  else __syncthreads();
   tc_fence_after();
+  if (PAIR) pdl_trigger();       // (with the pair's tensor memory in hand: that allocation waits for two SMs)
   const uint32_t tmem_base = *tmem_slot;
   const int num_kb = (p.K + BK - 1) / BK;
   pdl_wait();         // set-up above overlapped the previous kernel's tail; its results are needed from here on
@@ -328,7 +340,7 @@ gemm_tc_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_constant_
     // ---------------- TMA producers: warp 0 loads the A tile of every stage, warp 2 the W tile ----------------
     if (lane == 0) {
       const bool is_a = warp == 0;
-      Sched<BN> sched(p);
+      Sched<BN, PAIR> sched(p);
       Work w;
       int stage = 0; uint32_t phase = 0;
       bool ok = true;
@@ -338,7 +350,12 @@ gemm_tc_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_constant_
           if (!ok) break;
           const int kb = it < num_kb ? it : it - num_kb;
           const uint32_t sa = smem_base + stage * STAGE_BYTES;
-          if (is_a) {
+          if constexpr (PAIR) {      // own rows of A, own half of the tile's W rows; both CTAs' copies count on the leader's barrier
+            const uint32_t bar = map_to_rank(full_bar(stage), 0);
+            if (leader) mbar_expect_tx(full_bar(stage), 2 * (is_a ? T::A_BYTES : T::W_BYTES));
+            if (is_a) tma_load_2d_pair(sa, it < num_kb ? &map_a : &map_a2, kb * BK, w.m0, bar);
+            else tma_load_2d_pair(sa + T::A_BYTES, &map_w, kb * BK, w.n0 + (leader ? 0 : T::W_ROWS), bar);
+          } else if (is_a) {
             mbar_expect_tx(full_bar(stage), T::A_BYTES);
             tma_load_2d(sa, it < num_kb ? &map_a : &map_a2, kb * BK, w.m0, full_bar(stage));
           } else {
@@ -352,11 +369,11 @@ gemm_tc_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_constant_
     }
   } else if (warp == 1) {
     // ---------------- MMA issuer ----------------
-    if (lane == 0) {
+    if (lane == 0 && leader) {
       // operand formats: bits 7-9 (A) and 10-12 (B): 1 = bf16, 0 = IEEE half
       const uint32_t fmt = p.f16_operands ? 0u : ((1u << 7) | (1u << 10));
-      const uint32_t idesc = (1u << 4) | fmt | ((uint32_t)(BN >> 3) << 17) | ((uint32_t)(BM >> 4) << 24);
-      Sched<BN> sched(p);
+      const uint32_t idesc = (1u << 4) | fmt | ((uint32_t)(BN >> 3) << 17) | ((uint32_t)((PAIR ? 2 * BM : BM) >> 4) << 24);
+      Sched<BN, PAIR> sched(p);
       Work w;
       int stage = 0; uint32_t phase = 0;
       int acc = 0; uint32_t acc_phase = 0;
@@ -373,12 +390,16 @@ gemm_tc_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_constant_
           const uint32_t sa = smem_base + stage * STAGE_BYTES, sb = sa + T::A_BYTES;
           const uint64_t da = desc_kmajor(sa), db = desc_kmajor(sb);
 #pragma unroll
-          for (int k = 0; k < BK / 16; ++k)
-            tc_mma_bf16(d_tmem, da + 2u * k, db + 2u * k, idesc, (it > w.kb0 || k > 0) ? 1u : 0u);
-          tc_commit(empty_bar(stage));        // the slot is free once these MMAs have read it
+          for (int k = 0; k < BK / 16; ++k) {
+            if constexpr (PAIR) tc_mma_f16_pair(d_tmem, da + 2u * k, db + 2u * k, idesc, (it > w.kb0 || k > 0) ? 1u : 0u);
+            else tc_mma_bf16(d_tmem, da + 2u * k, db + 2u * k, idesc, (it > w.kb0 || k > 0) ? 1u : 0u);
+          }
+          if constexpr (PAIR) tc_commit_pair(empty_bar(stage));      // the slot is free once these MMAs have read it
+          else tc_commit(empty_bar(stage));
           if (++stage == STAGES) { stage = 0; phase ^= 1u; }
         }
-        if (ok) tc_commit(tfull_bar(acc));    // accumulator complete
+        if constexpr (PAIR) { if (ok) tc_commit_pair(tfull_bar(acc)); }      // accumulator complete
+        else { if (ok) tc_commit(tfull_bar(acc)); }
         if (++acc == 2) { acc = 0; acc_phase ^= 1u; }
       }
       if (!ok) drain_after_abort();
@@ -389,14 +410,14 @@ gemm_tc_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_constant_
     const int ew = warp - 3;                      // epilogue warp index
     constexpr int NH = EW / 4;                    // warps per lane quarter: each takes every NH-th block of 32 columns
     const int half = ew >> 2;
-    Sched<BN> sched(p);
+    Sched<BN, PAIR> sched(p);
     Work w;
     int acc = 0; uint32_t acc_phase = 0;
     bool ok = true;
     // fused norm (TC_RESID with H, every tile owned by one CTA): the old values of X arrive through this warp's ring
     constexpr bool fused = EPI == TC_RESID_NORM;
     const uint32_t xring = smem_base + STAGES * STAGE_BYTES + ew * (XS * X_SLOT_BYTES);
-    Sched<BN> pre(p);
+    Sched<BN, PAIR> pre(p);
     Work pw;
     bool pre_ok = fused && pre.next(pw);
     int pre_c = half;
@@ -643,16 +664,21 @@ gemm_tc_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_constant_
       }
       tc_fence_before();
       __syncwarp();
-      if (lane == 0) mbar_arrive(tempty_bar(acc));
+      if (lane == 0) {
+        if constexpr (PAIR) mbar_arrive_cluster(map_to_rank(tempty_bar(acc), 0));
+        else mbar_arrive(tempty_bar(acc));
+      }
       if (++acc == 2) { acc = 0; acc_phase ^= 1u; }
     }
     if ((EPI == TC_RESID || EPI == TC_RESID_NORM) && lane == 0) asm volatile("cp.async.bulk.wait_group 0;" ::: "memory");    // this warp's reduces have completed
   }
   tc_fence_before();
-  __syncthreads();
+  if constexpr (PAIR) cluster_sync();      // neither CTA leaves while the other's copies, MMAs or arrivals may still reach it
+  else __syncthreads();
   if (warp == 1) {
     tc_fence_after();
-    tmem_dealloc(tmem_base, 2 * T::ACC_STRIDE);
+    if constexpr (PAIR) tmem_dealloc_pair(tmem_base, 2 * T::ACC_STRIDE);
+    else tmem_dealloc(tmem_base, 2 * T::ACC_STRIDE);
   }
 }
 
@@ -662,13 +688,19 @@ bool make_map(CUtensorMap* m, const void* base, int rows, int cols, int ld, int 
   return tc_make_map_bf16(m, base, rows, cols, ld, box_rows);
 }
 
+template <int EPI, int BN, bool PAIR>
+cudaError_t go_form(const CUtensorMap& a, const CUtensorMap& a2, const CUtensorMap& w, const CUtensorMap& x, const Params& p, int grid, cudaStream_t st) {
+  constexpr int SMEM = Tile<BN, EPI, PAIR>::SMEM_BYTES;
+  static bool raised[TC_MAX_DEVICES] = {};
+  cudaError_t e = tc_raise_smem_limit(gemm_tc_kernel<EPI, BN, PAIR>, SMEM, raised);
+  if (e != cudaSuccess) return e;
+  return launch_overlapped_clusters(gemm_tc_kernel<EPI, BN, PAIR>, dim3(grid), dim3(Tile<BN, EPI, PAIR>::THREADS), PAIR ? 2 : 1, SMEM, st, a, a2, w, x, p);
+}
+constexpr int PAIR_BN = 256;           // the width of the tiles that CTA pairs take
 template <int EPI, int BN>
 cudaError_t go(const CUtensorMap& a, const CUtensorMap& a2, const CUtensorMap& w, const CUtensorMap& x, const Params& p, int grid, cudaStream_t st) {
-  constexpr int SMEM = Tile<BN, EPI>::SMEM_BYTES;
-  static bool raised[TC_MAX_DEVICES] = {};
-  cudaError_t e = tc_raise_smem_limit(gemm_tc_kernel<EPI, BN>, SMEM, raised);
-  if (e != cudaSuccess) return e;
-  return launch_overlapped(gemm_tc_kernel<EPI, BN>, dim3(grid), dim3(Tile<BN, EPI>::THREADS), SMEM, st, a, a2, w, x, p);
+  if constexpr (BN == PAIR_BN && EPI != TC_PAGED) { if (p.pair) return go_form<EPI, BN, true>(a, a2, w, x, p, grid, st); }
+  return p.pair ? cudaErrorInvalidValue : go_form<EPI, BN, false>(a, a2, w, x, p, grid, st);
 }
 
 // Which widths an epilogue takes: whole heads (TC_QKV: 192 only with head_dim 64), whole gate / up blocks (TC_SWIGLU), whole 64-column
@@ -695,27 +727,34 @@ cudaError_t go_epi(int epi, const CUtensorMap& a, const CUtensorMap& a2, const C
   }
 }
 
-// How a launch is cut: tile width, and whether the CTAs take whole tiles or (residual GEMM with one operand pass) equal shares of all
-// k blocks.  Costs in units of a k block of a 256-wide tile on one SM (0.41 us).  A CTA is bound by its shared-memory port (operands
-// written once and read once), so a k block costs almost the same whatever the width, and what counts is how many waves of tiles a
-// width leaves: with 128 and 256 columns only, 3776 x 1280 x 3456 took 3 waves or 2.03.  Fitted to 118 launches of 59 to 8192 rows,
-// N 1280 to 32000, K 1280 to 5632, 76 and 148 SMs, one and two passes: the geometric mean of the chosen cuts is 0.9 % above
-// that of the best ones (the rule before, 128 or 256 columns by tensor time: 18 %).
-struct Cut { int bn; bool shares; };
+// How a launch is cut: tile width, whether the CTAs take whole tiles or (residual GEMM with one operand pass) equal shares of all
+// k blocks, and whether they work in pairs (tiles of 256 x 256).  Costs in units of a k block of a 256-wide tile on one SM (0.41 us).
+// A CTA by itself is bound by its shared-memory port (operands written once and read once), so a k block costs almost the same
+// whatever the width, and what counts is how many waves of tiles a width leaves: with 128 and 256 columns only, 3776 x 1280 x 3456 took
+// 3 waves or 2.03.  Fitted to 118 launches of 59 to 8192 rows, N 1280 to 32000, K 1280 to 5632, 76 and 148 SMs, one and two passes: the
+// geometric mean of the chosen cuts is 0.9 % above that of the best ones (the rule before, 128 or 256 columns by tensor time: 18 %).
+// A pair's k block takes 0.91 to 0.94 of that (each CTA writes and reads half of the W tile only) and its launch 1 to 2 us more (two SMs
+// at once, tensor memory of both, a cluster barrier at either end).  us, single / pair: gate / up 25240 x 8192 x 1536 469 / 428, 65536 x
+// 6912 x 1280 863 / 813, 3776 x 6912 x 1280 54.3 / 51.9, 1024 x 6912 x 1280 21.0 / 21.3; down with the norm 25240 x 1536 x 4096 306 / 258,
+// in shares without it 251 / 226, 3776 x 1280 x 3456 28.9 / 29.3; QKV 25240 x 2304 x 1536 160 / 146, 1024 x 1920 x 1280 15.2 / 16.3; 2143 x 32000 x
+// 2048 in two passes 418 / 384.  Narrower tiles and the predictor (36.0 / 38.3 at K 384: its epilogue is the longer part) gain nothing as pairs.
+struct Cut { int bn; bool shares, pair; };
 Cut choose_cut(const TcGemm& g) {
   static const struct { int bn; double cost; } widths[] = {{256, 1.00}, {224, 0.95}, {192, 0.90}, {160, 0.87}, {128, 0.84}};
   const double kb = (double)((g.K + BK - 1) / BK) * (g.A2 ? 2 : 1);
-  Cut best{256, false};
+  Cut best{256, false, false};
   double least = -1.0;
-  for (const auto& w : widths) {
-    if (!width_ok(g, w.bn)) continue;
-    const long long tiles = (long long)((g.M + BM - 1) / BM) * ((g.N + w.bn - 1) / w.bn), waves = (tiles + g.n_sm - 1) / g.n_sm;
-    const double own = waves * (kb * w.cost + 2.0 + 2.0 * w.bn / 256);
-    if (least < 0 || own < least) { least = own; best = Cut{w.bn, false}; }
-    if (g.epi != TC_RESID || g.A2 || g.H || (w.bn != 128 && w.bn != 256)) continue;
-    const double per_sm = tiles * kb / g.n_sm, share = (per_sm > 1.0 ? per_sm : 1.0) * w.cost * 1.1 + 8.0 + 8.0 * w.bn / 256;
-    if (share < least) { least = share; best = Cut{w.bn, true}; }
-  }
+  auto consider = [&](int bn, bool pair, double cost, double launch_own, double launch_shares) {
+    const int rows = pair ? 2 * BM : BM, units = pair ? g.n_sm / 2 : g.n_sm;
+    const long long tiles = (long long)((g.M + rows - 1) / rows) * ((g.N + bn - 1) / bn), waves = (tiles + units - 1) / units;
+    const double own = waves * (kb * cost + 2.0 + 2.0 * bn / 256) + launch_own;
+    if (least < 0 || own < least) { least = own; best = Cut{bn, false, pair}; }
+    if (g.epi != TC_RESID || g.A2 || g.H || (bn != 128 && bn != 256)) return;
+    const double per_unit = tiles * kb / units, share = (per_unit > 1.0 ? per_unit : 1.0) * cost * 1.1 + 8.0 + 8.0 * bn / 256 + launch_shares;
+    if (share < least) { least = share; best = Cut{bn, true, pair}; }
+  };
+  for (const auto& w : widths) if (width_ok(g, w.bn)) consider(w.bn, false, w.cost, 0.0, 0.0);
+  if (g.pairs && g.epi != TC_PAGED && g.n_sm >= 2) consider(PAIR_BN, true, 0.92, 4.0, 5.0);
   return best;
 }
 
@@ -763,14 +802,14 @@ cudaError_t launch_gemm_tc(const TcGemm& g, int* status, cudaStream_t st, int64_
   CUtensorMap ma, ma2, mw, mx;
   if (g.H && g.epi != TC_RESID) return cudaErrorInvalidValue;
   if (!make_map(&ma, g.A, g.M, g.K, g.lda, BM)) return cudaErrorInvalidValue;
-  if (!make_map(&mw, g.W, g.N, g.K, g.ldw, bn)) return cudaErrorInvalidValue;
+  if (!make_map(&mw, g.W, g.N, g.K, g.ldw, cut.pair ? bn / 2 : bn)) return cudaErrorInvalidValue;
   if (g.A2) { if (!make_map(&ma2, g.A2, g.M, g.K, g.lda2, BM)) return cudaErrorInvalidValue; }
   else ma2 = ma;
   if (g.epi == TC_RESID) { if (!tc_make_map_f32(&mx, g.X, g.M, g.N, g.ldx, 32)) return cudaErrorInvalidValue; }
   else mx = ma;
   Params p{};
   p.M = g.M; p.N = g.N; p.K = g.K; p.split_begin = g.split_begin; p.has_a2 = g.A2 != nullptr; p.status = status;
-  p.stream_k = stream_k ? 1 : 0;
+  p.pair = cut.pair ? 1 : 0; p.stream_k = stream_k ? 1 : 0;
   p.C = g.C; p.ldc = g.ldc; p.X = g.X; p.ldx = g.ldx; p.C_lo = g.C_lo; p.ld_lo = g.ld_lo; p.lo_col_begin = g.lo_col_begin;
   p.q_gain = g.q_gain; p.k_gain = g.k_gain; p.q_cols = g.q_cols; p.eps = g.eps;
   p.rot_cols = g.rot_cols; p.hd = g.hd; p.rope_tab = g.rope_tab; p.tab_stride = g.tab_stride; p.tok_pos = g.tok_pos; p.ffn = g.ffn; p.paged = g.paged;
@@ -782,9 +821,11 @@ cudaError_t launch_gemm_tc(const TcGemm& g, int* status, cudaStream_t st, int64_
     for (int sg = 0; sg <= g.paged.n_seg; ++sg) if (g.paged.col0[sg] % 64) p.paged_wide = 0;
   }
   p.lo_is_half = g.lo_is_half; p.f16_operands = g.f16_operands; p.c_is_half = g.c_is_half; p.h_is_half = g.h_is_half;
-  const int tiles = ((g.M + BM - 1) / BM) * ((g.N + bn - 1) / bn);
+  const int rows = cut.pair ? 2 * BM : BM, units = cut.pair ? g.n_sm / 2 : g.n_sm;      // (a unit: a CTA or a pair)
+  const int tiles = ((g.M + rows - 1) / rows) * ((g.N + bn - 1) / bn);
   const long long kblocks = (long long)tiles * ((g.K + BK - 1) / BK);
-  int grid = stream_k ? (int)(kblocks < g.n_sm ? kblocks : g.n_sm) : (tiles < g.n_sm ? tiles : g.n_sm);
+  int grid = stream_k ? (int)(kblocks < units ? kblocks : units) : (tiles < units ? tiles : units);
+  if (cut.pair) grid *= 2;
   ++*n_launch;
   switch (bn) {
     case 160: return go_resid<160>(ma, ma2, mw, mx, p, grid, st);

@@ -41,6 +41,7 @@ struct TcGemm {
   int c_is_half;                   // TC_QKV: C is written as IEEE halves (for an attention that takes half operands)
   int f16_operands;                // A and W hold IEEE halves instead of bf16 (same 2 bytes; both operands alike)
   int n_sm;
+  int pairs;                       // pairs of CTAs may take tiles of 256 rows (both SMs of a pair have to be free at once)
 };
 
 bool tc_gemm_supported(const TcGemm& g);

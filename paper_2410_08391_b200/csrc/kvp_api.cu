@@ -215,6 +215,7 @@ bool ends_with(const std::string& s, const char* suf) {
 bool try_tc(kvp_handle* h, const LaunchCtx& ctx, TcGemm& t, int cls, cudaError_t* err) {
   if (h->opt.dtype != KVP_BF16) return false;
   t.n_sm = h->gemm_sms;
+  t.pairs = h->gemm_sms == h->n_sm;      // (persistent pieces of the step hold SMs one by one, not in pairs)
   if (!tc_gemm_supported(t)) return false;
   TimedScope ts(h, ctx.st, cls);
   cudaError_t e = launch_gemm_tc(t, ctx.status, ctx.st, ctx.n_launch);
