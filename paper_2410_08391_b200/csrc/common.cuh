@@ -150,7 +150,7 @@ __host__ __device__ __forceinline__ int map_row(const RowMap& m, int r) {
   return 2 * blk * m.G + m.which * gb + (r - blk * m.G);
 }
 
-enum GemmEpi : int { EPI_STORE = 0, EPI_RESID = 1, EPI_PAGED = 2, EPI_STORE32 = 3 };
+enum GemmEpi : int { EPI_STORE = 0, EPI_RESID = 1, EPI_PAGED = 2, EPI_STORE32 = 3, EPI_ROPE = 4, EPI_GATED = 5 };   // the last two: fp32 mode only
 
 // bf16 mode carries the K/V path in split precision: a value v travels as hi = bf16(v) and
 // lo = bf16(v - hi), and a GEMM whose A operand has a lo part accumulates A_hi W^T + A_lo W^T.
@@ -165,6 +165,9 @@ struct GemmArgs {
   void* C; int ldc;              // EPI_STORE: run dtype [M, N]; EPI_STORE32: fp32 [M, N]
   float* X; int ldx;             // EPI_RESID: fp32 residual, X += A W^T
   PagedOut paged;                // EPI_PAGED
+  const float* gain; float eps;  // fp32 mode: the rows of A are RMS-normalised with this gain [K] first (null: they are not)
+  int hd, n_rot; float theta; const int* tok_pos;      // EPI_ROPE: heads of hd columns, the first n_rot of them rotated by their row's position
+  RowMap gate, up;               // EPI_GATED: C[m, c] = silu(gate column) * up column, N = twice the outputs, W's rows placed as packed
 };
 
 // ---- launchers (defined in the .cu files); all enqueue on `st` and count launches ----

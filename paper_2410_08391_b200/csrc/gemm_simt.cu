@@ -8,11 +8,18 @@ namespace {
 // next k block is on its way to registers while this one is multiplied.  Small problems are a chain of memory latencies: 32 x 32
 // tiles with 64 k at a time give them four times the CTAs and a quarter of the trips.
 // Every output is one chain of multiply-adds in the order of k, whatever the tile.
+// fp32 mode is a chain of launches of 2 to 4 us each, so what surrounds a product is part of it there:
+//   g.gain     the rows of A are RMS-normalised: products take x gain, the CTA sums its rows' squares as it reads them (all of k passes
+//              through every CTA) and scales its outputs by 1 / rms
+//   EPI_ROPE   tile columns 2 i and 2 i + 1 are the two halves of one rotated pair, whichever columns of W those are
+//   EPI_GATED  ... are the gate and the up column of one output
 template <class T, int EPI, int TS>
-__global__ void __launch_bounds__(256) gemm_simt_kernel(GemmArgs g, int vec) {
+__device__ __forceinline__ void gemm_simt_tile(const GemmArgs& g, const InvFreq* inv, int vec) {
   constexpr int R = TS / 16, BK = 2048 / TS, KT = BK / 8;
   __shared__ __align__(16) float As[BK][TS + 4];
   __shared__ __align__(16) float Ws[BK][TS + 4];
+  __shared__ float rinv[TS];
+  constexpr bool PAIRED = EPI == EPI_ROPE || EPI == EPI_GATED;
   const T* __restrict__ A = (const T*)g.A;
   const T* __restrict__ W = (const T*)g.W;
   int m0 = blockIdx.y * TS, n0 = blockIdx.x * TS;
@@ -20,8 +27,16 @@ __global__ void __launch_bounds__(256) gemm_simt_kernel(GemmArgs g, int vec) {
   int tid = threadIdx.x;
   int tx = tid & 15, ty = tid >> 4;
   float acc[R][R] = {};
-  const int lr = tid / KT, lk = (tid % KT) * 8, am = m0 + lr, wn = n0 + lr;
-  float av[8], wv[8];
+  const int lr = tid / KT, lk = (tid % KT) * 8, am = m0 + lr;
+  // the row of W behind a column of the tile
+  auto w_row = [&](int n) {
+    if (!PAIRED || n >= g.N) return n;
+    if (EPI == EPI_GATED) return map_row(n & 1 ? g.up : g.gate, n >> 1);
+    const int half = g.hd >> 1, u = n >> 1, h = u / half;
+    return h * g.hd + (u - h * half) + (n & 1) * half;
+  };
+  const int wn = w_row(n0 + lr);
+  float av[8], wv[8], gv[8], ss = 0.f;
   auto load8 = [&](const T* row, bool ok, int k, float* v) {
     if (!ok || k >= g.K) {
 #pragma unroll
@@ -47,10 +62,18 @@ __global__ void __launch_bounds__(256) gemm_simt_kernel(GemmArgs g, int vec) {
 #pragma unroll
       for (int i = 0; i < 8; ++i) av[i] += a2[i];
     }
+    if (g.gain) {
+#pragma unroll
+      for (int i = 0; i < 8; ++i) gv[i] = k0 + lk + i < g.K ? g.gain[k0 + lk + i] : 0.f;
+    }
   };
   load8(W + (size_t)wn * g.ldw, wn < g.N, lk, wv);
   load(0);
   for (int k0 = 0; k0 < g.K; k0 += BK) {
+    if (g.gain) {
+#pragma unroll
+      for (int i = 0; i < 8; ++i) { ss = fmaf(av[i], av[i], ss); av[i] *= gv[i]; }
+    }
 #pragma unroll
     for (int i = 0; i < 8; ++i) { As[lk + i][lr] = av[i]; Ws[lk + i][lr] = wv[i]; }
     __syncthreads();
@@ -70,10 +93,40 @@ __global__ void __launch_bounds__(256) gemm_simt_kernel(GemmArgs g, int vec) {
     }
     __syncthreads();
   }
+  if (g.gain) {      // KT neighbouring threads have read a row
+#pragma unroll
+    for (int o = KT / 2; o > 0; o >>= 1) ss += __shfl_xor_sync(0xffffffffu, ss, o);
+    if (tid % KT == 0) rinv[lr] = rsqrtf(ss / (float)g.K + g.eps);
+    __syncthreads();
+  }
 #pragma unroll
   for (int i = 0; i < R; ++i) {
     int m = m0 + ty * R + i;
     if (m >= g.M) continue;
+    if (g.gain) {
+      const float r = rinv[ty * R + i];
+#pragma unroll
+      for (int j = 0; j < R; ++j) acc[i][j] *= r;
+    }
+    if (PAIRED) {
+#pragma unroll
+      for (int j = 0; j < R; j += 2) {
+        const int n = n0 + tx * R + j;
+        if (n >= g.N) continue;
+        const float a = acc[i][j], b = acc[i][j + 1];
+        T* row = (T*)g.C + (size_t)m * g.ldc;
+        if (EPI == EPI_GATED) {
+          row[n >> 1] = from_f<T>(a / (1.f + __expf(-a)) * b);
+        } else {
+          const int half = g.hd >> 1, u = n >> 1, h = u / half, c = u - h * half;
+          float sn = 0.f, cs = 1.f;
+          if (h < g.n_rot) rope_sincos(g.tok_pos[m], inv->f[c], &sn, &cs);
+          row[h * g.hd + c] = from_f<T>(h < g.n_rot ? a * cs - b * sn : a);
+          row[h * g.hd + c + half] = from_f<T>(h < g.n_rot ? b * cs + a * sn : b);
+        }
+      }
+      continue;
+    }
     int slot = 0;
     if (EPI == EPI_PAGED) { slot = g.paged.tok_slot[m]; if (slot < 0) continue; }
 #pragma unroll
@@ -102,6 +155,15 @@ __global__ void __launch_bounds__(256) gemm_simt_kernel(GemmArgs g, int vec) {
     }
   }
 }
+template <class T, int EPI, int TS>
+__global__ void __launch_bounds__(256) gemm_simt_kernel(const __grid_constant__ GemmArgs g, int vec) {
+  gemm_simt_tile<T, EPI, TS>(g, nullptr, vec);
+}
+// The projection that leaves its heads rotated (fp32 mode; elsewhere rope_split_kernel follows the projection).
+template <int TS>
+__global__ void __launch_bounds__(256) gemm_rope_split_kernel(const __grid_constant__ GemmArgs g, const __grid_constant__ InvFreq inv, int vec) {
+  gemm_simt_tile<float, EPI_ROPE, TS>(g, &inv, vec);
+}
 }  // namespace
 
 void launch_gemm_simt(const LaunchCtx& ctx, const GemmArgs& g, int epi) {
@@ -118,8 +180,13 @@ void launch_gemm_simt(const LaunchCtx& ctx, const GemmArgs& g, int epi) {
   // 45 and 438; 8 x 100 97, now 86.
 #define GO(T, E) (small ? (gemm_simt_kernel<T, E, 32><<<grid, 256, 0, ctx.st>>>(g, vec)) \
                         : (gemm_simt_kernel<T, E, 64><<<grid, 256, 0, ctx.st>>>(g, vec)))
-  if (ctx.dtype == 0) {
-    if (epi == EPI_STORE) GO(float, EPI_STORE); else if (epi == EPI_RESID) GO(float, EPI_RESID); else if (epi == EPI_STORE32) GO(float, EPI_STORE32); else GO(float, EPI_PAGED);
+  if (epi == EPI_ROPE) {
+    InvFreq inv;
+    fill_inv_freq(&inv, g.hd, g.theta);
+    small ? gemm_rope_split_kernel<32><<<grid, 256, 0, ctx.st>>>(g, inv, vec) : gemm_rope_split_kernel<64><<<grid, 256, 0, ctx.st>>>(g, inv, vec);
+  } else if (ctx.dtype == 0) {
+    if (epi == EPI_GATED) GO(float, EPI_GATED);
+    else if (epi == EPI_STORE) GO(float, EPI_STORE); else if (epi == EPI_RESID) GO(float, EPI_RESID); else if (epi == EPI_STORE32) GO(float, EPI_STORE32); else GO(float, EPI_PAGED);
   } else {
     if (epi == EPI_STORE) GO(bf16, EPI_STORE); else if (epi == EPI_RESID) GO(bf16, EPI_RESID); else if (epi == EPI_STORE32) GO(bf16, EPI_STORE32); else GO(bf16, EPI_PAGED);
   }

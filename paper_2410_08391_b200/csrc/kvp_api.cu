@@ -238,11 +238,11 @@ bool step_uses_tc(const kvp_handle* h, int batch) {
 // gate/up row, or as they are; null: they are there already), output cleared first unless it is the residual stream.
 void step_proj_tc(kvp_handle* h, const LaunchCtx& ctx, const WsLayout& w, char* ws, int mode, const float* src, int ld_src,
                   int K, int batch, const float* gain, int G, const void* W, int N, float* Y, int ldy, bool clear,
-                  cudaError_t* err, const void* next_w = nullptr, size_t next_bytes = 0, bool overlapped = true) {
+                  cudaError_t* err, bool overlapped = true) {
   bf16* XB = (bf16*)(ws + w.xbt);
   if (src) KVP_TIMED(KVP_CLASS_STEP_GEMV, launch_step_prep(ctx, mode, src, ld_src, K, batch, gain, h->base.eps, G, XB, clear ? Y : nullptr, ldy, N, overlapped));
   TimedScope ts(h, ctx.st, KVP_CLASS_STEP_GEMV);
-  cudaError_t e = launch_step_gemm_tc((const bf16*)W, K, N, K, XB, batch, Y, ldy, h->step_grid_sms, ctx.status, ctx.st, ctx.n_launch, next_w, next_bytes);
+  cudaError_t e = launch_step_gemm_tc((const bf16*)W, K, N, K, XB, batch, Y, ldy, h->step_grid_sms, ctx.status, ctx.st, ctx.n_launch);
   if (e != cudaSuccess && *err == cudaSuccess) *err = e;
 }
 
@@ -263,14 +263,8 @@ void base_layer_step(kvp_handle* h, const LaunchCtx& ctx, int i, const kvp_cache
   // the first step needs q only (keys and values are the predicted ones); generation needs q, k, v
   int n_out = generation ? L.nqkv : L.dq;
   const bool tc = step_uses_tc(h, batch);
-  // every projection names the weights of the one after it (the next layer's queries, or the LM head, after the down projection)
-  const size_t es = (size_t)h->es;
-  const bool last_layer = i + 1 == B.n_layers;
-  const void* w_after = last_layer ? P + B.lm_head : P + B.L[last_layer ? i : i + 1].wqkv;
-  const size_t b_after = last_layer ? (size_t)B.vocab * B.d * es : (size_t)(generation ? B.L[i + 1].nqkv : B.L[i + 1].dq) * B.d * es;
   if (tc)
-    step_proj_tc(h, ctx, w, ws, PREP_NORM, xb, B.d, B.d, batch, (const float*)(P + L.attn_norm), 0, P + L.wqkv, n_out, qkvb, n_out, true, err,
-                 P + L.wo, (size_t)B.d * L.dq * es, !after_event);
+    step_proj_tc(h, ctx, w, ws, PREP_NORM, xb, B.d, B.d, batch, (const float*)(P + L.attn_norm), 0, P + L.wqkv, n_out, qkvb, n_out, true, err, !after_event);
   else
     KVP_TIMED(KVP_CLASS_STEP_GEMV, launch_step_gemv(ctx, P + L.wqkv, B.d, n_out, B.d, xb, B.d, batch, qkvb, n_out, GEMV_STORE, 0, 0,
                                                     (const float*)(P + L.attn_norm), B.eps, hb));
@@ -286,10 +280,9 @@ void base_layer_step(kvp_handle* h, const LaunchCtx& ctx, int i, const kvp_cache
   KVP_TIMED(KVP_CLASS_STEP_ATTN, in_xb = launch_step_attn(ctx, a));
   if (tc) {
     float* gub = (float*)(ws + w.gub);
-    step_proj_tc(h, ctx, w, ws, PREP_PLAIN, in_xb ? nullptr : ab, L.dq, L.dq, batch, nullptr, 0, P + L.wo, B.d, xb, B.d, false, err, P + L.wgu, (size_t)2 * L.ffn * B.d * es);
-    step_proj_tc(h, ctx, w, ws, PREP_NORM, xb, B.d, B.d, batch, (const float*)(P + L.ffn_norm), 0, P + L.wgu, 2 * L.ffn, gub, 2 * L.ffn, true, err,
-                 P + L.wd, (size_t)B.d * L.ffn * es);
-    step_proj_tc(h, ctx, w, ws, PREP_SWIGLU, gub, 2 * L.ffn, L.ffn, batch, nullptr, L.G, P + L.wd, B.d, xb, B.d, false, err, w_after, b_after);
+    step_proj_tc(h, ctx, w, ws, PREP_PLAIN, in_xb ? nullptr : ab, L.dq, L.dq, batch, nullptr, 0, P + L.wo, B.d, xb, B.d, false, err);
+    step_proj_tc(h, ctx, w, ws, PREP_NORM, xb, B.d, B.d, batch, (const float*)(P + L.ffn_norm), 0, P + L.wgu, 2 * L.ffn, gub, 2 * L.ffn, true, err);
+    step_proj_tc(h, ctx, w, ws, PREP_SWIGLU, gub, 2 * L.ffn, L.ffn, batch, nullptr, L.G, P + L.wd, B.d, xb, B.d, false, err);
     return;
   }
   KVP_TIMED(KVP_CLASS_STEP_GEMV, launch_step_gemv(ctx, P + L.wo, L.dq, B.d, L.dq, ab, L.dq, batch, xb, B.d, GEMV_RESID, 0, 0));
@@ -690,6 +683,8 @@ static kvp_status prefill_direct(kvp_handle* h, const int32_t* tokens, const int
   char* hbuf = ws + w.h;
   char* qkv = ws + w.qkv;
   const bool split = h->opt.dtype == KVP_BF16;   // K/V path in hi + lo bf16 parts
+  // fp32 mode: norms, rotation and SwiGLU are part of the products around them (gemm_simt.cu), 7 launches an auxiliary layer that were 11.
+  const bool f32 = !split;
   char* h_lo = split ? ws + w.h_lo : nullptr;
   char* kv_lo = split ? ws + w.kv_lo : nullptr;
   float* qkv32 = (float*)(ws + w.qkv32);
@@ -770,7 +765,7 @@ static kvp_status prefill_direct(kvp_handle* h, const int32_t* tokens, const int
     const bool qkv_fused = fused_in[2 * j] != 0, gu_fused = fused_in[2 * j + 1] != 0;
     const bool next_fused = !last && fused_in[2 * (j + 1)] != 0;
     const bool qkv_half = h->qkv_half[j] != 0;
-    if (!qkv_fused)
+    if (!qkv_fused && !f32)
       KVP_TIMED(KVP_CLASS_OTHER, launch_rmsnorm(ctx, x, (const float*)(P + L.attn_norm), A.eps, T, A.d, hbuf, h->opt.dtype, qkv_half ? nullptr : h_lo, qkv_half));
     if (pending_join) {      // the predictor of the layer before reads the key and value buffers that this projection overwrites
       cudaStreamWaitEvent(s, h->ev_join, 0);
@@ -839,8 +834,13 @@ static kvp_status prefill_direct(kvp_handle* h, const int32_t* tokens, const int
       g.split_begin = L.dq - col_begin;    // the K and V columns take the lo part of h as well
       g.W = P + L.wqkv + (size_t)col_begin * A.d * es; g.ldw = A.d; g.N = n_out;
       g.C = qkv32; g.ldc = g.N;
-      KVP_TIMED(KVP_CLASS_AUX_GEMM, launch_gemm_simt(ctx, g, EPI_STORE32));
-      KVP_TIMED(KVP_CLASS_OTHER, launch_rope_split(ctx, qkv32, g.N, T, g.N / L.hd, q_heads + L.nkv, L.hd, tok_pos, A.theta,
+      if (f32) { g.A = x; g.gain = (const float*)(P + L.attn_norm); g.eps = A.eps; }
+      const bool rope_here = f32 && !A.qk_norm;      // (the norm of a head needs all of its columns)
+      if (rope_here) {
+        g.C = qkv + (size_t)col_begin * es; g.ldc = L.nqkv; g.hd = L.hd; g.n_rot = q_heads + L.nkv; g.theta = A.theta; g.tok_pos = tok_pos;
+      }
+      KVP_TIMED(KVP_CLASS_AUX_GEMM, launch_gemm_simt(ctx, g, rope_here ? EPI_ROPE : EPI_STORE32));
+      if (!rope_here) KVP_TIMED(KVP_CLASS_OTHER, launch_rope_split(ctx, qkv32, g.N, T, g.N / L.hd, q_heads + L.nkv, L.hd, tok_pos, A.theta,
                                                    qkv + (size_t)col_begin * es, L.nqkv, kv_lo, 2 * L.dkv, q_heads, q_heads, qn, kn, A.eps));
     }
     if (pg.n_seg > 0) {
@@ -918,7 +918,7 @@ static kvp_status prefill_direct(kvp_handle* h, const int32_t* tokens, const int
       if (gu_fused) return fail(h, KVP_ERR_CUDA, "internal: fused norm planned for a projection the tensor-core kernel refuses");
       KVP_TIMED(KVP_CLASS_AUX_GEMM, launch_gemm_simt(ctx, o, EPI_RESID));
     }
-    if (!gu_fused)
+    if (!gu_fused && !f32)
       KVP_TIMED(KVP_CLASS_OTHER, launch_rmsnorm(ctx, x, (const float*)(P + L.ffn_norm), A.eps, T, A.d, hbuf, h->opt.dtype));
     GemmArgs f{};
     f.A = hbuf; f.lda = A.d; f.W = P + L.wgu; f.ldw = A.d; f.M = T; f.N = 2 * L.ffn; f.K = A.d; f.C = gu; f.ldc = 2 * L.ffn;
@@ -928,8 +928,12 @@ static kvp_status prefill_direct(kvp_handle* h, const int32_t* tokens, const int
     if (gu_fused) { tf.ss_in = norm_ss + (size_t)(2 * j + 1) * T; tf.rms_eps = A.eps; }
     if (!try_tc(h, ctx, tf, KVP_CLASS_AUX_GEMM, &tc_err)) {
       if (gu_fused) return fail(h, KVP_ERR_CUDA, "internal: fused norm planned for a projection the tensor-core kernel refuses");
-      KVP_TIMED(KVP_CLASS_AUX_GEMM, launch_gemm_simt(ctx, f, EPI_STORE));
-      KVP_TIMED(KVP_CLASS_OTHER, launch_swiglu(ctx, gu, T, L.ffn, L.G, act));
+      if (f32) {
+        f.A = x; f.gain = (const float*)(P + L.ffn_norm); f.eps = A.eps; f.C = act; f.ldc = L.ffn;
+        f.gate = RowMap{0, L.G, 0, L.ffn}; f.up = RowMap{L.G == 0 ? L.ffn : 0, L.G, 1, L.ffn};
+      }
+      KVP_TIMED(KVP_CLASS_AUX_GEMM, launch_gemm_simt(ctx, f, f32 ? EPI_GATED : EPI_STORE));
+      if (!f32) KVP_TIMED(KVP_CLASS_OTHER, launch_swiglu(ctx, gu, T, L.ffn, L.G, act));
     }
     GemmArgs d{};
     d.A = act; d.lda = L.ffn; d.W = P + L.wd; d.ldw = L.ffn; d.M = T; d.N = A.d; d.K = L.ffn; d.X = x; d.ldx = A.d;

@@ -6,7 +6,7 @@
 // are the N side (2 * Bp columns: each row as a bf16 hi part and a bf16 lo part of its fp32
 // value, so that the activations lose nothing that matters), and the 128 x 2Bp accumulator
 // lives in tensor memory.  All k blocks of all row tiles form one sequence that is cut into
-// equal contiguous shares, one per SM, so every SM streams weights for the whole launch
+// equal contiguous shares, two per SM, so every SM streams weights for the whole launch
 // whatever the number of row tiles; a share's partial sums are added to the fp32 output with
 // red.global (lanes = consecutive n: 128 contiguous bytes per instruction).
 // Warp 0 feeds a ring of shared-memory stages with TMA, warp 1 issues the MMAs, warps 2-5 drain
@@ -20,12 +20,16 @@ using namespace tcp;
 constexpr int BM = 128, BK = 64;
 constexpr int W_BYTES = BM * BK * 2;
 constexpr int N_THREADS = 192;
-constexpr int SMEM_LIMIT = 220 * 1024;
-// Fewest k blocks of a CTA: a narrow projection (2048 x 2048: 512 blocks) takes 52 SMs, not all.  Every CTA adds a block of partial sums
-// to the output for each tile it touches and holds its SM through the wait for the launch before it, so more CTAs cost other work more
-// than they give: 64 x 123 keys among steps of other batches 1191 -> 1093 us, 8 x 300 974 -> 877; a step by itself 1549 -> 1714.
-constexpr int MIN_KB = 10;
-constexpr size_t STEP_PREFETCH_MAX = 32u << 20;   // bytes of the next weight matrix asked into L2 (L2 holds 126 MB; this kernel streams through it too)
+// Half of an SM's shared memory: a CTA waits for the launch before it and for its first tiles most of its time, so two share an SM,
+// the next projection's or another call's.  With all of it, us, generation step among other calls / by itself, all -> half: 1.1B shape 8 x 300
+// 823 / 1465 -> 652 / 1331, 32 x 200 964 / 1580 -> 808 / 1537, 64 x 123 1035 / 1724 -> 936 / 1771 (three stages of 32 KB are few for one
+// call), 3B shape 16 x 1000 2084 / 2807 -> 1802 / 2832, 4 x 16000 2766 / 3666 -> 2525 / 3573.  A third: 8 x 300 634 / 1371, but 64 x 123 1080 / 2570.
+constexpr int SMEM_LIMIT = 112 * 1024;
+// Fewest k blocks of a CTA: a narrow projection (2048 x 2048: 512 blocks) takes 64 CTAs, a wide one two on every SM.  Every CTA adds a
+// block of partial sums to the output for each tile it touches, so more CTAs serve one call and fewer many.  With one CTA an SM at most /
+// 8 blocks / 6 / 4, among other calls: 64 x 123 918 / 946 / 975 / 990, 3B shape 4 x 16000 2518 / 2559 / 2621 / 2731, 8 x 300 655 / 663 / 677 / 702; by
+// itself: 1787 / 1630 / 1642 / 1520, 3603 / 3455 / 3412 / 3370, 1355 / 1318 / 1330 / 1303.
+constexpr int MIN_KB = 8, CTAS_PER_SM = 2;
 
 struct Params {
   int N, K, batch, Bp;
@@ -33,10 +37,6 @@ struct Params {
   int acc_stride;           // tensor-memory columns between the two accumulators
   float* Y; int ldy;
   int* status;
-  // The weights the NEXT projection will stream (null = none): once this kernel has requested all of its own tiles, every CTA
-  // asks for its share of them to be brought into L2, so HBM keeps streaming through this kernel's tail, the operand
-  // preparation and the launch gap.
-  const char* next_w; long long next_bytes;
 };
 
 __device__ __forceinline__ void red_add(float* dst, float v) {
@@ -80,7 +80,6 @@ step_gemm_kernel(const __grid_constant__ CUtensorMap map_w, const __grid_constan
   auto tempty_bar = [&](int a) { return bar_base + 8u * (2 * S + 2 + a); };
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const uint32_t tmem_cols = max(32, 2 * p.acc_stride);
-  pdl_trigger();      // the next kernel's CTAs may take SMs as this kernel's CTAs leave them
   if (threadIdx.x == 32) { prefetch_tensormap(&map_w); prefetch_tensormap(&map_x); }   // on their way while the rest is set up
 
   if (threadIdx.x == 0) {
@@ -117,6 +116,9 @@ step_gemm_kernel(const __grid_constant__ CUtensorMap map_w, const __grid_constan
         }
       }
       pdl_wait();
+      // Only now, with tensor memory in hand and no wait ahead but for this kernel's own copies: a CTA that waits holds half an SM, which
+      // other calls can use.  Against the trigger at the kernel's start: 64 x 123 936 / 1771 -> 911 / 1775, 32 x 200 - / 1537 -> - / 1454.
+      pdl_trigger();
       int issued = 0;
       while (ok && sched.next(w)) {
         for (int kb = w.kb0; kb < w.kb1 && ok; ++kb, ++issued) {
@@ -129,14 +131,6 @@ step_gemm_kernel(const __grid_constant__ CUtensorMap map_w, const __grid_constan
           }
           tma_load_2d(sw + W_BYTES, &map_x, kb * BK, 0, full_bar(stage));
           if (++stage == S) { stage = 0; phase ^= 1u; }
-        }
-      }
-      if (ok && p.next_w) {
-        constexpr long long CHUNK = 64 * 1024;
-        const long long n_chunks = (p.next_bytes + CHUNK - 1) / CHUNK;
-        for (long long c = blockIdx.x; c < n_chunks; c += gridDim.x) {
-          const long long off = c * CHUNK, len = min(CHUNK, p.next_bytes - off) & ~15ll;
-          if (len > 0) bulk_prefetch_l2(p.next_w + off, (uint32_t)len);
         }
       }
       if (!ok) drain_after_abort();
@@ -306,15 +300,13 @@ void launch_step_prep(const LaunchCtx& ctx, int mode, const float* x, int ldx, i
 }
 
 cudaError_t launch_step_gemm_tc(const bf16* W, int ldw, int N, int K, const bf16* XB, int batch, float* Y, int ldy, int n_sm,
-                                int* status, cudaStream_t st, int64_t* n_launch, const void* next_w, size_t next_bytes) {
+                                int* status, cudaStream_t st, int64_t* n_launch) {
   const int Bp = step_tc_rows(batch);
   CUtensorMap mw, mx;
   if (!tc_make_map_bf16(&mw, W, N, K, ldw, BM)) return cudaErrorInvalidValue;
   if (!tc_make_map_bf16(&mx, XB, 2 * Bp, K, K, 2 * Bp)) return cudaErrorInvalidValue;
   Params p{};
   p.N = N; p.K = K; p.batch = batch; p.Bp = Bp; p.Y = Y; p.ldy = ldy; p.status = status;
-  p.next_w = (((uintptr_t)next_w & 15) == 0) ? (const char*)next_w : nullptr;
-  p.next_bytes = (long long)(next_bytes < STEP_PREFETCH_MAX ? next_bytes : STEP_PREFETCH_MAX);
   p.x_bytes = (2 * Bp * BK * 2 + 1023) / 1024 * 1024;
   p.stages = (SMEM_LIMIT - 2048) / (W_BYTES + p.x_bytes);
   if (p.stages > 12) p.stages = 12;
@@ -325,7 +317,7 @@ cudaError_t launch_step_gemm_tc(const bf16* W, int ldw, int N, int K, const bf16
   if (e != cudaSuccess) return e;
   const long long total = (long long)((N + BM - 1) / BM) * ((K + BK - 1) / BK);
   const long long want = (total + MIN_KB - 1) / MIN_KB;
-  const int grid = (int)(want < n_sm ? want : n_sm);
+  const int grid = (int)(want < CTAS_PER_SM * n_sm ? want : CTAS_PER_SM * n_sm);
   ++*n_launch;
   return launch_overlapped(step_gemm_kernel, dim3(grid), dim3(N_THREADS), (size_t)smem, st, mw, mx, p);
 }
