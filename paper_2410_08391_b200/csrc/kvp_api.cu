@@ -147,10 +147,10 @@ WsLayout ws_layout(const kvp_handle* h, int64_t Bm, int64_t Tm) {
   const int64_t k_max = std::max((int64_t)B.d, std::max((int64_t)B.max_dq, (int64_t)B.max_ffn));
   w.xbt = take(2 * Bp * k_max * 2);
   w.gub = take(Bm * 2 * (size_t)B.max_ffn * 4);
-  // The persistent kernel of small batches uses none of the seven buffers above: its tagged values (64 bits each) take
+  // The persistent kernels of small batches use none of the seven buffers above: its tagged values (64 bits each) take
   // their place, at the end, so that they and its split partials in w.part are cleared as one range.
   const size_t Bq = (size_t)std::min<int64_t>(Bm, 4);
-  const size_t ll = h->opt.dtype == KVP_BF16 ? Bq * ((size_t)B.max_nqkv + B.max_dq + 2 * (size_t)B.d + B.max_ffn) * 8 + 5 * 256 : 0;
+  const size_t ll = Bq * ((size_t)B.max_nqkv + B.max_dq + 2 * (size_t)B.d + B.max_ffn) * 8 + 5 * 256;
   off = std::max(off, align_up(step0 + ll, 256));
   w.ll = off - align_up(ll, 256);
   w.part = take((size_t)(2 * std::max(148, h->n_sm) + Bm * B.max_nkv) * B.max_group * (B.L[0].hd + 2) * 4);
@@ -346,7 +346,6 @@ bool mega_prepare(kvp_handle* h, const LaunchCtx& ctx, const kvp_cache* cache, c
   p.tokens = tokens; p.gather_idx = gather_idx;
   p.embed = P + B.embed; p.final_norm = (const float*)(P + B.final_norm); p.lm_head = P + B.lm_head;
   p.block_table = cache->block_table; p.mpps = cache->max_pages_per_seq; p.n_pages = cache->n_pages; p.seq_lens = cache->seq_lens;
-  p.xb = (float*)(ws + w.xb); p.qkvb = (float*)(ws + w.qkvb); p.ab = (float*)(ws + w.ab); p.actb = (float*)(ws + w.actb);
   p.part = (float*)(ws + w.part);
   p.attn_done = (int*)(ws + w.attn_done);
   p.logits = logits; p.token_out = token_out; p.status = ctx.status;
@@ -379,14 +378,15 @@ bool mega_prepare(kvp_handle* h, const LaunchCtx& ctx, const kvp_cache* cache, c
   return true;
 }
 
-// What has to be zero in the workspace before the first launch of a step: the tagged values of the tensor-core kernel (with
-// its split partials behind them), or the split counters of the other one.
+// What has to be zero in the workspace before the first launch of a step: the tagged values, and behind them the split partials of
+// the tensor-core kernel, or the split counters of the other one.
 void mega_clear(kvp_handle* h, const MegaParams& p, const WsLayout& w, char* ws, cudaStream_t st) {
   const ModelPlan& B = h->base;
-  if (mega_uses_mma(h, p.batch))
-    cudaMemsetAsync(ws + w.ll, 0, w.part - w.ll + (size_t)h->n_sm * B.max_group * (B.L[0].hd + 2) * 8, st);
-  else
-    cudaMemsetAsync(p.attn_done, 0, (size_t)p.batch * B.max_nkv * 4, st);
+  const bool mma = mega_uses_mma(h, p.batch);
+  cudaMemsetAsync(ws + w.ll, 0, w.part - w.ll + (mma ? (size_t)h->n_sm * B.max_group * (B.L[0].hd + 2) * 8 : 0), st);
+  bool splits = false;
+  for (int i = 0; i < B.n_layers; ++i) splits = splits || p.layers[i].n_split > 1;
+  if (!mma && splits) cudaMemsetAsync(p.attn_done, 0, (size_t)p.batch * B.max_nkv * 4, st);
 }
 
 // The whole base step (all layers, LM head, argmax) as one persistent kernel; false = not applicable.

@@ -2,15 +2,18 @@
 //
 // A step is ~170 dependent, bandwidth-bound operations of a few microseconds each; as separate
 // kernels their launch and ramp-up latency is several times the time the weights need to stream
-// from HBM.  Here one CTA of 16 warps per SM stays resident for the whole step.  The operations
-// become phases separated by a grid-wide barrier (one global counter, bounded spin):
-//   per layer:  q(kv) projection (RMSNorm fused) | [append k,v] | attention over cache pages |
-//               (key-range splits merged by the CTA that finishes a group's last split) | O projection + residual | gate/up + SwiGLU (RMSNorm
+// from HBM.  Here one CTA of 16 warps per SM stays resident for the whole step.  The operations become phases:
+//   per layer:  q(kv) projection (RMSNorm fused) | attention over cache pages, which takes the step's own key and value in (key-range
+//               splits merged by the CTA that finishes a group's last split) | O projection + residual | gate/up + SwiGLU (RMSNorm
 //               fused) | down projection + residual;   then LM head (final RMSNorm fused) + argmax.
+// No grid-wide barrier stands between them: every value that crosses CTAs is one 64-bit word {fp32 value, layer tag}, and who needs
+// it polls the word itself (step_waits.cuh).  Barrier, fence and counter took 4 of a phase's 6 us on models of test size.
+// A word is written again, one layer on, only by who has seen values that all of its readers had a part in: every phase needs every
+// output of the phase before it, and CTAs without a row (or an attention item) of a phase don't read its input.
 // Weights never pass through registers on their way from HBM: every warp owns a small ring of
 // shared-memory slots that it fills with bulk asynchronous copies (cp.async.bulk, completion on
 // an mbarrier) of the weight rows it will need, in schedule order.  The schedule is static, so a
-// warp keeps its ring full ACROSS phase boundaries: while the SMs wait at a barrier, or run
+// warp keeps its ring full ACROSS phase boundaries: while the SMs wait for one another, or run
 // attention, the first rows of the next projection are already landing.  About 190 KB per SM are
 // in flight, which is what HBM latency times bandwidth asks for.
 #include <math.h>
@@ -18,6 +21,7 @@
 #include "common.cuh"
 #include "tc_ptx.cuh"
 #include "step_mega.h"
+#include "step_waits.cuh"
 
 namespace {
 using namespace tcp;
@@ -26,30 +30,6 @@ constexpr int NT = 512;                 // threads per CTA, one CTA per SM
 constexpr int NW = NT / 32;
 constexpr int MAXG = 8;
 constexpr int NSLOT = 3;                // ring slots per warp
-
-
-// Grid-wide barrier: every CTA adds one to *counter and waits until it reaches `target`.
-// Returns false when the wait ran out (or some role already gave up): the caller leaves.
-__device__ __forceinline__ bool grid_barrier(unsigned* counter, unsigned target, int* status, volatile int* s_abort, int* s_flag) {
-  __syncthreads();
-  if (threadIdx.x == 0) {
-    int ok = *s_abort ? 0 : 1;
-    __threadfence();
-    atomicAdd(counter, 1u);
-    unsigned it = 0;
-    while (ok) {
-      unsigned v;
-      asm volatile("ld.acquire.gpu.global.u32 %0, [%1];" : "=r"(v) : "l"(counter) : "memory");
-      if (v >= target) break;
-      if (++it > L2_POLL_LIMIT) { dev_flag(status, DEV_TIMEOUT); ok = 0; break; }
-      if ((it & 255u) == 0u && *reinterpret_cast<volatile int*>(status) == DEV_TIMEOUT) { ok = 0; break; }
-    }
-    if (ok && *reinterpret_cast<volatile int*>(status) == DEV_TIMEOUT) ok = 0;
-    *s_flag = ok;
-  }
-  __syncthreads();
-  return *s_flag != 0;
-}
 
 struct GemvDesc {
   const void* W; int N, K;          // rows, row length (= leading dimension)
@@ -148,13 +128,23 @@ template <> __device__ __forceinline__ float dot_w8<float>(const unsigned char* 
   return a + b;
 }
 
-// One projection phase for this warp: y[b, n] (op)= sum_k W[n, k] xs[b, k] over the warp's rows,
+// A row of the residual stream: tagged values, or (before the first layer) the embedding of the row's token.
+template <class T> struct Stream {
+  const u64* x; uint32_t tag; const T* embed[4];
+};
+// The residual of row n of a projection on its way (lane 0, which stores the row).
+template <class T, int BB>
+__device__ __forceinline__ void ask_residual(const MegaParams& p, const Stream<T>& in, int n, int N, int lane, u64 (&old)[BB]) {
+#pragma unroll
+  for (int b = 0; b < BB; ++b) old[b] = in.x && lane == 0 && b < p.batch && n < N ? ll_load(in.x + (size_t)b * N + n) : 0ull;
+}
+// One projection phase for this warp: y[b, n] = sum_k W[n, k] xs[b, k] (+ residual) over the warp's rows,
 // consuming the warp's chunk stream.  xs is the staged (normalised) input in shared memory and
-// ring_ptr the address of the warp's first slot.
+// ring_ptr the address of the warp's first slot.  y: tagged values, or (null) the logits.
 template <class T, int BB>
 __device__ __forceinline__ void gemv_phase(const MegaParams& p, const GemvDesc g, WarpStream& ws, const unsigned char* ring_ptr,
-                                           const float* xs, float* y, int ldy, int gw, int GW, int lane,
-                                           unsigned long long* best, volatile int* s_abort) {
+                                           const float* xs, u64* y, uint32_t tag, const Stream<T>* resid, u64 (&old)[BB], int gw, int GW,
+                                           int lane, unsigned long long* best, volatile int* s_abort, bool& dead) {
   const int K = g.K, row_bytes = K * (int)sizeof(T);
   const int cpr = (row_bytes + ws.slot_bytes - 1) / ws.slot_bytes;
   const int R = g.mode == GEMV_SWIGLU ? 2 : 1;
@@ -165,6 +155,8 @@ __device__ __forceinline__ void gemv_phase(const MegaParams& p, const GemvDesc g
 #pragma unroll
   for (int b = 0; b < BB; ++b) { acc[b] = 0.f; accu[b] = 0.f; }
   for (int n = gw; n < g.N; n += GW) {
+    if (n != gw && resid) ask_residual<T, BB>(p, *resid, n, g.N, lane, old);      // (the first row's were asked for in front of the phase)
+    bool refill = false;
     for (int which = 0; which < R; ++which) {
       for (int part = 0; part < cpr; ++part) {
         const unsigned slot = ws.consumed % NSLOT;
@@ -201,7 +193,9 @@ __device__ __forceinline__ void gemv_phase(const MegaParams& p, const GemvDesc g
         ++ws.consumed;
         __syncwarp();
         asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
-        if (got) stream_fill<T>(p, ws, gw, GW, lane);
+        // the ring is filled again behind the output, which others wait for (filled first it took 300 to 500 cycles of every phase)
+        refill = got;
+        if (got && !(which == R - 1 && part == cpr - 1)) stream_fill<T>(p, ws, gw, GW, lane);
       }
     }
     // all pieces of this output are in: reduce, apply, store
@@ -210,11 +204,14 @@ __device__ __forceinline__ void gemv_phase(const MegaParams& p, const GemvDesc g
       float v = warp_sum(acc[b]);
       float u = R == 2 ? warp_sum(accu[b]) : 0.f;
       if (lane == 0 && b < p.batch && !*s_abort) {
-        float* dst = y + (size_t)b * ldy + n;
-        if (g.mode == GEMV_SWIGLU) *dst = v / (1.f + __expf(-v)) * u;
-        else if (g.mode == GEMV_RESID) *dst = __ldcg(dst) + v;
+        if (g.mode == GEMV_SWIGLU) v = v / (1.f + __expf(-v)) * u;
+        if (resid) {
+          if (!resid->x) v += resid->embed[b] ? to_f(resid->embed[b][n]) : 0.f;
+          else v += ll_tag(old[b]) == resid->tag ? ll_val(old[b]) : ll_wait(resid->x + (size_t)b * g.N + n, resid->tag, dead, s_abort, p.status);
+        }
+        if (y) ll_store(y + (size_t)b * g.N + n, v, tag);
         else {
-          *dst = v;
+          p.logits[(size_t)b * g.N + n] = v;
           if (best) {   // running argmax: larger value wins, then the lower index
             unsigned bits = __float_as_uint(v);
             bits = (bits & 0x80000000u) ? ~bits : (bits | 0x80000000u);
@@ -224,57 +221,62 @@ __device__ __forceinline__ void gemv_phase(const MegaParams& p, const GemvDesc g
       }
       acc[b] = 0.f; accu[b] = 0.f;
     }
+    if (refill) stream_fill<T>(p, ws, gw, GW, lane);
   }
 }
 
 // Stage `batch` activation rows of length K into shared memory, optionally RMS-normalised
-// (one pass: the row is held in registers between the sum of squares and the scaled store).
-template <int BB>
-__device__ __noinline__ void stage_x(const float* x, int ldx, int K, int batch, const float* gain, float eps, float* xs,
-                                     float* red) {
-  const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+// (one pass: the row is held in registers between the sum of squares and the scaled store).  J: elements a thread holds.
+template <class T, int BB, int J>
+__device__ __noinline__ void stage_rows(const MegaParams& p, const Stream<T>& in, int K, const float* gain, float* xs, float* red,
+                                     volatile int* s_abort, bool& dead) {
+  const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31, batch = p.batch;
   const int KS = xs_stride(K);
-  if (gain && K <= 8 * NT) {
-    float v[BB][8];
+  if (K <= J * NT) {
+    float v[BB][J], g[J];
     float ss[BB];
+#pragma unroll
+    for (int j = 0; j < J; ++j) { const int k = tid + j * NT; g[j] = gain && k < K ? __ldg(gain + k) : 1.f; }
+    constexpr int BS = J == 1 ? BB : 1;            // rows whose words are asked for together, until all have the tag
+#pragma unroll
+    for (int b0 = 0; b0 < BB; b0 += BS) {
+      if (in.x) {
+        bool ok;
+        unsigned it = 0;
+        do {
+          ok = true;
+#pragma unroll
+          for (int b = b0; b < b0 + BS; ++b)
+#pragma unroll
+            for (int j = 0; j < J; ++j) {
+              const int k = tid + j * NT;
+              const u64 w = k < K && b < batch ? ll_load(in.x + (size_t)b * K + k) : (u64)in.tag << 32;
+              ok = ok && ll_tag(w) == in.tag;
+              v[b][j] = ll_val(w);
+            }
+          if (!ok && !dead && !poll_more(it, s_abort, p.status)) dead = true;
+        } while (!ok && !dead);
+      } else {
+#pragma unroll
+        for (int b = b0; b < b0 + BS; ++b)
+#pragma unroll
+          for (int j = 0; j < J; ++j) {
+            const int k = tid + j * NT;
+            v[b][j] = k < K && in.embed[b] ? to_f(in.embed[b][k]) : 0.f;
+          }
+      }
+    }
 #pragma unroll
     for (int b = 0; b < BB; ++b) {
       ss[b] = 0.f;
 #pragma unroll
-      for (int j = 0; j < 8; ++j) {
-        int k = tid + j * NT;
-        v[b][j] = (k < K && b < batch) ? __ldcg(x + (size_t)b * ldx + k) : 0.f;
-        ss[b] = fmaf(v[b][j], v[b][j], ss[b]);
-      }
+      for (int j = 0; j < J; ++j) ss[b] = fmaf(v[b][j], v[b][j], ss[b]);
     }
-#pragma unroll
-    for (int b = 0; b < BB; ++b) { float t = warp_sum(ss[b]); if (lane == 0) red[warp * BB + b] = t; }
-    __syncthreads();
-#pragma unroll
-    for (int b = 0; b < BB; ++b) {
-      float t = 0.f;
-#pragma unroll
-      for (int w = 0; w < NW; ++w) t += red[w * BB + b];
-      float r = rsqrtf(t / (float)K + eps);
-#pragma unroll
-      for (int j = 0; j < 8; ++j) {
-        int k = tid + j * NT;
-        if (k < K) xs[b * KS + xs_index(k)] = gain[k] * v[b][j] * r;
-      }
-    }
-  } else {
     float r[BB];
 #pragma unroll
     for (int b = 0; b < BB; ++b) r[b] = 1.f;
+    __syncthreads();                               // (the staging area and `red` are free: the phase before this one has been read out)
     if (gain) {
-      float ss[BB];
-#pragma unroll
-      for (int b = 0; b < BB; ++b) ss[b] = 0.f;
-      for (int k = tid; k < K; k += NT) {
-#pragma unroll
-        for (int b = 0; b < BB; ++b)
-          if (b < batch) { float t = __ldcg(x + (size_t)b * ldx + k); ss[b] = fmaf(t, t, ss[b]); }
-      }
 #pragma unroll
       for (int b = 0; b < BB; ++b) { float t = warp_sum(ss[b]); if (lane == 0) red[warp * BB + b] = t; }
       __syncthreads();
@@ -283,16 +285,51 @@ __device__ __noinline__ void stage_x(const float* x, int ldx, int K, int batch, 
         float t = 0.f;
 #pragma unroll
         for (int w = 0; w < NW; ++w) t += red[w * BB + b];
-        r[b] = rsqrtf(t / (float)K + eps);
+        r[b] = rsqrtf(t / (float)K + p.eps);
       }
     }
-    for (int k = tid; k < K; k += NT) {
-      float g = gain ? gain[k] : 1.f;
 #pragma unroll
-      for (int b = 0; b < BB; ++b) xs[b * KS + xs_index(k)] = b < batch ? g * __ldcg(x + (size_t)b * ldx + k) * r[b] : 0.f;
+    for (int b = 0; b < BB; ++b)
+#pragma unroll
+      for (int j = 0; j < J; ++j) {
+        const int k = tid + j * NT;
+        if (k < K) xs[b * KS + xs_index(k)] = g[j] * v[b][j] * r[b];
+      }
+  } else {
+    float ss[BB];
+#pragma unroll
+    for (int b = 0; b < BB; ++b) ss[b] = 0.f;
+    __syncthreads();
+    for (int k = tid; k < K; k += NT) {
+#pragma unroll
+      for (int b = 0; b < BB; ++b) {
+        float t = 0.f;
+        if (b < batch) t = in.x ? ll_wait(in.x + (size_t)b * K + k, in.tag, dead, s_abort, p.status) : (in.embed[b] ? to_f(in.embed[b][k]) : 0.f);
+        ss[b] = fmaf(t, t, ss[b]);
+        xs[b * KS + xs_index(k)] = t;
+      }
+    }
+    if (gain) {
+#pragma unroll
+      for (int b = 0; b < BB; ++b) { float t = warp_sum(ss[b]); if (lane == 0) red[warp * BB + b] = t; }
+      __syncthreads();
+#pragma unroll
+      for (int b = 0; b < BB; ++b) {
+        float t = 0.f;
+#pragma unroll
+        for (int w = 0; w < NW; ++w) t += red[w * BB + b];
+        const float r = rsqrtf(t / (float)K + p.eps);
+        for (int k = tid; k < K; k += NT) xs[b * KS + xs_index(k)] = gain[k] * xs[b * KS + xs_index(k)] * r;      // (a thread's own elements)
+      }
     }
   }
   __syncthreads();
+}
+template <class T, int BB>
+__device__ __forceinline__ void stage_x(const MegaParams& p, const Stream<T>& in, int K, const float* gain, float* xs, float* red,
+                                        volatile int* s_abort, bool& dead) {
+  if (K <= NT) stage_rows<T, BB, 1>(p, in, K, gain, xs, red, s_abort, dead);      // (a model of test size: less code to fetch, all rows at once)
+  else stage_rows<T, BB, 8>(p, in, K, gain, xs, red, s_abort, dead);
 }
 
 // Attention of one (sequence, kv head, key-range split) over whole cache pages: the K and V page
@@ -301,7 +338,8 @@ __device__ __noinline__ void stage_x(const float* x, int ldx, int K, int batch, 
 // (dim, head subset).
 template <class T>
 __device__ __noinline__ void attn_item(const MegaParams& p, const MegaLayer& L, int b, int kvh, int sp, int n_split,
-                                       const float* q, int ldq, unsigned char* sm, float* part, float* out) {
+                                       const u64* q, int ldq, uint32_t tag, const float2* rope, unsigned char* sm, float* part,
+                                       u64* out, volatile int* s_abort, bool& dead) {
   const int hd = p.hd, nq = L.nq, nkv = L.nkv, group = nq / nkv;
   const int row_bytes = hd * (int)sizeof(T) + 16;
   unsigned char* Ks = sm;
@@ -311,52 +349,95 @@ __device__ __noinline__ void attn_item(const MegaParams& p, const MegaLayer& L, 
   float* m_run = ps + MAXG * PAGE_TOKENS;
   float* l_run = m_run + MAXG;
   float* alpha = l_run + MAXG;
+  float* rn = alpha + MAXG;                            // 1 / rms of the query heads, and of the new key
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
   const int n_keys = __ldcg(p.seq_lens + b) + (p.generation ? 1 : 0);
   const int pos = n_keys - 1;
   const float scale = rsqrtf((float)hd);
   const int half = hd >> 1;
   __syncthreads();                                   // shared memory free (previous item / phase)
-  if (L.q_norm) head_rnorm(q + (size_t)b * ldq + (size_t)kvh * group * hd, group, hd, p.eps, ps);   // ps is free until the first page's scores
-  for (int i = tid; i < group * half; i += NT) {
-    int h = i / half, c = i - h * half;
-    const float* qh = q + (size_t)b * ldq + (size_t)(kvh * group + h) * hd;
-    float sn, cs;
-    rope_sincos(pos, p.inv.f[c], &sn, &cs);
-    float x1 = __ldcg(qh + c), x2 = __ldcg(qh + c + half);
-    if (L.q_norm) { const float rn = ps[h]; x1 *= rn * L.q_norm[c]; x2 *= rn * L.q_norm[c + half]; }
-    qs[h * hd + c] = (x1 * cs - x2 * sn) * scale;
-    qs[h * hd + c + half] = (x2 * cs + x1 * sn) * scale;
-  }
-  if (tid < MAXG) { m_run[tid] = -INFINITY; l_run[tid] = 0.f; alpha[tid] = 1.f; }
+  typedef typename KvOf<T>::type KT;                   // cache element: fp32, or 16-bit half in bf16 mode
   const int n_pg = (n_keys + PAGE_TOKENS - 1) / PAGE_TOKENS;
   const int per = (n_pg + n_split - 1) / n_split;
   const int pg0 = sp * per, pg1 = min(n_pg, pg0 + per);
+  // the step's own key and value: the item whose range ends with their page takes them into its copy of the page and into the pool
+  const bool has_new = p.generation && pg0 < pg1 && pg1 == n_pg;
+  // A page into shared memory (every thread; its id, or -1).  The first one is fetched in front of the wait for the queries.
+  const int chunks_per_row = hd * (int)sizeof(KT) / 16;
+  const int n_chunks = PAGE_TOKENS * chunks_per_row;
+  auto load_page = [&](int pg) {
+    const int page = pg < p.mpps ? p.block_table[(size_t)b * p.mpps + pg] : -1;
+    if (page < 0 || page >= p.n_pages) {
+      if (tid == 0) dev_flag(p.status, DEV_BAD_PAGE);
+      return -1;
+    }
+    const uint4* ksrc = reinterpret_cast<const uint4*>((const KT*)L.kpool + ((size_t)page * nkv + kvh) * PAGE_TOKENS * hd);
+    const uint4* vsrc = reinterpret_cast<const uint4*>((const KT*)L.vpool + ((size_t)page * nkv + kvh) * PAGE_TOKENS * hd);
+    for (int i = tid; i < n_chunks; i += NT) {
+      int r = i / chunks_per_row, cc = i - r * chunks_per_row;
+      uint4 kx = __ldcg(ksrc + i), vx = __ldcg(vsrc + i);
+      *reinterpret_cast<uint4*>(Ks + r * row_bytes + cc * 16) = kx;
+      *reinterpret_cast<uint4*>(Vs + r * row_bytes + cc * 16) = vx;
+    }
+    return page;
+  };
+  int page = pg0 < pg1 ? load_page(pg0) : -1;
+  float* knew = ps;                                    // (ps is free until the first page's scores) [hd] key, [hd] value
+  for (int i = tid; i < group * hd; i += NT) qs[i] = ll_wait(q + (size_t)b * ldq + (size_t)kvh * group * hd + i, tag, dead, s_abort, p.status);
+  if (has_new)
+    for (int i = tid; i < 2 * hd; i += NT)
+      knew[i] = ll_wait(q + (size_t)b * ldq + L.dq + (size_t)((i < hd ? 0 : nkv) + kvh) * hd + (i < hd ? i : i - hd), tag, dead, s_abort, p.status);
+  __syncthreads();
+  if (L.q_norm) {
+    const int heads = group + (has_new ? 1 : 0);
+    if (warp < heads) {                                // (at most 9 of the 16 warps)
+      const float* x = warp < group ? qs + warp * hd : knew;
+      float ss = 0.f;
+      for (int c = lane; c < hd; c += 32) ss = fmaf(x[c], x[c], ss);
+      ss = warp_sum(ss);
+      if (lane == 0) rn[warp] = rsqrtf(ss / (float)hd + p.eps);
+    }
+    __syncthreads();
+  }
+  for (int i = tid; i < (group + (has_new ? 1 : 0)) * half; i += NT) {
+    const int h = i / half, c = i - h * half;
+    const bool key = h == group;
+    float* x = key ? knew : qs + h * hd;
+    const float cs = rope[c].x, sn = rope[c].y;
+    float x1 = x[c], x2 = x[c + half];
+    if (L.q_norm) { const float* gn = key ? L.k_norm : L.q_norm; x1 *= rn[h] * gn[c]; x2 *= rn[h] * gn[c + half]; }
+    const float f = key ? 1.f : scale;
+    x[c] = (x1 * cs - x2 * sn) * f;
+    x[c + half] = (x2 * cs + x1 * sn) * f;
+  }
+  KT* knew_kt = reinterpret_cast<KT*>(rn + MAXG + 8);   // [2][hd], as the cache holds them
+  __syncthreads();
+  if (has_new && tid < 2 * hd) knew_kt[tid] = from_f<KT>(knew[tid]);
+  if (tid < MAXG) { m_run[tid] = -INFINITY; l_run[tid] = 0.f; alpha[tid] = 1.f; }
   const int key = tid & 63, hh_s = tid >> 6;           // scores: thread = (key, head hh_s)
-  const int nhh = NT / hd;                             // value sum: heads hh_v, hh_v + nhh, ...
-  const int dim = tid % hd, hh_v = tid / hd;
+  // Value sum: NT / hd threads a dim.  They take a head each (and the one NT / hd further on), or, where there are more of them than heads,
+  // every key_step-th key of a head (one thread a head went through 64 keys, 900 cycles a page, while the others waited).
+  const int nhh = NT / hd, dim = tid % hd, slot_v = tid / hd;
+  const bool by_keys = nhh >= 2 * group;
+  const int key_step = by_keys ? nhh / group : 1, head0 = by_keys ? slot_v % group : slot_v, key0 = by_keys ? slot_v / group : 0;
+  const bool sums = key0 < key_step;
   float o[MAXG];
 #pragma unroll
   for (int i = 0; i < MAXG; ++i) o[i] = 0.f;
-  typedef typename KvOf<T>::type KT;                   // cache element: fp32, or 16-bit half in bf16 mode
-  const int chunks_per_row = hd * (int)sizeof(KT) / 16;
-  const int n_chunks = PAGE_TOKENS * chunks_per_row;
-  const KT* kpool = (const KT*)L.kpool;
-  const KT* vpool = (const KT*)L.vpool;
   for (int pg = pg0; pg < pg1; ++pg) {
-    int page = pg < p.mpps ? p.block_table[(size_t)b * p.mpps + pg] : -1;
-    bool page_ok = page >= 0 && page < p.n_pages;
-    if (!page_ok && tid == 0) dev_flag(p.status, DEV_BAD_PAGE);
-    const int nk = page_ok ? min(PAGE_TOKENS, n_keys - pg * PAGE_TOKENS) : 0;
-    __syncthreads();
-    if (page_ok) {
-      const uint4* ksrc = reinterpret_cast<const uint4*>(kpool + ((size_t)page * nkv + kvh) * PAGE_TOKENS * hd);
-      const uint4* vsrc = reinterpret_cast<const uint4*>(vpool + ((size_t)page * nkv + kvh) * PAGE_TOKENS * hd);
-      for (int i = tid; i < n_chunks; i += NT) {
-        int r = i / chunks_per_row, cc = i - r * chunks_per_row;
-        uint4 kx = __ldcg(ksrc + i), vx = __ldcg(vsrc + i);
-        *reinterpret_cast<uint4*>(Ks + r * row_bytes + cc * 16) = kx;
-        *reinterpret_cast<uint4*>(Vs + r * row_bytes + cc * 16) = vx;
+    if (pg != pg0) {
+      __syncthreads();
+      page = load_page(pg);
+    }
+    const int nk = page >= 0 ? min(PAGE_TOKENS, n_keys - pg * PAGE_TOKENS) : 0;
+    if (has_new && pg == n_pg - 1 && page >= 0) {
+      __syncthreads();
+      const int row = pos % PAGE_TOKENS;
+      for (int i = tid; i < 2 * hd; i += NT) {
+        const int c = i < hd ? i : i - hd;
+        const KT x = knew_kt[i];
+        reinterpret_cast<KT*>((i < hd ? Ks : Vs) + row * row_bytes)[c] = x;
+        ((KT*)(i < hd ? L.kpool : L.vpool))[(((size_t)page * nkv + kvh) * PAGE_TOKENS + row) * hd + c] = x;
       }
     }
     __syncthreads();
@@ -397,24 +478,31 @@ __device__ __noinline__ void attn_item(const MegaParams& p, const MegaLayer& L, 
     __syncthreads();
 #pragma unroll
     for (int i = 0; i < MAXG; ++i) {
-      int h = hh_v + nhh * i;
-      if (i * nhh < MAXG && h < group) {
+      const int h = head0 + nhh * i;
+      if (i * nhh < MAXG && (i == 0 || !by_keys) && h < group && sums) {
         float acc = o[i] * alpha[h];
         const float* pr = ps + h * PAGE_TOKENS;
-        for (int s = 0; s < nk; ++s) acc = fmaf(pr[s], to_f(reinterpret_cast<const KT*>(Vs + s * row_bytes)[dim]), acc);
+#pragma unroll 4
+        for (int s = key0; s < nk; s += key_step) acc = fmaf(pr[s], to_f(reinterpret_cast<const KT*>(Vs + s * row_bytes)[dim]), acc);
         o[i] = acc;
       }
     }
   }
   __syncthreads();
+  if (by_keys) {                                       // the parts of a sum meet in shared memory (the pages have been read)
+    float* parts = reinterpret_cast<float*>(sm);       // [key_step][group][hd]
+    if (sums) parts[(key0 * group + head0) * hd + dim] = o[0];
+    __syncthreads();
+    if (key0 == 0) for (int k = 1; k < key_step; ++k) o[0] += parts[(k * group + head0) * hd + dim];
+  }
   const int ldr = hd + 2;
 #pragma unroll
   for (int i = 0; i < MAXG; ++i) {
-    int h = hh_v + nhh * i;
-    if (i * nhh < MAXG && h < group) {
+    const int h = head0 + nhh * i;
+    if (i * nhh < MAXG && (i == 0 || !by_keys) && h < group && key0 == 0) {
       int qh = kvh * group + h;
       if (n_split == 1) {
-        out[(size_t)b * nq * hd + (size_t)qh * hd + dim] = o[i] / l_run[h];
+        ll_store(out + (size_t)b * nq * hd + (size_t)qh * hd + dim, o[i] / l_run[h], tag);
       } else {
         float* pr = part + (((size_t)b * nq + qh) * n_split + sp) * ldr;
         pr[dim] = o[i];
@@ -428,10 +516,10 @@ template <class T, int BB>
 __global__ void __launch_bounds__(NT, 1) step_mega_kernel(const __grid_constant__ MegaParams p) {
   extern __shared__ __align__(128) unsigned char sm_raw[];
   __shared__ float red[NW * BB];
-  __shared__ int s_flag;
   __shared__ int s_last;
   __shared__ int s_abort_mem;
   __shared__ __align__(8) unsigned long long s_bars[NW * NSLOT];
+  __shared__ float2 rope[BB][64];      // (cos, sin) of each sequence's last position
   volatile int* s_abort = &s_abort_mem;
   // dynamic shared memory: [ x staging / attention scratch | per-warp rings ]
   float* xs = reinterpret_cast<float*>(sm_raw);
@@ -455,64 +543,37 @@ __global__ void __launch_bounds__(NT, 1) step_mega_kernel(const __grid_constant_
   stream_load_phase<T>(p, ws, gw);
   stream_fill<T>(p, ws, gw, GW, lane);        // the first weight rows start streaming before anything else
 
-  unsigned phase = 0;
-#define BARRIER()                                                                                                   \
-  do {                                                                                                              \
-    ++phase;                                                                                                        \
-    if (p.trace && blockIdx.x == 0 && tid == 0 && phase < 900) p.trace[2 * phase] = clock64();                     \
-    if (!grid_barrier(counter, phase * gridDim.x, p.status, s_abort, &s_flag)) {                                    \
-      for (int i_ = 0; i_ < 2000; ++i_) __nanosleep(1000); /* let copies in flight land before the CTA goes */      \
-      return;                                                                                                       \
-    }                                                                                                               \
-    if (p.trace && blockIdx.x == 0 && tid == 0 && phase < 900) p.trace[2 * phase + 1] = clock64();                 \
-  } while (0)
-
-  // embedding gather (+ clear the argmax slots)
-  if (p.do_embed)
-  for (int i = blockIdx.x * NT + tid; i < batch * p.d; i += gridDim.x * NT) {
-    int b = i / p.d, c = i - b * p.d;
-    int tok = p.tokens[p.gather_idx ? p.gather_idx[b] : b];
-    bool ok = tok >= 0 && tok < p.vocab;
-    if (!ok && c == 0) dev_flag(p.status, DEV_BAD_TOKEN);
-    p.xb[(size_t)b * p.d + c] = ok ? to_f(((const T*)p.embed)[(size_t)tok * p.d + c]) : 0.f;
+  if (tid < batch * (p.hd >> 1)) {     // (once, not in every layer: 2000 cycles of 64-bit arithmetic)
+    const int b = tid / (p.hd >> 1), c = tid - b * (p.hd >> 1);
+    float sn, cs;
+    rope_sincos(__ldcg(p.seq_lens + b) + (p.generation ? 0 : -1), p.inv.f[c], &sn, &cs);
+    rope[b][c] = make_float2(cs, sn);
   }
-  if (blockIdx.x == 0 && tid < BB) best[tid] = 0ull;
-  BARRIER();
-
+  bool dead = false;                  // this thread has given up waiting
+  // the residual stream in front of the first layer
+  Stream<T> first{nullptr, 0u, {nullptr, nullptr, nullptr, nullptr}};
+  if (p.do_embed) {
+#pragma unroll
+    for (int b = 0; b < BB; ++b) {
+      if (b >= batch) continue;
+      const int tok = p.tokens[p.gather_idx ? p.gather_idx[b] : b];
+      const bool ok = tok >= 0 && tok < p.vocab;
+      if (!ok && blockIdx.x == 0 && tid == 0) dev_flag(p.status, DEV_BAD_TOKEN);
+      first.embed[b] = ok ? (const T*)p.embed + (size_t)tok * p.d : nullptr;
+    }
+  }
+  const int row0 = blockIdx.x * NW;   // the CTA's first row of a projection: without one it does not read the phase's input
   for (int i = p.layer_begin; i < p.layer_end; ++i) {
     const MegaLayer& L = p.layers[i];
     const int n_out = p.generation ? L.nqkv : L.dq;
+    const uint32_t tag = (uint32_t)i + 1u;
+    const Stream<T> x2{p.ll_x2, tag - 1u, {}}, x1{p.ll_x1, tag, {}}, a{p.ll_a, tag, {}}, h{p.ll_h, tag, {}};
+    const Stream<T>& in = p.do_embed && i == 0 ? first : x2;
+    u64 old[BB];        // the residual of the warp's first row
     // ---- q (k, v) projection
-    stage_x<BB>(p.xb, p.d, p.d, batch, L.attn_norm, p.eps, xs, red);
-    gemv_phase<T, BB>(p, stream_desc(p, 4 * i), ws, ring_ptr, xs, p.qkvb, n_out, gw, GW, lane, nullptr, s_abort);
-    BARRIER();
-    if (p.generation) {   // append the new key (after RoPE) and value at position seq_lens[b]
-      for (int b = blockIdx.x; b < batch; b += gridDim.x) {
-        int pos = __ldcg(p.seq_lens + b);
-        int pg = pos / PAGE_TOKENS;
-        int page = pg < p.mpps ? p.block_table[(size_t)b * p.mpps + pg] : -1;
-        if (page < 0 || page >= p.n_pages) { if (tid == 0) dev_flag(p.status, DEV_BAD_PAGE); continue; }
-        int row = pos % PAGE_TOKENS, half = p.hd >> 1;
-        const float* kin = p.qkvb + (size_t)b * n_out + L.dq;
-        const float* vin = kin + (size_t)L.nkv * p.hd;
-        float* rk = reinterpret_cast<float*>(sm_raw);     // the staging area is idle in this phase
-        __syncthreads();
-        if (L.k_norm) head_rnorm(kin, L.nkv, p.hd, p.eps, rk);
-        for (int e = tid; e < L.nkv * half; e += NT) {
-          int h = e / half, c = e - h * half;
-          float sn, cs;
-          rope_sincos(pos, p.inv.f[c], &sn, &cs);
-          float x1 = __ldcg(kin + h * p.hd + c), x2 = __ldcg(kin + h * p.hd + c + half);
-          if (L.k_norm) { x1 *= rk[h] * L.k_norm[c]; x2 *= rk[h] * L.k_norm[c + half]; }
-          size_t off = (((size_t)page * L.nkv + h) * PAGE_TOKENS + row) * p.hd;
-          typedef typename KvOf<T>::type KT;
-          ((KT*)L.kpool)[off + c] = from_f<KT>(x1 * cs - x2 * sn);
-          ((KT*)L.kpool)[off + c + half] = from_f<KT>(x2 * cs + x1 * sn);
-          ((KT*)L.vpool)[off + c] = from_f<KT>(__ldcg(vin + h * p.hd + c));
-          ((KT*)L.vpool)[off + c + half] = from_f<KT>(__ldcg(vin + h * p.hd + c + half));
-        }
-      }
-      BARRIER();
+    if (row0 < n_out) {
+      stage_x<T, BB>(p, in, p.d, L.attn_norm, xs, red, s_abort, dead);
+      gemv_phase<T, BB>(p, stream_desc(p, 4 * i), ws, ring_ptr, xs, p.ll_q, tag, nullptr, old, gw, GW, lane, nullptr, s_abort, dead);
     }
     // ---- attention over the cache.  With split key ranges the CTA that finishes the last split of a
     // (sequence, kv head) merges that group's partial results on the spot (a counter per group tells
@@ -522,7 +583,7 @@ __global__ void __launch_bounds__(NT, 1) step_mega_kernel(const __grid_constant_
       const int group = L.nq / L.nkv, ldr = p.hd + 2;
       for (int it = blockIdx.x; it < n_items; it += gridDim.x) {
         const int sp = it % n_split, r = it / n_split;
-        attn_item<T>(p, L, r / L.nkv, r % L.nkv, sp, n_split, p.qkvb, n_out, sm_raw, p.part, p.ab);
+        attn_item<T>(p, L, r / L.nkv, r % L.nkv, sp, n_split, p.ll_q, n_out, tag, rope[r / L.nkv], sm_raw, p.part, p.ll_a, s_abort, dead);
         if (n_split > 1) {
           __threadfence();                       // this CTA's partial results are visible before it counts itself done
           __syncthreads();
@@ -553,53 +614,69 @@ __global__ void __launch_bounds__(NT, 1) step_mega_kernel(const __grid_constant_
                 if (lane + 64 < p.hd) o2 = fmaf(__ldcg(rr + lane + 64), f, o2);
                 if (lane + 96 < p.hd) o3 = fmaf(__ldcg(rr + lane + 96), f, o3);
               }
-              float* dst = p.ab + (size_t)head * p.hd;
-              if (lane < p.hd) dst[lane] = o0 / ll;
-              if (lane + 32 < p.hd) dst[lane + 32] = o1 / ll;
-              if (lane + 64 < p.hd) dst[lane + 64] = o2 / ll;
-              if (lane + 96 < p.hd) dst[lane + 96] = o3 / ll;
+              u64* dst = p.ll_a + (size_t)head * p.hd;
+              if (lane < p.hd) ll_store(dst + lane, o0 / ll, tag);
+              if (lane + 32 < p.hd) ll_store(dst + lane + 32, o1 / ll, tag);
+              if (lane + 64 < p.hd) ll_store(dst + lane + 64, o2 / ll, tag);
+              if (lane + 96 < p.hd) ll_store(dst + lane + 96, o3 / ll, tag);
             }
           }
         }
       }
     }
-    BARRIER();
     // ---- O projection + residual
-    stage_x<BB>(p.ab, L.dq, L.dq, batch, nullptr, 0.f, xs, red);
-    gemv_phase<T, BB>(p, stream_desc(p, 4 * i + 1), ws, ring_ptr, xs, p.xb, p.d, gw, GW, lane, nullptr, s_abort);
-    BARRIER();
-    // ---- gate / up + SwiGLU
-    stage_x<BB>(p.xb, p.d, p.d, batch, L.ffn_norm, p.eps, xs, red);
-    gemv_phase<T, BB>(p, stream_desc(p, 4 * i + 2), ws, ring_ptr, xs, p.actb, L.ffn, gw, GW, lane, nullptr, s_abort);
-    BARRIER();
-    // ---- down projection + residual
-    stage_x<BB>(p.actb, L.ffn, L.ffn, batch, nullptr, 0.f, xs, red);
-    gemv_phase<T, BB>(p, stream_desc(p, 4 * i + 3), ws, ring_ptr, xs, p.xb, p.d, gw, GW, lane, nullptr, s_abort);
-    BARRIER();
-  }
-  if (!p.do_head) return;             // a later launch carries on from the residual stream in xb
-  // ---- LM head (final RMSNorm fused) with running argmax
-  stage_x<BB>(p.xb, p.d, p.d, batch, p.final_norm, p.eps, xs, red);
-  gemv_phase<T, BB>(p, stream_desc(p, 4 * p.n_layers), ws, ring_ptr, xs, p.logits, p.vocab, gw, GW, lane,
-                    p.token_out ? best : nullptr, s_abort);
-  BARRIER();
-  if (blockIdx.x == 0 && tid < batch) {
-    if (p.token_out) {
-      unsigned long long v;
-      asm volatile("ld.acquire.gpu.global.u64 %0, [%1];" : "=l"(v) : "l"(best + tid) : "memory");
-      p.token_out[tid] = (int)(0xFFFFFFFFu - (unsigned)(v & 0xFFFFFFFFull));
+    if (row0 < p.d) {
+      ask_residual<T, BB>(p, in, gw, p.d, lane, old);
+      stage_x<T, BB>(p, a, L.dq, nullptr, xs, red, s_abort, dead);
+      gemv_phase<T, BB>(p, stream_desc(p, 4 * i + 1), ws, ring_ptr, xs, p.ll_x1, tag, &in, old, gw, GW, lane, nullptr, s_abort, dead);
     }
-    if (p.generation) p.seq_lens[tid] += 1;
+    // ---- gate / up + SwiGLU
+    if (row0 < L.ffn) {
+      stage_x<T, BB>(p, x1, p.d, L.ffn_norm, xs, red, s_abort, dead);
+      gemv_phase<T, BB>(p, stream_desc(p, 4 * i + 2), ws, ring_ptr, xs, p.ll_h, tag, nullptr, old, gw, GW, lane, nullptr, s_abort, dead);
+    }
+    // ---- down projection + residual
+    if (row0 < p.d) {
+      ask_residual<T, BB>(p, x1, gw, p.d, lane, old);
+      stage_x<T, BB>(p, h, L.ffn, nullptr, xs, red, s_abort, dead);
+      gemv_phase<T, BB>(p, stream_desc(p, 4 * i + 3), ws, ring_ptr, xs, p.ll_x2, tag, &x1, old, gw, GW, lane, nullptr, s_abort, dead);
+    }
   }
-#undef BARRIER
+  if (p.do_head) {      // (else a later launch carries on from the residual stream in ll_x2)
+    // ---- LM head (final RMSNorm fused) with running argmax
+    if (row0 < p.vocab) {
+      const Stream<T> x2{p.ll_x2, (uint32_t)p.n_layers, {}};
+      stage_x<T, BB>(p, x2, p.d, p.final_norm, xs, red, s_abort, dead);
+      u64 none[BB];
+      gemv_phase<T, BB>(p, stream_desc(p, 4 * p.n_layers), ws, ring_ptr, xs, nullptr, 0u, nullptr, none, gw, GW, lane,
+                        p.token_out ? best : nullptr, s_abort, dead);
+    }
+    // the CTA that finishes last reads the argmax
+    __syncthreads();
+    if (tid == 0) {
+      __threadfence();
+      s_last = atomicAdd(counter, 1u) == gridDim.x - 1;
+    }
+    __syncthreads();
+    if (s_last && tid < batch) {
+      __threadfence();
+      if (p.token_out) {
+        unsigned long long v;
+        asm volatile("ld.acquire.gpu.global.u64 %0, [%1];" : "=l"(v) : "l"(best + tid) : "memory");
+        p.token_out[tid] = (int)(0xFFFFFFFFu - (unsigned)(v & 0xFFFFFFFFull));
+      }
+      if (p.generation) p.seq_lens[tid] += 1;
+    }
+  }
+  if (*s_abort) for (int i = 0; i < 2000; ++i) __nanosleep(1000);      // let copies in flight land before the CTA goes
 }
 
-constexpr int SMEM_LIMIT = 227 * 1024 - 2048;   // dynamic shared memory we allow ourselves per CTA
+constexpr int SMEM_LIMIT = 227 * 1024 - 3072;   // dynamic shared memory we allow ourselves per CTA
 
 size_t stage_region_bytes(int batch, int hd, int k_max, int es) {
   int bb = batch <= 1 ? 1 : (batch == 2 ? 2 : 4);
   size_t xs = (size_t)bb * ((k_max + 255) / 256 * 256) * 4;
-  size_t at = (size_t)2 * PAGE_TOKENS * (hd * es + 16) + (size_t)(MAXG * hd + MAXG * PAGE_TOKENS + 3 * MAXG) * 4;
+  size_t at = (size_t)2 * PAGE_TOKENS * (hd * es + 16) + (size_t)(MAXG * hd + MAXG * PAGE_TOKENS + 4 * MAXG + 8 + 2 * hd) * 4;
   size_t r = xs > at ? xs : at;
   return (r + 127) / 128 * 128;
 }
@@ -633,6 +710,8 @@ cudaError_t launch_step_mega(MegaParams p, int dtype, int k_max, int n_sm, cudaS
   size_t stage = stage_region_bytes(p.batch, p.hd, k_max, es);
   int slot = (int)((SMEM_LIMIT - stage) / (NW * NSLOT));
   slot = slot / 1024 * 1024;      // whole 256-element groups of either element size
+  const int row = (k_max * es + 1023) / 1024 * 1024;      // no more than the longest row
+  if (slot > row) slot = row;
   if (slot > 8192) slot = 8192;
   p.stage_bytes = (int)stage;
   p.slot_bytes = slot;

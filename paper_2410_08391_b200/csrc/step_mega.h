@@ -3,7 +3,7 @@
 #include "common.cuh"
 
 constexpr int MEGA_MAX_LAYERS = 64;
-constexpr int MEGA_COUNTERS = 32;      // counter words in the status block, one per launch of a step: grid barrier (step_mega_kernel), finished CTAs (step_mega_mma_kernel)
+constexpr int MEGA_COUNTERS = 32;      // counter words in the status block, one per launch of a step: finished CTAs
 constexpr int MEGA_STATUS_BYTES = 256; // what a caller clears before a step: status word, argmax slots, counters
 
 struct MegaLayer {
@@ -23,13 +23,13 @@ struct MegaParams {
   const void* embed; const float* final_norm; const void* lm_head;
   const int* block_table; int mpps, n_pages;
   int* seq_lens;
-  float *xb, *qkvb, *ab, *actb, *part;           // workspace: residual, projections, attention out, FFN act, partials
-  // step_mega_mma_kernel: {value, tag} words instead of the buffers above (cleared before a step): q(kv) rows, attention out,
-  // residual after attention / after the FFN, FFN act, split partials
+  float* part;                                   // step_mega_kernel: split partials
+  // {value, tag} words (cleared before a step): q(kv) rows, attention out, residual after attention / after the FFN, FFN act,
+  // split partials of step_mega_mma_kernel
   unsigned long long *ll_q, *ll_a, *ll_x1, *ll_x2, *ll_h, *ll_part;
   int* attn_done;                                // [batch * max n_kv] splits finished per (sequence, kv head); zero on entry, left zero
   float* logits; int* token_out;
-  // One launch may cover only base layers [layer_begin, layer_end): the residual stream stays in xb (ll_x2) between
+  // One launch may cover only base layers [layer_begin, layer_end): the residual stream stays in ll_x2 between
   // launches.  do_embed: start from the token embeddings; do_head: end with the LM head and the token.
   int layer_begin, layer_end, do_embed, do_head;
   int counter_idx;                               // which counter word this launch uses (zero on entry)

@@ -1,5 +1,5 @@
-// Bounded waits of the barrier-free step kernel (step_mega_mma.cu): tagged values in global memory, and the waits of its loader
-// warps.  In a header of their own so that the self-test of selftest.cu runs the same code.
+// Bounded waits of the persistent step kernels (step_mega_mma.cu, step_mega.cu): tagged values in global memory, and the waits of the
+// former's loader warps.  In a header of their own so that the self-test of selftest.cu runs the same code.
 #pragma once
 #include "common.cuh"
 #include "tc_ptx.cuh"
