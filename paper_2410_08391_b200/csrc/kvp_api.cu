@@ -632,13 +632,17 @@ kvp_status kvp_load_weights(kvp_handle* h, const kvp_tensor* tensors, int32_t n,
 }
 
 // SMs that the step's pieces take beside the prefill of a call; 0: the step runs after it, on all of them.  Both are estimated in
-// microseconds, the prefill from its launches and operations, the step (on all SMs) from its weights.  Prompts whose prefill is the
-// longer by far want the SMs themselves; where it is over long before the step, a caller that waits is served sooner by one after the
-// other (while other calls keep the GPU busy, 72 SMs get more done).  Alone / among other calls, us, with 0, 48, 72, 88 SMs:
-//   1.1B 1 x 59 (prefill / step 0.7): 1394 / 1107, 1562 / 885, 1370 / 969, 1295 / 1230;  1 x 1024 (1.6): 2087 / 1756, 1911 / 1606,
-//   1911 / 1677, 2027 / 1858;  3 x 1000 (2.5): 3486 / 3266, 3227 / 3038, 3446 / 3211, 3755 / 3398;  1 x 3500 (3.7): 4001 / 3878, 3904 / 3849,
-//   4151 / 3810, 4807 / 3919;  layer-pruned 1 x 1000 (2.5): 2567 / 2356, 2313 / 2170, 2605 / 2252, 2892 / 2437;
-//   3B 1 x 59 (0.35): 2678 / 2281, 4053 / 1912, 3113 / 2057, 2840 / 2769;  1 x 800 (0.8): 3677 / 3126, 4449 / 2872, 3550 / 2931, 3431 / 3263.
+// microseconds, the prefill from its launches and operations, the step (on all SMs) from its weights.  A caller that waits is served
+// soonest where the two end together, and by one after the other where the prefill is over long before the step; while other calls keep
+// the GPU busy, few SMs for the step get more done, down to where its pieces last longer than the prefill.  By itself / among other calls, us,
+// with 0, 48, 64, 72, 88 SMs (prefill / step in brackets):
+//   1.1B 1 x 59 (0.8): 1395 / 1095, 1567 / 877, 1379 / 925, 1377 / 969, 1299 / 1232;  1 x 300 (1.0): 1672 / 1315, 1666 / 1089, 1524 / 1123,
+//   1493 / 1174, 1467 / 1335;  1 x 600 (1.3): 1930 / 1505, 1732 / 1259, 1604 / 1363, 1629 / 1379, 1811 / 1555;  1 x 1024 (1.7): 2069 / 1748,
+//   1935 / 1618, 1894 / 1678, 1920 / 1668, 2034 / 1856;  1 x 1500 (2.2): 2570 / 2212, 2262 / 2003, 2286 / 2062, 2382 / 2098, 2530 / 2225;
+//   4 x 100 (0.8): 2027 / 1681, 2313 / 1415, 2021 / 1450, 1932 / 1490, 1862 / 1790;  layer-pruned 1 x 600 (1.9): 2212 / 1855, 1989 / 1627,
+//   1933 / 1699, 2011 / 1727, 2184 / 1867;  scaled 1 x 500: 1719 / 1254, 1538 / 1029, 1409 / 1087, 1397 / 1128, 1405 / 1293;
+//   3B 1 x 59 (0.4): 2681 / 2273, 4064 / 1913, 3239 / 1969, 3128 / 2039, 2852 / 2769;  1 x 1000 (0.9): 3796 / 3269, 4457 / 3033, 3735 / 3022,
+//   3658 / 3138, 3572 / 3452.
 int step_piece_sms(const kvp_handle* h, int batch, const CallShape& cs, bool blocking) {
   if (h->step_sms == 0 || h->opt.dtype != KVP_BF16) return h->step_sms;
   const ModelPlan &A = h->aux, &B = h->base;
@@ -647,12 +651,12 @@ int step_piece_sms(const kvp_handle* h, int batch, const CallShape& cs, bool blo
   for (int j = 0; j <= h->j_max; ++j) ops += 2.0 * cs.total * A.d * (A.L[j].nqkv + A.L[j].dq + 3.0 * A.L[j].ffn) + 4.0 * A.L[j].dq * pairs;
   for (const LayerPlan& L : B.L) bytes += (2.0 * L.dq + 3.0 * L.ffn) * B.d * h->es;
   const double prefill = 36.0 * (h->j_max + 1) + ops / 8e8, step = bytes / 3.2e6 * (1.0 + 0.1 * (batch - 1));      // microseconds
-  if (prefill > 1.9 * step) {
-    const int few = 48;
-    return few < h->step_sms && step_mega_mma_supported(batch, B.L[0].hd, B.max_group, B.d, few) ? few : h->step_sms;
-  }
-  if (blocking && prefill < 0.5 * step) return 0;
-  return h->step_sms;
+  int sms = h->step_sms;
+  if (prefill > (blocking ? 1.9 : 1.5) * step) sms = 48;
+  else if (blocking && prefill < 0.5 * step) return 0;
+  else if (blocking && prefill < step) sms = 88;
+  else if (prefill >= 0.6 * step) sms = 64;
+  return sms <= h->n_sm - 32 && step_mega_mma_supported(batch, B.L[0].hd, B.max_group, B.d, sms) ? sms : h->step_sms;
 }
 
 // Enqueues every kernel of the time-to-first-token path on `stream` (validates first).
