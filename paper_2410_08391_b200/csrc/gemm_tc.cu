@@ -334,7 +334,9 @@ gemm_tc_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_constant_
   if (PAIR) pdl_trigger();       // (with the pair's tensor memory in hand: that allocation waits for two SMs)
   const uint32_t tmem_base = *tmem_slot;
   const int num_kb = (p.K + BK - 1) / BK;
-  pdl_wait();         // set-up above overlapped the previous kernel's tail; its results are needed from here on
+  // Set-up above overlapped the previous kernel's tail; its results are needed from here on.  W does not come from any kernel of the
+  // chain: its loader fills the ring without waiting.
+  if (warp != 2) pdl_wait();
 
   if (warp == 0 || warp == 2) {
     // ---------------- TMA producers: warp 0 loads the A tile of every stage, warp 2 the W tile ----------------
