@@ -631,8 +631,18 @@ kvp_status kvp_load_weights(kvp_handle* h, const kvp_tensor* tensors, int32_t n,
   return check_cuda(h, "kvp_load_weights");
 }
 
-// SMs that the step's pieces take beside the prefill of a call; 0: the step runs after it, on all of them.  Both are estimated in
-// microseconds, the prefill from its launches and operations, the step (on all SMs) from its weights.  A caller that waits is served
+// The two halves of a call in microseconds: the prefill from its launches and operations, the step (on all SMs) from its weights.
+struct CallTimes { double prefill, step; };
+CallTimes estimate_call(const kvp_handle* h, int batch, const CallShape& cs) {
+  const ModelPlan &A = h->aux, &B = h->base;
+  double pairs = 0, ops = 0, bytes = (double)B.vocab * B.d * h->es;
+  for (int b = 0; b < batch; ++b) { const double n = cs.cu[b + 1] - cs.cu[b]; pairs += n * (n + 1) / 2; }
+  for (int j = 0; j <= h->j_max; ++j) ops += 2.0 * cs.total * A.d * (A.L[j].nqkv + A.L[j].dq + 3.0 * A.L[j].ffn) + 4.0 * A.L[j].dq * pairs;
+  for (const LayerPlan& L : B.L) bytes += (2.0 * L.dq + 3.0 * L.ffn) * B.d * h->es;
+  return {36.0 * (h->j_max + 1) + ops / 8e8, bytes / 3.2e6 * (1.0 + 0.1 * (batch - 1))};
+}
+
+// SMs that the step's pieces take beside the prefill of a call; 0: the step runs after it, on all of them.  A caller that waits is served
 // soonest where the two end together, and by one after the other where the prefill is over long before the step; while other calls keep
 // the GPU busy, few SMs for the step get more done, down to where its pieces last longer than the prefill.  By itself / among other calls, us,
 // with 0, 48, 64, 72, 88 SMs (prefill / step in brackets):
@@ -645,18 +655,31 @@ kvp_status kvp_load_weights(kvp_handle* h, const kvp_tensor* tensors, int32_t n,
 //   3658 / 3138, 3572 / 3452.
 int step_piece_sms(const kvp_handle* h, int batch, const CallShape& cs, bool blocking) {
   if (h->step_sms == 0 || h->opt.dtype != KVP_BF16) return h->step_sms;
-  const ModelPlan &A = h->aux, &B = h->base;
-  double pairs = 0, ops = 0, bytes = (double)B.vocab * B.d * h->es;
-  for (int b = 0; b < batch; ++b) { const double n = cs.cu[b + 1] - cs.cu[b]; pairs += n * (n + 1) / 2; }
-  for (int j = 0; j <= h->j_max; ++j) ops += 2.0 * cs.total * A.d * (A.L[j].nqkv + A.L[j].dq + 3.0 * A.L[j].ffn) + 4.0 * A.L[j].dq * pairs;
-  for (const LayerPlan& L : B.L) bytes += (2.0 * L.dq + 3.0 * L.ffn) * B.d * h->es;
-  const double prefill = 36.0 * (h->j_max + 1) + ops / 8e8, step = bytes / 3.2e6 * (1.0 + 0.1 * (batch - 1));      // microseconds
+  const ModelPlan& B = h->base;
+  const auto [prefill, step] = estimate_call(h, batch, cs);
   int sms = h->step_sms;
   if (prefill > (blocking ? 1.9 : 1.5) * step) sms = 48;
   else if (blocking && prefill < 0.5 * step) return 0;
   else if (blocking && prefill < step) sms = 88;
   else if (prefill >= 0.6 * step) sms = 64;
   return sms <= h->n_sm - 32 && step_mega_mma_supported(batch, B.L[0].hd, B.max_group, B.d, sms) ? sms : h->step_sms;
+}
+
+// Base layers that the pieces reach while the prefill of a caller that waits still runs; the others are one last piece on all SMs
+// (which take a layer in (n_sm / sms)^-0.6 of the pieces' time, measured from 24 SMs on).  From host memory to host memory, us, all
+// pieces on the same SMs / the last layers on all: 1.1B 1 x 59 1331 / 1225, 2 x 30 1433 / 1294, 4 x 100 1895 / 1786, 1 x 300 1475 / 1427, 1 x 600
+// 1632 / 1580, layer-pruned 1 x 200 1540 / 1479, scaled 1 x 300 1373 / 1285, 3B 1 x 400 3058 / 2867, 1 x 1000 3597 / 3566.
+int step_layers_beside(const kvp_handle* h, int batch, const CallShape& cs, int sms) {
+  const auto [whole, step] = estimate_call(h, batch, cs);
+  const double chain = 36.0 * (h->j_max + 1), prefill = chain + (whole - chain) * 0.9 * h->n_sm / (h->n_sm - sms);      // (on the SMs that the pieces leave)
+  const double layer = step / h->base.n_layers * pow((double)h->n_sm / sms, 0.6) + 4.0, aux = prefill / (h->j_max + 1);
+  double t = 0;
+  for (int i = 0; i < h->base.n_layers; ++i) {
+    t = std::max(t, aux * (h->map[i] + 1));
+    if (t >= prefill) return i;
+    t += layer;
+  }
+  return h->base.n_layers;
 }
 
 // Enqueues every kernel of the time-to-first-token path on `stream` (validates first).
@@ -736,6 +759,7 @@ static kvp_status prefill_direct(kvp_handle* h, const int32_t* tokens, const int
                           mega_prepare(h, ctx, cache, w, ws, batch, cs.max_len, false, tokens, last_idx, logits_out, first_token, &mp, &mega_kmax);
   const int piece_sms = one_kernel ? step_piece_sms(h, batch, cs, blocking) : 0;
   const bool piped = piece_sms > 0;
+  const int beside = piped && blocking && mega_uses_mma(h, batch) ? step_layers_beside(h, batch, cs, piece_sms) : h->base.n_layers;
   std::vector<int> ready_after(h->j_max + 2, 0);      // ready_after[j] = base layers runnable after auxiliary layer j
   if (piped) {
     int dep = 0, i = 0;
@@ -876,7 +900,7 @@ static kvp_status prefill_direct(kvp_handle* h, const int32_t* tokens, const int
         cudaEventRecord(h->ev_join, h->side);
         pending_join = true;
       }
-      if (piped && (ready_after[j] > base_done || last)) {
+      if (piped && (last || (ready_after[j] > base_done && base_done < beside))) {
         cudaStreamWaitEvent(h->step_st, h->ev_join, 0);
         MegaParams q = mp;
         q.layer_begin = base_done; q.layer_end = last ? h->base.n_layers : ready_after[j];

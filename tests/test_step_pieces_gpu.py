@@ -46,3 +46,34 @@ def test_a_step_that_is_the_longer_one_runs_in_pieces_or_after_the_prefill():
                 assert rel_fro(k, ref[b][0][i][0]) <= TOL["bf16"] and rel_fro(v, ref[b][0][i][1]) <= TOL["bf16"]
     finally:
         s.close()
+
+
+def test_the_last_layers_of_a_caller_that_waits_are_one_piece_on_all_sms():
+    """The prefill is estimated at 1.1 of the step (4 layers of 36 us, 0.42 GB of base weights): its pieces reach some of the base layers
+    meanwhile, and what is left is one launch.  Other callers get a piece per auxiliary layer."""
+    import torch
+
+    import paper_2410_08391_b200 as kvp
+    n = 4
+    pair = wl.PairCfg("waits", wl.uniform_model(n, 64, 2, 1, 64, 128, 500), wl.uniform_model(2 * n, 1024, 8, 2, 64, 8192, 500), tuple(i // 2 for i in range(2 * n)))
+    W = wl.make_weights(pair, seed=4, regime="fanin")
+    lens = [7]
+    pr = wl.custom_prompts(500, lens, seed=4)
+    ref = orc.prefill_predict(pair, W, pr)
+    assert len(recorded_prefill(pair, lens, W).grids("step_mega_mma_kernel")) == n
+    s = make_session(pair, W, pr)
+    try:
+        n0 = kvp.kvp_launch_count(s.h)
+        logits, _ = run_prefill(s, pr)
+        n1 = kvp.kvp_launch_count(s.h)
+        host, first = torch.zeros((1, 500)).pin_memory(), torch.zeros(1, dtype=torch.int32).pin_memory()
+        kvp.kvp_prefill_predict_host(s.h, torch.from_numpy(pr.tokens).pin_memory(), lens, s.cache, s.workspace, s.logits, host, first, s.stream)
+        s.poll()
+        fewer = (n1 - n0) - (kvp.kvp_launch_count(s.h) - n1)
+        assert 1 <= fewer < n - 1
+        assert rel_fro(logits[0], ref[0][1]) <= TOL["bf16"] and rel_fro(host[0].numpy(), ref[0][1]) <= TOL["bf16"]
+        for i in (0, n, 2 * n - 1):
+            k, v = s.cache.gather(i, 0, 7)
+            assert rel_fro(k, ref[0][0][i][0]) <= TOL["bf16"] and rel_fro(v, ref[0][0][i][1]) <= TOL["bf16"]
+    finally:
+        s.close()
