@@ -78,7 +78,6 @@ template <int HD, bool F16>
 __global__ void __launch_bounds__(NT, HD == 64 ? 4 : 2) attn_mma_kernel(const Params p) {
   constexpr int KS = HD / 16, NTL = HD / 8, TILE = Cfg<HD>::TILE;
   extern __shared__ __align__(128) unsigned char sm[];
-  pdl_trigger();
   pdl_wait();
   const int head = blockIdx.x, b = blockIdx.y;
   const int base = p.cu[b], L = p.cu[b + 1] - base;
@@ -178,6 +177,7 @@ __global__ void __launch_bounds__(NT, HD == 64 ? 4 : 2) attn_mma_kernel(const Pa
       }
     __syncthreads();             // this stage is free
   }
+  pdl_trigger();
 #pragma unroll
   for (int h = 0; h < 2; ++h) {
     l[h] += __shfl_xor_sync(0xffffffffu, l[h], 1);

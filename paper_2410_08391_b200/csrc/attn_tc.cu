@@ -146,7 +146,6 @@ attn_tc_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_constant_
   constexpr int BKV = C::BKV, QB = C::Q_BYTES, KB = C::KV_BYTES, NBOX = HD / 64, KS = C::K_STAGES, VS = C::V_STAGES;
   constexpr int KV_BOX = BKV * 128;     // bytes of one 64-column box of a K or V tile
   extern __shared__ uint8_t smem_raw[];
-  pdl_trigger();
   if (threadIdx.x == 32) { prefetch_tensormap(&map_q); prefetch_tensormap(&map_kv); }
   uint8_t* smem = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~uintptr_t(1023));
   const uint32_t sQ = smem_u32(smem), sK = sQ + 2 * QB, sV = sK + KS * KB;
@@ -224,6 +223,7 @@ attn_tc_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_constant_
 #pragma unroll
         for (int x = 0; x < NBOX; ++x) tma_load_2d(sV + st * KB + x * KV_BOX, &map_kv, vcol + x * 64, base + j * BKV, v_full(st));
       }
+      pdl_trigger();
       if (!ok) drain_after_abort();
     }
   } else if (warp == 1 || (warp == 2 && C::TWO_ISSUERS)) {

@@ -151,7 +151,6 @@ __global__ void __launch_bounds__(128) rmsnorm_vec_kernel(const float* __restric
   __shared__ float red[4];
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const int row = blockIdx.x * (4 / WPR) + warp / WPR, t = (warp % WPR) * 32 + lane;
-  pdl_trigger();
   float4 g[NV], v[NV];
 #pragma unroll
   for (int i = 0; i < NV; ++i) {            // the gain is a weight: it does not wait for the kernel before this one
@@ -167,6 +166,7 @@ __global__ void __launch_bounds__(128) rmsnorm_vec_kernel(const float* __restric
     const int c = 4 * (t + i * 32 * WPR);
     v[i] = c < d ? *reinterpret_cast<const float4*>(xr + c) : make_float4(0.f, 0.f, 0.f, 0.f);
   }
+  pdl_trigger();
 #pragma unroll
   for (int i = 0; i < NV; ++i) ss += (v[i].x * v[i].x + v[i].y * v[i].y) + (v[i].z * v[i].z + v[i].w * v[i].w);
   ss = warp_sum(ss);
