@@ -223,7 +223,7 @@ struct StepAttn {
   const int* seq_lens; int extra, batch, max_keys;
   int append;                          // the step's own keys (norm, RoPE) and values join the cache at position seq_lens[b]
   float* part; float* out;             // split partials; output rows [batch, nq * hd]
-  bf16* xb;                            // or null: the output goes here instead, as bf16 value and remainder rows (step_tc.h)
+  bf16* xb; int terms;                 // or null: the output goes here instead, as rows of two or three bf16 terms (step_tc.h)
   const float *q_gain, *k_gain; float eps;
   int* split_done;                     // [batch * nkv] ints, zero, left zero; or null (the kernels that merge their own splits need it)
 };

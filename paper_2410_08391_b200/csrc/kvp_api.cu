@@ -142,10 +142,9 @@ WsLayout ws_layout(const kvp_handle* h, int64_t Bm, int64_t Tm) {
   w.qkvb = take(Bm * B.max_nqkv * 4);
   w.ab = take(Bm * B.max_dq * 4);
   w.actb = take(Bm * (size_t)B.max_ffn * 4);
-  // tensor-core step projections: operand rows (hi + lo) of the widest input, fp32 gate/up outputs
-  const int64_t Bp = step_tc_rows((int)Bm);
+  // tensor-core step projections: operand rows (two or three terms each) of the widest input, fp32 gate/up outputs
   const int64_t k_max = std::max((int64_t)B.d, std::max((int64_t)B.max_dq, (int64_t)B.max_ffn));
-  w.xbt = take(2 * Bp * k_max * 2);
+  w.xbt = take((size_t)step_tc_operand_rows((int)Bm) * k_max * 2);
   w.gub = take(Bm * 2 * (size_t)B.max_ffn * 4);
   // The persistent kernels of small batches use none of the seven buffers above: its tagged values (64 bits each) take
   // their place, at the end, so that they and its split partials in w.part are cleared as one range.
@@ -226,7 +225,7 @@ bool try_tc(kvp_handle* h, const LaunchCtx& ctx, TcGemm& t, int cls, cudaError_t
 // Are the step's projections run on the tensor cores?  (Everything the persistent kernel does not take:
 // batches of more than 4 rows, and small batches over long caches.)
 bool step_uses_tc(const kvp_handle* h, int batch) {
-  if (h->opt.dtype != KVP_BF16 || step_tc_rows(batch) > 128) return false;
+  if (h->opt.dtype != KVP_BF16 || step_tc_operand_rows(batch) > 256) return false;
   const ModelPlan& B = h->base;
   if (B.d % 8) return false;
   for (int i = 0; i < B.n_layers; ++i)
@@ -240,9 +239,9 @@ void step_proj_tc(kvp_handle* h, const LaunchCtx& ctx, const WsLayout& w, char* 
                   int K, int batch, const float* gain, int G, const void* W, int N, float* Y, int ldy, bool clear,
                   cudaError_t* err, bool overlapped = true) {
   bf16* XB = (bf16*)(ws + w.xbt);
-  if (src) KVP_TIMED(KVP_CLASS_STEP_GEMV, launch_step_prep(ctx, mode, src, ld_src, K, batch, gain, h->base.eps, G, XB, clear ? Y : nullptr, ldy, N, overlapped));
+  if (src) KVP_TIMED(KVP_CLASS_STEP_GEMV, launch_step_prep(ctx, mode, src, ld_src, K, batch, h->step_terms, gain, h->base.eps, G, XB, clear ? Y : nullptr, ldy, N, overlapped));
   TimedScope ts(h, ctx.st, KVP_CLASS_STEP_GEMV);
-  cudaError_t e = launch_step_gemm_tc((const bf16*)W, K, N, K, XB, batch, Y, ldy, h->step_grid_sms, ctx.status, ctx.st, ctx.n_launch);
+  cudaError_t e = launch_step_gemm_tc((const bf16*)W, K, N, K, XB, batch, h->step_terms, Y, ldy, h->step_grid_sms, ctx.status, ctx.st, ctx.n_launch);
   if (e != cudaSuccess && *err == cudaSuccess) *err = e;
 }
 
@@ -272,6 +271,7 @@ void base_layer_step(kvp_handle* h, const LaunchCtx& ctx, int i, const kvp_cache
   a.q = qkvb; a.ldq = n_out; a.nq = L.nq; a.nkv = L.nkv; a.hd = L.hd; a.theta = B.theta; a.kpool = cache->k_pools[i]; a.vpool = cache->v_pools[i];
   a.block_table = cache->block_table; a.mpps = cache->max_pages_per_seq; a.n_pages = cache->n_pages; a.seq_lens = cache->seq_lens;
   a.extra = a.append = generation ? 1 : 0; a.batch = batch; a.max_keys = max_keys; a.part = (float*)(ws + w.part); a.out = ab;
+  a.terms = h->step_terms;
   a.xb = tc ? (bf16*)(ws + w.xbt) : nullptr;      // (the queries' own operand rows have been read)
   a.q_gain = B.qk_norm ? (const float*)(P + L.q_norm) : nullptr;
   a.k_gain = B.qk_norm ? (const float*)(P + L.k_norm) : nullptr;
@@ -315,6 +315,21 @@ cudaError_t launch_mega(kvp_handle* h, const MegaParams& p, int k_max, int n_sm,
   int ctas = std::max(16, (rows + 15) / 16);
   for (int i = p.layer_begin; i < p.layer_end; ++i) ctas = std::max(ctas, p.batch * p.layers[i].nkv * p.layers[i].n_split);
   return launch_step_mega(p, h->opt.dtype, k_max, std::min(n_sm, ctas), st, &h->n_launch);
+}
+
+// First steps of up to four sequences: is the chain of launches served sooner than the persistent tensor-core kernel?  (Both keep 24 bits
+// of an activation: the chain takes three terms then.)  Beside a prefill the chain takes SMs for some microseconds at a time and leaves
+// them to the prefill otherwise; the persistent kernel multiplies three or four rows on slower units, and a layer of it beside the prefill
+// takes the longer the more weights a layer has.  First token, us, persistent / chain by itself (among other calls): 3B pair 4 x 300 4662 / 3831
+// (3759 / 3321), 4 x 3000 16601 / 16381 (16922 / 15439), 2 x 300 3580 / 3146 (2617 / 2567), 1 x 300 3186 / 2968 (2336 / 2136), 1 x 1024 3574 / 3440
+// (2921 / 3027); 1.1B pair 4 x 300 2145 / 2077 (1853 / 1697), 3 x 1000 3321 / 3324 (3172 / 3068), 1 x 300 1409 / 1457 (1074 / 994), 1 x 1024 1801 /
+// 1981 (1608 / 1642); scaled 3 x 100 1627 / 1542 (1091 / 894).  Generation stays with the persistent kernel, which serves one call sooner.
+bool first_step_prefers_chain(const kvp_handle* h, int batch, double prefill_to_step, bool blocking) {
+  if (batch > 4 || !mega_uses_mma(h, batch) || !step_uses_tc(h, batch)) return false;
+  double mb = 0;        // weights of a layer
+  for (const LayerPlan& L : h->base.L) mb += (2.0 * L.dq + 3.0 * L.ffn) * h->base.d * h->es * 1e-6 / h->base.n_layers;
+  if (batch > 2) return mb >= 30.0 && !blocking;
+  return mb >= 150.0 && prefill_to_step < 0.75 && !blocking;
 }
 
 // Parameters of the persistent step kernel for this call; false = the kernel does not apply.
@@ -755,7 +770,14 @@ static kvp_status prefill_direct(kvp_handle* h, const int32_t* tokens, const int
   // layer below them) is complete once auxiliary layer j has gone through the predictor.
   MegaParams mp;
   int mega_kmax = 0, piece = 0, base_done = 0;
-  const bool one_kernel = fork && h->step_sms > 0 && h->j_max + 1 <= MEGA_COUNTERS &&
+  const CallTimes times = estimate_call(h, batch, cs);
+  const bool chain = first_step_prefers_chain(h, batch, times.prefill / times.step, blocking);
+  struct Terms {        // (the step's launches below, whichever way this function is left)
+    kvp_handle* h;
+    Terms(kvp_handle* h_, int n) : h(h_) { h->step_terms = n; }
+    ~Terms() { h->step_terms = 2; }
+  } terms(h, chain ? 3 : 2);
+  const bool one_kernel = fork && !chain && h->step_sms > 0 && h->j_max + 1 <= MEGA_COUNTERS &&
                           mega_prepare(h, ctx, cache, w, ws, batch, cs.max_len, false, tokens, last_idx, logits_out, first_token, &mp, &mega_kmax);
   const int piece_sms = one_kernel ? step_piece_sms(h, batch, cs, blocking) : 0;
   const bool piped = piece_sms > 0;
@@ -987,7 +1009,7 @@ static kvp_status prefill_direct(kvp_handle* h, const int32_t* tokens, const int
   }
   if (tc_err != cudaSuccess) return fail(h, KVP_ERR_CUDA, "kernel launch: %s", cudaGetErrorString(tc_err));
   // ---- stage 3: one base step per sequence on its last prompt token ----
-  if (!piped && !piped_tc && !base_step_fused(h, ctx, cache, w, ws, batch, cs.max_len, false, tokens, last_idx, logits_out, first_token, &tc_err)) {
+  if (!piped && !piped_tc && (chain || !base_step_fused(h, ctx, cache, w, ws, batch, cs.max_len, false, tokens, last_idx, logits_out, first_token, &tc_err))) {
     base_step_begin(h, ctx, w, ws, tokens, last_idx, batch);
     for (int i = 0; i < h->base.n_layers; ++i) base_layer_step(h, ctx, i, cache, w, ws, batch, cs.max_len, false, &tc_err);
     base_head(h, ctx, w, ws, batch, logits_out, first_token, &tc_err);

@@ -20,6 +20,7 @@
 #include <math.h>
 
 #include "common.cuh"
+#include "step_tc.h"
 #include "tc_ptx.cuh"
 
 namespace {
@@ -28,6 +29,7 @@ using namespace tcp;
 constexpr int NW = 4;                       // consumer warps
 constexpr int NT = (NW + 1) * 32;
 constexpr int BOX_BYTES = 64 * 128;         // one 64-key x 64-dim box
+constexpr float Q_UP = 16.f;                // scaled queries are multiplied by this before they are split, so that the remainder halves stay normal numbers
 
 template <int HD> struct MmaCfg {
   static constexpr int PAGE_BYTES = PAGE_TOKENS * HD * 2;
@@ -80,7 +82,7 @@ struct MmaParams {
   int per_pages;            // pages per CTA
   int stages;               // of its ring
   float* out;               // output rows [batch, nq * HD], or (null) as the next projection's operand rows:
-  bf16* xb; int Bp;         // row b = bf16(value), row Bp + b = bf16(remainder)
+  bf16* xb; int Bp, terms;  // row b = bf16(value), row Bp + b = bf16(remainder), with three terms row 2 Bp + b what that leaves
   // Generation: q's rows go on with the step's own keys and values.  They join the cache here: the CTA whose range ends with
   // their page takes them into its copy of the page and writes them to the pool (no launch of their own: 7.7 us a layer).
   int append; const float* k_gain; kv16* kpool; kv16* vpool;
@@ -90,7 +92,10 @@ __device__ __forceinline__ void emit(const MmaParams& p, int b, size_t width, in
   if (p.out) { p.out[(size_t)b * width + col] = v; return; }
   const bf16 h = __float2bfloat16_rn(v);
   p.xb[(size_t)b * width + col] = h;
-  p.xb[(size_t)(p.Bp + b) * width + col] = __float2bfloat16_rn(v - __bfloat162float(h));
+  const float rest = v - __bfloat162float(h);
+  const bf16 l = __float2bfloat16_rn(rest);
+  p.xb[(size_t)(p.Bp + b) * width + col] = l;
+  if (p.terms == 3) p.xb[(size_t)(2 * p.Bp + b) * width + col] = __float2bfloat16_rn(rest - __bfloat162float(l));
 }
 
 template <int HD>
@@ -182,7 +187,7 @@ step_attn_mma_kernel(const __grid_constant__ CUtensorMap map_k, const __grid_con
   if (p.q_gain) head_rnorm(p.q + (size_t)b * p.ldq + (size_t)kvh * group * HD, group, HD, p.eps, rq);
   else __syncthreads();
   {
-    const float scale = rsqrtf((float)HD);
+    const float scale = Q_UP * rsqrtf((float)HD);
     for (int i = tid; i < 8 * half; i += NT) {
       const int h = i / half, c = i - h * half;
       float r1 = 0.f, r2 = 0.f;
@@ -271,8 +276,8 @@ step_attn_mma_kernel(const __grid_constant__ CUtensorMap map_k, const __grid_con
         float sv4[4];
 #pragma unroll
         for (int t = 0; t < 2; ++t) {
-          sv4[2 * t] = sc[t][0] + sc[t][2];
-          sv4[2 * t + 1] = sc[t][1] + sc[t][3];
+          sv4[2 * t] = (sc[t][0] + sc[t][2]) * (1.f / Q_UP);
+          sv4[2 * t + 1] = (sc[t][1] + sc[t][3]) * (1.f / Q_UP);
           const int key0 = warp * 16 + t * 8 + 2 * qd;
           if (key0 >= nk) sv4[2 * t] = -INFINITY;
           if (key0 + 1 >= nk) sv4[2 * t + 1] = -INFINITY;
@@ -426,7 +431,7 @@ cudaError_t launch_step_attn_mma(const LaunchCtx& ctx, const StepAttn& a, int n_
   const long long rows = (long long)a.n_pages * nkv * PAGE_TOKENS;
   if (!make_pool_map(&mk, a.kpool, rows, hd) || !make_pool_map(&mv, a.vpool, rows, hd)) return cudaErrorInvalidValue;
   MmaParams p{a.q, a.ldq, nq, nkv, a.block_table, a.mpps, a.n_pages, a.seq_lens, a.extra, n_split, a.part, ctx.status, a.q_gain, a.eps,
-              a.split_done, per_pages, mma_stages(hd, per_pages), a.xb ? nullptr : a.out, a.xb, (a.batch + 7) / 8 * 8, a.append, a.k_gain, (kv16*)a.kpool, (kv16*)a.vpool};
+              a.split_done, per_pages, mma_stages(hd, per_pages), a.xb ? nullptr : a.out, a.xb, step_tc_rows(a.batch, a.terms), a.terms, a.append, a.k_gain, (kv16*)a.kpool, (kv16*)a.vpool};
   dim3 grid(n_split, nkv, a.batch);
   ++*ctx.n_launch;
   return hd == 64 ? go_mma<64>(mk, mv, inv, p, grid, ctx.st) : go_mma<128>(mk, mv, inv, p, grid, ctx.st);

@@ -3,8 +3,8 @@
 // y[b, n] = sum_k W[n, k] x[b, k] with W streamed once from HBM is bandwidth-bound only while
 // the multiply keeps up; beyond about 8 rows the CUDA cores do not.  Here the roles of the
 // operands are swapped: a tile of 128 weight rows is the M side of tcgen05.mma, the activations
-// are the N side (2 * Bp columns: each row as a bf16 hi part and a bf16 lo part of its fp32
-// value, so that the activations lose nothing that matters), and the 128 x 2Bp accumulator
+// are the N side (each row as a bf16 hi part and a bf16 lo part of its fp32 value, or, of up to four rows, as three parts,
+// so that the activations lose nothing that matters), and the 128 x (rows x parts) accumulator
 // lives in tensor memory.  All k blocks of all row tiles form one sequence that is cut into
 // equal contiguous shares, two per SM, so every SM streams weights for the whole launch
 // whatever the number of row tiles; a share's partial sums are added to the fp32 output with
@@ -31,8 +31,13 @@ constexpr int SMEM_LIMIT = 112 * 1024;
 // itself: 1787 / 1630 / 1642 / 1520, 3603 / 3455 / 3412 / 3370, 1355 / 1318 / 1330 / 1303.
 constexpr int MIN_KB = 8, CTAS_PER_SM = 2;
 
+// With three terms a sum is taken in eight parts, k blocks in turn, each in columns of its own, that the epilogue adds in fp32: the tensor
+// core rounds towards zero with every instruction, and 24-bit operands are worth no more than the sum.  (Changing columns with every
+// instruction instead cost 1 to 2 us a launch.)
+constexpr int PARTS = 8;
+
 struct Params {
-  int N, K, batch, Bp;
+  int N, K, batch, Bp, rows;      // rows of the operand buffer: the columns of an accumulator
   int stages, x_bytes;      // ring depth; bytes of the activation tile of a stage (multiple of 1024)
   int acc_stride;           // tensor-memory columns between the two accumulators
   float* Y; int ldy;
@@ -63,6 +68,7 @@ struct Sched {
   }
 };
 
+template <int TERMS>
 __global__ void __launch_bounds__(N_THREADS, 1)
 step_gemm_kernel(const __grid_constant__ CUtensorMap map_w, const __grid_constant__ CUtensorMap map_x, const Params p) {
   extern __shared__ uint8_t smem_raw[];
@@ -100,7 +106,7 @@ step_gemm_kernel(const __grid_constant__ CUtensorMap map_w, const __grid_constan
       Work w;
       int stage = 0; uint32_t phase = 0;
       bool ok = true;
-      const uint32_t tx = W_BYTES + 2 * p.Bp * BK * 2;
+      const uint32_t tx = W_BYTES + p.rows * BK * 2;
       // The weights do not depend on the kernel before this one: the W tiles of the first S k-blocks are
       // requested before the wait for that kernel, so they stream in while it finishes (all stages are free,
       // in order, on a fresh pipeline).  The activation tiles of those k-blocks follow after the wait.
@@ -137,7 +143,7 @@ step_gemm_kernel(const __grid_constant__ CUtensorMap map_w, const __grid_constan
     }
   } else if (warp == 1) {
     if (lane == 0) {
-      const uint32_t idesc = idesc_bf16(BM, 2 * p.Bp);
+      const uint32_t idesc = idesc_bf16(BM, p.rows);
       Sched sched(p);
       Work w;
       int stage = 0; uint32_t phase = 0;
@@ -155,7 +161,10 @@ step_gemm_kernel(const __grid_constant__ CUtensorMap map_w, const __grid_constan
           const uint32_t sw = smem_base + stage * stage_bytes;
           const uint64_t da = desc_kmajor(sw), db = desc_kmajor(sw + W_BYTES);
 #pragma unroll
-          for (int k = 0; k < BK / 16; ++k) tc_mma_bf16(d_tmem, da + 2u * k, db + 2u * k, idesc, (kb > w.kb0 || k > 0) ? 1u : 0u);
+          for (int k = 0; k < BK / 16; ++k) {
+            if (TERMS == 3) tc_mma_bf16(d_tmem + ((kb - w.kb0) & (PARTS - 1)) * 16, da + 2u * k, db + 2u * k, idesc, (kb - w.kb0 >= PARTS || k > 0) ? 1u : 0u);
+            else tc_mma_bf16(d_tmem, da + 2u * k, db + 2u * k, idesc, (kb > w.kb0 || k > 0) ? 1u : 0u);
+          }
           tc_commit(empty_bar(stage));
           if (++stage == S) { stage = 0; phase ^= 1u; }
         }
@@ -177,16 +186,39 @@ step_gemm_kernel(const __grid_constant__ CUtensorMap map_w, const __grid_constan
       tc_fence_after();
       const int n = w.n0 + quarter * 32 + lane;
       const uint32_t t_acc = tmem_base + ((uint32_t)(quarter * 32) << 16) + acc * p.acc_stride;
+      if constexpr (TERMS == 3) {   // four columns of each term, in as many parts as the range has k blocks, at most eight
+        const int parts = w.kb1 - w.kb0;
+        float hi[4] = {0.f, 0.f, 0.f, 0.f}, lo[4] = {0.f, 0.f, 0.f, 0.f};
 #pragma unroll 1
-      for (int c = 0; c < p.batch; c += 8) {
-        float hi[8], lo[8];
-        tmem_ld8(t_acc + c, hi);
-        tmem_ld8(t_acc + p.Bp + c, lo);
-        tmem_ld_wait();
+        for (int q0 = 0; q0 < PARTS && q0 < parts; q0 += 4) {
+          float v[64];
+          tmem_ld32(t_acc + 16 * q0, v);
+          tmem_ld32(t_acc + 16 * q0 + 32, v + 32);
+          tmem_ld_wait();
+#pragma unroll
+          for (int q = 0; q < 4; ++q)
+            if (q0 + q < parts) {
+#pragma unroll
+              for (int i = 0; i < 4; ++i) { hi[i] += v[16 * q + i]; lo[i] += v[16 * q + 4 + i] + v[16 * q + 8 + i]; }
+            }
+        }
         if (n < p.N) {
 #pragma unroll
-          for (int i = 0; i < 8; ++i)
-            if (c + i < p.batch) red_add(p.Y + (size_t)(c + i) * p.ldy + n, hi[i] + lo[i]);
+          for (int i = 0; i < 4; ++i)
+            if (i < p.batch) red_add(p.Y + (size_t)i * p.ldy + n, hi[i] + lo[i]);
+        }
+      } else {
+#pragma unroll 1
+        for (int c = 0; c < p.batch; c += 8) {
+          float hi[8], lo[8];
+          tmem_ld8(t_acc + c, hi);
+          tmem_ld8(t_acc + p.Bp + c, lo);
+          tmem_ld_wait();
+          if (n < p.N) {
+#pragma unroll
+            for (int i = 0; i < 8; ++i)
+              if (c + i < p.batch) red_add(p.Y + (size_t)(c + i) * p.ldy + n, hi[i] + lo[i]);
+          }
         }
       }
       tc_fence_before();
@@ -208,7 +240,7 @@ step_gemm_kernel(const __grid_constant__ CUtensorMap map_w, const __grid_constan
 // chunks need no second kernel.
 constexpr int PREP_CHUNK = 2048;
 
-__global__ void __launch_bounds__(256) step_prep_kernel(int mode, const float* __restrict__ x, int ldx, int K, int batch, int Bp,
+__global__ void __launch_bounds__(256) step_prep_kernel(int mode, const float* __restrict__ x, int ldx, int K, int batch, int Bp, int terms,
                                                         const float* __restrict__ gain, float eps, RowMap mg, RowMap mu,
                                                         bf16* __restrict__ XB, float* zero_ptr, int zero_ld, int zero_n) {
   __shared__ float red[8];
@@ -218,10 +250,12 @@ __global__ void __launch_bounds__(256) step_prep_kernel(int mode, const float* _
   const int k_begin = blockIdx.y * PREP_CHUNK, k_end = min(K, k_begin + PREP_CHUNK);
   bf16* hi = XB + (size_t)b * K;
   bf16* lo = XB + (size_t)(Bp + b) * K;
+  bf16* rest = terms == 3 ? XB + (size_t)(2 * Bp + b) * K : nullptr;
   if (b >= batch) {
     for (int k = k_begin + tid * 8; k < k_end; k += 2048) {
       *reinterpret_cast<uint4*>(hi + k) = make_uint4(0, 0, 0, 0);
       *reinterpret_cast<uint4*>(lo + k) = make_uint4(0, 0, 0, 0);
+      if (rest) *reinterpret_cast<uint4*>(rest + k) = make_uint4(0, 0, 0, 0);
     }
     return;
   }
@@ -262,7 +296,7 @@ __global__ void __launch_bounds__(256) step_prep_kernel(int mode, const float* _
         for (int i = 0; i < 8; ++i) v[i] = gg[i] * v[i] * r;
       }
     }
-    uint32_t h[4], l[4];
+    uint32_t h[4], l[4], r3[4];
 #pragma unroll
     for (int i = 0; i < 4; ++i) {
       const __nv_bfloat162 hh = __floats2bfloat162_rn(v[2 * i], v[2 * i + 1]);
@@ -270,9 +304,13 @@ __global__ void __launch_bounds__(256) step_prep_kernel(int mode, const float* _
       const __nv_bfloat162 ll = __floats2bfloat162_rn(v[2 * i] - hf.x, v[2 * i + 1] - hf.y);
       h[i] = *reinterpret_cast<const uint32_t*>(&hh);
       l[i] = *reinterpret_cast<const uint32_t*>(&ll);
+      const float2 lf = __bfloat1622float2(ll);
+      const __nv_bfloat162 rr = __floats2bfloat162_rn(v[2 * i] - hf.x - lf.x, v[2 * i + 1] - hf.y - lf.y);
+      r3[i] = *reinterpret_cast<const uint32_t*>(&rr);
     }
     *reinterpret_cast<uint4*>(hi + k) = make_uint4(h[0], h[1], h[2], h[3]);
     *reinterpret_cast<uint4*>(lo + k) = make_uint4(l[0], l[1], l[2], l[3]);
+    if (rest) *reinterpret_cast<uint4*>(rest + k) = make_uint4(r3[0], r3[1], r3[2], r3[3]);
   }
   if (zero_ptr) {
     const int n_chunks = gridDim.y;
@@ -280,44 +318,49 @@ __global__ void __launch_bounds__(256) step_prep_kernel(int mode, const float* _
   }
 }
 
+template <int TERMS>
+cudaError_t go_gemm(const CUtensorMap& mw, const CUtensorMap& mx, const Params& p, int grid, int smem, cudaStream_t st) {
+  static bool raised[TC_MAX_DEVICES] = {};
+  cudaError_t e = tc_raise_smem_limit(step_gemm_kernel<TERMS>, SMEM_LIMIT, raised);
+  if (e != cudaSuccess) return e;
+  return launch_overlapped(step_gemm_kernel<TERMS>, dim3(grid), dim3(N_THREADS), (size_t)smem, st, mw, mx, p);
+}
+
 int pow2_ceil(int v) { int p = 1; while (p < v) p <<= 1; return p; }
 
 }  // namespace
 
 bool step_tc_supported(int batch, int K, int ldw, const void* W, const void* XB) {
-  return batch >= 1 && step_tc_rows(batch) <= 128 && K % 8 == 0 && ldw % 8 == 0 && ((uintptr_t)W & 15) == 0 &&
+  return batch >= 1 && step_tc_operand_rows(batch) <= 256 && K % 8 == 0 && ldw % 8 == 0 && ((uintptr_t)W & 15) == 0 &&
          ((uintptr_t)XB & 15) == 0;
 }
 
-void launch_step_prep(const LaunchCtx& ctx, int mode, const float* x, int ldx, int K, int batch, const float* gain, float eps,
+void launch_step_prep(const LaunchCtx& ctx, int mode, const float* x, int ldx, int K, int batch, int terms, const float* gain, float eps,
                       int G, bf16* XB, float* zero_ptr, int zero_ld, int zero_n, bool overlapped) {
-  const int Bp = step_tc_rows(batch);
+  const int Bp = step_tc_rows(batch, terms);
   RowMap mg{0, G, 0, K}, mu{G == 0 ? K : 0, G, 1, K};
   const dim3 grid(Bp, (K + PREP_CHUNK - 1) / PREP_CHUNK);
   ++*ctx.n_launch;
-  if (overlapped) launch_overlapped(step_prep_kernel, grid, dim3(256), 0, ctx.st, mode, x, ldx, K, batch, Bp, gain, eps, mg, mu, XB, zero_ptr, zero_ld, zero_n);
-  else step_prep_kernel<<<grid, 256, 0, ctx.st>>>(mode, x, ldx, K, batch, Bp, gain, eps, mg, mu, XB, zero_ptr, zero_ld, zero_n);
+  if (overlapped) launch_overlapped(step_prep_kernel, grid, dim3(256), 0, ctx.st, mode, x, ldx, K, batch, Bp, terms, gain, eps, mg, mu, XB, zero_ptr, zero_ld, zero_n);
+  else step_prep_kernel<<<grid, 256, 0, ctx.st>>>(mode, x, ldx, K, batch, Bp, terms, gain, eps, mg, mu, XB, zero_ptr, zero_ld, zero_n);
 }
 
-cudaError_t launch_step_gemm_tc(const bf16* W, int ldw, int N, int K, const bf16* XB, int batch, float* Y, int ldy, int n_sm,
+cudaError_t launch_step_gemm_tc(const bf16* W, int ldw, int N, int K, const bf16* XB, int batch, int terms, float* Y, int ldy, int n_sm,
                                 int* status, cudaStream_t st, int64_t* n_launch) {
-  const int Bp = step_tc_rows(batch);
+  const int Bp = step_tc_rows(batch, terms), rows = step_tc_operand_rows(batch, terms);
   CUtensorMap mw, mx;
   if (!tc_make_map_bf16(&mw, W, N, K, ldw, BM)) return cudaErrorInvalidValue;
-  if (!tc_make_map_bf16(&mx, XB, 2 * Bp, K, K, 2 * Bp)) return cudaErrorInvalidValue;
+  if (!tc_make_map_bf16(&mx, XB, rows, K, K, rows)) return cudaErrorInvalidValue;
   Params p{};
-  p.N = N; p.K = K; p.batch = batch; p.Bp = Bp; p.Y = Y; p.ldy = ldy; p.status = status;
-  p.x_bytes = (2 * Bp * BK * 2 + 1023) / 1024 * 1024;
+  p.N = N; p.K = K; p.batch = batch; p.Bp = Bp; p.rows = rows; p.Y = Y; p.ldy = ldy; p.status = status;
+  p.x_bytes = (rows * BK * 2 + 1023) / 1024 * 1024;
   p.stages = (SMEM_LIMIT - 2048) / (W_BYTES + p.x_bytes);
   if (p.stages > 12) p.stages = 12;
-  p.acc_stride = pow2_ceil(2 * Bp < 16 ? 16 : 2 * Bp);
+  p.acc_stride = terms == 3 ? PARTS * 16 : pow2_ceil(rows);
   const int smem = p.stages * (W_BYTES + p.x_bytes) + 1024 + 8 * (2 * p.stages + 4) + 64;
-  static bool raised[TC_MAX_DEVICES] = {};
-  cudaError_t e = tc_raise_smem_limit(step_gemm_kernel, SMEM_LIMIT, raised);
-  if (e != cudaSuccess) return e;
   const long long total = (long long)((N + BM - 1) / BM) * ((K + BK - 1) / BK);
   const long long want = (total + MIN_KB - 1) / MIN_KB;
   const int grid = (int)(want < CTAS_PER_SM * n_sm ? want : CTAS_PER_SM * n_sm);
   ++*n_launch;
-  return launch_overlapped(step_gemm_kernel, dim3(grid), dim3(N_THREADS), (size_t)smem, st, mw, mx, p);
+  return terms == 3 ? go_gemm<3>(mw, mx, p, grid, smem, st) : go_gemm<2>(mw, mx, p, grid, smem, st);
 }
