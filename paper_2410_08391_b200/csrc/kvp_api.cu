@@ -128,13 +128,14 @@ WsLayout ws_layout(const kvp_handle* h, int64_t Bm, int64_t Tm) {
   w.tok_slot = take(Tm * 4);
   w.rope_tab = take(Tm * (size_t)((A.L[0].hd / 2 + 1) & ~1) * 8);     // entries hold two frequencies: an even number of them
   w.x = take(Tm * A.d * 4);
-  w.h = take(Tm * A.d * es);
-  w.h_lo = take(Tm * A.d * es);
+  const bool f32 = h->opt.dtype == KVP_F32;       // (norms and SwiGLU are part of the products there, keys and values one term)
+  w.h = take(f32 ? 0 : Tm * A.d * es);
+  w.h_lo = take(f32 ? 0 : Tm * A.d * es);
   w.qkv = take(Tm * A.max_nqkv * es);
   w.qkv32 = take(Tm * A.max_nqkv * 4);
-  w.kv_lo = take(Tm * 2 * (size_t)A.max_dkv * es);
+  w.kv_lo = take(f32 ? 0 : Tm * 2 * (size_t)A.max_dkv * es);
   w.attn = take(Tm * A.max_dq * es);
-  w.gu = take(Tm * 2 * (size_t)A.max_ffn * es);
+  w.gu = take(f32 ? 0 : Tm * 2 * (size_t)A.max_ffn * es);
   w.act = take(Tm * (size_t)A.max_ffn * es);
   const size_t step0 = off;
   w.xb = take(Bm * B.d * 4);
