@@ -322,6 +322,9 @@ gemm_tc_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_constant_
     *abort_flag = 0;
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
   }
+  // The allocation for a pair works on the tensor memory of both SMs: it may only be asked for once the other CTA is known to run, and
+  // neither CTA may leave while the other's release is still to come.
+  if constexpr (PAIR) cluster_sync();
   if (warp == 1) {   // tensor memory: two accumulators of BN columns (a power of two is allocated)
     if constexpr (PAIR) tmem_alloc_pair(smem_u32(tmem_slot), 2 * T::ACC_STRIDE);
     else tmem_alloc(smem_u32(tmem_slot), 2 * T::ACC_STRIDE);
@@ -684,6 +687,7 @@ gemm_tc_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_constant_
     if constexpr (PAIR) tmem_dealloc_pair(tmem_base, 2 * T::ACC_STRIDE);
     else tmem_dealloc(tmem_base, 2 * T::ACC_STRIDE);
   }
+  if constexpr (PAIR) cluster_sync();
 }
 
 // ---- host side ----------------------------------------------------------------------------
@@ -738,8 +742,8 @@ cudaError_t go_epi(int epi, const CUtensorMap& a, const CUtensorMap& a2, const C
 // 3 waves or 2.03.  Fitted to 118 launches of 59 to 8192 rows, N 1280 to 32000, K 1280 to 5632, 76 and 148 SMs, one and two passes: the
 // geometric mean of the chosen cuts is 0.9 % above that of the best ones (the rule before, 128 or 256 columns by tensor time: 18 %).
 // A pair's k block takes 0.91 to 0.94 of that (each CTA writes and reads half of the W tile only) and its launch 1 to 2 us more (two SMs
-// at once, tensor memory of both, a cluster barrier at either end).  us, single / pair: gate / up 25240 x 8192 x 1536 469 / 428, 65536 x
-// 6912 x 1280 863 / 813, 3776 x 6912 x 1280 54.3 / 51.9, 1024 x 6912 x 1280 21.0 / 21.3; down with the norm 25240 x 1536 x 4096 306 / 258,
+// at once, tensor memory of both, cluster barriers at either end).  us, single / pair (without the second barrier at either end, 0.3 to 0.5 us): gate /
+// up 25240 x 8192 x 1536 469 / 428, 65536 x 6912 x 1280 863 / 813, 3776 x 6912 x 1280 54.3 / 51.9, 1024 x 6912 x 1280 21.0 / 21.3; down with the norm 25240 x 1536 x 4096 306 / 258,
 // in shares without it 251 / 226, 3776 x 1280 x 3456 28.9 / 29.3; QKV 25240 x 2304 x 1536 160 / 146, 1024 x 1920 x 1280 15.2 / 16.3; 2143 x 32000 x
 // 2048 in two passes 418 / 384.  Narrower tiles and the predictor (36.0 / 38.3 at K 384: its epilogue is the longer part) gain nothing as pairs.
 struct Cut { int bn; bool shares, pair; };

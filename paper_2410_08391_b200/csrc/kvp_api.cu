@@ -215,7 +215,7 @@ bool ends_with(const std::string& s, const char* suf) {
 bool try_tc(kvp_handle* h, const LaunchCtx& ctx, TcGemm& t, int cls, cudaError_t* err) {
   if (h->opt.dtype != KVP_BF16) return false;
   t.n_sm = h->gemm_sms;
-  t.pairs = h->gemm_sms == h->n_sm;      // (persistent pieces of the step hold SMs one by one, not in pairs)
+  t.pairs = h->gemm_pairs && h->gemm_sms == h->n_sm;
   if (!tc_gemm_supported(t)) return false;
   TimedScope ts(h, ctx.st, cls);
   cudaError_t e = launch_gemm_tc(t, ctx.status, ctx.st, ctx.n_launch);
@@ -766,6 +766,8 @@ static kvp_status prefill_direct(kvp_handle* h, const int32_t* tokens, const int
   // ---- stage 1 + 2: auxiliary prefill, each layer's K/V pushed through the predictor ----
   // (only worth it while a layer's kernels leave SMs idle: with many tokens every kernel fills the GPU by itself)
   const bool fork = h->side != nullptr && !h->timing && T <= 4096;
+  // Pairs of CTAs need both of their SMs at once, which kernels on the other streams hold one by one (64 x 59 with pairs 1 % faster or not at all).
+  h->gemm_pairs = !fork;
   bool pending_join = false;
   // The base step in pieces beside the prefill: piece j = the base layers whose cache (and that of every
   // layer below them) is complete once auxiliary layer j has gone through the predictor.
@@ -1004,6 +1006,7 @@ static kvp_status prefill_direct(kvp_handle* h, const int32_t* tokens, const int
   }
   if (pending_join) cudaStreamWaitEvent(s, h->ev_join, 0);     // the base step reads what the predictor wrote
   h->gemm_sms = h->step_grid_sms = h->n_sm;
+  h->gemm_pairs = true;
   if (piped || piped_tc) {     // the step is already enqueued in pieces: join its stream
     cudaEventRecord(h->ev_step, h->step_st);
     cudaStreamWaitEvent(s, h->ev_step, 0);

@@ -88,6 +88,7 @@ struct kvp_handle {
   cudaStream_t step_st = nullptr;
   cudaEvent_t ev_step = nullptr;
   int step_sms = 72;
+  bool gemm_pairs = true;               // may pairs of CTAs take a GEMM's tiles
   int gemm_sms = 148;                   // SMs the tensor-core GEMMs of the current call size their grids for
   int step_tc_sms = 96;                 // grid of the step's projections when its per-layer kernels (batch > 4) run beside the prefill
   int step_terms = 2;                   // bf16 terms of an activation in the step's tensor-core projections
