@@ -45,7 +45,7 @@ __device__ __forceinline__ void dev_flag(int* status, int code) { atomicCAS(stat
 // returns when the earlier kernel has finished and its writes, and those of all before it, are
 // visible.  Every kernel of a chain calls it, in at least one CTA, before it writes or reads what a kernel
 // of the chain writes.  Before it a kernel may read only what was complete when the chain's last ordinary
-// launch started: weights (RMSNorm's gain, the matrices of the step's projections), and, in the step's
+// launch started: weights (RMSNorm's gain, the matrices of all products), and, in the step's
 // attention, lengths, block table and cache pages.  So the embedding, with which every pass starts, and the
 // first launch behind a wait for another stream are ordinary launches: recorded into a graph, a dependent
 // launch behind such a wait may start while the other stream's kernel still runs.  Both calls do

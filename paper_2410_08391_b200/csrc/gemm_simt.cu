@@ -13,6 +13,7 @@ namespace {
 //              through every CTA) and scales its outputs by 1 / rms
 //   EPI_ROPE   tile columns 2 i and 2 i + 1 are the two halves of one rotated pair, whichever columns of W those are
 //   EPI_GATED  ... are the gate and the up column of one output
+// (with launches of their own for the four: 64 x 16 tokens 100.6 -> 96.1 us, 8 x 100 84.9 -> 81.8, 1 x 64 45.3 -> 44.1).
 template <class T, int EPI, int TS>
 __device__ __forceinline__ void gemm_simt_tile(const GemmArgs& g, const InvFreq* inv, int vec) {
   constexpr int R = TS / 16, BK = 2048 / TS, KT = BK / 8;

@@ -121,7 +121,7 @@ WsLayout ws_layout(const kvp_handle* h, int64_t Bm, int64_t Tm) {
   auto take = [&](size_t bytes) { size_t o = off; off = align_up(off + bytes, 256); return o; };
   const ModelPlan &A = h->aux, &B = h->base;
   size_t es = h->es;
-  w.status = take(16384);     // status word, barrier counter, argmax slots; from byte 256: optional phase trace
+  w.status = take(16384);     // status word, counters of finished CTAs, argmax slots; from byte 256: optional phase trace
   w.cu = take((Bm + 1) * 4);
   w.last_idx = take(Bm * 4);
   w.tok_pos = take(Tm * 4);
@@ -306,10 +306,10 @@ bool mega_uses_mma(const kvp_handle* h, int batch) {
 }
 cudaError_t launch_mega(kvp_handle* h, const MegaParams& p, int k_max, int n_sm, cudaStream_t st) {
   if (mega_uses_mma(h, p.batch)) return launch_step_mega_mma(p, h->base.max_group, n_sm, st, &h->n_launch);
-  // The CUDA-core kernel gives a row to a warp, 16 warps to a CTA, and its grid-wide barriers cost the more the more CTAs meet (and a
-  // launch that takes every SM keeps other calls off them): a model whose widest projection has fewer rows takes fewer CTAs, but no
+  // The CUDA-core kernel gives a row to a warp, 16 warps to a CTA, and a launch that takes every SM keeps other calls off them: a model whose widest projection has fewer rows takes fewer CTAs, but no
   // fewer than attention has items (key ranges of a sequence and kv head), which would then take several rounds.
-  // fp32 test pair, us by itself / among other calls, with 43 CTAs (rows / 16), 64, 96 and 148: first token of 1 x 64 (4 items) 139 / 45,
+  // fp32 test pair, us by itself / among other calls, with 43 CTAs (rows / 16), 64, 96 and 148 (all of it with the kernel that still had
+  // grid-wide barriers; first token of 1 x 64 with 43 now 125 / 39): first token of 1 x 64 (4 items) 139 / 45,
   // 139 / 55, 139 / 98, 141 / 99; step over 1 x 1000 keys (64 items) 188 / 55, 157 / 64, 158 / 124, 157 / 127; 4 x 300 (80) 224 / 67, 228 / 96,
   // 196 / 161, 198 / 165; 1 x 4000 (252) 361 / 111, 320 / 142, 272 / 238, 225 / 193; 4 x 4000 (304) 545 / 178, 441 / 203, 394 / 356, 311 / 274.
   const int rows = std::max(std::max(2 * h->base.max_ffn, h->base.max_nqkv), std::max(h->base.d, h->base.vocab));
