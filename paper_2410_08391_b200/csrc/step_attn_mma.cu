@@ -261,6 +261,13 @@ step_attn_mma_kernel(const __grid_constant__ CUtensorMap map_k, const __grid_con
           }
           __syncwarp();
         }
+        if (warp * 16 + 16 > nk) {
+          // Rows at or beyond the sequence's end may hold anything, and 0 x NaN is NaN: the values of this warp's 16 become zero in the CTA's
+          // copy.  (Their scores are never looked at.  Only a sequence's last page has such rows, and no copy into its stage follows.)
+          for (int i = lane; i < (warp * 16 + 16 - nk) * (HD / 8); i += 32)
+            asm volatile("st.shared.v4.b32 [%0], {%1, %1, %1, %1};" ::"r"(sv + piece(nk + i / (HD / 8), i % (HD / 8))), "r"(0u) : "memory");
+          __syncwarp();
+        }
         // ---- scores of this warp's 16 keys: two 8-key blocks
         float sc[2][4];
 #pragma unroll
