@@ -29,7 +29,6 @@ using namespace tcp;
 constexpr int NW = 4;                       // consumer warps
 constexpr int NT = (NW + 1) * 32;
 constexpr int BOX_BYTES = 64 * 128;         // one 64-key x 64-dim box
-constexpr float Q_UP = 16.f;                // scaled queries are multiplied by this before they are split, so that the remainder halves stay normal numbers
 
 template <int HD> struct MmaCfg {
   static constexpr int PAGE_BYTES = PAGE_TOKENS * HD * 2;
@@ -187,7 +186,7 @@ step_attn_mma_kernel(const __grid_constant__ CUtensorMap map_k, const __grid_con
   if (p.q_gain) head_rnorm(p.q + (size_t)b * p.ldq + (size_t)kvh * group * HD, group, HD, p.eps, rq);
   else __syncthreads();
   {
-    const float scale = Q_UP * rsqrtf((float)HD);
+    const float scale = rsqrtf((float)HD);
     for (int i = tid; i < 8 * half; i += NT) {
       const int h = i / half, c = i - h * half;
       float r1 = 0.f, r2 = 0.f;
@@ -229,11 +228,23 @@ step_attn_mma_kernel(const __grid_constant__ CUtensorMap map_k, const __grid_con
   if (warp < NW) {
     // ---------------- consumers: warp w takes keys 16 w .. 16 w + 15 of every page ----------------
     uint32_t qa[KS][4];                             // A fragments of Q: rows g = value part, g + 8 = remainder part
+    // A head's queries are split after a multiplication by the power of two that puts its largest between 2^13 and 2^14 (`down` takes it
+    // off the scores): no finite query is too large for a half, and remainders are normal halves down to 2^-16 of the largest.
+    float mx = 0.f;
 #pragma unroll
     for (int ks = 0; ks < KS; ++ks) {
       const float* qrow = qs + g * HD + ks * 16 + 2 * qd;
-      split2(qrow[0], qrow[1], qa[ks][0], qa[ks][1]);
-      split2(qrow[8], qrow[9], qa[ks][2], qa[ks][3]);
+      mx = fmaxf(mx, fmaxf(fmaxf(fabsf(qrow[0]), fabsf(qrow[1])), fmaxf(fabsf(qrow[8]), fabsf(qrow[9]))));
+    }
+    mx = fmaxf(mx, __shfl_xor_sync(0xffffffffu, mx, 1));
+    mx = fmaxf(mx, __shfl_xor_sync(0xffffffffu, mx, 2));
+    const int up_exp = min(253, 267 - (int)(__float_as_uint(mx) >> 23));
+    const float up = __uint_as_float((uint32_t)up_exp << 23), down = __uint_as_float((uint32_t)(254 - up_exp) << 23);
+#pragma unroll
+    for (int ks = 0; ks < KS; ++ks) {
+      const float* qrow = qs + g * HD + ks * 16 + 2 * qd;
+      split2(qrow[0] * up, qrow[1] * up, qa[ks][0], qa[ks][1]);
+      split2(qrow[8] * up, qrow[9] * up, qa[ks][2], qa[ks][3]);
     }
     const int k_lane = warp * 16 + (lane & 7);      // key row this lane addresses in matrix loads (+ 8 for the second key block)
     const int mi = lane >> 3;                        // which of the four 8 x 8 matrices of a load this lane addresses
@@ -283,8 +294,8 @@ step_attn_mma_kernel(const __grid_constant__ CUtensorMap map_k, const __grid_con
         float sv4[4];
 #pragma unroll
         for (int t = 0; t < 2; ++t) {
-          sv4[2 * t] = (sc[t][0] + sc[t][2]) * (1.f / Q_UP);
-          sv4[2 * t + 1] = (sc[t][1] + sc[t][3]) * (1.f / Q_UP);
+          sv4[2 * t] = (sc[t][0] + sc[t][2]) * down;
+          sv4[2 * t + 1] = (sc[t][1] + sc[t][3]) * down;
           const int key0 = warp * 16 + t * 8 + 2 * qd;
           if (key0 >= nk) sv4[2 * t] = -INFINITY;
           if (key0 + 1 >= nk) sv4[2 * t + 1] = -INFINITY;

@@ -1,5 +1,6 @@
 """What the base step's attention may meet in its inputs, whichever kernel serves it: cache rows at or beyond a sequence's length, which
 are unspecified and here hold NaN.  First step and generation step, against the oracle on the cache that the GPU left."""
+import numpy as np
 import pytest
 
 import workloads as wl
@@ -57,3 +58,23 @@ def test_rows_beyond_a_sequence_may_hold_anything(kernel, pair, lens):
     W = wl.make_weights(pair, seed=6, regime="fanin")
     assert recorded_prefill(pair, lens, W).find(kernel)
     _compare(pair, W, lens, fill=float("nan"))
+
+
+@pytest.mark.parametrize("kernel,pair,lens", [
+    ("step_attn_mma", _pair(64, (24, 8), 1544, 2568), [9, 130, 65]),
+    ("step_attn_mma", _pair(64, (8, 2)), [1, 63, 64, 65, 200]),
+    ("step_attn_mma", _pair(128, (6, 2)), [15, 16, 17, 33, 118]),
+    ("step_mega_mma", _pair(64, (8, 2)), [3, 100]),
+], ids=str)
+@pytest.mark.parametrize("up", [-12, 0, 14, 17])
+def test_queries_of_any_size(kernel, pair, lens, up):
+    """Queries of 2^up times the ordinary size (up to about 4 x 2^up; halves end at 65504 and lose bits below 6e-5) on keys of 2^-up of it, so
+    that the scores stay as they are; the cache is what the GPU holds, so that small keys are what they are."""
+    W = wl.make_weights(pair, seed=6, regime="fanin")
+    for i in range(2):
+        W[f"base.L{i}.wq"] = W[f"base.L{i}.wq"] * np.float32(2.0 ** up)
+        down = np.float32(2.0 ** min(12, -up))      # (keys of up to some thousand: halves, too)
+        W[f"base.L{i}.wk"] = W[f"base.L{i}.wk"] * down
+        W[f"pred.L{i}.fk"] = W[f"pred.L{i}.fk"] * down
+    assert recorded_prefill(pair, lens, W).find(kernel)
+    _compare(pair, W, lens)
