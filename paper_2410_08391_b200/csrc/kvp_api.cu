@@ -238,13 +238,26 @@ bool step_uses_tc(const kvp_handle* h, int batch) {
 // gate/up row, or as they are; null: they are there already), output cleared first unless it is the residual stream.
 void step_proj_tc(kvp_handle* h, const LaunchCtx& ctx, const WsLayout& w, char* ws, int mode, const float* src, int ld_src,
                   int K, int batch, const float* gain, int G, const void* W, int N, float* Y, int ldy, bool clear,
-                  cudaError_t* err, bool overlapped = true) {
+                  cudaError_t* err, bool overlapped = true, const StepSum& sum = StepSum()) {
   bf16* XB = (bf16*)(ws + w.xbt);
-  if (src) KVP_TIMED(KVP_CLASS_STEP_GEMV, launch_step_prep(ctx, mode, src, ld_src, K, batch, h->step_terms, gain, h->base.eps, G, XB, clear ? Y : nullptr, ldy, N, overlapped));
+  if (src) KVP_TIMED(KVP_CLASS_STEP_GEMV, launch_step_prep(ctx, mode, src, ld_src, K, batch, h->step_terms, gain, h->base.eps, G, XB, clear ? Y : nullptr, ldy, N, overlapped, sum));
   TimedScope ts(h, ctx.st, KVP_CLASS_STEP_GEMV);
   cudaError_t e = launch_step_gemm_tc((const bf16*)W, K, N, K, XB, batch, h->step_terms, Y, ldy, h->step_grid_sms, ctx.status, ctx.st, ctx.n_launch);
   if (e != cudaSuccess && *err == cudaSuccess) *err = e;
 }
+
+// The residual stream of a step with three terms: it goes back and forth between w.xb and x2, and partial sums onto it meet in o and down
+// (StepSum).  All in buffers that the other forms of the step use.
+struct StepStream { float *x2, *o, *down; };
+StepStream step_stream(const kvp_handle* h, const WsLayout& w, char* ws, int batch) {
+  float* sums = (float*)(ws + w.ab);            // (w.actb lies behind it)
+  return {(float*)(ws + w.hb), sums, sums + (size_t)batch * h->base.d};
+}
+bool step_stream_fits(const kvp_handle* h) {
+  const ModelPlan& B = h->base;
+  return 2 * (int64_t)B.d <= (int64_t)B.max_dq + B.max_ffn && B.max_dq <= 2 * B.max_ffn;
+}
+
 
 // one base-model layer of a single-token step (shared by the first step and generation)
 // after_event: the launch before it on this stream is a wait for another stream's kernels, which wrote the cache pages.  A dependent
@@ -263,15 +276,18 @@ void base_layer_step(kvp_handle* h, const LaunchCtx& ctx, int i, const kvp_cache
   // the first step needs q only (keys and values are the predicted ones); generation needs q, k, v
   int n_out = generation ? L.nqkv : L.dq;
   const bool tc = step_uses_tc(h, batch);
+  const StepStream x3 = step_stream(h, w, ws, batch);
+  const bool exact = tc && h->step_terms == 3;
   if (tc)
-    step_proj_tc(h, ctx, w, ws, PREP_NORM, xb, B.d, B.d, batch, (const float*)(P + L.attn_norm), 0, P + L.wqkv, n_out, qkvb, n_out, true, err, !after_event);
+    step_proj_tc(h, ctx, w, ws, PREP_NORM, exact && i > 0 ? x3.x2 : xb, B.d, B.d, batch, (const float*)(P + L.attn_norm), 0, P + L.wqkv, n_out, qkvb, n_out, true, err, !after_event,
+                 exact ? StepSum{i > 0 ? x3.down : nullptr, i > 0 ? xb : nullptr, x3.o} : StepSum());
   else
     KVP_TIMED(KVP_CLASS_STEP_GEMV, launch_step_gemv(ctx, P + L.wqkv, B.d, n_out, B.d, xb, B.d, batch, qkvb, n_out, GEMV_STORE, 0, 0,
                                                     (const float*)(P + L.attn_norm), B.eps, hb));
   StepAttn a{};
   a.q = qkvb; a.ldq = n_out; a.nq = L.nq; a.nkv = L.nkv; a.hd = L.hd; a.theta = B.theta; a.kpool = cache->k_pools[i]; a.vpool = cache->v_pools[i];
   a.block_table = cache->block_table; a.mpps = cache->max_pages_per_seq; a.n_pages = cache->n_pages; a.seq_lens = cache->seq_lens;
-  a.extra = a.append = generation ? 1 : 0; a.batch = batch; a.max_keys = max_keys; a.part = (float*)(ws + w.part); a.out = ab;
+  a.extra = a.append = generation ? 1 : 0; a.batch = batch; a.max_keys = max_keys; a.part = (float*)(ws + w.part); a.out = exact ? (float*)(ws + w.gub) : ab;
   a.terms = h->step_terms;
   a.xb = tc ? (bf16*)(ws + w.xbt) : nullptr;      // (the queries' own operand rows have been read)
   a.q_gain = B.qk_norm ? (const float*)(P + L.q_norm) : nullptr;
@@ -281,9 +297,10 @@ void base_layer_step(kvp_handle* h, const LaunchCtx& ctx, int i, const kvp_cache
   KVP_TIMED(KVP_CLASS_STEP_ATTN, in_xb = launch_step_attn(ctx, a));
   if (tc) {
     float* gub = (float*)(ws + w.gub);
-    step_proj_tc(h, ctx, w, ws, PREP_PLAIN, in_xb ? nullptr : ab, L.dq, L.dq, batch, nullptr, 0, P + L.wo, B.d, xb, B.d, false, err);
-    step_proj_tc(h, ctx, w, ws, PREP_NORM, xb, B.d, B.d, batch, (const float*)(P + L.ffn_norm), 0, P + L.wgu, 2 * L.ffn, gub, 2 * L.ffn, true, err);
-    step_proj_tc(h, ctx, w, ws, PREP_SWIGLU, gub, 2 * L.ffn, L.ffn, batch, nullptr, L.G, P + L.wd, B.d, xb, B.d, false, err);
+    step_proj_tc(h, ctx, w, ws, PREP_PLAIN, in_xb ? nullptr : a.out, L.dq, L.dq, batch, nullptr, 0, P + L.wo, B.d, exact ? x3.o : xb, B.d, false, err);
+    step_proj_tc(h, ctx, w, ws, PREP_NORM, xb, B.d, B.d, batch, (const float*)(P + L.ffn_norm), 0, P + L.wgu, 2 * L.ffn, gub, 2 * L.ffn, true, err, true,
+                 exact ? StepSum{x3.o, x3.x2, x3.down} : StepSum());
+    step_proj_tc(h, ctx, w, ws, PREP_SWIGLU, gub, 2 * L.ffn, L.ffn, batch, nullptr, L.G, P + L.wd, B.d, exact ? x3.down : xb, B.d, false, err);
     return;
   }
   KVP_TIMED(KVP_CLASS_STEP_GEMV, launch_step_gemv(ctx, P + L.wo, L.dq, B.d, L.dq, ab, L.dq, batch, xb, B.d, GEMV_RESID, 0, 0));
@@ -326,7 +343,7 @@ cudaError_t launch_mega(kvp_handle* h, const MegaParams& p, int k_max, int n_sm,
 // (2921 / 3027); 1.1B pair 4 x 300 2145 / 2077 (1853 / 1697), 3 x 1000 3321 / 3324 (3172 / 3068), 1 x 300 1409 / 1457 (1074 / 994), 1 x 1024 1801 /
 // 1981 (1608 / 1642); scaled 3 x 100 1627 / 1542 (1091 / 894).  Generation stays with the persistent kernel, which serves one call sooner.
 bool first_step_prefers_chain(const kvp_handle* h, int batch, double prefill_to_step, bool blocking) {
-  if (batch > 4 || !mega_uses_mma(h, batch) || !step_uses_tc(h, batch)) return false;
+  if (batch > 4 || !mega_uses_mma(h, batch) || !step_uses_tc(h, batch) || !step_stream_fits(h)) return false;
   double mb = 0;        // weights of a layer
   for (const LayerPlan& L : h->base.L) mb += (2.0 * L.dq + 3.0 * L.ffn) * h->base.d * h->es * 1e-6 / h->base.n_layers;
   if (batch > 2) return mb >= 30.0 && !blocking;
@@ -426,8 +443,11 @@ void base_head(kvp_handle* h, const LaunchCtx& ctx, const WsLayout& w, char* ws,
   const char* P = h->packed;
   float* xb = (float*)(ws + w.xb);
   float* hb = (float*)(ws + w.hb);
+  const StepStream x3 = step_stream(h, w, ws, batch);
+  const bool exact = h->step_terms == 3;
   if (step_uses_tc(h, batch))
-    step_proj_tc(h, ctx, w, ws, PREP_NORM, xb, B.d, B.d, batch, (const float*)(P + B.final_norm), 0, P + B.lm_head, B.vocab, logits, B.vocab, true, err);
+    step_proj_tc(h, ctx, w, ws, PREP_NORM, exact ? x3.x2 : xb, B.d, B.d, batch, (const float*)(P + B.final_norm), 0, P + B.lm_head, B.vocab, logits, B.vocab, true, err, true,
+                 exact ? StepSum{x3.down, nullptr, nullptr} : StepSum());
   else
   KVP_TIMED(KVP_CLASS_STEP_GEMV, launch_step_gemv(ctx, P + B.lm_head, B.d, B.vocab, B.d, xb, B.d, batch, logits, B.vocab, GEMV_STORE, 0, 0,
                                                   (const float*)(P + B.final_norm), B.eps, hb));

@@ -230,11 +230,12 @@ step_attn_mma_kernel(const __grid_constant__ CUtensorMap map_k, const __grid_con
     uint32_t qa[KS][4];                             // A fragments of Q: rows g = value part, g + 8 = remainder part
     // A head's queries are split after a multiplication by the power of two that puts its largest between 2^13 and 2^14 (`down` takes it
     // off the scores): no finite query is too large for a half, and remainders are normal halves down to 2^-16 of the largest.
+    float2 qv[2 * KS];
     float mx = 0.f;
 #pragma unroll
-    for (int ks = 0; ks < KS; ++ks) {
-      const float* qrow = qs + g * HD + ks * 16 + 2 * qd;
-      mx = fmaxf(mx, fmaxf(fmaxf(fabsf(qrow[0]), fabsf(qrow[1])), fmaxf(fabsf(qrow[8]), fabsf(qrow[9]))));
+    for (int i = 0; i < 2 * KS; ++i) {
+      qv[i] = *reinterpret_cast<const float2*>(qs + g * HD + i * 8 + 2 * qd);
+      mx = fmaxf(mx, fmaxf(fabsf(qv[i].x), fabsf(qv[i].y)));
     }
     mx = fmaxf(mx, __shfl_xor_sync(0xffffffffu, mx, 1));
     mx = fmaxf(mx, __shfl_xor_sync(0xffffffffu, mx, 2));
@@ -242,9 +243,8 @@ step_attn_mma_kernel(const __grid_constant__ CUtensorMap map_k, const __grid_con
     const float up = __uint_as_float((uint32_t)up_exp << 23), down = __uint_as_float((uint32_t)(254 - up_exp) << 23);
 #pragma unroll
     for (int ks = 0; ks < KS; ++ks) {
-      const float* qrow = qs + g * HD + ks * 16 + 2 * qd;
-      split2(qrow[0] * up, qrow[1] * up, qa[ks][0], qa[ks][1]);
-      split2(qrow[8] * up, qrow[9] * up, qa[ks][2], qa[ks][3]);
+      split2(qv[2 * ks].x * up, qv[2 * ks].y * up, qa[ks][0], qa[ks][1]);
+      split2(qv[2 * ks + 1].x * up, qv[2 * ks + 1].y * up, qa[ks][2], qa[ks][3]);
     }
     const int k_lane = warp * 16 + (lane & 7);      // key row this lane addresses in matrix loads (+ 8 for the second key block)
     const int mi = lane >> 3;                        // which of the four 8 x 8 matrices of a load this lane addresses

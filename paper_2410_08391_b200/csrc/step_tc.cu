@@ -31,15 +31,19 @@ constexpr int SMEM_LIMIT = 112 * 1024;
 // itself: 1787 / 1630 / 1642 / 1520, 3603 / 3455 / 3412 / 3370, 1355 / 1318 / 1330 / 1303.
 constexpr int MIN_KB = 8, CTAS_PER_SM = 2;
 
-// With three terms a sum is taken in eight parts, k blocks in turn, each in columns of its own, that the epilogue adds in fp32: the tensor
+// With three terms a sum is taken in sixteen parts, k blocks in turn, each in columns of its own, that the epilogue adds in fp32: the tensor
 // core rounds towards zero with every instruction, and 24-bit operands are worth no more than the sum.  (Changing columns with every
-// instruction instead cost 1 to 2 us a launch.)
-constexpr int PARTS = 8;
+// instruction instead cost 1 to 2 us a launch.)  There is one accumulator then, not two: two CTAs still share an SM's 512 columns.
+// Distance of the first step's logits from 64 bits on the same cache, persistent kernel / eight parts added to x one by one / sixteen
+// / sixteen and x in StepSum's way: 3B shape 4 x 300 1.60e-6 / 2.00e-6 / 1.80e-6 / 1.55e-6, 1.1B 1.30 / 1.39 / 1.42 / 1.21, scaled 3 x 100 2.25 / 2.10 /
+// 2.10 / 1.96; first token of them 3270 -> 3305 us, 1668 -> 1672, 845 -> 859.
+constexpr int PARTS = 16;
+template <int TERMS> constexpr int N_ACC = TERMS == 3 ? 1 : 2;
 
 struct Params {
   int N, K, batch, Bp, rows;      // rows of the operand buffer: the columns of an accumulator
   int stages, x_bytes;      // ring depth; bytes of the activation tile of a stage (multiple of 1024)
-  int acc_stride;           // tensor-memory columns between the two accumulators
+  int acc_stride;           // tensor-memory columns of an accumulator
   float* Y; int ldy;
   int* status;
 };
@@ -85,7 +89,7 @@ step_gemm_kernel(const __grid_constant__ CUtensorMap map_w, const __grid_constan
   auto tfull_bar = [&](int a) { return bar_base + 8u * (2 * S + a); };
   auto tempty_bar = [&](int a) { return bar_base + 8u * (2 * S + 2 + a); };
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  const uint32_t tmem_cols = max(32, 2 * p.acc_stride);
+  const uint32_t tmem_cols = max(32, N_ACC<TERMS> * p.acc_stride);
   if (threadIdx.x == 32) { prefetch_tensormap(&map_w); prefetch_tensormap(&map_x); }   // on their way while the rest is set up
 
   if (threadIdx.x == 0) {
@@ -169,7 +173,7 @@ step_gemm_kernel(const __grid_constant__ CUtensorMap map_w, const __grid_constan
           if (++stage == S) { stage = 0; phase ^= 1u; }
         }
         if (ok) tc_commit(tfull_bar(acc));
-        if (++acc == 2) { acc = 0; acc_phase ^= 1u; }
+        if (++acc == N_ACC<TERMS>) { acc = 0; acc_phase ^= 1u; }
       }
       if (!ok) drain_after_abort();
     }
@@ -186,7 +190,7 @@ step_gemm_kernel(const __grid_constant__ CUtensorMap map_w, const __grid_constan
       tc_fence_after();
       const int n = w.n0 + quarter * 32 + lane;
       const uint32_t t_acc = tmem_base + ((uint32_t)(quarter * 32) << 16) + acc * p.acc_stride;
-      if constexpr (TERMS == 3) {   // four columns of each term, in as many parts as the range has k blocks, at most eight
+      if constexpr (TERMS == 3) {   // four columns of each term, in as many parts as the range has k blocks, at most PARTS
         const int parts = w.kb1 - w.kb0;
         float hi[4] = {0.f, 0.f, 0.f, 0.f}, lo[4] = {0.f, 0.f, 0.f, 0.f};
 #pragma unroll 1
@@ -224,7 +228,7 @@ step_gemm_kernel(const __grid_constant__ CUtensorMap map_w, const __grid_constan
       tc_fence_before();
       __syncwarp();
       if (lane == 0) mbar_arrive(tempty_bar(acc));
-      if (++acc == 2) { acc = 0; acc_phase ^= 1u; }
+      if (++acc == N_ACC<TERMS>) { acc = 0; acc_phase ^= 1u; }
     }
   }
   tc_fence_before();
@@ -240,9 +244,10 @@ step_gemm_kernel(const __grid_constant__ CUtensorMap map_w, const __grid_constan
 // chunks need no second kernel.
 constexpr int PREP_CHUNK = 2048;
 
+template <bool SUM>
 __global__ void __launch_bounds__(256) step_prep_kernel(int mode, const float* __restrict__ x, int ldx, int K, int batch, int Bp, int terms,
                                                         const float* __restrict__ gain, float eps, RowMap mg, RowMap mu,
-                                                        bf16* __restrict__ XB, float* zero_ptr, int zero_ld, int zero_n) {
+                                                        bf16* __restrict__ XB, float* zero_ptr, int zero_ld, int zero_n, StepSum sum) {
   __shared__ float red[8];
   pdl_trigger();
   pdl_wait();         // everything below reads or overwrites what earlier kernels of the step use
@@ -260,11 +265,17 @@ __global__ void __launch_bounds__(256) step_prep_kernel(int mode, const float* _
     return;
   }
   const float* xr = x + (size_t)b * ldx;
+  const float* ar = SUM && sum.add ? sum.add + (size_t)b * K : nullptr;
+  auto load4 = [&](int k) {
+    float4 v = *reinterpret_cast<const float4*>(xr + k);
+    if (ar) { const float4 a = *reinterpret_cast<const float4*>(ar + k); v.x += a.x; v.y += a.y; v.z += a.z; v.w += a.w; }
+    return v;
+  };
   float r = 1.f;
   if (mode == PREP_NORM) {
     float ss = 0.f;
     for (int k = tid * 4; k < K; k += 1024) {
-      const float4 v = *reinterpret_cast<const float4*>(xr + k);
+      const float4 v = load4(k);
       ss = fmaf(v.x, v.x, ss); ss = fmaf(v.y, v.y, ss); ss = fmaf(v.z, v.z, ss); ss = fmaf(v.w, v.w, ss);
     }
     ss = warp_sum(ss);
@@ -287,7 +298,11 @@ __global__ void __launch_bounds__(256) step_prep_kernel(int mode, const float* _
 #pragma unroll
       for (int i = 0; i < 8; ++i) v[i] = __fdividef(gv[i], 1.f + __expf(-gv[i])) * uv[i];
     } else {
-      const float4 a0 = *reinterpret_cast<const float4*>(xr + k), a1 = *reinterpret_cast<const float4*>(xr + k + 4);
+      const float4 a0 = load4(k), a1 = load4(k + 4);
+      if (SUM && sum.out) {
+        float* o = sum.out + (size_t)b * K + k;
+        *reinterpret_cast<float4*>(o) = a0; *reinterpret_cast<float4*>(o + 4) = a1;
+      }
       v[0] = a0.x; v[1] = a0.y; v[2] = a0.z; v[3] = a0.w; v[4] = a1.x; v[5] = a1.y; v[6] = a1.z; v[7] = a1.w;
       if (mode == PREP_NORM) {
         const float4 c0 = *reinterpret_cast<const float4*>(gain + k), c1 = *reinterpret_cast<const float4*>(gain + k + 4);
@@ -316,6 +331,7 @@ __global__ void __launch_bounds__(256) step_prep_kernel(int mode, const float* _
     const int n_chunks = gridDim.y;
     for (int i = blockIdx.y * 256 + tid; i < zero_n; i += n_chunks * 256) zero_ptr[(size_t)b * zero_ld + i] = 0.f;
   }
+  if (SUM && sum.clear) for (int k = k_begin + tid; k < k_end; k += 256) sum.clear[(size_t)b * K + k] = 0.f;
 }
 
 template <int TERMS>
@@ -336,13 +352,14 @@ bool step_tc_supported(int batch, int K, int ldw, const void* W, const void* XB)
 }
 
 void launch_step_prep(const LaunchCtx& ctx, int mode, const float* x, int ldx, int K, int batch, int terms, const float* gain, float eps,
-                      int G, bf16* XB, float* zero_ptr, int zero_ld, int zero_n, bool overlapped) {
+                      int G, bf16* XB, float* zero_ptr, int zero_ld, int zero_n, bool overlapped, const StepSum& sum) {
   const int Bp = step_tc_rows(batch, terms);
   RowMap mg{0, G, 0, K}, mu{G == 0 ? K : 0, G, 1, K};
   const dim3 grid(Bp, (K + PREP_CHUNK - 1) / PREP_CHUNK);
   ++*ctx.n_launch;
-  if (overlapped) launch_overlapped(step_prep_kernel, grid, dim3(256), 0, ctx.st, mode, x, ldx, K, batch, Bp, terms, gain, eps, mg, mu, XB, zero_ptr, zero_ld, zero_n);
-  else step_prep_kernel<<<grid, 256, 0, ctx.st>>>(mode, x, ldx, K, batch, Bp, terms, gain, eps, mg, mu, XB, zero_ptr, zero_ld, zero_n);
+  const auto kernel = terms == 3 ? step_prep_kernel<true> : step_prep_kernel<false>;
+  if (overlapped) launch_overlapped(kernel, grid, dim3(256), 0, ctx.st, mode, x, ldx, K, batch, Bp, terms, gain, eps, mg, mu, XB, zero_ptr, zero_ld, zero_n, sum);
+  else kernel<<<grid, 256, 0, ctx.st>>>(mode, x, ldx, K, batch, Bp, terms, gain, eps, mg, mu, XB, zero_ptr, zero_ld, zero_n, sum);
 }
 
 cudaError_t launch_step_gemm_tc(const bf16* W, int ldw, int N, int K, const bf16* XB, int batch, int terms, float* Y, int ldy, int n_sm,

@@ -13,11 +13,19 @@ bool step_tc_supported(int batch, int K, int ldw, const void* W, const void* XB)
 
 // XB[b, :] = bf16(v_b), XB[Bp + b, :] = bf16(v_b - bf16(v_b)) (and so on) for b < batch (zero rows up to Bp), where
 //   PREP_PLAIN:  v_b = x[b, 0:K]
-//   PREP_NORM:   v_b = gain * x[b] / sqrt(mean(x[b]^2) + eps)
+//   PREP_NORM:   v_b = gain * x[b] / sqrt(mean(x[b]^2) + eps), x plus `add` where there is one (and their sum to `out`)
 //   PREP_SWIGLU: v_b[c] = silu(x[b, gate row c]) * x[b, up row c], c < K = ffn, rows placed as in the packed w_gate/w_up
 // Also clears zero_ptr[b, 0:zero_n] (row stride zero_ld) for b < batch when zero_ptr is given.
+//
+// With three terms the partial sums of a projection onto the residual stream x (up to 24 a row) meet in a buffer of their own, and the next
+// PREP_NORM adds them to x at once: added to x one by one, each sum rounds to x, which is several times as large.
+struct StepSum {            // rows of K floats
+  const float* add = nullptr;
+  float* out = nullptr;     // (not x: other CTAs still read it)
+  float* clear = nullptr;   // where the next such projection's partial sums will meet
+};
 void launch_step_prep(const LaunchCtx&, int mode, const float* x, int ldx, int K, int batch, int terms, const float* gain, float eps,
-                      int G, bf16* XB, float* zero_ptr, int zero_ld, int zero_n, bool overlapped = true);
+                      int G, bf16* XB, float* zero_ptr, int zero_ld, int zero_n, bool overlapped = true, const StepSum& sum = StepSum());
 
 // Y[b, n] += sum_k W[n, k] (XB[b, k] + XB[Bp + b, k] + ...) for b < batch, n < N; fp32 atomic adds.
 cudaError_t launch_step_gemm_tc(const bf16* W, int ldw, int N, int K, const bf16* XB, int batch, int terms, float* Y, int ldy,
