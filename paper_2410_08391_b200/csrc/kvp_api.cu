@@ -335,19 +335,21 @@ cudaError_t launch_mega(kvp_handle* h, const MegaParams& p, int k_max, int n_sm,
   return launch_step_mega(p, h->opt.dtype, k_max, std::min(n_sm, ctas), st, &h->n_launch);
 }
 
-// First steps of up to four sequences: is the chain of launches served sooner than the persistent tensor-core kernel?  (Both keep 24 bits
-// of an activation: the chain takes three terms then.)  Beside a prefill the chain takes SMs for some microseconds at a time and leaves
-// them to the prefill otherwise; the persistent kernel multiplies three or four rows on slower units, and a layer of it beside the prefill
-// takes the longer the more weights a layer has.  First token, us, persistent / chain by itself (among other calls): 3B pair 4 x 300 4662 / 3831
-// (3759 / 3321), 4 x 3000 16601 / 16381 (16922 / 15439), 2 x 300 3580 / 3146 (2617 / 2567), 1 x 300 3186 / 2968 (2336 / 2136), 1 x 1024 3574 / 3440
-// (2921 / 3027); 1.1B pair 4 x 300 2145 / 2077 (1853 / 1697), 3 x 1000 3321 / 3324 (3172 / 3068), 1 x 300 1409 / 1457 (1074 / 994), 1 x 1024 1801 /
-// 1981 (1608 / 1642); scaled 3 x 100 1627 / 1542 (1091 / 894).  Generation stays with the persistent kernel, which serves one call sooner.
-bool first_step_prefers_chain(const kvp_handle* h, int batch, double prefill_to_step, bool blocking) {
-  if (batch > 4 || !mega_uses_mma(h, batch) || !step_uses_tc(h, batch) || !step_stream_fits(h)) return false;
+// First steps of three and four sequences: the chain of launches, or the persistent tensor-core kernel?  (The chain takes three terms then
+// and sums as exactly, step_tc.cu.)  Beside a prefill the chain takes SMs for some microseconds at a time and leaves them to the prefill
+// otherwise; the persistent kernel multiplies three or four rows on slower units.  First token among other calls (by itself), us,
+// persistent / chain: 3B pair 4 x 300 3759 / 3305 (4662 / 3831), 4 x 3000 16922 / 15587 (16601 / 16381); 1.1B pair 4 x 300 1853 / 1672 (2145 / 2077), 3 x 1000
+// 3172 / 3068 (3321 / 3324); scaled 3 x 100 1091 / 859 (1627 / 1542).  The weights of a layer are 189, 86
+// and on average 68 MB there; nothing was measured between them and pairs of test size, where launches count: the line at 30 MB is set, not found.
+// A caller that waits is served by the persistent kernel: from host memory to host memory scaled 3 x 100 1394 / 1461; but 1.1B 3 x 40 1444 / 1395,
+// 4 x 300 2075 / 1950, 3 x 1000 3280 / 3208, layer-pruned 4 x 300 2756 / 2686, 3B 3 x 60 3277 / 2578, 4 x 300 4034 / 3707, so a finer line would pay there.
+// One and two sequences stay with the persistent kernel: it is the more exact one for them (3B shape 1 x 300 1.30e-6 of 64 bits, the chain
+// 1.46e-6), though the chain is served sooner on the 3B pair (2336 / 2065).  Generation stays with it too, which serves one call sooner.
+bool first_step_prefers_chain(const kvp_handle* h, int batch, bool blocking) {
+  if (batch <= 2 || batch > 4 || blocking || !mega_uses_mma(h, batch) || !step_uses_tc(h, batch) || !step_stream_fits(h)) return false;
   double mb = 0;        // weights of a layer
   for (const LayerPlan& L : h->base.L) mb += (2.0 * L.dq + 3.0 * L.ffn) * h->base.d * h->es * 1e-6 / h->base.n_layers;
-  if (batch > 2) return mb >= 30.0 && !blocking;
-  return mb >= 150.0 && prefill_to_step < 0.75 && !blocking;
+  return mb >= 30.0;
 }
 
 // Parameters of the persistent step kernel for this call; false = the kernel does not apply.
@@ -793,8 +795,7 @@ static kvp_status prefill_direct(kvp_handle* h, const int32_t* tokens, const int
   // layer below them) is complete once auxiliary layer j has gone through the predictor.
   MegaParams mp;
   int mega_kmax = 0, piece = 0, base_done = 0;
-  const CallTimes times = estimate_call(h, batch, cs);
-  const bool chain = first_step_prefers_chain(h, batch, times.prefill / times.step, blocking);
+  const bool chain = first_step_prefers_chain(h, batch, blocking);
   struct Terms {        // (the step's launches below, whichever way this function is left)
     kvp_handle* h;
     Terms(kvp_handle* h_, int n) : h(h_) { h->step_terms = n; }

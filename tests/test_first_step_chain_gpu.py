@@ -76,3 +76,11 @@ def test_the_chain_is_as_exact_as_the_persistent_kernel(pair, lens):
         assert chain <= persistent
     finally:
         s.close()
+
+
+@pytest.mark.parametrize("lens", [[20], [20, 9]], ids=str)
+def test_one_and_two_sequences_stay_with_the_persistent_kernel(lens):
+    """It is the more exact one for them, however many weights a layer has (here 193 MB) and however short the prompt."""
+    pair = wl.PairCfg("large_layer", wl.uniform_model(1, 64, 1, 1, 128, 64, 300), wl.uniform_model(1, 4104, 8, 2, 128, 7176, 300), (0,))
+    g = recorded_prefill(pair, lens)
+    assert g.find("step_mega_mma_kernel") and not g.find("step_gemm_kernel")
