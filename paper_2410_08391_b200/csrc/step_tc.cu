@@ -20,16 +20,20 @@ using namespace tcp;
 constexpr int BM = 128, BK = 64;
 constexpr int W_BYTES = BM * BK * 2;
 constexpr int N_THREADS = 192;
-// Half of an SM's shared memory: a CTA waits for the launch before it and for its first tiles most of its time, so two share an SM,
-// the next projection's or another call's.  With all of it, us, generation step among other calls / by itself, all -> half: 1.1B shape 8 x 300
-// 823 / 1465 -> 652 / 1331, 32 x 200 964 / 1580 -> 808 / 1537, 64 x 123 1035 / 1724 -> 936 / 1771 (three stages of 32 KB are few for one
-// call), 3B shape 16 x 1000 2084 / 2807 -> 1802 / 2832, 4 x 16000 2766 / 3666 -> 2525 / 3573.  A third: 8 x 300 634 / 1371, but 64 x 123 1080 / 2570.
-constexpr int SMEM_LIMIT = 112 * 1024;
+// Two CTAs share an SM wherever their accumulators fit its tensor memory: a CTA waits for the launch before it and for its first tiles most
+// of its time.  A CTA with the whole SM / half of its shared memory, us, generation step among other calls and by itself: 1.1B shape 8 x 300
+// 823 and 1465 / 652 and 1331, 32 x 200 964 and 1580 / 808 and 1537, 64 x 123 1035 and 1724 / 936 and 1771 (three stages of 32 KB are few for
+// one call), 3B shape 16 x 1000 2084 and 2807 / 1802 and 2832, 4 x 16000 2766 and 3666 / 2525 and 3573; a third: 8 x 300 634 and 1371, 64 x 123 1080 and 2570.
+// From 65 sequences on two accumulators take all 512 columns.  A second CTA would wait for the first to leave before it asks for a weight: us
+// among other calls and of a new state's first pass, two CTAs an SM / one with all of its shared memory: 83 x 123 1374 and 2590 / 1200 and 1850, 128
+// x 123 1639 and 3270 / 1569 and 2220, 3B shape 96 x 200 3520 and 4860 / 3128 and 3530.  (Two CTAs with one accumulator each: 1171 and 2040, 1482 and
+// 2430, 3111 and 3680: calls of a batch this large that come alone lose what others gain.)
+constexpr int SMEM_SHARED = 112 * 1024, SMEM_WHOLE = 220 * 1024;
 // Fewest k blocks of a CTA: a narrow projection (2048 x 2048: 512 blocks) takes 64 CTAs, a wide one two on every SM.  Every CTA adds a
 // block of partial sums to the output for each tile it touches, so more CTAs serve one call and fewer many.  With one CTA an SM at most /
 // 8 blocks / 6 / 4, among other calls: 64 x 123 918 / 946 / 975 / 990, 3B shape 4 x 16000 2518 / 2559 / 2621 / 2731, 8 x 300 655 / 663 / 677 / 702; by
 // itself: 1787 / 1630 / 1642 / 1520, 3603 / 3455 / 3412 / 3370, 1355 / 1318 / 1330 / 1303.
-constexpr int MIN_KB = 8, CTAS_PER_SM = 2;
+constexpr int MIN_KB = 8;
 
 // With three terms a sum is taken in sixteen parts, k blocks in turn, each in columns of its own, that the epilogue adds in fp32: the tensor
 // core rounds towards zero with every instruction, and 24-bit operands are worth no more than the sum.  (Changing columns with every
@@ -337,7 +341,7 @@ __global__ void __launch_bounds__(256) step_prep_kernel(int mode, const float* _
 template <int TERMS>
 cudaError_t go_gemm(const CUtensorMap& mw, const CUtensorMap& mx, const Params& p, int grid, int smem, cudaStream_t st) {
   static bool raised[TC_MAX_DEVICES] = {};
-  cudaError_t e = tc_raise_smem_limit(step_gemm_kernel<TERMS>, SMEM_LIMIT, raised);
+  cudaError_t e = tc_raise_smem_limit(step_gemm_kernel<TERMS>, SMEM_WHOLE, raised);
   if (e != cudaSuccess) return e;
   return launch_overlapped(step_gemm_kernel<TERMS>, dim3(grid), dim3(N_THREADS), (size_t)smem, st, mw, mx, p);
 }
@@ -371,13 +375,15 @@ cudaError_t launch_step_gemm_tc(const bf16* W, int ldw, int N, int K, const bf16
   Params p{};
   p.N = N; p.K = K; p.batch = batch; p.Bp = Bp; p.rows = rows; p.Y = Y; p.ldy = ldy; p.status = status;
   p.x_bytes = (rows * BK * 2 + 1023) / 1024 * 1024;
-  p.stages = (SMEM_LIMIT - 2048) / (W_BYTES + p.x_bytes);
-  if (p.stages > 12) p.stages = 12;
   p.acc_stride = terms == 3 ? PARTS * 16 : pow2_ceil(rows);
+  const bool shared = (terms == 3 ? N_ACC<3> : N_ACC<2>) * p.acc_stride <= 256;      // two CTAs' accumulators fit an SM's tensor memory
+  p.stages = ((shared ? SMEM_SHARED : SMEM_WHOLE) - 2048) / (W_BYTES + p.x_bytes);
+  if (p.stages > 12) p.stages = 12;
   const int smem = p.stages * (W_BYTES + p.x_bytes) + 1024 + 8 * (2 * p.stages + 4) + 64;
   const long long total = (long long)((N + BM - 1) / BM) * ((K + BK - 1) / BK);
   const long long want = (total + MIN_KB - 1) / MIN_KB;
-  const int grid = (int)(want < CTAS_PER_SM * n_sm ? want : CTAS_PER_SM * n_sm);
+  const long long most = (shared ? 2 : 1) * n_sm;
+  const int grid = (int)(want < most ? want : most);
   ++*n_launch;
   return terms == 3 ? go_gemm<3>(mw, mx, p, grid, smem, st) : go_gemm<2>(mw, mx, p, grid, smem, st);
 }
