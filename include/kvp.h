@@ -25,7 +25,11 @@
  *   - Calls that take a stream only enqueue work on it and return without
  *     synchronising (except the *_host variant, which synchronises the stream);
  *     arguments are validated on the host before anything is launched.
- *   - Device-side waits are bounded; a kernel that gives up, or that meets an
+ *   - Device-side waits are bounded, except where the hardware has no bounded form: a
+ *     block's request for tensor memory, which waits for the block on its SM that holds
+ *     it, and the barriers between the two blocks of a pair in the matrix products of
+ *     prefills above 4096 tokens and of kvp_train_forward(), whose two blocks run at the
+ *     same time by construction.  A kernel that gives up, or that meets an
  *     out-of-range token id or page index, records a code in a status word inside
  *     the workspace and skips the access.  kvp_poll_status() reads it.  The status
  *     word is cleared by kvp_prefill_predict() at its start and by kvp_poll_status();

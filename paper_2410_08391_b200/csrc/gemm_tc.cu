@@ -36,7 +36,7 @@ constexpr int N_THREADS = 224;                             // warps: 0 A loads, 
 constexpr int N_THREADS_NORM = 352;                        // fused-norm residual kernel: 8 epilogue warps (3-10), two per lane quarter
 constexpr int TC_RESID_NORM = 100;                         // internal: TC_RESID with the folded RMSNorm producer (own shared-memory plan)
 constexpr int SMEM_LIMIT = 227 * 1024;
-template <int BN, int EPI = TC_STORE, bool PAIR = false> struct Tile {
+template <int BN, int EPI, bool PAIR> struct Tile {
   static constexpr int XS = (EPI == TC_PAGED || EPI == TC_QKV) ? 1 : 2;        // 4 KiB slots per epilogue warp
   // epilogues that move every element through shared memory get eight warps (two per tensor-memory lane quarter)
   static constexpr int EPI_WARPS = (EPI == TC_RESID_NORM || EPI == TC_PAGED || EPI == TC_QKV || EPI == TC_SWIGLU) ? 8 : 4;
@@ -163,18 +163,7 @@ struct Sched {
 template <int EPI, int BN>
 __device__ __forceinline__ void epilogue_tile(const Params& p, uint32_t tmem_acc, int m, int n0, bool row_ok, int part, int n_parts, uint32_t slot, int row_base) {
   // tmem_acc already carries this warp's lane quarter in its upper half
-  if (EPI == TC_STORE) {
-#pragma unroll 1
-    for (int c = part * 32; c < BN; c += 32 * n_parts) {
-      int n = n0 + c;
-      int n_valid = p.N - n;
-      if (n_valid <= 0) break;           // uniform over the warp
-      float v[32];
-      tmem_ld32(tmem_acc + c, v);
-      tmem_ld_wait();
-      if (row_ok) store32_bf16(p.C + (size_t)m * p.ldc + n, v, n_valid);
-    }
-  } else if (EPI == TC_SWIGLU) {
+  if (EPI == TC_SWIGLU) {
     // every 128 columns of the tile: [0, 64) gate rows, [64, 128) the matching up rows
     const float rinv = (p.ss_in && row_ok) ? rsqrtf(p.ss_in[m] / (float)p.K + p.rms_eps) : 1.f;
 #pragma unroll 1
@@ -727,7 +716,6 @@ cudaError_t go_resid(const CUtensorMap& a, const CUtensorMap& a2, const CUtensor
 template <int BN>
 cudaError_t go_epi(int epi, const CUtensorMap& a, const CUtensorMap& a2, const CUtensorMap& w, const CUtensorMap& x, const Params& p, int grid, cudaStream_t st) {
   switch (epi) {
-    case TC_STORE: return go<TC_STORE, BN>(a, a2, w, x, p, grid, st);
     case TC_RESID: return go_resid<BN>(a, a2, w, x, p, grid, st);
     case TC_SWIGLU: return go<TC_SWIGLU, BN>(a, a2, w, x, p, grid, st);
     case TC_QKV: return go<TC_QKV, BN>(a, a2, w, x, p, grid, st);
@@ -783,7 +771,6 @@ bool tc_gemm_supported(const TcGemm& g) {
   if (g.K % 8 || g.lda % 8 || g.ldw % 8 || !al16(g.A) || !al16(g.W)) return false;
   if (g.A2 && (g.lda2 % 8 || !al16(g.A2))) return false;
   switch (g.epi) {
-    case TC_STORE: return g.N % 8 == 0 && g.ldc % 8 == 0 && al16(g.C);
     case TC_RESID:
       if (g.H && (g.N % 8 || g.ldh % 8 || !al16(g.H) || (g.H_lo && !al16(g.H_lo)) || !g.gain_next || !g.ss_out || g.A2)) return false;
       return g.N % 4 == 0 && g.ldx % 4 == 0 && al16(g.X);

@@ -3,7 +3,6 @@
 #include "common.cuh"
 
 enum TcEpi : int {
-  TC_STORE = 0,   // C[m, n] = bf16(acc)
   TC_RESID = 1,   // X[m, n] += acc (fp32 residual stream)
   TC_SWIGLU = 2,  // W rows interleaved (64 gate rows, 64 up rows); C[m, c] = bf16(silu(gate_c) * up_c) (+ remainder to C_lo)
   TC_QKV = 3,     // RoPE on columns < rot_cols, bf16 hi to C, bf16 lo of columns >= lo_col_begin to C_lo

@@ -323,12 +323,14 @@ bool mega_uses_mma(const kvp_handle* h, int batch) {
 }
 cudaError_t launch_mega(kvp_handle* h, const MegaParams& p, int k_max, int n_sm, cudaStream_t st) {
   if (mega_uses_mma(h, p.batch)) return launch_step_mega_mma(p, h->base.max_group, n_sm, st, &h->n_launch);
-  // The CUDA-core kernel gives a row to a warp, 16 warps to a CTA, and a launch that takes every SM keeps other calls off them: a model whose widest projection has fewer rows takes fewer CTAs, but no
-  // fewer than attention has items (key ranges of a sequence and kv head), which would then take several rounds.
-  // fp32 test pair, us by itself / among other calls, with 43 CTAs (rows / 16), 64, 96 and 148 (all of it with the kernel that still had
-  // grid-wide barriers; first token of 1 x 64 with 43 now 125 / 39): first token of 1 x 64 (4 items) 139 / 45,
-  // 139 / 55, 139 / 98, 141 / 99; step over 1 x 1000 keys (64 items) 188 / 55, 157 / 64, 158 / 124, 157 / 127; 4 x 300 (80) 224 / 67, 228 / 96,
-  // 196 / 161, 198 / 165; 1 x 4000 (252) 361 / 111, 320 / 142, 272 / 238, 225 / 193; 4 x 4000 (304) 545 / 178, 441 / 203, 394 / 356, 311 / 274.
+  // The CUDA-core kernel gives a row to a warp, 16 warps to a CTA, and a launch that takes every SM keeps other calls off them: a model
+  // whose widest projection has fewer rows takes fewer CTAs, but no fewer than attention has items (key ranges of a sequence and kv head),
+  // which would then take several rounds.  fp32 test pair, us by itself / among other calls, with 43 CTAs (rows / 16), 64, 96 and 148:
+  //   first token of 1 x 64 (4 items)    121 / 39, 121 / 40, 122 / 42, 121 / 63
+  //   step over 1 x 1000 keys (64 items) 161 / 48, 129 / 49, 128 / 80, 130 / 95
+  //   4 x 300 (80)                       192 / 59, 194 / 82, 169 / 108, 162 / 129
+  //   1 x 4000 (252)                     340 / 108, 295 / 131, 246 / 178, 201 / 162
+  //   4 x 4000 (304)                     593 / 197, 469 / 221, 414 / 328, 321 / 282
   const int rows = std::max(std::max(2 * h->base.max_ffn, h->base.max_nqkv), std::max(h->base.d, h->base.vocab));
   int ctas = std::max(16, (rows + 15) / 16);
   for (int i = p.layer_begin; i < p.layer_end; ++i) ctas = std::max(ctas, p.batch * p.layers[i].nkv * p.layers[i].n_split);
@@ -788,7 +790,8 @@ static kvp_status prefill_direct(kvp_handle* h, const int32_t* tokens, const int
   // ---- stage 1 + 2: auxiliary prefill, each layer's K/V pushed through the predictor ----
   // (only worth it while a layer's kernels leave SMs idle: with many tokens every kernel fills the GPU by itself)
   const bool fork = h->side != nullptr && !h->timing && T <= 4096;
-  // Pairs of CTAs need both of their SMs at once, which kernels on the other streams hold one by one (64 x 59 with pairs 1 % faster or not at all).
+  // Pairs of CTAs need both of their SMs at once, which kernels on the other streams hold one by one, and wait for each other without a limit:
+  // calls with streams of their own take single CTAs (pairs measured 1.2 and 1.9 % ahead on 64 x 59 and on 8 ragged prompts of the layer-pruned pair).
   h->gemm_pairs = !fork;
   bool pending_join = false;
   // The base step in pieces beside the prefill: piece j = the base layers whose cache (and that of every
@@ -821,7 +824,7 @@ static kvp_status prefill_direct(kvp_handle* h, const int32_t* tokens, const int
       mp.layers[i].n_split = std::max(1, std::min(mp.layers[i].n_split, piece_sms / (batch * h->base.L[i].nkv)));
   }
   // More than 4 sequences: the step is a chain of short per-layer kernels bound by launch latency; the same
-  // pieces go to the step stream as plain launches.  Their projections size their grids for step_tc_sms SMs;
+  // pieces go to the step stream as plain launches.  Their projections size their grids for step_tc_sms SMs (kvp_internal.h);
   // the prefill's GEMMs keep the whole GPU (measured: restricting them costs more than the step gains).
   const bool piped_tc = !one_kernel && fork && h->step_sms > 0 && h->step_tc_sms > 0 && step_uses_tc(h, batch);
   if (piped_tc) {

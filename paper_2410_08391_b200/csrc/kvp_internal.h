@@ -90,7 +90,11 @@ struct kvp_handle {
   int step_sms = 72;
   bool gemm_pairs = true;               // may pairs of CTAs take a GEMM's tiles
   int gemm_sms = 148;                   // SMs the tensor-core GEMMs of the current call size their grids for
-  int step_tc_sms = 96;                 // grid of the step's projections when its per-layer kernels (batch > 4) run beside the prefill
+  // SMs that the step's projections size their grids for when its per-layer kernels run beside the prefill: up to 192 CTAs (96 from 65
+  // sequences on), which the hardware spreads over all SMs.  First token, us among other calls / by itself, with 32, 48, 64, 96, 148: 64 x 59
+  // 3612 / 3838, 3618 / 3859, 3627 / 3801, 3654 / 3769, 3678 / 3781; layer-pruned 8 ragged 3814 / 4194, 3834 / 4068, 3822 / 4173, 3794 / 4066, 3865 / 4225; 3B
+  // shape 8 x 300 4575 / 5032, 4592 / 4899, 4621 / 4950, 4678 / 4870, 4716 / 4897; 96 x 40 3938 / 4521, 3904 / 4240, 3948 / 4152, 3975 / 4108, 4052 / 4099.
+  int step_tc_sms = 96;
   int step_terms = 2;                   // bf16 terms of an activation in the step's tensor-core projections
   int step_grid_sms = 148;              // SMs the step's tensor-core projections size their grids for
   // instrumentation

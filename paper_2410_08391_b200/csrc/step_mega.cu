@@ -578,7 +578,7 @@ __global__ void __launch_bounds__(NT, 1) step_mega_kernel(const __grid_constant_
     }
     // ---- attention over the cache.  With split key ranges the CTA that finishes the last split of a
     // (sequence, kv head) merges that group's partial results on the spot (a counter per group tells
-    // it so), which saves a separate merge phase and its grid barrier.
+    // it so), which saves a merge phase of its own.
     {
       const int n_split = L.n_split, n_items = batch * L.nkv * n_split;
       const int group = L.nq / L.nkv, ldr = p.hd + 2;
