@@ -34,8 +34,9 @@ template <int HD> struct MmaCfg {
   static constexpr int PAGE_BYTES = PAGE_TOKENS * HD * 2;
   static constexpr int STAGES = HD == 64 ? 5 : 3;          // most stages: two CTAs per SM
   static constexpr int PER_SM = HD == 64 ? 4 : 2;          // most CTAs per SM (registers)
-  // after the ring: q [8][HD] fp32, then the warps' partial results [NW][8][HD + 2] fp32 (reuses the ring when it is idle)
-  static constexpr int smem(int stages) { return 1024 + stages * 2 * PAGE_BYTES + 8 * HD * 4 + 256; }
+  static constexpr int LDQ = HD + 8;                       // floats from head to head of the staged queries: no two heads' pieces in the same banks
+  // after the ring: q [8][LDQ] fp32, then the warps' partial results [NW][8][HD + 2] fp32 (reuses the ring when it is idle)
+  static constexpr int smem(int stages) { return 1024 + stages * 2 * PAGE_BYTES + 8 * LDQ * 4 + 256; }
 };
 // Ring stages of a launch whose CTAs walk `per_pages` pages, and how many of its CTAs an SM holds.  A short range needs no deep ring:
 // with 2 or 3 stages four CTAs of head_dim 64 share an SM instead of two, and their set-up and merge overlap (64 x 59 keys: 512 CTAs
@@ -102,13 +103,13 @@ __global__ void __launch_bounds__(NT, MmaCfg<HD>::PER_SM)
 step_attn_mma_kernel(const __grid_constant__ CUtensorMap map_k, const __grid_constant__ CUtensorMap map_v,
                      const __grid_constant__ InvFreq inv, const MmaParams p) {
   using Cfg = MmaCfg<HD>;
-  constexpr int PB = Cfg::PAGE_BYTES, KS = HD / 16, NTL = HD / 8;
+  constexpr int PB = Cfg::PAGE_BYTES, LDQ = Cfg::LDQ, KS = HD / 16, NTL = HD / 8;
   extern __shared__ uint8_t sm_raw[];
   uint8_t* smem = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(sm_raw) + 1023) & ~uintptr_t(1023));
   const uint32_t ring = smem_u32(smem);
   const int STG = p.stages;
-  float* qs = reinterpret_cast<float*>(smem + STG * 2 * PB);                     // [8][HD], scaled, after RoPE
-  uint64_t* bars = reinterpret_cast<uint64_t*>(smem + STG * 2 * PB + 8 * HD * 4);   // full[STG], empty[STG]
+  float* qs = reinterpret_cast<float*>(smem + STG * 2 * PB);                     // [8][LDQ], scaled, after RoPE
+  uint64_t* bars = reinterpret_cast<uint64_t*>(smem + STG * 2 * PB + 8 * LDQ * 4);   // full[STG], empty[STG]
   __shared__ int s_abort_mem;
   __shared__ float rq[8];
   __shared__ float rk;
@@ -198,8 +199,8 @@ step_attn_mma_kernel(const __grid_constant__ CUtensorMap map_k, const __grid_con
         r1 = (x1 * cs.x - x2 * cs.y) * scale;
         r2 = (x2 * cs.x + x1 * cs.y) * scale;
       }
-      qs[h * HD + c] = r1;
-      qs[h * HD + c + half] = r2;
+      qs[h * LDQ + c] = r1;
+      qs[h * LDQ + c + half] = r2;
     }
     if (has_new)
       for (int c = tid; c < half; c += NT) {
@@ -234,7 +235,7 @@ step_attn_mma_kernel(const __grid_constant__ CUtensorMap map_k, const __grid_con
     float mx = 0.f;
 #pragma unroll
     for (int i = 0; i < 2 * KS; ++i) {
-      qv[i] = *reinterpret_cast<const float2*>(qs + g * HD + i * 8 + 2 * qd);
+      qv[i] = *reinterpret_cast<const float2*>(qs + g * LDQ + i * 8 + 2 * qd);
       mx = fmaxf(mx, fmaxf(fabsf(qv[i].x), fabsf(qv[i].y)));
     }
     mx = fmaxf(mx, __shfl_xor_sync(0xffffffffu, mx, 1));
@@ -275,6 +276,7 @@ step_attn_mma_kernel(const __grid_constant__ CUtensorMap map_k, const __grid_con
         if (warp * 16 + 16 > nk) {
           // Rows at or beyond the sequence's end may hold anything, and 0 x NaN is NaN: the values of this warp's 16 become zero in the CTA's
           // copy.  (Their scores are never looked at.  Only a sequence's last page has such rows, and no copy into its stage follows.)
+#pragma unroll 1
           for (int i = lane; i < (warp * 16 + 16 - nk) * (HD / 8); i += 32)
             asm volatile("st.shared.v4.b32 [%0], {%1, %1, %1, %1};" ::"r"(sv + piece(nk + i / (HD / 8), i % (HD / 8))), "r"(0u) : "memory");
           __syncwarp();
