@@ -108,7 +108,8 @@ typedef struct {
  *                          stream outgrows 32 MB (calls of some five thousand tokens and
  *                          more), RMSNorm is folded into the GEMMs around it: the residual GEMM that completes x also
  *                          writes x * gain as the next GEMM's 16-bit operand and the rows' sums of squares, the next GEMM
- *                          scales its rows by 1 / rms. */
+ *                          scales its rows by 1 / rms.  (KVP_F32 mode: no effect, the prefill's products normalise the rows
+ *                          that they read.) */
 enum { KVP_OPT_FUSED_KV_PRED = 1, KVP_OPT_SEPARATE_NORM = 2 };
 
 /* A named tensor handed to kvp_load_weights().  Names:
