@@ -345,8 +345,8 @@ cudaError_t launch_mega(kvp_handle* h, const MegaParams& p, int k_max, int n_sm,
 // and on average 68 MB there; nothing was measured between them and pairs of test size, where launches count: the line at 30 MB is set, not found.
 // A caller that waits is served by the persistent kernel: from host memory to host memory scaled 3 x 100 1394 / 1461; but 1.1B 3 x 40 1444 / 1395,
 // 4 x 300 2075 / 1950, 3 x 1000 3280 / 3208, layer-pruned 4 x 300 2756 / 2686, 3B 3 x 60 3277 / 2578, 4 x 300 4034 / 3707, so a finer line would pay there.
-// One and two sequences stay with the persistent kernel: it is the more exact one for them (3B shape 1 x 300 1.30e-6 of 64 bits, the chain
-// 1.46e-6), though the chain is served sooner on the 3B pair (2336 / 2065).  Generation stays with it too, which serves one call sooner.
+// One and two sequences stay with the persistent kernel: it is the more exact one for them (distance from 64 bits, rms of 12
+// prompts on the 3B shape, persistent / chain: 1 x 300 1.37e-6 / 1.55e-6, 2 x 300 1.55e-6 / 1.59e-6), though the chain is served sooner there (1 x 300 2336 / 2065).  Generation stays with it too, which serves one call sooner.
 bool first_step_prefers_chain(const kvp_handle* h, int batch, bool blocking) {
   if (batch <= 2 || batch > 4 || blocking || !mega_uses_mma(h, batch) || !step_uses_tc(h, batch) || !step_stream_fits(h)) return false;
   double mb = 0;        // weights of a layer
